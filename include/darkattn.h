@@ -54,8 +54,10 @@ typedef enum { DARKATTN_F32 = 0, DARKATTN_BF16 = 1 } darkattn_dtype_t;
 
 /* Which kernels carry the work.
  *   AUTO   : F32 -> SIMT; BF16 -> TENSOR where the shape is covered, else SIMT.
- *   SIMT   : FP32 FFMA kernels with FP32 accumulation (any shape; the only path that meets the
- *            1e-4 tolerance, because TF32/BF16 operands round the exponent's argument).
+ *   SIMT   : FP32 operands and FP32 accumulation (any shape; the only path that meets the 1e-4
+ *            tolerance, because a single TF32/BF16 operand rounds the exponent's argument). Its
+ *            products run on the tensor cores with every FP32 operand split exactly into three BF16
+ *            parts, everything else on the FP32 pipes.
  *   TENSOR : tcgen05 / TMEM / TMA kernels, BF16 operands, FP32 accumulation (BF16 dtype only;
  *            DARKATTN_ERR_UNSUPPORTED at plan time if the shape is not covered).               */
 typedef enum { DARKATTN_PATH_AUTO = 0, DARKATTN_PATH_SIMT = 1, DARKATTN_PATH_TENSOR = 2 } darkattn_path_t;
@@ -192,7 +194,7 @@ darkattn_status_t darkattn_selftest_wait_limit(int32_t *device_status, double *s
  *    device; cudaDeviceReset invalidates it (the library is not meant to outlive a reset).
  *  - No cudaMalloc, cudaFree or other allocating routine is called by the library, now or later.
  *  - The status word of this call lives in the library's own array, out of reach of
- *    darkattn_last_device_status: the FP32 kernels it runs never write one.
+ *    darkattn_last_device_status.
  *  - All calls on a device share the one array, and it keeps the previous call's contents; the call
  *    clears the words that must start at zero itself. Two calls whose GPU work overlaps (different
  *    streams, or different host threads) race on the array: serialise them on one stream.         */

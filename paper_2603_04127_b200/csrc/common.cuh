@@ -25,30 +25,30 @@ struct Dims {
     float s;         // sqrt(scale), applied to Mq and to Mk
 };
 
-// Offsets (bytes) into the caller's workspace of the SIMT path's intermediates.
+// Offsets (bytes) into the caller's workspace of the FP32 path's intermediates (all fp32).
 struct SimtLayout {
     size_t status;                 // device status word (first 256 bytes)
-    size_t Qf, Kf, Vf, Mf, Wf, Gf; // fp32 copies of bf16 inputs (unused for f32 storage)
     size_t xtQ, xtK;               // x~            [BH, N, r]
-    size_t nQ, nK;                 // |x~|^2 / 2    [BH, N]
-    size_t fQ, fK;                 // exponents, then features  [BH, Npad, m]
-    size_t cK;                     // per-feature key shift     [BH, m]
-    size_t Va;                     // [V | 1]       [BH, Npad, dva]
-    size_t Sloc;                   // chunk states, then exclusive prefixes [BH, nc, m, dva]
+    size_t nK;                     // sums of squares of x~_K's rows, one per 128 columns  [ceil(r/128), BH, N]
+    size_t fQ, fK;                 // exponents, then features  [BH, N, m]
+    size_t cK;                     // per-feature key shift, order keys  [BH, m]
+    size_t Sloc, zloc;             // causal: state of every chunk, then before it; else of every token block, the first then holds the sum
+                                   // [BH, nb, m, dv], [BH, nb, m]
     size_t P;                      // masked intra-chunk kernel  [BH, nc, C, C]   (causal)
-    size_t num;                    // numerators and normaliser  [BH, Npad, dva]
     // backward only
-    size_t Ga;                     // [dO/den | -delta/den]      [BH, Npad, dva]
+    size_t Ga;                     // dO / den      [BH, N, dv]
+    size_t gd;                     // -(dO . O) / den, one part per 128 columns  [ceil(dv/128), BH, N]
     size_t dP;                     // [BH, nc, C, C]             (causal)
-    size_t Rloc;                   // reverse states             [BH, nc, m, dva]
-    size_t dA, dBf;                // feature gradients, then E  [BH, Npad, m]
-    size_t dVa;                    // [BH, Npad, dva]
-    size_t esQ, esK;               // rowsum(E)                  [BH, N]
+    size_t Rloc, rloc;             // reverse states, as Sloc and zloc
+    size_t dA, dBf;                // E = feature gradients times features  [BH, N, m]
+    size_t esK;                    // rowsum(E_K), one part per 128 columns  [ceil(m/128), BH, N]
     size_t dxtQ, dxtK;             // dx~                        [BH, N, r]
-    size_t dXf;                    // fp32 dX before the cast    [BH, N, d]
-    size_t dMp;                    // per-(b,h) dM               [BH, r, d]
-    size_t dWp;                    // per-(b,h) dW               [BH, m, r]
+    size_t dKh, dVh;               // grouped key/value heads: dK and dV per query head  [BH, N, d], [BH, N, dv]
+    size_t dMp;                    // dM per (b,h) and token block  [BH, nsM, r, d]
+    size_t dWp;                    // dW per (b,h) and token block  [BH, nsW, m, r]
     size_t fwd_bytes, total_bytes;
+    int C, nb, blk;                // tokens per chunk (causal) or block, blocks per (b,h)
+    int nsM, nsW, blkM, blkW;      // token blocks of the dM and dW products, tokens in each
 };
 
 // Offsets (bytes) into the workspace of the tensor-core forward path.
@@ -168,11 +168,10 @@ inline cudaError_t ensure_aux(const darkattn_plan_s *plan)
 // Records an event in front of the kernel `name` (nullptr: after the last kernel of a call) when timing is on.
 void timer_mark(const darkattn_plan_s *plan, cudaStream_t st, const char *name);
 
-// SIMT (FP32 FFMA) path
+// FP32 path (products of split operands on the tensor cores)
 void simt_make_layout(darkattn_plan_s *plan);
 darkattn_status_t simt_forward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
-                               const void *M, const void *W, void *O, char *ws, cudaStream_t st,
-                               bool keep_for_backward);
+                               const void *M, const void *W, void *O, char *ws, cudaStream_t st);
 darkattn_status_t simt_backward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
                                 const void *M, const void *W, const void *dO, void *dQ, void *dK,
                                 void *dV, float *dM, char *ws, cudaStream_t st);

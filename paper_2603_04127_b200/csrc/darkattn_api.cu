@@ -76,9 +76,9 @@ darkattn_status_t darkattn_plan(const darkattn_desc_t *desc, darkattn_plan_t *ou
     p->workspace_bytes = p->simt.total_bytes;
     p->saved_bytes = 0;
     {
-        const int stage = (D.bf16 ? 5 : 0) + 4 + 6 + (D.causal ? 5 : 2);
-        p->launches_fwd = stage + 1;
-        p->launches_bwd = stage + (D.bf16 ? 1 : 0) + 1 + (D.causal ? 9 : 4) + 1 + 2 * 6 + 1;
+        const int scan = (D.causal || p->simt.nb > 1) ? 1 : 0;
+        p->launches_fwd = 5 + scan;
+        p->launches_bwd = 5 + scan + 1 + scan + 4 + (D.G > 1 ? 2 : 0);
     }
     if (path == DARKATTN_PATH_TENSOR) tensor_make_layout(p);
     *out = p;
@@ -98,13 +98,13 @@ darkattn_status_t darkattn_forward(darkattn_plan_t plan, const void *Q, const vo
     if (plan->workspace_bytes && !workspace) return DARKATTN_ERR_WORKSPACE;
     if (!aligned16(workspace) || !aligned16(saved)) return DARKATTN_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    DARKATTN_CUDA_TRY(cudaMemsetAsync(workspace, 0, 256, st), "forward: clear status word");
     darkattn_status_t rc;
     if (plan->path == DARKATTN_PATH_TENSOR) {
+        DARKATTN_CUDA_TRY(cudaMemsetAsync(workspace, 0, 256, st), "forward: clear status word");
         rc = tensor_forward(plan, Q, K, V, M, W, O, saved, static_cast<char *>(workspace), st, saved != nullptr);
     } else {
         timer_mark(plan, st, "simt_forward (all kernels)");
-        rc = simt_forward(plan, Q, K, V, M, W, O, static_cast<char *>(workspace), st, false);
+        rc = simt_forward(plan, Q, K, V, M, W, O, static_cast<char *>(workspace), st);
     }
     timer_mark(plan, st, nullptr);
     return rc;
@@ -122,9 +122,9 @@ darkattn_status_t darkattn_backward(darkattn_plan_t plan, const void *Q, const v
     if (plan->workspace_bytes && !workspace) return DARKATTN_ERR_WORKSPACE;
     if (!aligned16(workspace) || !aligned16(saved) || !aligned16(O)) return DARKATTN_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    DARKATTN_CUDA_TRY(cudaMemsetAsync(workspace, 0, 256, st), "backward: clear status word");
     darkattn_status_t rc;
     if (plan->path == DARKATTN_PATH_TENSOR) {
+        DARKATTN_CUDA_TRY(cudaMemsetAsync(workspace, 0, 256, st), "backward: clear status word");
         rc = tensor_backward(plan, Q, K, V, M, W, O, dO, saved, dQ, dK, dV, dM, static_cast<char *>(workspace), st);
     } else {
         timer_mark(plan, st, "simt_backward (all kernels)");

@@ -1,429 +1,337 @@
-// FP32 path of libdarkattn: every step of DARK attention as FP32 FFMA kernels with FP32 accumulation.
+// FP32 path of libdarkattn: every step of DARK attention with fp32 operands and fp32 accumulation.
 //
-// This is the path that meets the 1e-4 tolerance (tensor-core operand types round the argument of
-// the exponential too coarsely), and the path that accepts any shape. It is built from one strided
-// batched GEMM kernel plus small row-wise kernels, and keeps its intermediates in the workspace.
+// This is the path that meets the 1e-4 tolerance (a single bf16 or TF32 operand rounds the argument of the exponential
+// too coarsely), and the path that accepts any shape. Its products run on the tensor cores with every fp32 operand split
+// into three bf16 numbers (split_gemm.cu); what surrounds them is done on the way into or out of a product, so that the
+// intermediates are written once and read by the next product:
+//   forward    x~ = s X M^T (both sides; row norms of the keys) | u = x~ W^T (keys: minus the norm; column maxima) |
+//              features in place | chunk states and masked kernel tiles | prefix over the chunks | output rows
+//   backward   the forward steps with the output rows turned into dO / den and -delta / den | dP and the reverse states |
+//              suffix over the chunks | E of both sides and dV | dx~ | dQ, dK and dM | sums over batch and token blocks
+// Each line's items between bars are one launch each; all but the first start while the one before drains
+// (programmatic dependent launch).
 //
 // Stabiliser (cancels in O): keys use one shift per (batch, head, feature), c_l = max_j (u_jl - n_j),
 // queries use e_il = u_il + c_l - max_l(u_il + c_l); the query's own norm term is a per-row constant
-// and is dropped. The product phi(q_i)_l phi(k_j)_l is then the unshifted one times a per-row factor.
+// and is dropped (so is its gradient, which is zero). The product phi(q_i)_l phi(k_j)_l is then the unshifted one times
+// a per-row factor.
 #include "common.cuh"
+#include "split_gemm.cuh"
+#include "tc_common.cuh"
 
 #include <math.h>
 
 namespace darkattn {
 
+using sg::launch_pdl;
+
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16;
-
-struct GemmP {
-    const float *A, *B;
-    float *C;
-    int M, N, K;
-    long long sAm, sAk, sBk, sBn, sCm, sCn;   // element strides
-    int nb1;                                  // batch index z = z0 * nb1 + z1
-    long long A0, A1, B0, B1, C0, C1;         // batch strides for z0, z1
-    float alpha;
-    int accumulate;                           // C += instead of C =
-    int mask;                                 // 0 none; 1 keep col <= row (others written as 0)
-    int tilesM, tilesN;
-};
-
-// C[z] (+)= alpha * A[z] * B[z], A is M x K, B is K x N, all with arbitrary element strides.
-__global__ void __launch_bounds__(256) gemm_kernel(GemmP p)
+// Features in place, one warp per row: query rows exp(u_l + c_l - max_l(u_l + c_l)), key rows exp(u_l - c_l) (u already
+// has the key's norm taken off). V: elements per load. A row is read twice (the second time from L1 or L2).
+template <int V>
+__global__ void __launch_bounds__(256) features_kernel(float *fQ, float *fK, const int *cK, int N, int m, long long rows)
 {
-    __shared__ float As[BK][BM + 4];
-    __shared__ float Bs[BK][BN + 4];
-    const int tiles = p.tilesM * p.tilesN;
-    const long long z = blockIdx.x / tiles;
-    const int t = blockIdx.x % tiles;
-    const int m0 = (t / p.tilesN) * BM, n0 = (t % p.tilesN) * BN;
-    const long long z0 = z / p.nb1, z1 = z % p.nb1;
-    const float *A = p.A + z0 * p.A0 + z1 * p.A1;
-    const float *B = p.B + z0 * p.B0 + z1 * p.B1;
-    float *C = p.C + z0 * p.C0 + z1 * p.C1;
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    float acc[4][4];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    const long long w = (blockIdx.x * 256LL + threadIdx.x) / 32;
+    const int lane = threadIdx.x & 31;
+    if (w >= 2 * rows) return;
+    const bool keys = w >= rows;
+    const long long row = keys ? w - rows : w;
+    float *f = (keys ? fK : fQ) + row * m;
+    const int *c = cK + row / N * m;
+    float mx = 0.f;
+    auto load = [&](int l, float (&x)[V], float (&s)[V]) {
+        if constexpr (V == 4) {
+            const float4 a = *reinterpret_cast<const float4 *>(f + l);
+            const int4 k = __ldg(reinterpret_cast<const int4 *>(c + l));
+            x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
+            s[0] = tc::float_from_order_key(k.x); s[1] = tc::float_from_order_key(k.y); s[2] = tc::float_from_order_key(k.z); s[3] = tc::float_from_order_key(k.w);
+        } else { x[0] = f[l]; s[0] = tc::float_from_order_key(__ldg(c + l)); }
+    };
+    if (!keys) {
+        mx = -INFINITY;
+        for (int l = lane * V; l < m; l += 32 * V) {
+            float x[V], s[V];
+            load(l, x, s);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-
-    const bool dead = (p.mask == 1 && n0 > m0 + BM - 1);   // tile entirely above the diagonal
-    if (!dead) {
-        for (int k0 = 0; k0 < p.K; k0 += BK) {
-            if (p.sAk == 1) {
-                const int row = tid / 4, kk = (tid % 4) * 4;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int k = k0 + kk + i;
-                    As[kk + i][row] = (m0 + row < p.M && k < p.K) ? A[(long long)(m0 + row) * p.sAm + k] : 0.f;
-                }
-            } else {
-                const int kk = tid / 16, mm = (tid % 16) * 4;
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    As[kk][mm + i] = (m0 + mm + i < p.M && k0 + kk < p.K)
-                                         ? A[(long long)(m0 + mm + i) * p.sAm + (long long)(k0 + kk) * p.sAk] : 0.f;
-            }
-            if (p.sBk == 1) {
-                const int col = tid / 4, kk = (tid % 4) * 4;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int k = k0 + kk + i;
-                    Bs[kk + i][col] = (n0 + col < p.N && k < p.K) ? B[(long long)(n0 + col) * p.sBn + k] : 0.f;
-                }
-            } else {
-                const int kk = tid / 16, nn = (tid % 16) * 4;
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    Bs[kk][nn + i] = (n0 + nn + i < p.N && k0 + kk < p.K)
-                                         ? B[(long long)(k0 + kk) * p.sBk + (long long)(n0 + nn + i) * p.sBn] : 0.f;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int kk = 0; kk < BK; ++kk) {
-                float a[4], b[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-            }
-            __syncthreads();
+            for (int j = 0; j < V; ++j) mx = fmaxf(mx, x[j] + s[j]);
         }
+        for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     }
+    for (int l = lane * V; l < m; l += 32 * V) {
+        float x[V], s[V];
+        load(l, x, s);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int row = m0 + ty * 4 + i;
-        if (row >= p.M) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int col = n0 + tx * 4 + j;
-            if (col >= p.N) continue;
-            float v = p.alpha * acc[i][j];
-            if (p.mask == 1 && col > row) v = 0.f;
-            float *dst = C + (long long)row * p.sCm + (long long)col * p.sCn;
-            *dst = p.accumulate ? (*dst + v) : v;
-        }
+        for (int j = 0; j < V; ++j) x[j] = expf(keys ? x[j] - s[j] : x[j] + s[j] - mx);
+        if constexpr (V == 4) *reinterpret_cast<float4 *>(f + l) = make_float4(x[0], x[1], x[2], x[3]);
+        else f[l] = x[0];
     }
 }
 
-__global__ void cast_bf16_f32_kernel(const __nv_bfloat16 *in, float *out, long long n)
+// Over the token blocks of S[pair, block, e] and z[pair, block, l], in place: what came before each block (forward) or
+// comes after it (reverse), or the sum over all of them into the first. One thread per V neighbouring elements; eight
+// blocks' loads are in flight at a time (the sum is a serial chain, the loads are not).
+enum { SCAN_FORWARD = 0, SCAN_REVERSE = 1, SCAN_TOTAL = 2 };
+template <int V>
+__global__ void __launch_bounds__(256) chunk_scan_kernel(float *S, float *z, int nb, long long E, int m, long long pairs, int mode)
 {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        out[i] = __bfloat162float(in[i]);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    long long i = (blockIdx.x * 256LL + threadIdx.x) * V;
+    float *base;
+    long long step;
+    if (i < pairs * E) { base = S + i / E * nb * E + i % E; step = E; }
+    else {
+        i -= pairs * E;
+        if (i >= pairs * m) return;
+        base = z + i / m * nb * m + i % m;
+        step = m;
+    }
+    float run[V];
+#pragma unroll
+    for (int j = 0; j < V; ++j) run[j] = 0.f;
+    for (int k0 = 0; k0 < nb; k0 += 8) {
+        float x[8][V];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int c = mode == SCAN_REVERSE ? nb - 1 - (k0 + k) : k0 + k;
+            if (k0 + k < nb) {
+                if constexpr (V == 4) { const float4 a = *reinterpret_cast<const float4 *>(base + c * step); x[k][0] = a.x; x[k][1] = a.y; x[k][2] = a.z; x[k][3] = a.w; }
+                else x[k][0] = base[c * step];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (k0 + k >= nb) break;
+            const int c = mode == SCAN_REVERSE ? nb - 1 - (k0 + k) : k0 + k;
+            if (mode != SCAN_TOTAL) {
+                if constexpr (V == 4) *reinterpret_cast<float4 *>(base + c * step) = make_float4(run[0], run[1], run[2], run[3]);
+                else base[c * step] = run[0];
+            }
+#pragma unroll
+            for (int j = 0; j < V; ++j) run[j] += x[k][j];
+        }
+    }
+    if (mode == SCAN_TOTAL) {
+        if constexpr (V == 4) *reinterpret_cast<float4 *>(base) = make_float4(run[0], run[1], run[2], run[3]);
+        else base[0] = run[0];
+    }
 }
 
-__global__ void fill_kernel(float *p, float v, long long n)
+// out[o, e] = sum of src over `n1` outer and `n2` inner slices: src[(i1 * stride1 + o) * n2 + i2, e]. dM sums over the batch
+// and the token blocks (o = head), dW also over the heads where they share W (o = 0).
+__global__ void __launch_bounds__(256) reduce_kernel(const float *src, float *out, int n1, long long stride1, int n2, long long E, long long total)
 {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) p[i] = v;
-}
-
-// n[row] = 0.5 * |xt[row,:]|^2, one warp per row.
-__global__ void half_sqnorm_kernel(const float *xt, float *n, long long rows, int r)
-{
-    const long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32;
-    const int lane = threadIdx.x % 32;
-    if (row >= rows) return;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const long long t = blockIdx.x * 256LL + threadIdx.x;
+    if (t >= total) return;
+    const long long o = t / E, e = t % E;
     float acc = 0.f;
-    for (int a = lane; a < r; a += 32) { const float v = xt[row * r + a]; acc = fmaf(v, v, acc); }
-    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) n[row] = 0.5f * acc;
-}
-
-__device__ __forceinline__ void atomic_max_float(float *addr, float v)
-{
-    if (v >= 0.f) atomicMax(reinterpret_cast<int *>(addr), __float_as_int(v));
-    else atomicMin(reinterpret_cast<unsigned int *>(addr), __float_as_uint(v));
-}
-
-// cK[bh,l] = max_j (u[bh,j,l] - n[bh,j]); block = (rows block of 128, bh); thread per column.
-__global__ void key_colmax_kernel(const float *u, const float *n, float *cK, int N, int Npad, int m)
-{
-    const int bh = blockIdx.y;
-    const int j0 = blockIdx.x * 128, j1 = min(N, j0 + 128);
-    for (int l = threadIdx.x; l < m; l += blockDim.x) {
-        float mx = -INFINITY;
-        for (int j = j0; j < j1; ++j) mx = fmaxf(mx, u[((long long)bh * Npad + j) * m + l] - n[(long long)bh * N + j]);
-        if (j1 > j0) atomic_max_float(&cK[(long long)bh * m + l], mx);
+    for (int i1 = 0; i1 < n1; ++i1) {
+        const float *p = src + (i1 * stride1 + o) * n2 * E + e;
+#pragma unroll 8
+        for (int i2 = 0; i2 < n2; ++i2) acc += p[i2 * E];
     }
+    out[t] = acc;
 }
 
-// f[bh,j,l] = exp(u - n_j - cK_l) for j < N, 0 for padding rows.
-__global__ void key_features_kernel(float *f, const float *n, const float *cK, int N, int Npad, int m, long long total)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const int l = (int)(i % m);
-        const long long row = i / m;
-        const int j = (int)(row % Npad);
-        const long long bh = row / Npad;
-        f[i] = (j < N) ? expf(f[i] - n[bh * N + j] - cK[bh * m + l]) : 0.f;
-    }
-}
-
-// f[bh,i,l] = exp(u + cK_l - max_l(u + cK_l)) for i < N, 0 for padding rows; one warp per row.
-__global__ void query_features_kernel(float *f, const float *cK, int N, int Npad, int m, long long rows)
-{
-    const long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32;
-    const int lane = threadIdx.x % 32;
-    if (row >= rows) return;
-    const int i = (int)(row % Npad);
-    const long long bh = row / Npad;
-    float *fr = f + row * m;
-    if (i >= N) { for (int l = lane; l < m; l += 32) fr[l] = 0.f; return; }
-    const float *c = cK + bh * m;
-    float mx = -INFINITY;
-    for (int l = lane; l < m; l += 32) mx = fmaxf(mx, fr[l] + c[l]);
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    for (int l = lane; l < m; l += 32) fr[l] = expf(fr[l] + c[l] - mx);
-}
-
-// Va[bh,j,:] = [V_j | 1] for j < N, 0 for padding rows.
-__global__ void augment_values_kernel(const float *V, float *Va, int N, int Npad, int dv, long long total)
-{
-    const int dva = dv + 1;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i % dva);
-        const long long row = i / dva;
-        const int j = (int)(row % Npad);
-        const long long bh = row / Npad;
-        Va[i] = (j >= N) ? 0.f : (c < dv ? V[(bh * N + j) * dv + c] : 1.f);
-    }
-}
-
-// In-place exclusive scan over the chunk index of S[bh, c, e] (forward or reverse order).
-__global__ void chunk_scan_kernel(float *S, int nc, long long E, long long total, int reverse)
-{
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= total) return;
-    const long long bh = i / E, e = i % E;
-    float *base = S + bh * nc * E + e;
-    float run = 0.f;
-    for (int k = 0; k < nc; ++k) {
-        const int c = reverse ? nc - 1 - k : k;
-        const float v = base[(long long)c * E];
-        base[(long long)c * E] = run;
-        run += v;
-    }
-}
-
-// out[bh,i,c] = src[bh,i,c] (/ src[bh,i,div_col]) for i < N, c < w, cast to the storage type.
-template <typename T>
-__global__ void emit_rows_kernel(T *out, const float *src, int N, int w, long long src_batch, int src_row,
-                                 int div_col, long long total)
-{
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(t % w);
-        const long long row = t / w;
-        const int i = (int)(row % N);
-        const long long bh = row / N;
-        const float *s = src + bh * src_batch + (long long)i * src_row;
-        float v = s[c];
-        if (div_col >= 0) v = v / s[div_col];
-        if constexpr (sizeof(T) == 2) out[t] = __float2bfloat16_rn(v);
-        else out[t] = v;
-    }
-}
-
-// Grouped key/value heads. out[(b,hk),i,c] = sum_g src[(b, hk G + g),i,c]: the gradient of a shared key or value row
+// Grouped key/value heads: out[(b,hk), e] = sum_g src[(b, hk G + g), e]: the gradient of a shared key or value row
 // collects the parts of the G query heads that read it.
 template <typename T>
-__global__ void emit_grouped_kernel(T *out, const float *src, int N, int w, long long src_batch, int src_row, int H, int Hkv,
-                                    long long total)
+__global__ void __launch_bounds__(256) group_sum_f32_kernel(T *out, const float *src, int G, long long E, long long total)
 {
-    const int G = H / Hkv;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(t % w);
-        const long long row = t / w;
-        const int i = (int)(row % N);
-        const long long bhk = row / N, b = bhk / Hkv, hk = bhk % Hkv;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (long long t = blockIdx.x * 256LL + threadIdx.x; t < total; t += gridDim.x * 256LL) {
+        const long long kv = t / E, e = t % E;
         float v = 0.f;
-        for (int g = 0; g < G; ++g) v += src[(b * H + hk * G + g) * src_batch + (long long)i * src_row + c];
+        for (int g = 0; g < G; ++g) v += src[(kv * G + g) * E + e];
         if constexpr (sizeof(T) == 2) out[t] = __float2bfloat16_rn(v);
         else out[t] = v;
     }
 }
 
-// out[(b,h),i,c] = in[(b, h / G),i,c] as fp32: every query head gets its own copy of the key/value head it reads.
-template <typename T>
-__global__ void expand_kv_kernel(const T *in, float *out, long long per_head, int H, int Hkv, long long total)
-{
-    const int G = H / Hkv;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
-        const long long bh = t / per_head, e = t % per_head, b = bh / H, h = bh % H;
-        const T x = in[(b * Hkv + h / G) * per_head + e];
-        if constexpr (sizeof(T) == 2) out[t] = __bfloat162float(x);
-        else out[t] = x;
-    }
-}
-
-// Ga[bh,i,:] = [G_i / den_i | -(G_i . O_i) / den_i], O_i = num_i / den_i; one warp per row.
-__global__ void grad_aug_kernel(const float *G, const float *num, float *Ga, int N, int Npad, int dv, long long rows)
-{
-    const long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32;
-    const int lane = threadIdx.x % 32;
-    if (row >= rows) return;
-    const int dva = dv + 1;
-    const int i = (int)(row % Npad);
-    const long long bh = row / Npad;
-    float *g = Ga + row * dva;
-    if (i >= N) { for (int c = lane; c < dva; c += 32) g[c] = 0.f; return; }
-    const float *nr = num + row * dva;
-    const float *Gr = G + (bh * N + i) * dv;
-    const float inv = 1.f / nr[dv];
-    float delta = 0.f;
-    for (int c = lane; c < dv; c += 32) { const float gv = Gr[c]; g[c] = gv * inv; delta = fmaf(gv, nr[c] * inv, delta); }
-    for (int o = 16; o; o >>= 1) delta += __shfl_xor_sync(0xffffffffu, delta, o);
-    if (lane == 0) g[dv] = -delta * inv;
-}
-
-// E = dphi .* phi in place (into dphi); es[bh,i] = sum_l E_il for i < N; one warp per row.
-__global__ void feature_grad_kernel(float *dphi, const float *phi, float *es, int N, int Npad, int m, long long rows)
-{
-    const long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32;
-    const int lane = threadIdx.x % 32;
-    if (row >= rows) return;
-    const int i = (int)(row % Npad);
-    const long long bh = row / Npad;
-    float acc = 0.f;
-    for (int l = lane; l < m; l += 32) { const float e = dphi[row * m + l] * phi[row * m + l]; dphi[row * m + l] = e; acc += e; }
-    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0 && i < N) es[bh * N + i] = acc;
-}
-
-// dxt[row,a] -= es[row] * xt[row,a]
-__global__ void norm_term_kernel(float *dxt, const float *xt, const float *es, int r, long long total)
-{
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x)
-        dxt[t] = fmaf(-es[t / r], xt[t], dxt[t]);
-}
-
-// dM[h,:] = sum_b dMp[b,h,:]
-__global__ void reduce_batch_kernel(const float *dMp, float *dM, int B, long long per_b, long long total)
-{
-    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (t >= total) return;
-    float acc = 0.f;
-    for (int b = 0; b < B; ++b) acc += dMp[b * per_b + t];
-    dM[t] = acc;
-}
-
-struct Launcher {
+struct Runner {
+    const darkattn_plan_s *plan;
+    char *ws;
     cudaStream_t st;
-    int count = 0;
+    bool dependent = false;         // a kernel of this call has been launched
     cudaError_t err = cudaSuccess;
-    void check() { cudaError_t e = cudaGetLastError(); if (e != cudaSuccess && err == cudaSuccess) err = e; ++count; }
-    static int blocks(long long n, int per) { long long b = (n + per - 1) / per; return (int)(b < 1 ? 1 : (b > 148LL * 64 ? 148LL * 64 : b)); }
 
-    void gemm(const float *A, const float *B, float *C, int M, int N, int K, long long sAm, long long sAk,
-              long long sBk, long long sBn, long long sCm, long long sCn, long long nbatch, int nb1,
-              long long A0, long long A1, long long B0, long long B1, long long C0, long long C1, float alpha,
-              int accumulate, int mask)
+    const Dims &D() const { return plan->dims; }
+    float *f(size_t off) const { return reinterpret_cast<float *>(ws + off); }
+    void keep(cudaError_t e) { if (e != cudaSuccess && err == cudaSuccess) err = e; dependent = true; }
+    void gemms(sg::Launch &L) { L.status = reinterpret_cast<int *>(ws); keep(sg::run(L, st, dependent)); }
+    template <typename... K, typename... A>
+    void kernel(void (*k)(K...), long long threads, A... args)
     {
-        GemmP p{A, B, C, M, N, K, sAm, sAk, sBk, sBn, sCm, sCn, nb1, A0, A1, B0, B1, C0, C1, alpha, accumulate, mask,
-                (M + BM - 1) / BM, (N + BN - 1) / BN};
-        const long long grid = nbatch * p.tilesM * p.tilesN;
-        gemm_kernel<<<(unsigned)grid, 256, 0, st>>>(p);
-        check();
+        // (the same division of the SM's memory as the products' kernel: a change between launches costs microseconds)
+        keep(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+        keep(launch_pdl(k, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, st, dependent, args...));
     }
-    void cast(const void *in, float *out, long long n)
+
+    // ---- operands
+    // tensors [B, H (or H_kv), N, w] in the storage type; cut into blocks of `blk` tokens
+    sg::Op input(const void *p, int w, bool kv, int mn, int blk = 0) const
     {
-        cast_bf16_f32_kernel<<<blocks(n, 1024), 256, 0, st>>>((const __nv_bfloat16 *)in, out, n);
-        check();
+        sg::Op o;
+        const long long per = (long long)D().N * w;
+        o.p = p; o.sh = per; o.sb = per * (kv ? D().Hkv : D().H); o.kv = kv; o.sc = (long long)blk * w;
+        o.ld = w; o.bf16 = D().bf16; o.mn = mn;
+        return o;
     }
-    void fill(float *p, float v, long long n) { fill_kernel<<<blocks(n, 1024), 256, 0, st>>>(p, v, n); check(); }
-    void expand_kv(const void *in, int bf16, float *out, long long per_head, int B, int H, int Hkv)
+    // fp32 intermediates [BH, N, w]
+    sg::Op rows(size_t off, int w, int mn, int blk = 0) const
     {
-        const long long total = (long long)B * H * per_head;
-        if (bf16) expand_kv_kernel<__nv_bfloat16><<<blocks(total, 1024), 256, 0, st>>>((const __nv_bfloat16 *)in, out, per_head, H, Hkv, total);
-        else expand_kv_kernel<float><<<blocks(total, 1024), 256, 0, st>>>((const float *)in, out, per_head, H, Hkv, total);
-        check();
+        sg::Op o;
+        const long long per = (long long)D().N * w;
+        o.p = f(off); o.sh = per; o.sb = per * D().H; o.sc = (long long)blk * w; o.ld = w; o.mn = mn;
+        return o;
     }
-    void emit_grouped(void *out, int bf16, const float *src, int B, int H, int Hkv, int N, int w, long long src_batch, int src_row)
+    // fp32 per block [BH, nb, rows, w] (one_block: the first block stands for all)
+    sg::Op blocks(size_t off, int nb, long long nrows, int w, int mn, bool one_block = false) const
     {
-        const long long total = (long long)B * Hkv * N * w;
-        if (bf16) emit_grouped_kernel<__nv_bfloat16><<<blocks(total, 1024), 256, 0, st>>>((__nv_bfloat16 *)out, src, N, w, src_batch, src_row, H, Hkv, total);
-        else emit_grouped_kernel<float><<<blocks(total, 1024), 256, 0, st>>>((float *)out, src, N, w, src_batch, src_row, H, Hkv, total);
-        check();
+        sg::Op o;
+        const long long per = nrows * w;
+        o.p = f(off); o.sh = per * nb; o.sb = per * nb * D().H; o.sc = one_block ? 0 : per; o.ld = w; o.mn = mn;
+        return o;
     }
-    void emit(void *out, int bf16, const float *src, long long BH, int N, int w, long long src_batch, int src_row, int div_col)
+    // parameters M [H, r, d], W [m, r] or [H, m, r]
+    sg::Op paramM(const void *M, int mn) const
     {
-        const long long total = BH * N * w;
-        if (bf16) emit_rows_kernel<__nv_bfloat16><<<blocks(total, 1024), 256, 0, st>>>((__nv_bfloat16 *)out, src, N, w, src_batch, src_row, div_col, total);
-        else emit_rows_kernel<float><<<blocks(total, 1024), 256, 0, st>>>((float *)out, src, N, w, src_batch, src_row, div_col, total);
-        check();
+        sg::Op o; o.p = M; o.sh = (long long)D().r * D().d; o.ld = D().d; o.bf16 = D().bf16; o.mn = mn; return o;
+    }
+    sg::Op paramW(const void *W, int mn) const
+    {
+        sg::Op o; o.p = W; o.sh = D().w_per_head ? (long long)D().m * D().r : 0; o.ld = D().r; o.bf16 = D().bf16; o.mn = mn; return o;
+    }
+    // ---- products over the whole sequence of every (batch, head)
+    sg::Prob whole() const
+    {
+        sg::Prob p;
+        p.H = D().H; p.G = D().G; p.batch = D().BH; p.ntok = D().N; p.nblk = 1; p.block = 0;
+        return p;
+    }
+    // ... or over blocks of it
+    sg::Prob blocked(int nb, int blk) const
+    {
+        sg::Prob p = whole();
+        p.nblk = nb; p.block = blk;
+        return p;
+    }
+    void out_rows(sg::Prob &p, void *o, int w, bool storage, int blk = 0) const      // [BH, N, w]
+    {
+        const long long per = (long long)D().N * w;
+        p.out = o; p.osh = per; p.osb = per * D().H; p.osc = (long long)blk * w; p.old_ = w; p.obf16 = storage && D().bf16;
+    }
+    void out_blocks(sg::Prob &p, size_t off, int nb, long long nrows, int w) const
+    {
+        const long long per = nrows * w;
+        p.out = f(off); p.osh = per * nb; p.osb = per * nb * D().H; p.osc = per; p.old_ = w;
     }
 };
 
-inline int warp_rows_grid(long long rows) { return (int)((rows * 32 + 255) / 256); }
+inline int tiles(int n) { return (n + 127) / 128; }
 
-struct Bufs {
-    const float *Q, *K, *V, *M, *W;
-    float *xtQ, *xtK, *nQ, *nK, *fQ, *fK, *cK, *Va, *Sloc, *P, *num;
-};
-
-// Steps shared by forward and backward: features, states, numerators (all left in the workspace).
-void run_forward_stages(const darkattn_plan_s *plan, Launcher &L, const void *Q, const void *K, const void *V,
-                        const void *M, const void *W, char *ws, Bufs &b)
+// Features, states and output rows. With dO given the rows dO / den and -delta / den are formed in place of O.
+void run_forward_stages(Runner &R, const void *Q, const void *K, const void *V, const void *M, const void *W, void *O, const void *dO)
 {
-    const Dims &D = plan->dims;
-    const SimtLayout &Y = plan->simt;
-    const long long BH = D.BH, N = D.N, Np = D.Npad, d = D.d, r = D.r, m = D.m, dv = D.dv, dva = D.dva, C = D.C, nc = D.nc;
-    auto F = [&](size_t off) { return reinterpret_cast<float *>(ws + off); };
-    if (D.bf16) {
-        L.cast(Q, F(Y.Qf), BH * N * d);
-        L.cast(M, F(Y.Mf), (long long)D.H * r * d); L.cast(W, F(Y.Wf), (long long)(D.w_per_head ? D.H : 1) * m * r);
-        b.Q = F(Y.Qf); b.M = F(Y.Mf); b.W = F(Y.Wf);
-    } else {
-        b.Q = (const float *)Q; b.M = (const float *)M; b.W = (const float *)W;
+    const Dims &D = R.D();
+    const SimtLayout &Y = R.plan->simt;
+    const int N = D.N, d = D.d, r = D.r, m = D.m, dv = D.dv, C = Y.C, nb = Y.nb;
+    const long long BH = D.BH;
+    {   // x~ = s X M^T
+        sg::Launch L;
+        for (int side = 0; side < 2; ++side) {
+            sg::Prob p = R.whole();
+            p.A[0] = R.input(side ? K : Q, d, side, 0); p.B[0] = R.paramM(M, 0); p.K[0] = d;
+            p.mtok = 1; p.N = r; p.alpha = D.s;
+            R.out_rows(p, R.f(side ? Y.xtK : Y.xtQ), r, false);
+            p.chain = 1;                    // (the exponent's argument: the most sensitive)
+            if (side) { p.epi = sg::EPI_SQUARES; p.sums = R.f(Y.nK); }
+            sg::add(L, p);
+        }
+        L.init = reinterpret_cast<int *>(R.f(Y.cK)); L.init_n = (int)(BH * m);
+        R.gemms(L);
     }
-    if (D.G > 1) {          // grouped key/value heads: every query head works on its own fp32 copy of the head it reads
-        L.expand_kv(K, D.bf16, F(Y.Kf), N * d, D.B, D.H, D.Hkv); L.expand_kv(V, D.bf16, F(Y.Vf), N * dv, D.B, D.H, D.Hkv);
-        b.K = F(Y.Kf); b.V = F(Y.Vf);
-    } else if (D.bf16) {
-        L.cast(K, F(Y.Kf), BH * N * d); L.cast(V, F(Y.Vf), BH * N * dv);
-        b.K = F(Y.Kf); b.V = F(Y.Vf);
-    } else {
-        b.K = (const float *)K; b.V = (const float *)V;
+    {   // u = x~ W^T, for the keys minus half the squared norm of x~
+        sg::Launch L;
+        for (int side = 0; side < 2; ++side) {
+            sg::Prob p = R.whole();
+            p.A[0] = R.rows(side ? Y.xtK : Y.xtQ, r, 0); p.B[0] = R.paramW(W, 0); p.K[0] = r;
+            p.mtok = 1; p.N = m; p.chain = 1;
+            R.out_rows(p, R.f(side ? Y.fK : Y.fQ), m, false);
+            if (side) {
+                p.epi = sg::EPI_KEY_EXPONENT; p.row = {R.f(Y.nK), BH * N, tiles(r), 0.5f};
+                p.colmax = reinterpret_cast<int *>(R.f(Y.cK));
+            }
+            sg::add(L, p);
+        }
+        R.gemms(L);
     }
-    b.xtQ = F(Y.xtQ); b.xtK = F(Y.xtK); b.nQ = F(Y.nQ); b.nK = F(Y.nK); b.fQ = F(Y.fQ); b.fK = F(Y.fK);
-    b.cK = F(Y.cK); b.Va = F(Y.Va); b.Sloc = F(Y.Sloc); b.P = F(Y.P); b.num = F(Y.num);
-    const long long wb1 = D.w_per_head ? m * r : 0;
-
-    for (int side = 0; side < 2; ++side) {
-        const float *X = side ? b.K : b.Q;
-        float *xt = side ? b.xtK : b.xtQ, *f = side ? b.fK : b.fQ;
-        // x~ = s X M^T
-        L.gemm(X, b.M, xt, (int)N, (int)r, (int)d, d, 1, 1, d, r, 1, BH, D.H, D.H * N * d, N * d, 0, r * d, D.H * N * r, N * r, D.s, 0, 0);
-        // u = x~ W^T
-        L.gemm(xt, b.W, f, (int)N, (int)m, (int)r, r, 1, 1, r, m, 1, BH, D.H, D.H * N * r, N * r, 0, wb1, D.H * Np * m, Np * m, 1.f, 0, 0);
+    if (m % 4 == 0) R.kernel(features_kernel<4>, 2 * BH * N * 32, R.f(Y.fQ), R.f(Y.fK), reinterpret_cast<const int *>(R.f(Y.cK)), N, m, BH * N);
+    else R.kernel(features_kernel<1>, 2 * BH * N * 32, R.f(Y.fQ), R.f(Y.fK), reinterpret_cast<const int *>(R.f(Y.cK)), N, m, BH * N);
+    {   // S_c = phi(K_c)^T V_c, z_c = phi(K_c)^T 1 per token block; causal: P_c = tril(phi(Q_c) phi(K_c)^T)
+        sg::Launch L;
+        sg::Prob p = R.blocked(nb, Y.blk);
+        p.A[0] = R.rows(Y.fK, m, 1, Y.blk); p.B[0] = R.input(V, dv, true, 1, Y.blk); p.K[0] = N; p.ktok[0] = 1;
+        p.M = m; p.N = dv; p.dot[0] = sg::DOT_ONES; p.dot_out = R.f(Y.zloc);
+        R.out_blocks(p, Y.Sloc, nb, m, dv);
+        sg::add(L, p);
+        if (D.causal) {
+            sg::Prob q = R.blocked(nb, C);
+            q.A[0] = R.rows(Y.fQ, m, 0, C); q.B[0] = R.rows(Y.fK, m, 0, C); q.K[0] = m;
+            q.mtok = q.ntok_dim = 1; q.epi = sg::EPI_MASK;
+            R.out_blocks(q, Y.P, nb, C, C);
+            sg::add(L, q);
+        }
+        R.gemms(L);
     }
-    half_sqnorm_kernel<<<warp_rows_grid(BH * N), 256, 0, L.st>>>(b.xtK, b.nK, BH * N, (int)r); L.check();
-    L.fill(b.cK, -INFINITY, BH * m);
-    key_colmax_kernel<<<dim3((unsigned)((N + 127) / 128), (unsigned)BH), 256, 0, L.st>>>(b.fK, b.nK, b.cK, (int)N, (int)Np, (int)m); L.check();
-    key_features_kernel<<<Launcher::blocks(BH * Np * m, 1024), 256, 0, L.st>>>(b.fK, b.nK, b.cK, (int)N, (int)Np, (int)m, BH * Np * m); L.check();
-    query_features_kernel<<<warp_rows_grid(BH * Np), 256, 0, L.st>>>(b.fQ, b.cK, (int)N, (int)Np, (int)m, BH * Np); L.check();
-    augment_values_kernel<<<Launcher::blocks(BH * Np * dva, 1024), 256, 0, L.st>>>(b.V, b.Va, (int)N, (int)Np, (int)dv, BH * Np * dva); L.check();
-
-    if (!D.causal) {
-        // S = phi(K)^T [V|1]; num = phi(Q) S
-        L.gemm(b.fK, b.Va, b.Sloc, (int)m, (int)dva, (int)Np, 1, m, dva, 1, dva, 1, BH, 1, Np * m, 0, Np * dva, 0, m * dva, 0, 1.f, 0, 0);
-        L.gemm(b.fQ, b.Sloc, b.num, (int)Np, (int)dva, (int)m, m, 1, dva, 1, dva, 1, BH, 1, Np * m, 0, m * dva, 0, Np * dva, 0, 1.f, 0, 0);
-    } else {
-        const long long Z = BH * nc;
-        // chunk-local states, then exclusive prefix over chunks
-        L.gemm(b.fK, b.Va, b.Sloc, (int)m, (int)dva, (int)C, 1, m, dva, 1, dva, 1, Z, (int)nc, Np * m, C * m, Np * dva, C * dva, nc * m * dva, m * dva, 1.f, 0, 0);
-        chunk_scan_kernel<<<(unsigned)((BH * m * dva + 255) / 256), 256, 0, L.st>>>(b.Sloc, (int)nc, m * dva, BH * m * dva, 0); L.check();
-        // P = tril(phi(Q_c) phi(K_c)^T); num = P [V|1] + phi(Q_c) S_prev
-        L.gemm(b.fQ, b.fK, b.P, (int)C, (int)C, (int)m, m, 1, 1, m, C, 1, Z, (int)nc, Np * m, C * m, Np * m, C * m, nc * C * C, C * C, 1.f, 0, 1);
-        L.gemm(b.P, b.Va, b.num, (int)C, (int)dva, (int)C, C, 1, dva, 1, dva, 1, Z, (int)nc, nc * C * C, C * C, Np * dva, C * dva, Np * dva, C * dva, 1.f, 0, 0);
-        L.gemm(b.fQ, b.Sloc, b.num, (int)C, (int)dva, (int)m, m, 1, dva, 1, dva, 1, Z, (int)nc, Np * m, C * m, nc * m * dva, m * dva, Np * dva, C * dva, 1.f, 1, 0);
+    const long long E = (long long)m * dv;
+    auto scan = [&](size_t S, size_t z, int mode) {
+        if (nb == 1 && mode == SCAN_TOTAL) return;
+        if (m % 4 == 0) R.kernel(chunk_scan_kernel<4>, BH * (E + m) / 4, R.f(S), R.f(z), nb, E, m, BH, mode);
+        else R.kernel(chunk_scan_kernel<1>, BH * (E + m), R.f(S), R.f(z), nb, E, m, BH, mode);
+    };
+    scan(Y.Sloc, Y.zloc, D.causal ? SCAN_FORWARD : SCAN_TOTAL);
+    {   // O = (P V + phi(Q) S_prev) / (P 1 + phi(Q) z_prev)
+        sg::Launch L;
+        sg::Prob p = D.causal ? R.blocked(nb, C) : R.whole();
+        const int s = D.causal ? 1 : 0, blk = D.causal ? C : 0;
+        if (D.causal) {
+            p.A[0] = R.blocks(Y.P, nb, C, C, 0); p.B[0] = R.input(V, dv, true, 1, C); p.K[0] = C; p.ktok[0] = 1; p.dot[0] = sg::DOT_ONES;
+            p.skip2_first = 1;
+        }
+        p.A[s] = R.rows(Y.fQ, m, 0, blk); p.B[s] = R.blocks(Y.Sloc, nb, m, dv, 1, !D.causal); p.K[s] = m; p.dot[s] = sg::DOT_FEATURES;
+        p.dotf = R.f(Y.zloc); p.vec_pair = (long long)nb * m; p.vec_blk = D.causal ? m : 0;
+        p.mtok = 1; p.N = dv; p.epi = dO ? sg::EPI_GRAD : sg::EPI_DIVIDE;
+        if (dO) {
+            p.x = R.input(dO, dv, false, 0, blk); p.sums = R.f(Y.gd);
+            R.out_rows(p, R.f(Y.Ga), dv, false, blk);
+        } else R.out_rows(p, O, dv, true, blk);
+        sg::add(L, p);
+        R.gemms(L);
     }
+    if (!dO) return;
+    const sg::TokVec gd = {R.f(Y.gd), BH * N, tiles(dv), 1.f};
+    {   // R_c = phi(Q_c)^T Ga_c, rho_c = phi(Q_c)^T gd_c; causal: dP_c = tril(Ga_c V_c^T + gd_c)
+        sg::Launch L;
+        sg::Prob p = R.blocked(nb, Y.blk);
+        p.A[0] = R.rows(Y.fQ, m, 1, Y.blk); p.B[0] = R.rows(Y.Ga, dv, 1, Y.blk); p.K[0] = N; p.ktok[0] = 1;
+        p.M = m; p.N = dv; p.dot[0] = sg::DOT_TOKENS; p.dott = gd; p.dot_out = R.f(Y.rloc);
+        R.out_blocks(p, Y.Rloc, nb, m, dv);
+        sg::add(L, p);
+        if (D.causal) {
+            sg::Prob q = R.blocked(nb, C);
+            q.A[0] = R.rows(Y.Ga, dv, 0, C); q.B[0] = R.input(V, dv, true, 0, C); q.K[0] = dv;
+            q.mtok = q.ntok_dim = 1; q.epi = sg::EPI_MASK; q.row = gd;
+            R.out_blocks(q, Y.dP, nb, C, C);
+            sg::add(L, q);
+        }
+        R.gemms(L);
+    }
+    scan(Y.Rloc, Y.rloc, D.causal ? SCAN_REVERSE : SCAN_TOTAL);
 }
 
 size_t take(size_t &off, long long floats)
@@ -433,53 +341,69 @@ size_t take(size_t &off, long long floats)
     return at;
 }
 
+// Cuts N tokens into blocks (multiples of 64 tokens) so that `units` products of one block each are at least one wave of
+// two CTAs per SM, none shorter than two stages of the contraction.
+void cut_tokens(int N, long long units, int most, int &nblk, int &blk)
+{
+    long long want = (2 * 148 + units - 1) / units;
+    if (want > (N + 127) / 128) want = (N + 127) / 128;
+    if (want > most) want = most;
+    if (want < 1) want = 1;
+    blk = (int)(((N + want - 1) / want + 63) / 64 * 64);
+    nblk = (N + blk - 1) / blk;
+}
+
 }  // namespace
 
 void simt_make_layout(darkattn_plan_s *plan)
 {
     const Dims &D = plan->dims;
     SimtLayout &Y = plan->simt;
-    const long long BH = D.BH, N = D.N, Np = D.Npad, d = D.d, r = D.r, m = D.m, dv = D.dv, dva = D.dva, C = D.C, nc = D.nc;
+    const long long BH = D.BH, N = D.N, d = D.d, r = D.r, m = D.m, dv = D.dv;
+    if (D.causal) {
+        Y.C = (int)(N < D.C ? (N + 3) / 4 * 4 : D.C);
+        if (Y.C > D.C) Y.C = D.C;
+        Y.blk = Y.C;
+        Y.nb = (int)((N + Y.C - 1) / Y.C);
+    } else {
+        Y.C = 0;
+        // (the extra partial states never take more room than two rows of values per token)
+        cut_tokens(D.N, BH * tiles(D.m) * tiles(D.dv), (int)(1 + 2 * N / m > 64 ? 64 : 1 + 2 * N / m), Y.nb, Y.blk);
+    }
+    const long long nb = Y.nb, C = Y.C;
     size_t off = 0;
     Y.status = take(off, 64);
-    Y.Qf = Y.Kf = Y.Vf = Y.Mf = Y.Wf = 0;
-    if (D.bf16) {
-        Y.Qf = take(off, BH * N * d);
-        Y.Mf = take(off, (long long)D.H * r * d); Y.Wf = take(off, (long long)(D.w_per_head ? D.H : 1) * m * r);
-    }
-    if (D.bf16 || D.G > 1) { Y.Kf = take(off, BH * N * d); Y.Vf = take(off, BH * N * dv); }
     Y.xtQ = take(off, BH * N * r); Y.xtK = take(off, BH * N * r);
-    Y.nQ = take(off, BH * N); Y.nK = take(off, BH * N);
-    Y.fQ = take(off, BH * Np * m); Y.fK = take(off, BH * Np * m);
+    Y.fQ = take(off, BH * N * m); Y.fK = take(off, BH * N * m);
     Y.cK = take(off, BH * m);
-    Y.Va = take(off, BH * Np * dva);
-    Y.Sloc = take(off, BH * nc * m * dva);
-    Y.P = D.causal ? take(off, BH * nc * C * C) : 0;
-    Y.num = take(off, BH * Np * dva);
+    Y.Sloc = take(off, BH * nb * m * dv); Y.zloc = take(off, BH * nb * m);
+    Y.P = D.causal ? take(off, BH * nb * C * C) : 0;
+    {   // the key norms are done with before the states are written: they share their place
+        size_t end = Y.Sloc;
+        Y.nK = take(end, tiles(D.r) * BH * N);
+        if (end > off) off = end;
+    }
     Y.fwd_bytes = off;
-    Y.Gf = D.bf16 ? take(off, BH * N * dv) : 0;
-    Y.Ga = take(off, BH * Np * dva);
-    Y.dP = D.causal ? take(off, BH * nc * C * C) : 0;
-    Y.Rloc = take(off, BH * nc * m * dva);
-    Y.dA = take(off, BH * Np * m); Y.dBf = take(off, BH * Np * m);
-    Y.dVa = take(off, BH * Np * dva);
-    Y.esQ = take(off, BH * N); Y.esK = take(off, BH * N);
+    Y.Ga = take(off, BH * N * dv); Y.gd = take(off, tiles(D.dv) * BH * N);
+    Y.dP = D.causal ? take(off, BH * nb * C * C) : 0;
+    Y.Rloc = take(off, BH * nb * m * dv); Y.rloc = take(off, BH * nb * m);
+    Y.dA = take(off, BH * N * m); Y.dBf = take(off, BH * N * m);
+    Y.esK = take(off, tiles(D.m) * BH * N);
     Y.dxtQ = take(off, BH * N * r); Y.dxtK = take(off, BH * N * r);
-    Y.dXf = take(off, BH * N * d);
-    Y.dMp = take(off, BH * r * d);
-    Y.dWp = take(off, BH * m * r);
+    Y.dKh = D.G > 1 ? take(off, BH * N * d) : 0; Y.dVh = D.G > 1 ? take(off, BH * N * dv) : 0;
+    cut_tokens(D.N, BH * tiles(D.r) * tiles(D.d), 64, Y.nsM, Y.blkM);
+    cut_tokens(D.N, BH * tiles(D.m) * tiles(D.r), 64, Y.nsW, Y.blkW);
+    Y.dMp = take(off, BH * Y.nsM * r * d);
+    Y.dWp = take(off, BH * Y.nsW * m * r);
     Y.total_bytes = off;
 }
 
 darkattn_status_t simt_forward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
-                               const void *M, const void *W, void *O, char *ws, cudaStream_t st, bool)
+                               const void *M, const void *W, void *O, char *ws, cudaStream_t st)
 {
-    const Dims &D = plan->dims;
-    Launcher L{st};
-    Bufs b;
-    run_forward_stages(plan, L, Q, K, V, M, W, ws, b);
-    L.emit(O, D.bf16, b.num, D.BH, D.N, D.dv, (long long)D.Npad * D.dva, D.dva, D.dv);
-    if (L.err != cudaSuccess) { set_cuda_error(L.err, "simt_forward"); return DARKATTN_ERR_CUDA; }
+    Runner R{plan, ws, st};
+    run_forward_stages(R, Q, K, V, M, W, O, nullptr);
+    if (R.err != cudaSuccess) { set_cuda_error(R.err, "simt_forward"); return DARKATTN_ERR_CUDA; }
     return DARKATTN_OK;
 }
 
@@ -489,97 +413,118 @@ darkattn_status_t simt_backward(const darkattn_plan_s *plan, const void *Q, cons
 {
     const Dims &D = plan->dims;
     const SimtLayout &Y = plan->simt;
-    const long long BH = D.BH, N = D.N, Np = D.Npad, d = D.d, r = D.r, m = D.m, dv = D.dv, dva = D.dva, C = D.C, nc = D.nc;
-    auto F = [&](size_t off) { return reinterpret_cast<float *>(ws + off); };
-    Launcher L{st};
-    Bufs b;
-    run_forward_stages(plan, L, Q, K, V, M, W, ws, b);
+    const int N = D.N, d = D.d, r = D.r, m = D.m, dv = D.dv, C = Y.C, nb = Y.nb;
+    const long long BH = D.BH;
+    Runner R{plan, ws, st};
+    run_forward_stages(R, Q, K, V, M, W, nullptr, dO);
 
-    const float *G;
-    if (D.bf16) { L.cast(dO, F(Y.Gf), BH * N * dv); G = F(Y.Gf); } else G = (const float *)dO;
-    float *Ga = F(Y.Ga), *dP = F(Y.dP), *Rl = F(Y.Rloc), *dA = F(Y.dA), *dBf = F(Y.dBf), *dVa = F(Y.dVa);
-    grad_aug_kernel<<<warp_rows_grid(BH * Np), 256, 0, st>>>(G, b.num, Ga, (int)N, (int)Np, (int)dv, BH * Np); L.check();
-
-    if (!D.causal) {
-        // dA = Ga S^T ; R = phi(Q)^T Ga ; dBf = [V|1] R^T ; d[V|1] = phi(K) R
-        L.gemm(Ga, b.Sloc, dA, (int)Np, (int)m, (int)dva, dva, 1, 1, dva, m, 1, BH, 1, Np * dva, 0, m * dva, 0, Np * m, 0, 1.f, 0, 0);
-        L.gemm(b.fQ, Ga, Rl, (int)m, (int)dva, (int)Np, 1, m, dva, 1, dva, 1, BH, 1, Np * m, 0, Np * dva, 0, m * dva, 0, 1.f, 0, 0);
-        L.gemm(b.Va, Rl, dBf, (int)Np, (int)m, (int)dva, dva, 1, 1, dva, m, 1, BH, 1, Np * dva, 0, m * dva, 0, Np * m, 0, 1.f, 0, 0);
-        L.gemm(b.fK, Rl, dVa, (int)Np, (int)dva, (int)m, m, 1, dva, 1, dva, 1, BH, 1, Np * m, 0, m * dva, 0, Np * dva, 0, 1.f, 0, 0);
-    } else {
-        const long long Z = BH * nc;
-        const long long sP0 = nc * C * C, sP1 = C * C, sF0 = Np * m, sF1 = C * m, sV0 = Np * dva, sV1 = C * dva, sS0 = nc * m * dva, sS1 = m * dva;
-        // dP = tril(Ga_c [V|1]_c^T)
-        L.gemm(Ga, b.Va, dP, (int)C, (int)C, (int)dva, dva, 1, 1, dva, C, 1, Z, (int)nc, sV0, sV1, sV0, sV1, sP0, sP1, 1.f, 0, 1);
-        // dA_c = dP_c phi(K_c) + Ga_c S_prev^T
-        L.gemm(dP, b.fK, dA, (int)C, (int)m, (int)C, C, 1, m, 1, m, 1, Z, (int)nc, sP0, sP1, sF0, sF1, sF0, sF1, 1.f, 0, 0);
-        L.gemm(Ga, b.Sloc, dA, (int)C, (int)m, (int)dva, dva, 1, 1, dva, m, 1, Z, (int)nc, sV0, sV1, sS0, sS1, sF0, sF1, 1.f, 1, 0);
-        // reverse states R_c = phi(Q_c)^T Ga_c, exclusive suffix over chunks
-        L.gemm(b.fQ, Ga, Rl, (int)m, (int)dva, (int)C, 1, m, dva, 1, dva, 1, Z, (int)nc, sF0, sF1, sV0, sV1, sS0, sS1, 1.f, 0, 0);
-        chunk_scan_kernel<<<(unsigned)((BH * m * dva + 255) / 256), 256, 0, st>>>(Rl, (int)nc, m * dva, BH * m * dva, 1); L.check();
-        // dBf_c = dP_c^T phi(Q_c) + [V|1]_c R_next^T
-        L.gemm(dP, b.fQ, dBf, (int)C, (int)m, (int)C, 1, C, m, 1, m, 1, Z, (int)nc, sP0, sP1, sF0, sF1, sF0, sF1, 1.f, 0, 0);
-        L.gemm(b.Va, Rl, dBf, (int)C, (int)m, (int)dva, dva, 1, 1, dva, m, 1, Z, (int)nc, sV0, sV1, sS0, sS1, sF0, sF1, 1.f, 1, 0);
-        // d[V|1]_c = P_c^T Ga_c + phi(K_c) R_next
-        L.gemm(b.P, Ga, dVa, (int)C, (int)dva, (int)C, 1, C, dva, 1, dva, 1, Z, (int)nc, sP0, sP1, sV0, sV1, sV0, sV1, 1.f, 0, 0);
-        L.gemm(b.fK, Rl, dVa, (int)C, (int)dva, (int)m, m, 1, dva, 1, dva, 1, Z, (int)nc, sF0, sF1, sS0, sS1, sV0, sV1, 1.f, 1, 0);
+    const bool grouped = D.G > 1;
+    const sg::TokVec gd = {R.f(Y.gd), BH * N, tiles(dv), 1.f};
+    const int blk = D.causal ? C : 0, s = D.causal ? 1 : 0;
+    auto per_block = [&]() { return D.causal ? R.blocked(nb, C) : R.whole(); };
+    {
+        sg::Launch L;
+        {   // E_Q = phi(Q) .* (dP phi(K) + Ga S_prev^T + gd z_prev^T)
+            sg::Prob p = per_block();
+            if (D.causal) { p.A[0] = R.blocks(Y.dP, nb, C, C, 0); p.B[0] = R.rows(Y.fK, m, 1, C); p.K[0] = C; p.ktok[0] = 1; p.skip2_first = 1; }
+            p.A[s] = R.rows(Y.Ga, dv, 0, blk); p.B[s] = R.blocks(Y.Sloc, nb, m, dv, 0, !D.causal); p.K[s] = dv;
+            p.epi = sg::EPI_RANK1; p.row = gd; p.rank1 = R.f(Y.zloc); p.vec_pair = (long long)nb * m; p.vec_blk = D.causal ? m : 0;
+            p.x = R.rows(Y.fQ, m, 0, blk);
+            p.mtok = 1; p.N = m;
+            R.out_rows(p, R.f(Y.dA), m, false, blk);
+            sg::add(L, p);
+        }
+        {   // E_K = phi(K) .* (dP^T phi(Q) + V R_next^T + rho_next^T), and its row sums
+            sg::Prob p = per_block();
+            if (D.causal) { p.A[0] = R.blocks(Y.dP, nb, C, C, 1); p.B[0] = R.rows(Y.fQ, m, 1, C); p.K[0] = C; p.ktok[0] = 1; }
+            p.A[s] = R.input(V, dv, true, 0, blk); p.B[s] = R.blocks(Y.Rloc, nb, m, dv, 0, !D.causal); p.K[s] = dv;
+            p.epi = sg::EPI_RANK1; p.rank1 = R.f(Y.rloc); p.vec_pair = (long long)nb * m; p.vec_blk = D.causal ? m : 0;
+            p.x = R.rows(Y.fK, m, 0, blk); p.sums = R.f(Y.esK);
+            p.mtok = 1; p.N = m;
+            R.out_rows(p, R.f(Y.dBf), m, false, blk);
+            sg::add(L, p);
+        }
+        {   // dV = P^T Ga + phi(K) R_next
+            sg::Prob p = per_block();
+            if (D.causal) { p.A[0] = R.blocks(Y.P, nb, C, C, 1); p.B[0] = R.rows(Y.Ga, dv, 1, C); p.K[0] = C; p.ktok[0] = 1; }
+            p.A[s] = R.rows(Y.fK, m, 0, blk); p.B[s] = R.blocks(Y.Rloc, nb, m, dv, 1, !D.causal); p.K[s] = m;
+            p.mtok = 1; p.N = dv;
+            if (grouped) R.out_rows(p, R.f(Y.dVh), dv, false, blk);
+            else R.out_rows(p, dV, dv, true, blk);
+            sg::add(L, p);
+        }
+        R.gemms(L);
     }
-    if (D.G > 1) L.emit_grouped(dV, D.bf16, dVa, D.B, D.H, D.Hkv, (int)N, (int)dv, Np * dva, (int)dva);
-    else L.emit(dV, D.bf16, dVa, BH, (int)N, (int)dv, Np * dva, (int)dva, -1);
-
-    const long long wb1 = D.w_per_head ? m * r : 0;
-    for (int side = 0; side < 2; ++side) {
-        float *dphi = side ? dBf : dA;
-        const float *phi = side ? b.fK : b.fQ, *xt = side ? b.xtK : b.xtQ, *X = side ? b.K : b.Q;
-        float *es = F(side ? Y.esK : Y.esQ), *dxt = F(side ? Y.dxtK : Y.dxtQ), *dXf = F(Y.dXf);
-        feature_grad_kernel<<<warp_rows_grid(BH * Np), 256, 0, st>>>(dphi, phi, es, (int)N, (int)Np, (int)m, BH * Np); L.check();
-        // dx~ = E W - rowsum(E) x~
-        L.gemm(dphi, b.W, dxt, (int)N, (int)r, (int)m, m, 1, r, 1, r, 1, BH, D.H, D.H * Np * m, Np * m, 0, wb1, D.H * N * r, N * r, 1.f, 0, 0);
-        norm_term_kernel<<<Launcher::blocks(BH * N * r, 1024), 256, 0, st>>>(dxt, xt, es, (int)r, BH * N * r); L.check();
-        // dX = s dx~ M
-        L.gemm(dxt, b.M, dXf, (int)N, (int)d, (int)r, r, 1, d, 1, d, 1, BH, D.H, D.H * N * r, N * r, 0, r * d, D.H * N * d, N * d, D.s, 0, 0);
-        if (side && D.G > 1) L.emit_grouped(dK, D.bf16, dXf, D.B, D.H, D.Hkv, (int)N, (int)d, N * d, (int)d);
-        else L.emit(side ? dK : dQ, D.bf16, dXf, BH, (int)N, (int)d, N * d, (int)d, -1);
-        // dM_(b,h) (+)= s dx~^T X
-        L.gemm(dxt, X, F(Y.dMp), (int)r, (int)d, (int)N, 1, r, d, 1, d, 1, BH, 1, N * r, 0, N * d, 0, r * d, 0, D.s, side, 0);
+    {   // dx~ = E W, for the keys minus rowsum(E) x~
+        sg::Launch L;
+        for (int side = 0; side < 2; ++side) {
+            sg::Prob p = R.whole();
+            p.A[0] = R.rows(side ? Y.dBf : Y.dA, m, 0); p.B[0] = R.paramW(W, 1); p.K[0] = m;
+            p.mtok = 1; p.N = r;
+            if (side) { p.epi = sg::EPI_SUBX; p.x = R.rows(Y.xtK, r, 0); p.row = {R.f(Y.esK), BH * N, tiles(m), 1.f}; }
+            R.out_rows(p, R.f(side ? Y.dxtK : Y.dxtQ), r, false);
+            sg::add(L, p);
+        }
+        R.gemms(L);
     }
-    reduce_batch_kernel<<<(unsigned)(((long long)D.H * r * d + 255) / 256), 256, 0, st>>>(F(Y.dMp), dM, D.B, (long long)D.H * r * d, (long long)D.H * r * d); L.check();
-    if (L.err != cudaSuccess) { set_cuda_error(L.err, "simt_backward"); return DARKATTN_ERR_CUDA; }
+    {   // dX = s dx~ M; dM = s sum dx~^T X over the tokens of both sides, per (b,h) and token block
+        sg::Launch L;
+        for (int side = 0; side < 2; ++side) {
+            sg::Prob p = R.whole();
+            p.A[0] = R.rows(side ? Y.dxtK : Y.dxtQ, r, 0); p.B[0] = R.paramM(M, 1); p.K[0] = r;
+            p.mtok = 1; p.N = d; p.alpha = D.s;
+            if (side && grouped) R.out_rows(p, R.f(Y.dKh), d, false);
+            else R.out_rows(p, side ? dK : dQ, d, true);
+            sg::add(L, p);
+        }
+        sg::Prob p = R.blocked(Y.nsM, Y.blkM);
+        for (int side = 0; side < 2; ++side) {
+            p.A[side] = R.rows(side ? Y.dxtK : Y.dxtQ, r, 1, Y.blkM); p.B[side] = R.input(side ? K : Q, d, side, 1, Y.blkM);
+            p.K[side] = N; p.ktok[side] = 1;
+        }
+        p.M = r; p.N = d; p.alpha = D.s;
+        R.out_blocks(p, Y.dMp, Y.nsM, r, d);
+        sg::add(L, p);
+        R.gemms(L);
+    }
+    const long long E = (long long)r * d;
+    R.kernel(reduce_kernel, D.H * E, R.f(Y.dMp), dM, D.B, (long long)D.H, Y.nsM, E, D.H * E);
+    if (grouped) {
+        const long long BHkv = (long long)D.B * D.Hkv, nv = BHkv * N * dv, nk = BHkv * N * d;
+        auto threads = [](long long n) { return n < 148LL * 16 * 256 ? n : 148LL * 16 * 256; };
+        if (D.bf16) {
+            R.kernel(group_sum_f32_kernel<__nv_bfloat16>, threads(nv), (__nv_bfloat16 *)dV, R.f(Y.dVh), D.G, (long long)N * dv, nv);
+            R.kernel(group_sum_f32_kernel<__nv_bfloat16>, threads(nk), (__nv_bfloat16 *)dK, R.f(Y.dKh), D.G, (long long)N * d, nk);
+        } else {
+            R.kernel(group_sum_f32_kernel<float>, threads(nv), (float *)dV, R.f(Y.dVh), D.G, (long long)N * dv, nv);
+            R.kernel(group_sum_f32_kernel<float>, threads(nk), (float *)dK, R.f(Y.dKh), D.G, (long long)N * d, nk);
+        }
+    }
+    if (R.err != cudaSuccess) { set_cuda_error(R.err, "simt_backward"); return DARKATTN_ERR_CUDA; }
     return DARKATTN_OK;
 }
 
 // dW_l = sum_i E_il x~_i over queries and keys: E (in the buffers dA, dBf) and x~ are still in the workspace after
-// simt_backward. Per (b,h) products, then the sum over the batch (and over the heads when W is shared).
-__global__ void reduce_dw_kernel(const float *dWp, float *dW, int B, int H, long long per_head, int w_per_head, long long total)
-{
-    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (t >= total) return;
-    float acc = 0.f;
-    if (w_per_head) {
-        const long long h = t / per_head, e = t % per_head;
-        for (int b = 0; b < B; ++b) acc += dWp[((long long)b * H + h) * per_head + e];
-    } else {
-        for (int bh = 0; bh < B * H; ++bh) acc += dWp[(long long)bh * per_head + t];
-    }
-    dW[t] = acc;
-}
-
+// simt_backward. Per (b,h) and token block, then the sum over those (and over the heads when W is shared).
 darkattn_status_t simt_backward_dw(const darkattn_plan_s *plan, float *dW, char *ws, cudaStream_t st)
 {
     const Dims &D = plan->dims;
     const SimtLayout &Y = plan->simt;
-    const long long BH = D.BH, N = D.N, Np = D.Npad, r = D.r, m = D.m;
-    auto F = [&](size_t off) { return reinterpret_cast<float *>(ws + off); };
-    Launcher L{st};
+    Runner R{plan, ws, st};
+    sg::Launch L;
+    sg::Prob p = R.blocked(Y.nsW, Y.blkW);
     for (int side = 0; side < 2; ++side) {
-        const float *E = F(side ? Y.dBf : Y.dA), *xt = F(side ? Y.xtK : Y.xtQ);
-        // dWp_(b,h) (+)= E^T x~   [m x r], contraction over the N tokens (padding rows of E are zero, but x~ has only N rows)
-        L.gemm(E, xt, F(Y.dWp), (int)m, (int)r, (int)N, 1, m, r, 1, r, 1, BH, 1, Np * m, 0, N * r, 0, m * r, 0, 1.f, side, 0);
+        p.A[side] = R.rows(side ? Y.dBf : Y.dA, D.m, 1, Y.blkW); p.B[side] = R.rows(side ? Y.xtK : Y.xtQ, D.r, 1, Y.blkW);
+        p.K[side] = D.N; p.ktok[side] = 1;
     }
-    const long long per_head = m * r, total = (D.w_per_head ? D.H : 1) * per_head;
-    reduce_dw_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(F(Y.dWp), dW, D.B, D.H, per_head, D.w_per_head, total);
-    L.check();
-    if (L.err != cudaSuccess) { set_cuda_error(L.err, "simt_backward_dw"); return DARKATTN_ERR_CUDA; }
+    p.M = D.m; p.N = D.r;
+    R.out_blocks(p, Y.dWp, Y.nsW, D.m, D.r);
+    sg::add(L, p);
+    R.gemms(L);
+    const long long E = (long long)D.m * D.r;
+    if (D.w_per_head) R.kernel(reduce_kernel, D.H * E, R.f(Y.dWp), dW, D.B, (long long)D.H, Y.nsW, E, D.H * E);
+    else R.kernel(reduce_kernel, E, R.f(Y.dWp), dW, D.BH, 1LL, Y.nsW, E, E);
+    if (R.err != cudaSuccess) { set_cuda_error(R.err, "simt_backward_dw"); return DARKATTN_ERR_CUDA; }
     return DARKATTN_OK;
 }
 

@@ -59,9 +59,7 @@ extern "C" darkattn_status_t darkattn_forward_static(darkattn_plan_t plan, const
     darkattn_status_t s = scratch_for_current_device(&scratch);
     if (s != DARKATTN_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    // the array still holds the previous call's data: the status word must start at zero; every other
-    // region is written by this call before it is read (the per-feature maxima are re-initialised by
-    // the forward stages themselves)
-    DARKATTN_CUDA_TRY(cudaMemsetAsync(scratch, 0, 256, st), "forward_static: clear status word");
-    return simt_forward(plan, Q, K, V, M, W, O, scratch, st, false);
+    // the array still holds the previous call's data: the first kernel clears the status word and the per-feature maxima,
+    // every other region is written by this call before it is read
+    return simt_forward(plan, Q, K, V, M, W, O, scratch, st);
 }

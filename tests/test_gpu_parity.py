@@ -59,6 +59,35 @@ def test_small_shapes_forward_backward_simt(binding, name, kw, dtype):
     _compare(got, want, TOL[dtype], name)
 
 
+# The FP32 path's products at the edges of their 128 x 128 x 64 tiles: one more or one less than a tile in every dimension,
+# rows that do not start on 16 bytes (every width odd), several tiles of features and values, one token, a chunk of two
+# tiles with a short last block, grouped heads.
+SPLIT_EDGES = [
+    dict(B=1, H=2, N=129, d=65, m=129, r=63, dv=127, causal=True),
+    dict(B=1, H=2, N=127, d=33, m=50, r=17, dv=15, causal=False),
+    dict(B=2, H=1, N=191, d=128, m=260, r=132, dv=136, causal=True),
+    dict(B=1, H=1, N=1, d=64, m=64, dv=64, causal=False),
+    dict(B=1, H=2, N=700, d=16, m=24, r=8, dv=8, causal=True, chunk=256),
+    dict(B=2, H=4, N=65, d=40, m=72, r=20, dv=36, causal=False),
+]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("i", range(len(SPLIT_EDGES)))
+def test_fp32_products_at_tile_edges(binding, i, dtype):
+    kw = dict(SPLIT_EDGES[i])
+    chunk = kw.pop("chunk", 0)
+    wl = inputs.small(name=f"split{i}", wid=400 + i, dtype=dtype, backward=True, **kw)
+    t = inputs.generate(wl)
+    got = run_gpu(binding, wl, t, path=binding.PATH_SIMT, chunk=chunk, want_dw=True)
+    want = _oracle(t, wl)
+    want["dW"] = ref.backward(t.Q, t.K, t.V, t.M, t.W, t.dO, causal=wl.causal)[4]
+    if wl.N == 1:               # O_0 = V_0 whatever Q, K, M and W are: those gradients are exactly zero
+        for k in ("dQ", "dK", "dM", "dW"):
+            assert np.abs(want.pop(k)).max() < 1e-12 and np.abs(got[k]).max() < TOL[dtype]
+    _compare(got, want, TOL[dtype], f"split{i}")
+
+
 @pytest.mark.parametrize("chunk", [16, 64, 256])
 def test_chunk_length_does_not_change_the_result(binding, chunk):
     wl = inputs.small(name="chunks", wid=31, B=1, H=2, N=300, d=32, m=64, causal=True, dtype="f32")
