@@ -5,7 +5,15 @@
 // Stabiliser (cancels in o, and is the same at every step, so the state of one step is valid for the next): keys use
 // the per-feature shift c_l = |w_l|^2 / 2, i.e. phi(k)_l = exp(u_l - |x~|^2/2 - c_l) = exp(-|x~ - w_l|^2 / 2) <= 1;
 // queries use exp(u_l + c_l - max_l(u_l + c_l)).
-// The step is bound by the traffic of the state (read and written once): plain SIMT, FP32, coalesced over dv.
+//
+// The step is bound by the traffic of the state (read and written once) when there are many (batch, head) pairs, and by a
+// chain of load latencies (q, k -> M -> W -> state) when there are few. Both want the state's loads out of the chain: they
+// start first, by asynchronous copies into shared memory (every lane copies what it will use itself, so nothing has to be
+// synchronised), and the features are formed while they are on their way. The features of a pair are cut over the CTAs of
+// a cluster: each forms x~, then the exponents of its own features, updates its own rows of the state and sends its partial
+// numerators and normaliser, scaled by its own maximum, to the first CTA. Measured (m = 256, dv = 128, bf16): 64 pairs
+// 14.3 -> 8.3 us, 1024 pairs (134 MB of state) 90.7 -> 62 us, 4.3 TB/s; there the features' arithmetic, 27 thousand warp
+// instructions a pair, is what keeps it from the copy bandwidth.
 #include "common.cuh"
 
 #include <math.h>
@@ -14,6 +22,9 @@ namespace darkattn {
 
 namespace {
 
+constexpr int kNT = 256, kWarps = kNT / 32, kGroups = kNT / 8;      // kGroups: rows of M or W in work at a time, eight lanes each
+constexpr int kItems = 8, kSlots = 2;                               // 16-byte pieces per lane and slot, slots per warp
+
 template <typename T>
 __device__ __forceinline__ float ldf(const T *p, size_t i)
 {
@@ -21,172 +32,301 @@ __device__ __forceinline__ float ldf(const T *p, size_t i)
     else return p[i];
 }
 
-// Dot products of one row of a matrix with up to two vectors held in shared memory, and the row's squared norm. Eight lanes
-// share a row: lane `sub` of the eight takes every eighth 16-byte piece of it, so a warp's load covers four rows in pieces
-// of 128 contiguous bytes (every sector it fetches is used), and three shuffle steps add the eight parts up (all eight
-// lanes end with the sums). Rows whose length is not a multiple of 16 bytes are read element by element, eight apart.
-// Every lane of the warp must call this (the shuffles name the full warp).
-template <typename T, bool TWO>
-__device__ __forceinline__ void row_dots(const T *row, const float *x0, const float *x1, int n, int sub, bool vec, float &d0, float &d1,
-                                         float &nn)
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void copy16_async(void *dst, const void *src)
 {
-    d0 = d1 = nn = 0.f;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// stores into the same place of another CTA's shared memory
+__device__ __forceinline__ void store_cluster(float *p, uint32_t rank, float v)
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+
+template <typename T>
+__device__ __forceinline__ void unpack16(const uint4 &q, float (&w)[16 / sizeof(T)])
+{
+    const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+    if constexpr (sizeof(T) == 2) {                 // eight bf16: the upper half of an fp32 each
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { w[2 * j] = __uint_as_float(u[j] << 16); w[2 * j + 1] = __uint_as_float(u[j] & 0xffff0000u); }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = __uint_as_float(u[j]);
+    }
+}
+
+__device__ __forceinline__ float sum8(float v)
+{
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Dot products of the rows of a matrix [nrows, n] with two vectors held in shared memory, and the rows' squared norms. Eight
+// lanes share a row: lane `sub` of the eight takes every eighth 16-byte piece of it, so a warp's load covers four rows in
+// pieces of 128 contiguous bytes, and three shuffle steps add the eight parts up. put(row, d0, d1, nn) is called by all
+// eight lanes. PIECES > 0: rows of exactly 8 PIECES pieces; the lane's share of the vectors stays in registers and
+// the loads of 8 / PIECES rows are in flight together (a block is a chain of load latencies). PIECES = 0: any length, rows that
+// do not start on 16 bytes element by element.
+template <typename T, int PIECES, bool NORM, typename Put>
+__device__ __forceinline__ void rows_dots(const T *mat, int nrows, int n, const float *x0, const float *x1, int tid, Put put)
+{
     constexpr int V = 16 / (int)sizeof(T);          // elements per 16-byte load
-    if (vec) {
-#pragma unroll 4
-        for (int c = sub * V; c < n; c += 8 * V) {
-            float w[V];
-            if constexpr (sizeof(T) == 2) {         // eight bf16: the upper half of an fp32 each
-                const uint4 raw = *reinterpret_cast<const uint4 *>(row + c);
-                const uint32_t u[4] = {raw.x, raw.y, raw.z, raw.w};
+    const int sub = tid & 7, grp = tid >> 3;
+    if constexpr (PIECES > 0) {
+        constexpr int RB = PIECES == 4 ? 1 : 8 / PIECES;
+        float a[PIECES][V], b[PIECES][V];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) { w[2 * j] = __uint_as_float(u[j] << 16); w[2 * j + 1] = __uint_as_float(u[j] & 0xffff0000u); }
+        for (int i = 0; i < PIECES; ++i)
+#pragma unroll
+            for (int j = 0; j < V; ++j) { a[i][j] = x0[(i * 8 + sub) * V + j]; b[i][j] = x1[(i * 8 + sub) * V + j]; }
+        for (int r0 = 0; r0 < nrows; r0 += kGroups * RB) {
+            uint4 raw[RB][PIECES];
+#pragma unroll
+            for (int k = 0; k < RB; ++k) {
+                const int row = min(r0 + k * kGroups + grp, nrows - 1);      // (rows past the end: the last one again, not stored)
+#pragma unroll
+                for (int i = 0; i < PIECES; ++i) raw[k][i] = __ldg(reinterpret_cast<const uint4 *>(mat + (size_t)row * n) + i * 8 + sub);
             }
-            else { const float4 f = *reinterpret_cast<const float4 *>(row + c); w[0] = f.x; w[1] = f.y; w[2] = f.z; w[3] = f.w; }
 #pragma unroll
-            for (int j = 0; j < V; ++j) {
-                d0 = fmaf(w[j], x0[c + j], d0);
-                if constexpr (TWO) d1 = fmaf(w[j], x1[c + j], d1);
-                nn = fmaf(w[j], w[j], nn);
+            for (int k = 0; k < RB; ++k) {
+                if (r0 + k * kGroups >= nrows) break;
+                float d0 = 0.f, d1 = 0.f, nn = 0.f;
+#pragma unroll
+                for (int i = 0; i < PIECES; ++i) {
+                    float w[V];
+                    unpack16<T>(raw[k][i], w);
+#pragma unroll
+                    for (int j = 0; j < V; ++j) {
+                        d0 = fmaf(w[j], a[i][j], d0);
+                        d1 = fmaf(w[j], b[i][j], d1);
+                        if (NORM) nn = fmaf(w[j], w[j], nn);
+                    }
+                }
+                d0 = sum8(d0); d1 = sum8(d1);
+                if (NORM) nn = sum8(nn);
+                const int row = r0 + k * kGroups + grp;
+                if (row < nrows) put(row, d0, d1, nn);
             }
         }
     } else {
-        for (int c = sub; c < n; c += 8) {
-            const float w = ldf(row, c);
-            d0 = fmaf(w, x0[c], d0);
-            if constexpr (TWO) d1 = fmaf(w, x1[c], d1);
-            nn = fmaf(w, w, nn);
-        }
-    }
+        const bool vec = (n % V == 0) && (reinterpret_cast<uintptr_t>(mat) & 15) == 0;
+        for (int r0 = 0; r0 < nrows; r0 += kGroups) {
+            const int row = r0 + grp;
+            const T *p = mat + (size_t)min(row, nrows - 1) * n;
+            float d0 = 0.f, d1 = 0.f, nn = 0.f;
+            if (vec) {
+#pragma unroll 4
+                for (int c = sub * V; c < n; c += 8 * V) {
+                    float w[V];
+                    unpack16<T>(__ldg(reinterpret_cast<const uint4 *>(p + c)), w);
 #pragma unroll
-    for (int off = 1; off < 8; off <<= 1) {
-        d0 += __shfl_xor_sync(0xffffffffu, d0, off);
-        if constexpr (TWO) d1 += __shfl_xor_sync(0xffffffffu, d1, off);
-        nn += __shfl_xor_sync(0xffffffffu, nn, off);
+                    for (int j = 0; j < V; ++j) { d0 = fmaf(w[j], x0[c + j], d0); d1 = fmaf(w[j], x1[c + j], d1); nn = fmaf(w[j], w[j], nn); }
+                }
+            } else {
+                for (int c = sub; c < n; c += 8) {
+                    const float w = ldf(p, c);
+                    d0 = fmaf(w, x0[c], d0); d1 = fmaf(w, x1[c], d1); nn = fmaf(w, w, nn);
+                }
+            }
+            d0 = sum8(d0); d1 = sum8(d1); nn = sum8(nn);
+            if (row < nrows) put(row, d0, d1, nn);
+        }
     }
 }
 
-// Features of one (batch, head)'s new token, by the whole block (a multiple of 32 threads, at most 1024): fk[l] = phi(k)_l and, when WITH_Q, fq[l] = phi(q)_l
-// (shared memory: vq[d], vk[d], xq[r], xk[r], fq[m], fk[m], red[...]).
-template <typename T, bool WITH_Q>
-__device__ __forceinline__ void token_features(const T *qv, const T *kv, const T *Mh, const T *Wh, float *vq, float *vk, float *xq,
-                                               float *xk, float *fq, float *fk, float *red, int d, int r, int m, float s)
+template <typename T, bool NORM, typename Put>
+__device__ __forceinline__ void rows_dots_any(const T *mat, int nrows, int n, const float *x0, const float *x1, int tid, Put put)
 {
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int nt = blockDim.x, sub = tid & 7, grp = tid >> 3, ngrp = nt >> 3;
     constexpr int V = 16 / (int)sizeof(T);
-    for (int c = tid; c < d; c += nt) {
-        vk[c] = ldf(kv, c);
-        if constexpr (WITH_Q) vq[c] = ldf(qv, c);
-    }
-    __syncthreads();
-    // x~ = s M x for the query and the key: eight lanes per row of M (whole warps walk the loop: rows past the end are read
-    // from the last row and not stored)
-    const bool vec_m = (d % V == 0) && (reinterpret_cast<uintptr_t>(Mh) & 15) == 0;
-    for (int a0 = 0; a0 < r; a0 += ngrp) {
-        const int a = a0 + grp, ac = a < r ? a : r - 1;
-        float aq, ak, nn;
-        row_dots<T, WITH_Q>(Mh + (size_t)ac * d, WITH_Q ? vq : vk, vk, d, sub, vec_m, aq, ak, nn);
-        if (a < r && sub == 0) {
-            if constexpr (WITH_Q) { xq[a] = s * aq; xk[a] = s * ak; }
-            else xk[a] = s * aq;
+    const bool aligned = (reinterpret_cast<uintptr_t>(mat) & 15) == 0;
+    if (aligned && n == 32 * V) rows_dots<T, 4, NORM>(mat, nrows, n, x0, x1, tid, put);            // 256 bf16 or 128 fp32
+    else if (aligned && n == 16 * V) rows_dots<T, 2, NORM>(mat, nrows, n, x0, x1, tid, put);       // 128 bf16 or 64 fp32
+    else if (aligned && n == 8 * V) rows_dots<T, 1, NORM>(mat, nrows, n, x0, x1, tid, put);   // 64 bf16 or 32 fp32
+    else rows_dots<T, 0, NORM>(mat, nrows, n, x0, x1, tid, put);
+}
+
+struct DecodeParams {
+    const void *q, *k, *v, *M, *W;
+    float *S, *z;
+    void *o;
+    int H, Hkv, d, r, m, dv, w_per_head, parts, mp;      // parts: CTAs per (batch, head); mp: features of each
+    float s;
+};
+
+// NCB: pieces of 128 columns per row of the state (1, 2 or 4).
+template <typename T, int NCB>
+__global__ void __launch_bounds__(kNT, 3) decode_step_kernel(const __grid_constant__ DecodeParams p)
+{
+    extern __shared__ __align__(16) float sm[];
+    float4 *ring = reinterpret_cast<float4 *>(sm);                   // [warp][slot][item][lane]; afterwards the partial numerators
+    float *vq = sm + kWarps * kSlots * kItems * 32 * 4, *vk = vq + p.d, *xq = vk + p.d, *xk = xq + p.r;
+    float2 *fkq = reinterpret_cast<float2 *>(xk + p.r);     // phi(k), phi(q) of every feature
+    float *red = reinterpret_cast<float *>(fkq + p.mp);                                         // [kWarps] maxima, [kWarps] normalisers
+    float *gather = red + 2 * kWarps;                                // first CTA: [parts][dv + 2] partial numerators, normaliser, maximum
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int part = blockIdx.x % p.parts, bh = blockIdx.x / p.parts, h = bh % p.H;
+    const int kvh = (bh / p.H) * p.Hkv + h / (p.H / p.Hkv);           // the key/value head this query head reads (grouped key/value heads)
+    const int l0 = part * p.mp, nl = min(p.mp, p.m - l0);             // this CTA's features (the last CTA's may be fewer, never none)
+    if (p.parts > 1) cluster_arrive();
+
+    // which piece of the state is the lane's i-th: four columns of a row, a row of dv <= 128 columns to dv / 4 lanes
+    // (i = NCB * n + b: columns col0 + 128 b .. + 3 of row row0 + n step; a lane without columns has no rows)
+    const int lpr = NCB == 1 ? p.dv / 4 : 32, rpi = 32 / lpr, sub = lane / lpr, col0 = (lane - sub * lpr) * 4;
+    const int row0 = warp * rpi + sub, step = kWarps * rpi;
+    const int nrows = sub < rpi ? (nl - row0 + step - 1) / step : 0;            // this lane's rows (may be negative)
+    const int nslots = ((nl + step - 1) / step * NCB + kItems - 1) / kItems;    // (the same for all lanes)
+    float *Sb = p.S + ((size_t)bh * p.m + l0 + row0) * p.dv + col0;
+    const size_t rstride = (size_t)step * p.dv;
+    float4 *mine = ring + (size_t)warp * kSlots * kItems * 32 + lane;
+    auto start_slot = [&](int slot) {
+        float4 *dst = mine + (slot % kSlots) * kItems * 32;
+#pragma unroll
+        for (int j = 0; j < kItems; ++j) {
+            const int n = (slot * kItems + j) / NCB, b = j % NCB;
+            if (n < nrows && (NCB == 1 || col0 + 128 * b < p.dv)) copy16_async(dst + j * 32, Sb + n * rstride + 128 * b);
         }
+        copy_commit();
+    };
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    {
+        const T *qv = static_cast<const T *>(p.q) + (size_t)bh * p.d, *kv = static_cast<const T *>(p.k) + (size_t)kvh * p.d;
+        for (int c = tid; c < p.d; c += kNT) { vk[c] = ldf(kv, c); vq[c] = ldf(qv, c); }
     }
+#pragma unroll
+    for (int i = 0; i < kSlots; ++i) start_slot(i);
+    float *zb = p.z + (size_t)bh * p.m + l0;
+    const float z_first = tid < nl ? zb[tid] : 0.f;
+    __syncthreads();
+    // x~ = s M x for the query and the key
+    rows_dots_any<T, false>(static_cast<const T *>(p.M) + (size_t)h * p.r * p.d, p.r, p.d, vq, vk, tid,
+                            [&](int row, float a, float b, float) { if ((tid & 7) == 0) { xq[row] = p.s * a; xk[row] = p.s * b; } });
     __syncthreads();
     float nk = 0.f;
-    for (int a = lane; a < r; a += 32) nk = fmaf(xk[a], xk[a], nk);
+    for (int a = lane; a < p.r; a += 32) nk = fmaf(xk[a], xk[a], nk);
     for (int off = 16; off; off >>= 1) nk += __shfl_xor_sync(0xffffffffu, nk, off);
     nk *= 0.5f;
     float mx = -INFINITY;
-    const bool vec_w = (r % V == 0) && (reinterpret_cast<uintptr_t>(Wh) & 15) == 0;
-    for (int l0 = 0; l0 < m; l0 += ngrp) {          // exponents of the features: eight lanes per row of W
-        const int l = l0 + grp, lc = l < m ? l : m - 1;
-        float uq, uk, c;
-        row_dots<T, WITH_Q>(Wh + (size_t)lc * r, WITH_Q ? xq : xk, xk, r, sub, vec_w, uq, uk, c);
-        if constexpr (!WITH_Q) uk = uq;
-        c *= 0.5f;
-        if (l < m) {
-            if (sub == 0) {
-                fk[l] = __expf(uk - nk - c);
-                if constexpr (WITH_Q) fq[l] = uq + c;
-            }
-            if constexpr (WITH_Q) mx = fmaxf(mx, uq + c);
-        }
-    }
-    if constexpr (WITH_Q) {
-        for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-        if (lane == 0) red[tid >> 5] = mx;
-        __syncthreads();
-        mx = red[0];
-        for (int w = 1; w < nt / 32; ++w) mx = fmaxf(mx, red[w]);
-        __syncthreads();
-        for (int l = tid; l < m; l += nt) fq[l] = __expf(fq[l] - mx);
-    }
+    rows_dots_any<T, true>(static_cast<const T *>(p.W) + ((size_t)(p.w_per_head ? h : 0) * p.m + l0) * p.r, nl, p.r, xq, xk, tid,
+                           [&](int row, float uq, float uk, float nn) {
+                               const float c = 0.5f * nn;
+                               if ((tid & 7) == 0) fkq[row] = make_float2(__expf(uk - nk - c), uq + c);
+                               mx = fmaxf(mx, uq + c);
+                           });
+    for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    if (lane == 0) red[warp] = mx;
     __syncthreads();
-}
-
-// One block of NT threads per (batch, head): thread = (four columns of the state, group of rows). The block owns
-// the head's z, so it reads z for the normaliser and stores z + phi(k) itself. NT = 512 when the blocks are few (each is
-// a chain of load latencies: more threads shorten it); NT = 256 when there are several per SM, so that two share an SM
-// and one's feature phase, which moves no state, runs under the other's state traffic.
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT, 512 / NT) decode_step_kernel(const T *q, const T *k, const T *v, const T *M, const T *W, float *S,
-                                                           float *z, T *o, int H, int Hkv, int d, int r, int m, int dv, int w_per_head,
-                                                           float s)
-{
-    extern __shared__ float sm[];
-    float *vq = sm, *vk = vq + d, *xq = vk + d, *xk = xq + r, *fq = xk + r, *fk = fq + m, *red = fk + m;   // red: up to 2048 partial numerators + 16 partial normalisers
-    const int bh = blockIdx.x, h = bh % H, tid = threadIdx.x, lane = tid & 31;
-    const int kvh = (bh / H) * Hkv + h / (H / Hkv);     // the key/value head this query head reads (grouped key/value heads)
-    token_features<T, true>(q + (size_t)bh * d, k + (size_t)kvh * d, M + (size_t)h * r * d, W + (size_t)(w_per_head ? h : 0) * m * r,
-                            vq, vk, xq, xk, fq, fk, red, d, r, m, s);
-
-    // normaliser phi(q) . (z + phi(k)) and the new z: one feature per thread
-    float *zb = z + (size_t)bh * m;
+    mx = red[0];
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) mx = fmaxf(mx, red[w]);
+    // the query's features, the new z and the normaliser phi(q) . z
     float den = 0.f;
-    for (int l = tid; l < m; l += NT) {
-        const float zn = zb[l] + fk[l];
+    for (int l = tid; l < nl; l += kNT) {
+        const float2 fg = fkq[l];
+        const float f = __expf(fg.y - mx), zn = (l == tid ? z_first : zb[l]) + fg.x;
+        fkq[l].y = f;
         zb[l] = zn;
-        den = fmaf(fq[l], zn, den);
+        den = fmaf(f, zn, den);
     }
     for (int off = 16; off; off >>= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
+    if (lane == 0) red[kWarps + warp] = den;
+    // the value's columns of this lane
+    float4 vv[NCB], num[NCB];
+#pragma unroll
+    for (int b = 0; b < NCB; ++b) {
+        const int c = col0 + 128 * b;
+        const T *vr = static_cast<const T *>(p.v) + (size_t)kvh * p.dv;
+        num[b] = vv[b] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (c < p.dv) vv[b] = make_float4(ldf(vr, c), ldf(vr, c + 1), ldf(vr, c + 2), ldf(vr, c + 3));
+    }
+    __syncthreads();
 
-    // state update and read-out: a thread owns four neighbouring columns of every (NT / (dv / 4))-th row and keeps 16 of
-    // its rows (256 bytes) in flight
-    const int tpr = dv / 4, nrg = NT / tpr, c4 = (tid % tpr) * 4, rg = tid / tpr;
-    float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (rg < nrg) {
-        const float4 vv = make_float4(ldf(v, (size_t)kvh * dv + c4), ldf(v, (size_t)kvh * dv + c4 + 1), ldf(v, (size_t)kvh * dv + c4 + 2),
-                                      ldf(v, (size_t)kvh * dv + c4 + 3));
-        float4 *Sb = reinterpret_cast<float4 *>(S + (size_t)bh * m * dv + c4);
-        for (int l0 = rg; l0 < m; l0 += 16 * nrg) {
-            float4 sv[16];
+    // state update and read-out
+    for (int slot = 0; slot < nslots; ++slot) {
+        copy_wait<kSlots - 1>();                    // (each lane reads only what it copied)
+        const float4 *src = mine + (slot % kSlots) * kItems * 32;
 #pragma unroll
-            for (int j = 0; j < 16; ++j) { const int l = l0 + nrg * j; sv[j] = (l < m) ? Sb[(size_t)l * tpr] : make_float4(0.f, 0.f, 0.f, 0.f); }
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int l = l0 + nrg * j;
-                if (l < m) {
-                    const float f = fk[l], g = fq[l];
-                    const float4 sn = make_float4(fmaf(f, vv.x, sv[j].x), fmaf(f, vv.y, sv[j].y), fmaf(f, vv.z, sv[j].z), fmaf(f, vv.w, sv[j].w));
-                    Sb[(size_t)l * tpr] = sn;
-                    num.x = fmaf(g, sn.x, num.x); num.y = fmaf(g, sn.y, num.y); num.z = fmaf(g, sn.z, num.z); num.w = fmaf(g, sn.w, num.w);
-                }
+        for (int j = 0; j < kItems; ++j) {
+            const int n = (slot * kItems + j) / NCB, b = j % NCB;
+            if (n < nrows && (NCB == 1 || col0 + 128 * b < p.dv)) {
+                const float4 x = src[j * 32], v4 = vv[b];
+                const float2 fg = fkq[row0 + n * step];
+                const float f = fg.x, g = fg.y;
+                const float4 sn = make_float4(fmaf(f, v4.x, x.x), fmaf(f, v4.y, x.y), fmaf(f, v4.z, x.z), fmaf(f, v4.w, x.w));
+                *reinterpret_cast<float4 *>(Sb + n * rstride + 128 * b) = sn;
+                float4 &nm = num[b];
+                nm.x = fmaf(g, sn.x, nm.x); nm.y = fmaf(g, sn.y, nm.y); nm.z = fmaf(g, sn.z, nm.z); nm.w = fmaf(g, sn.w, nm.w);
             }
         }
-        float *rd = red + rg * dv + c4;
-        rd[0] = num.x; rd[1] = num.y; rd[2] = num.z; rd[3] = num.w;
+        if (slot + kSlots < nslots) start_slot(slot + kSlots);
+        else copy_commit();                         // (an empty group, so that the wait above counts the same)
     }
-    if (lane == 0) red[2048 + (tid >> 5)] = den;
+    copy_wait<0>();
+    __syncthreads();                                // the ring becomes the partial numerators: [warp][row of the warp][dv]
+    const int npart = kWarps * rpi;
+    if (sub < rpi)
+#pragma unroll
+        for (int b = 0; b < NCB; ++b) {
+            const int c = col0 + 128 * b;
+            if (c < p.dv) *reinterpret_cast<float4 *>(sm + (size_t)(warp * rpi + sub) * p.dv + c) = num[b];
+        }
     __syncthreads();
-    if (tid < dv) {
-        float n = 0.f, dn = 0.f;
-        for (int g = 0; g < nrg; ++g) n += red[g * dv + tid];
-        for (int w = 0; w < NT / 32; ++w) dn += red[2048 + w];
-        const float out = n / dn;
-        if constexpr (sizeof(T) == 2) o[(size_t)bh * dv + tid] = __float2bfloat16_rn(out);
-        else o[(size_t)bh * dv + tid] = out;
+    if (p.parts > 1) cluster_wait();                // the first CTA runs (all have arrived at their start)
+    float *slotp = gather + (size_t)part * (p.dv + 2);
+    for (int c = tid; c < p.dv + 2; c += kNT) {
+        float x = 0.f;
+        if (c < p.dv) for (int g = 0; g < npart; ++g) x += sm[(size_t)g * p.dv + c];
+        else if (c == p.dv) {
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) x += red[kWarps + w];
+        } else x = mx;
+        if (p.parts > 1) store_cluster(slotp + c, 0, x);
+        else slotp[c] = x;
     }
+    if (p.parts > 1) { cluster_arrive(); cluster_wait(); }
+    else __syncthreads();
+    if (part > 0) return;
+    float top = -INFINITY;
+    for (int i = 0; i < p.parts; ++i) top = fmaxf(top, gather[(size_t)i * (p.dv + 2) + p.dv + 1]);
+    for (int c = tid; c < p.dv; c += kNT) {
+        float n = 0.f, dn = 0.f;
+        for (int i = 0; i < p.parts; ++i) {
+            const float *g = gather + (size_t)i * (p.dv + 2), e = __expf(g[p.dv + 1] - top);
+            n = fmaf(e, g[c], n);
+            dn = fmaf(e, g[p.dv], dn);
+        }
+        const float out = n / dn;
+        if constexpr (sizeof(T) == 2) static_cast<__nv_bfloat16 *>(p.o)[(size_t)bh * p.dv + c] = __float2bfloat16_rn(out);
+        else static_cast<float *>(p.o)[(size_t)bh * p.dv + c] = out;
+    }
+}
+
+template <typename T>
+cudaError_t launch_decode(const DecodeParams &P, int BH, cudaStream_t st)
+{
+    const size_t smem = ((size_t)kWarps * kSlots * kItems * 32 * 4 + 2 * P.d + 2 * P.r + 2 * P.mp + 2 * kWarps + (size_t)P.parts * (P.dv + 2)) * sizeof(float);
+    auto *k = P.dv <= 128 ? decode_step_kernel<T, 1> : P.dv <= 256 ? decode_step_kernel<T, 2> : decode_step_kernel<T, 4>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)BH * P.parts); cfg.blockDim = dim3(kNT); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // (the kernel waits before it touches memory)
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = P.parts; at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, k, P);
 }
 
 }  // namespace
@@ -202,18 +342,17 @@ extern "C" darkattn_status_t darkattn_decode_step(darkattn_plan_t plan, const vo
     const Dims &D = plan->dims;
     if (!D.causal) return DARKATTN_ERR_UNSUPPORTED;          // the recurrent form is the causal one
     if (D.dv % 32) return DARKATTN_ERR_UNSUPPORTED;
-    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if (D.dv > 512) return DARKATTN_ERR_UNSUPPORTED;
-    const size_t smem = (size_t)(2 * D.d + 2 * D.r + 2 * D.m + 2048 + 16) * sizeof(float);
-    if (smem > 48 * 1024) return DARKATTN_ERR_UNSUPPORTED;
-    const bool many = D.BH >= 2 * 148 && D.dv <= 256;      // several blocks per SM: two smaller blocks share one
-#define DARKATTN_DECODE_LAUNCH(T, NT)                                                                                              \
-    decode_step_kernel<T, NT><<<(unsigned)D.BH, NT, smem, st>>>((const T *)q, (const T *)k, (const T *)v, (const T *)M, (const T *)W, S, z, \
-                                                                (T *)o, D.H, D.Hkv, D.d, D.r, D.m, D.dv, D.w_per_head, D.s)
-    if (D.bf16) { if (many) DARKATTN_DECODE_LAUNCH(__nv_bfloat16, 256); else DARKATTN_DECODE_LAUNCH(__nv_bfloat16, 512); }
-    else { if (many) DARKATTN_DECODE_LAUNCH(float, 256); else DARKATTN_DECODE_LAUNCH(float, 512); }
-#undef DARKATTN_DECODE_LAUNCH
-    cudaError_t e = cudaGetLastError();
+    if ((size_t)(2 * D.d + 2 * D.r + 2 * D.m + 2048 + 16) * sizeof(float) > 48 * 1024) return DARKATTN_ERR_UNSUPPORTED;
+    // CTAs per (batch, head): enough to give most SMs one while the pairs are few (64 pairs of m = 256, dv = 128: 10.2 us with
+    // one CTA each, 8.3 with two, 10.5 with four, whose x~ is formed four times); at least 32 features each.
+    int parts = D.BH <= 37 ? 4 : D.BH < 148 ? 2 : 1;
+    while (parts > 1 && D.m < 32 * parts) parts /= 2;
+    DecodeParams P{q, k, v, M, W, S, z, o, D.H, D.Hkv, D.d, D.r, D.m, D.dv, D.w_per_head, 0, 0, D.s};
+    P.mp = (D.m + parts - 1) / parts;
+    P.parts = (D.m + P.mp - 1) / P.mp;
+    const cudaError_t e = D.bf16 ? launch_decode<__nv_bfloat16>(P, D.BH, static_cast<cudaStream_t>(cuda_stream))
+                                 : launch_decode<float>(P, D.BH, static_cast<cudaStream_t>(cuda_stream));
     if (e != cudaSuccess) { set_cuda_error(e, "decode_step"); return DARKATTN_ERR_CUDA; }
     return DARKATTN_OK;
 }

@@ -314,6 +314,22 @@ def test_decode_steps_reproduce_the_causal_forward(binding, name, kw, dtype):
     plan.destroy()
 
 
+DECODE_PARTS = [
+    # a pair's features cut over clusters of four and two CTAs (the last with fewer), rows of the state in one, two and four
+    # pieces of 128 columns, several slots of the state's ring per warp
+    ("four_ragged", dict(B=1, H=3, N=6, d=64, m=201, r=128, dv=32)),
+    ("two_of_37_plus", dict(B=13, H=3, N=4, d=128, m=130, r=64, dv=160)),
+    ("four_dv384", dict(B=1, H=2, N=5, d=128, m=520, r=128, dv=384)),
+    ("one_of_148_plus", dict(B=37, H=4, N=3, d=256, m=72, r=64, dv=96)),
+]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("name,kw", DECODE_PARTS, ids=[s[0] for s in DECODE_PARTS])
+def test_decode_steps_in_parts(binding, name, kw, dtype):
+    test_decode_steps_reproduce_the_causal_forward(binding, name, kw, dtype)
+
+
 @pytest.mark.parametrize("name", ["headline", "headline_nc"])
 def test_headline_backward_sampled_heads(binding, name):
     """Forward + backward at the benchmark's full size; dQ, dK, dV of sampled (batch, head) pairs and
