@@ -183,7 +183,8 @@ darkattn_status_t darkattn_selftest_wait_limit(int32_t *device_status, double *s
  * image: every GPU that loads the library holds that much memory until the process exits.
  *
  *  - The caller still passes Q, K, V, M, W (inputs) and O (output), laid out as for darkattn_forward.
- *  - darkattn_static_scratch_needed(plan) tells how much of the array a plan would use. A plan that
+ *  - darkattn_static_scratch_needed(plan) tells how much of the array a plan would use (when all
+ *    heads of the batch together need more than the array, they are computed one after the other). A plan that
  *    needs more than DARKATTN_STATIC_SCRATCH_BYTES is refused with DARKATTN_ERR_WORKSPACE before
  *    anything touches the GPU; use darkattn_forward with a workspace of your own for it.
  *  - The first call on each device looks up the array's device address (with that device current).
@@ -198,7 +199,7 @@ darkattn_status_t darkattn_selftest_wait_limit(int32_t *device_status, double *s
  *  - All calls on a device share the one array, and it keeps the previous call's contents; the call
  *    clears the words that must start at zero itself. Two calls whose GPU work overlaps (different
  *    streams, or different host threads) race on the array: serialise them on one stream.         */
-#define DARKATTN_STATIC_SCRATCH_BYTES (16u << 20)
+#define DARKATTN_STATIC_SCRATCH_BYTES (32u << 20)
 size_t darkattn_static_scratch_needed(darkattn_plan_t plan);
 darkattn_status_t darkattn_forward_static(darkattn_plan_t plan, const void *Q, const void *K, const void *V,
                                           const void *M, const void *W, void *O, void *cuda_stream);

@@ -28,7 +28,7 @@ EXPORTS = [
 ]
 # instruments of the benchmark, in a library of their own (include/darkattn_bench.h)
 BENCH_EXPORTS = ["darkattn_plan_launches", "darkattn_kernel_timing", "darkattn_kernel_times", "darkattn_measure_mma_cycles"]
-STATIC_SCRATCH_BYTES = 16 << 20
+STATIC_SCRATCH_BYTES = 32 << 20
 
 
 class Desc(ctypes.Structure):

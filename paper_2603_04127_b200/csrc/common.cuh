@@ -25,29 +25,33 @@ struct Dims {
     float s;         // sqrt(scale), applied to Mq and to Mk
 };
 
-// Offsets (bytes) into the caller's workspace of the FP32 path's intermediates (all fp32).
+// Offsets (bytes) into the caller's workspace of the FP32 path's intermediates. "planes": fp32 numbers as three bf16 parts,
+// [3][batch][rows][width rounded up to 8]; the others are fp32.
 struct SimtLayout {
     size_t status;                 // device status word (first 256 bytes)
-    size_t xtQ, xtK;               // x~            [BH, N, r]
-    size_t nK;                     // sums of squares of x~_K's rows, one per 128 columns  [ceil(r/128), BH, N]
-    size_t fQ, fK;                 // exponents, then features  [BH, N, m]
-    size_t cK;                     // per-feature key shift, order keys  [BH, m]
-    size_t Sloc, zloc;             // causal: state of every chunk, then before it; else of every token block, the first then holds the sum
-                                   // [BH, nb, m, dv], [BH, nb, m]
-    size_t P;                      // masked intra-chunk kernel  [BH, nc, C, C]   (causal)
+    size_t in[5];                  // Q, K, V, M, W as planes (one plane when bf16), where they cannot be read as they are
+    bool conv[5];
+    size_t xtQ, xtK;               // x~            planes [BH, N, r]
+    size_t nK;                     // sums of squares of x~_K's rows, one per 32 columns  [4 ceil(r/128), BH, N]
+    size_t rmax;                   // maxima of the query exponents' rows, one per 32 columns  [4 ceil(m/128), BH, N]
+    size_t cK;                     // per-feature key shift, order keys  [BH, m4]  (m4: m rounded up to 4)
+    size_t fQ, fK;                 // features      planes [BH, N, m]
+    size_t Sloc, zloc;             // state of every chunk or token block  [BH, nb, m, dv], [BH, nb, m4]; z then before the chunk, or the sum
+    size_t Sp;                     // causal: state before every chunk, else their sum   planes [BH, nb or 1, m, dv]
+    size_t P;                      // masked intra-chunk kernel  planes [BH, nb, 128, 128]   (causal)
     // backward only
-    size_t Ga;                     // dO / den      [BH, N, dv]
-    size_t gd;                     // -(dO . O) / den, one part per 128 columns  [ceil(dv/128), BH, N]
-    size_t dP;                     // [BH, nc, C, C]             (causal)
-    size_t Rloc, rloc;             // reverse states, as Sloc and zloc
-    size_t dA, dBf;                // E = feature gradients times features  [BH, N, m]
-    size_t esK;                    // rowsum(E_K), one part per 128 columns  [ceil(m/128), BH, N]
-    size_t dxtQ, dxtK;             // dx~                        [BH, N, r]
+    size_t Ga;                     // dO / den      planes [BH, N, dv]
+    size_t gd;                     // -(dO . O) / den, one part per 32 columns  [4 ceil(dv/128), BH, N]
+    size_t dP;                     // planes [BH, nb, 128, 128]  (causal)
+    size_t Rloc, rloc, Rp;         // reverse states, as Sloc, zloc, Sp
+    size_t dA, dBf;                // E = feature gradients times features  planes [BH, N, m]
+    size_t esK;                    // rowsum(E_K), one part per 32 columns  [4 ceil(m/128), BH, N]
+    size_t dxtQ, dxtK;             // dx~           planes [BH, N, r]
     size_t dKh, dVh;               // grouped key/value heads: dK and dV per query head  [BH, N, d], [BH, N, dv]
     size_t dMp;                    // dM per (b,h) and token block  [BH, nsM, r, d]
     size_t dWp;                    // dW per (b,h) and token block  [BH, nsW, m, r]
-    size_t fwd_bytes, total_bytes;
-    int C, nb, blk;                // tokens per chunk (causal) or block, blocks per (b,h)
+    size_t bytes;
+    int nb, blk;                   // chunks or token blocks per (b,h), tokens in each
     int nsM, nsW, blkM, blkW;      // token blocks of the dM and dW products, tokens in each
 };
 
@@ -140,7 +144,7 @@ struct darkattn_plan_s {
     darkattn_desc_t desc;
     darkattn::Dims dims;
     int path;                      // resolved DARKATTN_PATH_*
-    darkattn::SimtLayout simt;
+    darkattn::SimtLayout simt, simt_fwd;   // with the backward pass; forward pass alone
     darkattn::TensorLayout tensor;
     size_t workspace_bytes;
     size_t saved_bytes;
@@ -170,6 +174,7 @@ void timer_mark(const darkattn_plan_s *plan, cudaStream_t st, const char *name);
 
 // FP32 path (products of split operands on the tensor cores)
 void simt_make_layout(darkattn_plan_s *plan);
+void simt_launches(const darkattn_plan_s *plan, int &fwd, int &bwd);     // kernels of a forward and of a backward call
 darkattn_status_t simt_forward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
                                const void *M, const void *W, void *O, char *ws, cudaStream_t st);
 darkattn_status_t simt_backward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,

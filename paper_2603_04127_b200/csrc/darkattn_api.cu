@@ -73,13 +73,9 @@ darkattn_status_t darkattn_plan(const darkattn_desc_t *desc, darkattn_plan_t *ou
     p->path = path;
 
     simt_make_layout(p);
-    p->workspace_bytes = p->simt.total_bytes;
+    p->workspace_bytes = p->simt.bytes > p->simt_fwd.bytes ? p->simt.bytes : p->simt_fwd.bytes;
     p->saved_bytes = 0;
-    {
-        const int scan = (D.causal || p->simt.nb > 1) ? 1 : 0;
-        p->launches_fwd = 5 + scan;
-        p->launches_bwd = 5 + scan + 1 + scan + 4 + (D.G > 1 ? 2 : 0);
-    }
+    simt_launches(p, p->launches_fwd, p->launches_bwd);
     if (path == DARKATTN_PATH_TENSOR) tensor_make_layout(p);
     *out = p;
     return DARKATTN_OK;

@@ -2,19 +2,23 @@
 //
 // This is the path that meets the 1e-4 tolerance (a single bf16 or TF32 operand rounds the argument of the exponential
 // too coarsely), and the path that accepts any shape. Its products run on the tensor cores with every fp32 operand split
-// into three bf16 numbers (split_gemm.cu); what surrounds them is done on the way into or out of a product, so that the
-// intermediates are written once and read by the next product:
-//   forward    x~ = s X M^T (both sides; row norms of the keys) | u = x~ W^T (keys: minus the norm; column maxima) |
-//              features in place | chunk states and masked kernel tiles | prefix over the chunks | output rows
+// into three bf16 numbers (split_gemm.cu); what surrounds them is done on the way out of a product, and intermediates are
+// written as the bf16 parts that the next product reads:
+//   forward    inputs into parts (fp32, or rows that do not start on 16 bytes) | x~ = s X M^T (row norms of the keys) |
+//              key shifts c_l = max_j (u_jl - n_j), from the large parts alone | row maxima of the query exponents, likewise
+//              (several tiles of features) | features phi = exp(x~ W^T ...) | chunk states and masked kernel tiles |
+//              prefix over the chunks | output rows
 //   backward   the forward steps with the output rows turned into dO / den and -delta / den | dP and the reverse states |
 //              suffix over the chunks | E of both sides and dV | dx~ | dQ, dK and dM | sums over batch and token blocks
 // Each line's items between bars are one launch each; all but the first start while the one before drains
-// (programmatic dependent launch).
+// (programmatic dependent launch). Chunks are 128 tokens, a tile's rows, whatever chunk length the descriptor names (the
+// result does not depend on it).
 //
 // Stabiliser (cancels in O): keys use one shift per (batch, head, feature), c_l = max_j (u_jl - n_j),
 // queries use e_il = u_il + c_l - max_l(u_il + c_l); the query's own norm term is a per-row constant
 // and is dropped (so is its gradient, which is zero). The product phi(q_i)_l phi(k_j)_l is then the unshifted one times
-// a per-row factor.
+// a per-row factor. Any constants near these maxima serve, so the maxima are taken from one bf16 product (x~'s and W's large
+// parts: off by a few 2^-9 of the terms' size); the features themselves use the whole of both.
 #include "common.cuh"
 #include "split_gemm.cuh"
 #include "tc_common.cuh"
@@ -24,100 +28,131 @@
 namespace darkattn {
 
 using sg::launch_pdl;
+using sg::Mat;
 
 namespace {
 
-// Features in place, one warp per row: query rows exp(u_l + c_l - max_l(u_l + c_l)), key rows exp(u_l - c_l) (u already
-// has the key's norm taken off). V: elements per load. A row is read twice (the second time from L1 or L2).
-template <int V>
-__global__ void __launch_bounds__(256) features_kernel(float *fQ, float *fK, const int *cK, int N, int m, long long rows)
+inline int tiles(int n) { return (n + 127) / 128; }
+inline int up4(int n) { return (n + 3) & ~3; }
+inline int up8(int n) { return (n + 7) & ~7; }
+
+// Inputs into bf16 planes with rows a multiple of 8 apart: three of an fp32 tensor, one of a bf16 tensor. A thread handles eight
+// columns of a row.
+struct SplitJob { const void *in; __nv_bfloat16 *out; int w, ld, vec; long long rows, first; };     // first: threads of the jobs before
+struct SplitJobs { SplitJob j[5]; int n; long long total; };
+
+template <typename T>
+__global__ void __launch_bounds__(256) split_inputs_kernel(const __grid_constant__ SplitJobs J)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
-    const long long w = (blockIdx.x * 256LL + threadIdx.x) / 32;
-    const int lane = threadIdx.x & 31;
-    if (w >= 2 * rows) return;
-    const bool keys = w >= rows;
-    const long long row = keys ? w - rows : w;
-    float *f = (keys ? fK : fQ) + row * m;
-    const int *c = cK + row / N * m;
-    float mx = 0.f;
-    auto load = [&](int l, float (&x)[V], float (&s)[V]) {
-        if constexpr (V == 4) {
-            const float4 a = *reinterpret_cast<const float4 *>(f + l);
-            const int4 k = __ldg(reinterpret_cast<const int4 *>(c + l));
-            x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
-            s[0] = tc::float_from_order_key(k.x); s[1] = tc::float_from_order_key(k.y); s[2] = tc::float_from_order_key(k.z); s[3] = tc::float_from_order_key(k.w);
-        } else { x[0] = f[l]; s[0] = tc::float_from_order_key(__ldg(c + l)); }
-    };
-    if (!keys) {
-        mx = -INFINITY;
-        for (int l = lane * V; l < m; l += 32 * V) {
-            float x[V], s[V];
-            load(l, x, s);
+    for (long long i = blockIdx.x * 256LL + threadIdx.x; i < J.total; i += gridDim.x * 256LL) {
+        int k = 0;
+        while (k + 1 < J.n && i >= J.j[k + 1].first) ++k;
+        const SplitJob &b = J.j[k];
+        const long long e = i - b.first;
+        const int per = b.ld / 8, c = (int)(e % per) * 8;
+        const long long row = e / per;
+        const T *src = static_cast<const T *>(b.in) + row * b.w + c;
+        __nv_bfloat16 *dst = b.out + row * b.ld + c;
+        if constexpr (sizeof(T) == 2) {
+            for (int j = 0; j < 8; ++j) dst[j] = c + j < b.w ? src[j] : __float2bfloat16_rn(0.f);
+        } else {
+            float x[8];
+            if (b.vec) {
+                const float4 a = *reinterpret_cast<const float4 *>(src), d = *(reinterpret_cast<const float4 *>(src) + 1);
+                x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = d.x; x[5] = d.y; x[6] = d.z; x[7] = d.w;
+            } else {
 #pragma unroll
-            for (int j = 0; j < V; ++j) mx = fmaxf(mx, x[j] + s[j]);
+                for (int j = 0; j < 8; ++j) x[j] = c + j < b.w ? src[j] : 0.f;
+            }
+#pragma unroll
+            for (int pl = 0; pl < 3; ++pl) {
+                uint32_t u[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    u[j] = tc::pack_bf16(x[2 * j], x[2 * j + 1]);
+                    x[2 * j] -= __uint_as_float(u[j] << 16);
+                    x[2 * j + 1] -= __uint_as_float(u[j] & 0xffff0000u);
+                }
+                *reinterpret_cast<uint4 *>(dst + pl * b.rows * b.ld) = make_uint4(u[0], u[1], u[2], u[3]);
+            }
         }
-        for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    }
-    for (int l = lane * V; l < m; l += 32 * V) {
-        float x[V], s[V];
-        load(l, x, s);
-#pragma unroll
-        for (int j = 0; j < V; ++j) x[j] = expf(keys ? x[j] - s[j] : x[j] + s[j] - mx);
-        if constexpr (V == 4) *reinterpret_cast<float4 *>(f + l) = make_float4(x[0], x[1], x[2], x[3]);
-        else f[l] = x[0];
     }
 }
 
-// Over the token blocks of S[pair, block, e] and z[pair, block, l], in place: what came before each block (forward) or
-// comes after it (reverse), or the sum over all of them into the first. One thread per V neighbouring elements; eight
-// blocks' loads are in flight at a time (the sum is a serial chain, the loads are not).
+// Over the token blocks of S[pair, block, row, col]: what came before each block (forward) or comes after it (reverse), or the
+// sum over all of them, as bf16 planes Sp [3][pair, block (or one)][m][ld]; z[pair, block, m4] the same in place (the sum into the
+// first block). One thread per V neighbouring elements of a row; eight blocks' loads are in flight at a time (the sum is
+// a serial chain, the loads are not).
 enum { SCAN_FORWARD = 0, SCAN_REVERSE = 1, SCAN_TOTAL = 2 };
 template <int V>
-__global__ void __launch_bounds__(256) chunk_scan_kernel(float *S, float *z, int nb, long long E, int m, long long pairs, int mode)
+__global__ void __launch_bounds__(256) chunk_scan_kernel(const float *S, float *z, __nv_bfloat16 *Sp, int nb, int m, int dv, int ld, int m4, long long pairs, int mode)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
-    long long i = (blockIdx.x * 256LL + threadIdx.x) * V;
-    float *base;
-    long long step;
-    if (i < pairs * E) { base = S + i / E * nb * E + i % E; step = E; }
-    else {
-        i -= pairs * E;
-        if (i >= pairs * m) return;
-        base = z + i / m * nb * m + i % m;
-        step = m;
-    }
-    float run[V];
+    const long long E = (long long)m * dv;
+    long long i = blockIdx.x * 256LL + threadIdx.x;
+    const int nout = mode == SCAN_TOTAL ? 1 : nb;
+    if (i < pairs * E / V) {
+        const long long pair = i * V / E, e = i * V % E;
+        const float *src = S + pair * nb * E + e;
+        __nv_bfloat16 *dst = Sp + (pair * nout * m + e / dv) * ld + e % dv;
+        const long long dstep = (long long)m * ld, plane = pairs * nout * dstep;
+        float run[V];
 #pragma unroll
-    for (int j = 0; j < V; ++j) run[j] = 0.f;
-    for (int k0 = 0; k0 < nb; k0 += 8) {
-        float x[8][V];
+        for (int j = 0; j < V; ++j) run[j] = 0.f;
+        auto emit = [&](__nv_bfloat16 *d) {
+            float x[V];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int c = mode == SCAN_REVERSE ? nb - 1 - (k0 + k) : k0 + k;
-            if (k0 + k < nb) {
-                if constexpr (V == 4) { const float4 a = *reinterpret_cast<const float4 *>(base + c * step); x[k][0] = a.x; x[k][1] = a.y; x[k][2] = a.z; x[k][3] = a.w; }
-                else x[k][0] = base[c * step];
+            for (int j = 0; j < V; ++j) x[j] = run[j];
+#pragma unroll
+            for (int pl = 0; pl < 3; ++pl, d += plane) {
+                if constexpr (V == 4) {
+                    const uint32_t u0 = tc::pack_bf16(x[0], x[1]), u1 = tc::pack_bf16(x[2], x[3]);
+                    *reinterpret_cast<uint2 *>(d) = make_uint2(u0, u1);
+                    x[0] -= __uint_as_float(u0 << 16); x[1] -= __uint_as_float(u0 & 0xffff0000u);
+                    x[2] -= __uint_as_float(u1 << 16); x[3] -= __uint_as_float(u1 & 0xffff0000u);
+                } else {
+                    const __nv_bfloat16 b = __float2bfloat16_rn(x[0]);
+                    *d = b;
+                    x[0] -= __bfloat162float(b);
+                }
+            }
+        };
+        for (int k0 = 0; k0 < nb; k0 += 8) {
+            float x[8][V];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int c = mode == SCAN_REVERSE ? nb - 1 - (k0 + k) : k0 + k;
+                if (k0 + k < nb) {
+                    if constexpr (V == 4) { const float4 a = __ldg(reinterpret_cast<const float4 *>(src + c * E)); x[k][0] = a.x; x[k][1] = a.y; x[k][2] = a.z; x[k][3] = a.w; }
+                    else x[k][0] = __ldg(src + c * E);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (k0 + k >= nb) break;
+                const int c = mode == SCAN_REVERSE ? nb - 1 - (k0 + k) : k0 + k;
+                if (mode != SCAN_TOTAL && k0 + k > 0) emit(dst + c * dstep);       // (the first one's state is zero and is not read)
+#pragma unroll
+                for (int j = 0; j < V; ++j) run[j] += x[k][j];
             }
         }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            if (k0 + k >= nb) break;
-            const int c = mode == SCAN_REVERSE ? nb - 1 - (k0 + k) : k0 + k;
-            if (mode != SCAN_TOTAL) {
-                if constexpr (V == 4) *reinterpret_cast<float4 *>(base + c * step) = make_float4(run[0], run[1], run[2], run[3]);
-                else base[c * step] = run[0];
-            }
-#pragma unroll
-            for (int j = 0; j < V; ++j) run[j] += x[k][j];
-        }
+        if (mode == SCAN_TOTAL) emit(dst);
+        return;
     }
-    if (mode == SCAN_TOTAL) {
-        if constexpr (V == 4) *reinterpret_cast<float4 *>(base) = make_float4(run[0], run[1], run[2], run[3]);
-        else base[0] = run[0];
+    i -= pairs * E / V;
+    if (i >= pairs * m) return;
+    float *base = z + i / m * nb * m4 + i % m;
+    float run = 0.f;
+    for (int k = 0; k < nb; ++k) {
+        float *p = base + (long long)(mode == SCAN_REVERSE ? nb - 1 - k : k) * m4;
+        const float x = *p;
+        if (mode != SCAN_TOTAL) *p = run;
+        run += x;
     }
+    if (mode == SCAN_TOTAL) base[0] = run;
 }
 
 // out[o, e] = sum of src over `n1` outer and `n2` inner slices: src[(i1 * stride1 + o) * n2 + i2, e]. dM sums over the batch
@@ -154,198 +189,216 @@ __global__ void __launch_bounds__(256) group_sum_f32_kernel(T *out, const float 
 
 struct Runner {
     const darkattn_plan_s *plan;
+    const SimtLayout &Y;
     char *ws;
     cudaStream_t st;
     bool dependent = false;         // a kernel of this call has been launched
     cudaError_t err = cudaSuccess;
+    Mat Q, K, V, M, W;
 
     const Dims &D() const { return plan->dims; }
     float *f(size_t off) const { return reinterpret_cast<float *>(ws + off); }
     void keep(cudaError_t e) { if (e != cudaSuccess && err == cudaSuccess) err = e; dependent = true; }
     void gemms(sg::Launch &L) { L.status = reinterpret_cast<int *>(ws); keep(sg::run(L, st, dependent)); }
-    template <typename... K, typename... A>
-    void kernel(void (*k)(K...), long long threads, A... args)
+    template <typename... KA, typename... A>
+    void kernel(void (*k)(KA...), long long threads, const A &...args)
     {
         // (the same division of the SM's memory as the products' kernel: a change between launches costs microseconds)
         keep(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
         keep(launch_pdl(k, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, st, dependent, args...));
     }
 
+    // ---- matrices
+    Mat planes(size_t off, long long batch, long long rows, int w) const
+    {
+        Mat m;
+        m.p = reinterpret_cast<__nv_bfloat16 *>(ws + off); m.w = w; m.ld = up8(w); m.rows = rows; m.batch = batch;
+        return m;
+    }
+    Mat tokens(size_t off, int w) const { return planes(off, D().BH, D().N, w); }
+    Mat input(int i, const void *p, long long batch, long long rows, int w) const
+    {
+        Mat m = planes(Y.in[i], batch, rows, w);
+        m.planes = D().bf16 ? 1 : 3;
+        if (!Y.conv[i]) { m.p = const_cast<__nv_bfloat16 *>(static_cast<const __nv_bfloat16 *>(p)); m.ld = w; }
+        return m;
+    }
     // ---- operands
-    // tensors [B, H (or H_kv), N, w] in the storage type; cut into blocks of `blk` tokens
-    sg::Op input(const void *p, int w, bool kv, int mn, int blk = 0) const
-    {
-        sg::Op o;
-        const long long per = (long long)D().N * w;
-        o.p = p; o.sh = per; o.sb = per * (kv ? D().Hkv : D().H); o.kv = kv; o.sc = (long long)blk * w;
-        o.ld = w; o.bf16 = D().bf16; o.mn = mn;
-        return o;
-    }
-    // fp32 intermediates [BH, N, w]
-    sg::Op rows(size_t off, int w, int mn, int blk = 0) const
-    {
-        sg::Op o;
-        const long long per = (long long)D().N * w;
-        o.p = f(off); o.sh = per; o.sb = per * D().H; o.sc = (long long)blk * w; o.ld = w; o.mn = mn;
-        return o;
-    }
-    // fp32 per block [BH, nb, rows, w] (one_block: the first block stands for all)
-    sg::Op blocks(size_t off, int nb, long long nrows, int w, int mn, bool one_block = false) const
-    {
-        sg::Op o;
-        const long long per = nrows * w;
-        o.p = f(off); o.sh = per * nb; o.sb = per * nb * D().H; o.sc = one_block ? 0 : per; o.ld = w; o.mn = mn;
-        return o;
-    }
-    // parameters M [H, r, d], W [m, r] or [H, m, r]
-    sg::Op paramM(const void *M, int mn) const
-    {
-        sg::Op o; o.p = M; o.sh = (long long)D().r * D().d; o.ld = D().d; o.bf16 = D().bf16; o.mn = mn; return o;
-    }
-    sg::Op paramW(const void *W, int mn) const
-    {
-        sg::Op o; o.p = W; o.sh = D().w_per_head ? (long long)D().m * D().r : 0; o.ld = D().r; o.bf16 = D().bf16; o.mn = mn; return o;
-    }
-    // ---- products over the whole sequence of every (batch, head)
-    sg::Prob whole() const
+    sg::Op op(const Mat &m, int batch, int mn, int tok = 0) const { sg::Op o; o.m = m; o.batch = batch; o.mn = mn; o.tok = tok; return o; }
+    sg::Op rows(const Mat &m, int mn) const { return op(m, sg::BATCH_PAIR, mn, 1); }       // token rows of the (batch, head)
+    sg::Op kv(const Mat &m, int mn) const { return op(m, sg::BATCH_KV, mn, 1); }           // ... of its key/value head
+    sg::Op block(const Mat &m, int mn) const { return op(m, sg::BATCH_BLOCK, mn); }
+    sg::Op state(const Mat &m, int mn) const { return op(m, D().causal ? sg::BATCH_BLOCK : sg::BATCH_PAIR, mn); }
+    sg::Op opM(int mn) const { return op(M, sg::BATCH_HEAD, mn); }
+    sg::Op opW(int mn) const { return op(W, D().w_per_head ? sg::BATCH_HEAD : sg::BATCH_NONE, mn); }
+    // ---- products over the whole sequence of every (batch, head), or over blocks of it
+    sg::Prob prob(int nb = 1, int blk = 0) const
     {
         sg::Prob p;
-        p.H = D().H; p.G = D().G; p.batch = D().BH; p.ntok = D().N; p.nblk = 1; p.block = 0;
+        p.H = D().H; p.G = D().G; p.batch = D().BH; p.ntok = D().N; p.nblk = nb; p.block = blk;
         return p;
     }
-    // ... or over blocks of it
-    sg::Prob blocked(int nb, int blk) const
+    sg::Prob per_chunk() const { return D().causal ? prob(Y.nb, 128) : prob(); }
+    void product(sg::Launch &L, sg::Prob &p, int s, const sg::Op &A, const sg::Op &B, int K, bool ktok = false, bool hi = false) const
     {
-        sg::Prob p = whole();
-        p.nblk = nb; p.block = blk;
-        return p;
+        sg::set_operand(L, p, 2 * s, A, hi);
+        sg::set_operand(L, p, 2 * s + 1, B, hi);
+        p.K[s] = K; p.ktok[s] = ktok;
     }
-    void out_rows(sg::Prob &p, void *o, int w, bool storage, int blk = 0) const      // [BH, N, w]
+    void out_rows(sg::Prob &p, const Mat &m) const          // [BH, N, w]
     {
-        const long long per = (long long)D().N * w;
-        p.out = o; p.osh = per; p.osb = per * D().H; p.osc = (long long)blk * w; p.old_ = w; p.obf16 = storage && D().bf16;
+        p.okind = sg::OUT_PLANES; p.out = m.p; p.old_ = m.ld; p.ops = m.ps(); p.os_pair = m.bs(); p.os_blk = (long long)p.block * m.ld;
     }
-    void out_blocks(sg::Prob &p, size_t off, int nb, long long nrows, int w) const
+    void out_blocks(sg::Prob &p, const Mat &m) const        // [BH, blocks, rows, w]
     {
-        const long long per = nrows * w;
-        p.out = f(off); p.osh = per * nb; p.osb = per * nb * D().H; p.osc = per; p.old_ = w;
+        p.okind = sg::OUT_PLANES; p.out = m.p; p.old_ = m.ld; p.ops = m.ps(); p.os_blk = m.bs(); p.os_pair = p.nblk * m.bs();
     }
+    void plain_rows(sg::Prob &p, void *o, int w, bool storage) const        // [BH, N, w]
+    {
+        p.out = o; p.old_ = w; p.os_pair = (long long)D().N * w; p.os_blk = (long long)p.block * w;
+        p.okind = storage && D().bf16 ? sg::OUT_BF16 : sg::OUT_F32;
+    }
+    void plain_blocks(sg::Prob &p, size_t off, int nb, long long nrows, int w) const       // [BH, nb, rows, w]
+    {
+        p.out = f(off); p.old_ = w; p.os_blk = nrows * w; p.os_pair = nb * p.os_blk; p.okind = sg::OUT_F32;
+    }
+    void x_planes(sg::Prob &p, const Mat &m) const { p.xkind = sg::X_PLANES; p.x = m.p; p.xld = m.ld; p.xps = m.ps(); }
+    // whether there are states at all: a causal sequence of one chunk has none
+    bool states() const { return !D().causal || Y.nb > 1; }
+    void scan(size_t S, size_t z, size_t Sp, int mode)
+    {
+        const long long E = (long long)D().m * D().dv, BH = D().BH;
+        const int ld = up8(D().dv), m4 = up4(D().m);
+        __nv_bfloat16 *out = reinterpret_cast<__nv_bfloat16 *>(ws + Sp);
+        if (D().dv % 4 == 0) kernel(chunk_scan_kernel<4>, BH * (E / 4 + D().m), (const float *)f(S), f(z), out, Y.nb, D().m, D().dv, ld, m4, BH, mode);
+        else kernel(chunk_scan_kernel<1>, BH * (E + D().m), (const float *)f(S), f(z), out, Y.nb, D().m, D().dv, ld, m4, BH, mode);
+    }
+    Mat state_planes(size_t off) const { return planes(off, (long long)D().BH * (D().causal ? Y.nb : 1), D().m, D().dv); }
 };
-
-inline int tiles(int n) { return (n + 127) / 128; }
 
 // Features, states and output rows. With dO given the rows dO / den and -delta / den are formed in place of O.
 void run_forward_stages(Runner &R, const void *Q, const void *K, const void *V, const void *M, const void *W, void *O, const void *dO)
 {
     const Dims &D = R.D();
-    const SimtLayout &Y = R.plan->simt;
-    const int N = D.N, d = D.d, r = D.r, m = D.m, dv = D.dv, C = Y.C, nb = Y.nb;
-    const long long BH = D.BH;
+    const SimtLayout &Y = R.Y;
+    const int N = D.N, d = D.d, r = D.r, m = D.m, dv = D.dv, nb = Y.nb, m4 = up4(m);
+    const long long BH = D.BH, BHkv = (long long)D.B * D.Hkv;
+    R.Q = R.input(0, Q, BH, N, d); R.K = R.input(1, K, BHkv, N, d); R.V = R.input(2, V, BHkv, N, dv);
+    R.M = R.input(3, M, D.H, r, d); R.W = R.input(4, W, D.w_per_head ? D.H : 1, m, r);
+    const Mat *in[5] = {&R.Q, &R.K, &R.V, &R.M, &R.W};
+    const void *src[5] = {Q, K, V, M, W};
+    SplitJobs J;
+    J.n = 0; J.total = 0;
+    for (int i = 0; i < 5; ++i)
+        if (Y.conv[i]) {
+            const Mat &x = *in[i];
+            J.j[J.n++] = {src[i], x.p, x.w, x.ld, x.w % 8 == 0, x.rows * x.batch, J.total};
+            J.total += x.rows * x.batch * (x.ld / 8);
+        }
+    if (J.n) {
+        const long long threads = J.total < 148LL * 8 * 256 ? J.total : 148LL * 8 * 256;
+        if (D.bf16) R.kernel(split_inputs_kernel<__nv_bfloat16>, threads, J);
+        else R.kernel(split_inputs_kernel<float>, threads, J);
+    }
+    const Mat xt[2] = {R.tokens(Y.xtQ, r), R.tokens(Y.xtK, r)}, phi[2] = {R.tokens(Y.fQ, m), R.tokens(Y.fK, m)};
+    int *cK = reinterpret_cast<int *>(R.f(Y.cK));
+    const sg::TokVec norm = {R.f(Y.nK), BH * N, 4 * tiles(r), 0.5f}, rmax = {R.f(Y.rmax), BH * N, 4 * tiles(m), 1.f};
     {   // x~ = s X M^T
         sg::Launch L;
         for (int side = 0; side < 2; ++side) {
-            sg::Prob p = R.whole();
-            p.A[0] = R.input(side ? K : Q, d, side, 0); p.B[0] = R.paramM(M, 0); p.K[0] = d;
-            p.mtok = 1; p.N = r; p.alpha = D.s;
-            R.out_rows(p, R.f(side ? Y.xtK : Y.xtQ), r, false);
-            p.chain = 1;                    // (the exponent's argument: the most sensitive)
+            sg::Prob p = R.prob();
+            R.product(L, p, 0, side ? R.kv(R.K, 0) : R.rows(R.Q, 0), R.opM(0), d);
+            p.mtok = 1; p.N = r; p.alpha = D.s; p.chain = 1;                // (the exponent's argument: the most sensitive)
             if (side) { p.epi = sg::EPI_SQUARES; p.sums = R.f(Y.nK); }
+            R.out_rows(p, xt[side]);
             sg::add(L, p);
         }
-        L.init = reinterpret_cast<int *>(R.f(Y.cK)); L.init_n = (int)(BH * m);
+        L.init = cK; L.init_n = (int)(BH * m4);
         R.gemms(L);
     }
-    {   // u = x~ W^T, for the keys minus half the squared norm of x~
+    auto exponents = [&](sg::Launch &L, int side, bool hi) {
+        sg::Prob p = R.prob();
+        R.product(L, p, 0, R.rows(xt[side], 0), R.opW(0), r, false, hi);
+        p.mtok = 1; p.N = m; p.chain = hi ? 2 : 1; p.colmax = cK; p.colkey_ld = m4;
+        return p;
+    };
+    {   // the keys' shifts
+        sg::Launch L;
+        sg::Prob p = exponents(L, 1, true);
+        p.epi = sg::EPI_COLMAX; p.row = norm;
+        sg::add(L, p);
+        R.gemms(L);
+    }
+    if (tiles(m) > 1) {     // the rows' maxima of the queries' exponents
+        sg::Launch L;
+        sg::Prob p = exponents(L, 0, true);
+        p.epi = sg::EPI_ROWMAX; p.sums = R.f(Y.rmax);
+        sg::add(L, p);
+        R.gemms(L);
+    }
+    {   // phi(Q), phi(K)
         sg::Launch L;
         for (int side = 0; side < 2; ++side) {
-            sg::Prob p = R.whole();
-            p.A[0] = R.rows(side ? Y.xtK : Y.xtQ, r, 0); p.B[0] = R.paramW(W, 0); p.K[0] = r;
-            p.mtok = 1; p.N = m; p.chain = 1;
-            R.out_rows(p, R.f(side ? Y.fK : Y.fQ), m, false);
-            if (side) {
-                p.epi = sg::EPI_KEY_EXPONENT; p.row = {R.f(Y.nK), BH * N, tiles(r), 0.5f};
-                p.colmax = reinterpret_cast<int *>(R.f(Y.cK));
-            }
+            sg::Prob p = exponents(L, side, false);
+            p.epi = side ? sg::EPI_PHI_K : sg::EPI_PHI_Q;
+            if (side) p.row = norm;
+            else if (tiles(m) > 1) p.row = rmax;
+            R.out_rows(p, phi[side]);
             sg::add(L, p);
         }
         R.gemms(L);
     }
-    if (m % 4 == 0) R.kernel(features_kernel<4>, 2 * BH * N * 32, R.f(Y.fQ), R.f(Y.fK), reinterpret_cast<const int *>(R.f(Y.cK)), N, m, BH * N);
-    else R.kernel(features_kernel<1>, 2 * BH * N * 32, R.f(Y.fQ), R.f(Y.fK), reinterpret_cast<const int *>(R.f(Y.cK)), N, m, BH * N);
+    const Mat Sp = R.state_planes(Y.Sp), P = R.planes(Y.P, BH * nb, 128, 128);
     {   // S_c = phi(K_c)^T V_c, z_c = phi(K_c)^T 1 per token block; causal: P_c = tril(phi(Q_c) phi(K_c)^T)
         sg::Launch L;
-        sg::Prob p = R.blocked(nb, Y.blk);
-        p.A[0] = R.rows(Y.fK, m, 1, Y.blk); p.B[0] = R.input(V, dv, true, 1, Y.blk); p.K[0] = N; p.ktok[0] = 1;
-        p.M = m; p.N = dv; p.dot[0] = sg::DOT_ONES; p.dot_out = R.f(Y.zloc);
-        R.out_blocks(p, Y.Sloc, nb, m, dv);
-        sg::add(L, p);
         if (D.causal) {
-            sg::Prob q = R.blocked(nb, C);
-            q.A[0] = R.rows(Y.fQ, m, 0, C); q.B[0] = R.rows(Y.fK, m, 0, C); q.K[0] = m;
+            sg::Prob q = R.prob(nb, 128);
+            R.product(L, q, 0, R.rows(phi[0], 0), R.rows(phi[1], 0), m);
             q.mtok = q.ntok_dim = 1; q.epi = sg::EPI_MASK;
-            R.out_blocks(q, Y.P, nb, C, C);
+            R.out_blocks(q, P);
             sg::add(L, q);
+        }
+        if (R.states()) {
+            sg::Prob p = R.prob(nb, Y.blk);
+            R.product(L, p, 0, R.rows(phi[1], 1), R.kv(R.V, 1), N, true);
+            p.M = m; p.N = dv; p.dot[0] = sg::DOT_ONES; p.dot_out = R.f(Y.zloc); p.dot_ld = m4;
+            if (!D.causal && nb == 1) R.out_blocks(p, Sp);
+            else R.plain_blocks(p, Y.Sloc, nb, m, dv);
+            sg::add(L, p);
         }
         R.gemms(L);
     }
-    const long long E = (long long)m * dv;
-    auto scan = [&](size_t S, size_t z, int mode) {
-        if (nb == 1 && mode == SCAN_TOTAL) return;
-        if (m % 4 == 0) R.kernel(chunk_scan_kernel<4>, BH * (E + m) / 4, R.f(S), R.f(z), nb, E, m, BH, mode);
-        else R.kernel(chunk_scan_kernel<1>, BH * (E + m), R.f(S), R.f(z), nb, E, m, BH, mode);
-    };
-    scan(Y.Sloc, Y.zloc, D.causal ? SCAN_FORWARD : SCAN_TOTAL);
+    if (nb > 1) R.scan(Y.Sloc, Y.zloc, Y.Sp, D.causal ? SCAN_FORWARD : SCAN_TOTAL);
     {   // O = (P V + phi(Q) S_prev) / (P 1 + phi(Q) z_prev)
         sg::Launch L;
-        sg::Prob p = D.causal ? R.blocked(nb, C) : R.whole();
-        const int s = D.causal ? 1 : 0, blk = D.causal ? C : 0;
-        if (D.causal) {
-            p.A[0] = R.blocks(Y.P, nb, C, C, 0); p.B[0] = R.input(V, dv, true, 1, C); p.K[0] = C; p.ktok[0] = 1; p.dot[0] = sg::DOT_ONES;
-            p.skip2_first = 1;
+        sg::Prob p = R.per_chunk();
+        if (D.causal) { R.product(L, p, 0, R.block(P, 0), R.kv(R.V, 1), 128, true); p.dot[0] = sg::DOT_ONES; p.skip2 = 0; }
+        if (R.states()) {
+            R.product(L, p, 1, R.rows(phi[0], 0), R.state(Sp, 1), m); p.dot[1] = sg::DOT_FEATURES;
+            p.dotf = R.f(Y.zloc); p.vec_pair = (long long)nb * m4; p.vec_blk = D.causal ? m4 : 0;
         }
-        p.A[s] = R.rows(Y.fQ, m, 0, blk); p.B[s] = R.blocks(Y.Sloc, nb, m, dv, 1, !D.causal); p.K[s] = m; p.dot[s] = sg::DOT_FEATURES;
-        p.dotf = R.f(Y.zloc); p.vec_pair = (long long)nb * m; p.vec_blk = D.causal ? m : 0;
         p.mtok = 1; p.N = dv; p.epi = dO ? sg::EPI_GRAD : sg::EPI_DIVIDE;
         if (dO) {
-            p.x = R.input(dO, dv, false, 0, blk); p.sums = R.f(Y.gd);
-            R.out_rows(p, R.f(Y.Ga), dv, false, blk);
-        } else R.out_rows(p, O, dv, true, blk);
+            p.xkind = D.bf16 ? sg::X_BF16 : sg::X_F32; p.x = dO; p.xld = dv; p.sums = R.f(Y.gd);
+            R.out_rows(p, R.tokens(Y.Ga, dv));
+        } else R.plain_rows(p, O, dv, true);
         sg::add(L, p);
         R.gemms(L);
     }
-    if (!dO) return;
-    const sg::TokVec gd = {R.f(Y.gd), BH * N, tiles(dv), 1.f};
-    {   // R_c = phi(Q_c)^T Ga_c, rho_c = phi(Q_c)^T gd_c; causal: dP_c = tril(Ga_c V_c^T + gd_c)
-        sg::Launch L;
-        sg::Prob p = R.blocked(nb, Y.blk);
-        p.A[0] = R.rows(Y.fQ, m, 1, Y.blk); p.B[0] = R.rows(Y.Ga, dv, 1, Y.blk); p.K[0] = N; p.ktok[0] = 1;
-        p.M = m; p.N = dv; p.dot[0] = sg::DOT_TOKENS; p.dott = gd; p.dot_out = R.f(Y.rloc);
-        R.out_blocks(p, Y.Rloc, nb, m, dv);
-        sg::add(L, p);
-        if (D.causal) {
-            sg::Prob q = R.blocked(nb, C);
-            q.A[0] = R.rows(Y.Ga, dv, 0, C); q.B[0] = R.input(V, dv, true, 0, C); q.K[0] = dv;
-            q.mtok = q.ntok_dim = 1; q.epi = sg::EPI_MASK; q.row = gd;
-            R.out_blocks(q, Y.dP, nb, C, C);
-            sg::add(L, q);
-        }
-        R.gemms(L);
-    }
-    scan(Y.Rloc, Y.rloc, D.causal ? SCAN_REVERSE : SCAN_TOTAL);
 }
 
-size_t take(size_t &off, long long floats)
+size_t take(size_t &off, size_t bytes)
 {
     const size_t at = off;
-    off += (((size_t)floats * sizeof(float)) + 255) / 256 * 256;
+    off += (bytes + 255) / 256 * 256;
     return at;
 }
 
-// Cuts N tokens into blocks (multiples of 64 tokens) so that `units` products of one block each are at least one wave of
-// two CTAs per SM, none shorter than two stages of the contraction.
+// Cuts N tokens into blocks (multiples of 64 tokens) so that `units` products of one block each are about one per SM, none
+// shorter than two stages of the contraction.
 void cut_tokens(int N, long long units, int most, int &nblk, int &blk)
 {
-    long long want = (2 * 148 + units - 1) / units;
+    long long want = (148 + units - 1) / units;
     if (want > (N + 127) / 128) want = (N + 127) / 128;
     if (want > most) want = most;
     if (want < 1) want = 1;
@@ -353,55 +406,85 @@ void cut_tokens(int N, long long units, int most, int &nblk, int &blk)
     nblk = (N + blk - 1) / blk;
 }
 
+SimtLayout make_layout(const Dims &D, bool backward)
+{
+    SimtLayout Y = {};
+    const size_t BH = D.BH, N = D.N, m = D.m, dv = D.dv, m4 = up4(D.m), BHkv = (size_t)D.B * D.Hkv;
+    if (D.causal) {
+        Y.blk = 128;
+        Y.nb = tiles(D.N);
+    } else {
+        // (the extra partial states never take more room than two rows of values per token)
+        cut_tokens(D.N, (long long)BH * tiles(D.m) * tiles(D.dv), (int)(1 + 2 * N / m > 64 ? 64 : 1 + 2 * N / m), Y.nb, Y.blk);
+    }
+    const size_t nb = Y.nb;
+    auto planes = [](size_t rows, int w) { return 3 * rows * up8(w) * 2; };
+    size_t off = 0;
+    Y.status = take(off, 256);
+    Y.cK = take(off, BH * m4 * 4);
+    const int widths[5] = {D.d, D.d, D.dv, D.d, D.r};
+    const size_t rows[5] = {BH * N, BHkv * N, BHkv * N, (size_t)D.H * D.r, (size_t)(D.w_per_head ? D.H : 1) * m};
+    for (int i = 0; i < 5; ++i) Y.conv[i] = !D.bf16 || widths[i] % 8;
+    auto take_in = [&](int i) { if (Y.conv[i]) Y.in[i] = take(off, (D.bf16 ? 1 : 3) * rows[i] * up8(widths[i]) * 2); };
+    take_in(2);
+    Y.fQ = take(off, planes(BH * N, D.m)); Y.fK = take(off, planes(BH * N, D.m));
+    // What is done with once the features are formed, unless the backward pass needs it again; there the states and kernel
+    // tiles take its place.
+    const size_t mark = off;
+    take_in(0); take_in(1); take_in(3); take_in(4);
+    Y.xtQ = take(off, planes(BH * N, D.r)); Y.xtK = take(off, planes(BH * N, D.r));
+    Y.nK = take(off, (size_t)4 * tiles(D.r) * BH * N * 4);
+    Y.rmax = tiles(D.m) > 1 ? take(off, (size_t)4 * tiles(D.m) * BH * N * 4) : 0;
+    const size_t end = off;
+    if (!backward) off = mark;
+    const bool states = !D.causal || nb > 1;
+    Y.zloc = states ? take(off, BH * nb * m4 * 4) : 0;
+    Y.Sloc = nb > 1 ? take(off, BH * nb * m * dv * 4) : 0;
+    Y.Sp = states ? take(off, planes(BH * (D.causal ? nb : 1) * m, D.dv)) : 0;
+    Y.P = D.causal ? take(off, planes(BH * nb * 128, 128)) : 0;
+    if (off < end) off = end;
+    if (backward) {
+        Y.Ga = take(off, planes(BH * N, D.dv)); Y.gd = take(off, (size_t)4 * tiles(D.dv) * BH * N * 4);
+        Y.dP = D.causal ? take(off, planes(BH * nb * 128, 128)) : 0;
+        Y.rloc = states ? take(off, BH * nb * m4 * 4) : 0;
+        Y.Rloc = nb > 1 ? take(off, BH * nb * m * dv * 4) : 0;
+        Y.Rp = states ? take(off, planes(BH * (D.causal ? nb : 1) * m, D.dv)) : 0;
+        Y.dA = take(off, planes(BH * N, D.m)); Y.dBf = take(off, planes(BH * N, D.m));
+        Y.esK = take(off, (size_t)4 * tiles(D.m) * BH * N * 4);
+        Y.dxtQ = take(off, planes(BH * N, D.r)); Y.dxtK = take(off, planes(BH * N, D.r));
+        Y.dKh = D.G > 1 ? take(off, BH * N * D.d * 4) : 0; Y.dVh = D.G > 1 ? take(off, BH * N * dv * 4) : 0;
+        cut_tokens(D.N, (long long)BH * tiles(D.r) * tiles(D.d), 64, Y.nsM, Y.blkM);
+        cut_tokens(D.N, (long long)BH * tiles(D.m) * tiles(D.r), 64, Y.nsW, Y.blkW);
+        Y.dMp = take(off, BH * Y.nsM * D.r * D.d * 4);
+        Y.dWp = take(off, BH * Y.nsW * m * D.r * 4);
+    }
+    Y.bytes = off;
+    return Y;
+}
+
 }  // namespace
 
 void simt_make_layout(darkattn_plan_s *plan)
 {
+    plan->simt = make_layout(plan->dims, true);
+    plan->simt_fwd = make_layout(plan->dims, false);
+}
+
+void simt_launches(const darkattn_plan_s *plan, int &fwd, int &bwd)
+{
     const Dims &D = plan->dims;
-    SimtLayout &Y = plan->simt;
-    const long long BH = D.BH, N = D.N, d = D.d, r = D.r, m = D.m, dv = D.dv;
-    if (D.causal) {
-        Y.C = (int)(N < D.C ? (N + 3) / 4 * 4 : D.C);
-        if (Y.C > D.C) Y.C = D.C;
-        Y.blk = Y.C;
-        Y.nb = (int)((N + Y.C - 1) / Y.C);
-    } else {
-        Y.C = 0;
-        // (the extra partial states never take more room than two rows of values per token)
-        cut_tokens(D.N, BH * tiles(D.m) * tiles(D.dv), (int)(1 + 2 * N / m > 64 ? 64 : 1 + 2 * N / m), Y.nb, Y.blk);
-    }
-    const long long nb = Y.nb, C = Y.C;
-    size_t off = 0;
-    Y.status = take(off, 64);
-    Y.xtQ = take(off, BH * N * r); Y.xtK = take(off, BH * N * r);
-    Y.fQ = take(off, BH * N * m); Y.fK = take(off, BH * N * m);
-    Y.cK = take(off, BH * m);
-    Y.Sloc = take(off, BH * nb * m * dv); Y.zloc = take(off, BH * nb * m);
-    Y.P = D.causal ? take(off, BH * nb * C * C) : 0;
-    {   // the key norms are done with before the states are written: they share their place
-        size_t end = Y.Sloc;
-        Y.nK = take(end, tiles(D.r) * BH * N);
-        if (end > off) off = end;
-    }
-    Y.fwd_bytes = off;
-    Y.Ga = take(off, BH * N * dv); Y.gd = take(off, tiles(D.dv) * BH * N);
-    Y.dP = D.causal ? take(off, BH * nb * C * C) : 0;
-    Y.Rloc = take(off, BH * nb * m * dv); Y.rloc = take(off, BH * nb * m);
-    Y.dA = take(off, BH * N * m); Y.dBf = take(off, BH * N * m);
-    Y.esK = take(off, tiles(D.m) * BH * N);
-    Y.dxtQ = take(off, BH * N * r); Y.dxtK = take(off, BH * N * r);
-    Y.dKh = D.G > 1 ? take(off, BH * N * d) : 0; Y.dVh = D.G > 1 ? take(off, BH * N * dv) : 0;
-    cut_tokens(D.N, BH * tiles(D.r) * tiles(D.d), 64, Y.nsM, Y.blkM);
-    cut_tokens(D.N, BH * tiles(D.m) * tiles(D.r), 64, Y.nsW, Y.blkW);
-    Y.dMp = take(off, BH * Y.nsM * r * d);
-    Y.dWp = take(off, BH * Y.nsW * m * r);
-    Y.total_bytes = off;
+    const SimtLayout &Y = plan->simt;
+    bool conv = false;
+    for (bool c : Y.conv) conv = conv || c;
+    const int scan = Y.nb > 1;
+    fwd = (conv ? 1 : 0) + 5 + (tiles(D.m) > 1 ? 1 : 0) + scan;
+    bwd = fwd + 1 + scan + 4 + (D.G > 1 ? 2 : 0);
 }
 
 darkattn_status_t simt_forward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
                                const void *M, const void *W, void *O, char *ws, cudaStream_t st)
 {
-    Runner R{plan, ws, st};
+    Runner R{plan, plan->simt_fwd, ws, st};
     run_forward_stages(R, Q, K, V, M, W, O, nullptr);
     if (R.err != cudaSuccess) { set_cuda_error(R.err, "simt_forward"); return DARKATTN_ERR_CUDA; }
     return DARKATTN_OK;
@@ -413,44 +496,66 @@ darkattn_status_t simt_backward(const darkattn_plan_s *plan, const void *Q, cons
 {
     const Dims &D = plan->dims;
     const SimtLayout &Y = plan->simt;
-    const int N = D.N, d = D.d, r = D.r, m = D.m, dv = D.dv, C = Y.C, nb = Y.nb;
+    const int N = D.N, d = D.d, r = D.r, m = D.m, dv = D.dv, nb = Y.nb, m4 = up4(m);
     const long long BH = D.BH;
-    Runner R{plan, ws, st};
+    Runner R{plan, Y, ws, st};
     run_forward_stages(R, Q, K, V, M, W, nullptr, dO);
 
     const bool grouped = D.G > 1;
-    const sg::TokVec gd = {R.f(Y.gd), BH * N, tiles(dv), 1.f};
-    const int blk = D.causal ? C : 0, s = D.causal ? 1 : 0;
-    auto per_block = [&]() { return D.causal ? R.blocked(nb, C) : R.whole(); };
+    const sg::TokVec gd = {R.f(Y.gd), BH * N, 4 * tiles(dv), 1.f}, es = {R.f(Y.esK), BH * N, 4 * tiles(m), 1.f};
+    const Mat xtK = R.tokens(Y.xtK, r), fQ = R.tokens(Y.fQ, m), fK = R.tokens(Y.fK, m), Ga = R.tokens(Y.Ga, dv), E[2] = {R.tokens(Y.dA, m), R.tokens(Y.dBf, m)};
+    const Mat Sp = R.state_planes(Y.Sp), Rp = R.state_planes(Y.Rp), P = R.planes(Y.P, BH * nb, 128, 128), dP = R.planes(Y.dP, BH * nb, 128, 128);
+    const Mat dxt[2] = {R.tokens(Y.dxtQ, r), R.tokens(Y.dxtK, r)};
+    {   // R_c = phi(Q_c)^T Ga_c, rho_c = phi(Q_c)^T gd_c; causal: dP_c = tril(Ga_c V_c^T + gd_c)
+        sg::Launch L;
+        if (D.causal) {
+            sg::Prob q = R.prob(nb, 128);
+            R.product(L, q, 0, R.rows(Ga, 0), R.kv(R.V, 0), dv);
+            q.mtok = q.ntok_dim = 1; q.epi = sg::EPI_MASK; q.row = gd;
+            R.out_blocks(q, dP);
+            sg::add(L, q);
+        }
+        if (R.states()) {
+            sg::Prob p = R.prob(nb, Y.blk);
+            R.product(L, p, 0, R.rows(fQ, 1), R.rows(Ga, 1), N, true);
+            p.M = m; p.N = dv; p.dot[0] = sg::DOT_TOKENS; p.dott = gd; p.dot_out = R.f(Y.rloc); p.dot_ld = m4;
+            if (!D.causal && nb == 1) R.out_blocks(p, Rp);
+            else R.plain_blocks(p, Y.Rloc, nb, m, dv);
+            sg::add(L, p);
+        }
+        R.gemms(L);
+    }
+    if (nb > 1) R.scan(Y.Rloc, Y.rloc, Y.Rp, D.causal ? SCAN_REVERSE : SCAN_TOTAL);
     {
         sg::Launch L;
+        auto vec = [&](sg::Prob &p, size_t v) { if (R.states()) { p.colvec = R.f(v); p.vec_pair = (long long)nb * m4; p.vec_blk = D.causal ? m4 : 0; } };
         {   // E_Q = phi(Q) .* (dP phi(K) + Ga S_prev^T + gd z_prev^T)
-            sg::Prob p = per_block();
-            if (D.causal) { p.A[0] = R.blocks(Y.dP, nb, C, C, 0); p.B[0] = R.rows(Y.fK, m, 1, C); p.K[0] = C; p.ktok[0] = 1; p.skip2_first = 1; }
-            p.A[s] = R.rows(Y.Ga, dv, 0, blk); p.B[s] = R.blocks(Y.Sloc, nb, m, dv, 0, !D.causal); p.K[s] = dv;
-            p.epi = sg::EPI_RANK1; p.row = gd; p.rank1 = R.f(Y.zloc); p.vec_pair = (long long)nb * m; p.vec_blk = D.causal ? m : 0;
-            p.x = R.rows(Y.fQ, m, 0, blk);
+            sg::Prob p = R.per_chunk();
+            if (D.causal) { R.product(L, p, 0, R.block(dP, 0), R.rows(fK, 1), 128, true); p.skip2 = 0; }
+            if (R.states()) R.product(L, p, 1, R.rows(Ga, 0), R.state(Sp, 0), dv);
+            p.epi = sg::EPI_RANK1; p.row = gd; vec(p, Y.zloc);
+            R.x_planes(p, fQ);
             p.mtok = 1; p.N = m;
-            R.out_rows(p, R.f(Y.dA), m, false, blk);
+            R.out_rows(p, E[0]);
             sg::add(L, p);
         }
         {   // E_K = phi(K) .* (dP^T phi(Q) + V R_next^T + rho_next^T), and its row sums
-            sg::Prob p = per_block();
-            if (D.causal) { p.A[0] = R.blocks(Y.dP, nb, C, C, 1); p.B[0] = R.rows(Y.fQ, m, 1, C); p.K[0] = C; p.ktok[0] = 1; }
-            p.A[s] = R.input(V, dv, true, 0, blk); p.B[s] = R.blocks(Y.Rloc, nb, m, dv, 0, !D.causal); p.K[s] = dv;
-            p.epi = sg::EPI_RANK1; p.rank1 = R.f(Y.rloc); p.vec_pair = (long long)nb * m; p.vec_blk = D.causal ? m : 0;
-            p.x = R.rows(Y.fK, m, 0, blk); p.sums = R.f(Y.esK);
+            sg::Prob p = R.per_chunk();
+            if (D.causal) { R.product(L, p, 0, R.block(dP, 1), R.rows(fQ, 1), 128, true); p.skip2 = nb - 1; }
+            if (R.states()) R.product(L, p, 1, R.kv(R.V, 0), R.state(Rp, 0), dv);
+            p.epi = sg::EPI_RANK1; vec(p, Y.rloc);
+            R.x_planes(p, fK); p.sums = R.f(Y.esK);
             p.mtok = 1; p.N = m;
-            R.out_rows(p, R.f(Y.dBf), m, false, blk);
+            R.out_rows(p, E[1]);
             sg::add(L, p);
         }
         {   // dV = P^T Ga + phi(K) R_next
-            sg::Prob p = per_block();
-            if (D.causal) { p.A[0] = R.blocks(Y.P, nb, C, C, 1); p.B[0] = R.rows(Y.Ga, dv, 1, C); p.K[0] = C; p.ktok[0] = 1; }
-            p.A[s] = R.rows(Y.fK, m, 0, blk); p.B[s] = R.blocks(Y.Rloc, nb, m, dv, 1, !D.causal); p.K[s] = m;
+            sg::Prob p = R.per_chunk();
+            if (D.causal) { R.product(L, p, 0, R.block(P, 1), R.rows(Ga, 1), 128, true); p.skip2 = nb - 1; }
+            if (R.states()) R.product(L, p, 1, R.rows(fK, 0), R.state(Rp, 1), m);
             p.mtok = 1; p.N = dv;
-            if (grouped) R.out_rows(p, R.f(Y.dVh), dv, false, blk);
-            else R.out_rows(p, dV, dv, true, blk);
+            if (grouped) R.plain_rows(p, R.f(Y.dVh), dv, false);
+            else R.plain_rows(p, dV, dv, true);
             sg::add(L, p);
         }
         R.gemms(L);
@@ -458,11 +563,11 @@ darkattn_status_t simt_backward(const darkattn_plan_s *plan, const void *Q, cons
     {   // dx~ = E W, for the keys minus rowsum(E) x~
         sg::Launch L;
         for (int side = 0; side < 2; ++side) {
-            sg::Prob p = R.whole();
-            p.A[0] = R.rows(side ? Y.dBf : Y.dA, m, 0); p.B[0] = R.paramW(W, 1); p.K[0] = m;
+            sg::Prob p = R.prob();
+            R.product(L, p, 0, R.rows(E[side], 0), R.opW(1), m);
             p.mtok = 1; p.N = r;
-            if (side) { p.epi = sg::EPI_SUBX; p.x = R.rows(Y.xtK, r, 0); p.row = {R.f(Y.esK), BH * N, tiles(m), 1.f}; }
-            R.out_rows(p, R.f(side ? Y.dxtK : Y.dxtQ), r, false);
+            if (side) { p.epi = sg::EPI_SUBX; R.x_planes(p, xtK); p.row = es; }
+            R.out_rows(p, dxt[side]);
             sg::add(L, p);
         }
         R.gemms(L);
@@ -470,34 +575,32 @@ darkattn_status_t simt_backward(const darkattn_plan_s *plan, const void *Q, cons
     {   // dX = s dx~ M; dM = s sum dx~^T X over the tokens of both sides, per (b,h) and token block
         sg::Launch L;
         for (int side = 0; side < 2; ++side) {
-            sg::Prob p = R.whole();
-            p.A[0] = R.rows(side ? Y.dxtK : Y.dxtQ, r, 0); p.B[0] = R.paramM(M, 1); p.K[0] = r;
+            sg::Prob p = R.prob();
+            R.product(L, p, 0, R.rows(dxt[side], 0), R.opM(1), r);
             p.mtok = 1; p.N = d; p.alpha = D.s;
-            if (side && grouped) R.out_rows(p, R.f(Y.dKh), d, false);
-            else R.out_rows(p, side ? dK : dQ, d, true);
+            if (side && grouped) R.plain_rows(p, R.f(Y.dKh), d, false);
+            else R.plain_rows(p, side ? dK : dQ, d, true);
             sg::add(L, p);
         }
-        sg::Prob p = R.blocked(Y.nsM, Y.blkM);
-        for (int side = 0; side < 2; ++side) {
-            p.A[side] = R.rows(side ? Y.dxtK : Y.dxtQ, r, 1, Y.blkM); p.B[side] = R.input(side ? K : Q, d, side, 1, Y.blkM);
-            p.K[side] = N; p.ktok[side] = 1;
-        }
+        sg::Prob p = R.prob(Y.nsM, Y.blkM);
+        R.product(L, p, 0, R.rows(dxt[0], 1), R.rows(R.Q, 1), N, true);
+        R.product(L, p, 1, R.rows(dxt[1], 1), R.kv(R.K, 1), N, true);
         p.M = r; p.N = d; p.alpha = D.s;
-        R.out_blocks(p, Y.dMp, Y.nsM, r, d);
+        R.plain_blocks(p, Y.dMp, Y.nsM, r, d);
         sg::add(L, p);
         R.gemms(L);
     }
-    const long long E = (long long)r * d;
-    R.kernel(reduce_kernel, D.H * E, R.f(Y.dMp), dM, D.B, (long long)D.H, Y.nsM, E, D.H * E);
+    const long long Em = (long long)r * d;
+    R.kernel(reduce_kernel, D.H * Em, (const float *)R.f(Y.dMp), dM, D.B, (long long)D.H, Y.nsM, Em, D.H * Em);
     if (grouped) {
         const long long BHkv = (long long)D.B * D.Hkv, nv = BHkv * N * dv, nk = BHkv * N * d;
         auto threads = [](long long n) { return n < 148LL * 16 * 256 ? n : 148LL * 16 * 256; };
         if (D.bf16) {
-            R.kernel(group_sum_f32_kernel<__nv_bfloat16>, threads(nv), (__nv_bfloat16 *)dV, R.f(Y.dVh), D.G, (long long)N * dv, nv);
-            R.kernel(group_sum_f32_kernel<__nv_bfloat16>, threads(nk), (__nv_bfloat16 *)dK, R.f(Y.dKh), D.G, (long long)N * d, nk);
+            R.kernel(group_sum_f32_kernel<__nv_bfloat16>, threads(nv), (__nv_bfloat16 *)dV, (const float *)R.f(Y.dVh), D.G, (long long)N * dv, nv);
+            R.kernel(group_sum_f32_kernel<__nv_bfloat16>, threads(nk), (__nv_bfloat16 *)dK, (const float *)R.f(Y.dKh), D.G, (long long)N * d, nk);
         } else {
-            R.kernel(group_sum_f32_kernel<float>, threads(nv), (float *)dV, R.f(Y.dVh), D.G, (long long)N * dv, nv);
-            R.kernel(group_sum_f32_kernel<float>, threads(nk), (float *)dK, R.f(Y.dKh), D.G, (long long)N * d, nk);
+            R.kernel(group_sum_f32_kernel<float>, threads(nv), (float *)dV, (const float *)R.f(Y.dVh), D.G, (long long)N * dv, nv);
+            R.kernel(group_sum_f32_kernel<float>, threads(nk), (float *)dK, (const float *)R.f(Y.dKh), D.G, (long long)N * d, nk);
         }
     }
     if (R.err != cudaSuccess) { set_cuda_error(R.err, "simt_backward"); return DARKATTN_ERR_CUDA; }
@@ -510,20 +613,18 @@ darkattn_status_t simt_backward_dw(const darkattn_plan_s *plan, float *dW, char 
 {
     const Dims &D = plan->dims;
     const SimtLayout &Y = plan->simt;
-    Runner R{plan, ws, st};
+    Runner R{plan, Y, ws, st};
     sg::Launch L;
-    sg::Prob p = R.blocked(Y.nsW, Y.blkW);
-    for (int side = 0; side < 2; ++side) {
-        p.A[side] = R.rows(side ? Y.dBf : Y.dA, D.m, 1, Y.blkW); p.B[side] = R.rows(side ? Y.xtK : Y.xtQ, D.r, 1, Y.blkW);
-        p.K[side] = D.N; p.ktok[side] = 1;
-    }
+    sg::Prob p = R.prob(Y.nsW, Y.blkW);
+    R.product(L, p, 0, R.rows(R.tokens(Y.dA, D.m), 1), R.rows(R.tokens(Y.xtQ, D.r), 1), D.N, true);
+    R.product(L, p, 1, R.rows(R.tokens(Y.dBf, D.m), 1), R.rows(R.tokens(Y.xtK, D.r), 1), D.N, true);
     p.M = D.m; p.N = D.r;
-    R.out_blocks(p, Y.dWp, Y.nsW, D.m, D.r);
+    R.plain_blocks(p, Y.dWp, Y.nsW, D.m, D.r);
     sg::add(L, p);
     R.gemms(L);
     const long long E = (long long)D.m * D.r;
-    if (D.w_per_head) R.kernel(reduce_kernel, D.H * E, R.f(Y.dWp), dW, D.B, (long long)D.H, Y.nsW, E, D.H * E);
-    else R.kernel(reduce_kernel, E, R.f(Y.dWp), dW, D.BH, 1LL, Y.nsW, E, E);
+    if (D.w_per_head) R.kernel(reduce_kernel, D.H * E, (const float *)R.f(Y.dWp), dW, D.B, (long long)D.H, Y.nsW, E, D.H * E);
+    else R.kernel(reduce_kernel, E, (const float *)R.f(Y.dWp), dW, D.BH, 1LL, Y.nsW, E, E);
     if (R.err != cudaSuccess) { set_cuda_error(R.err, "simt_backward_dw"); return DARKATTN_ERR_CUDA; }
     return DARKATTN_OK;
 }

@@ -35,6 +35,17 @@ darkattn_status_t scratch_for_current_device(char **out)
     return DARKATTN_OK;
 }
 
+// The plan of one (batch, head) pair of `plan`: what the array has to hold when all pairs at once are too much for it.
+void single_pair(const darkattn_plan_s *plan, darkattn_plan_s &one)
+{
+    one.desc = plan->desc;
+    one.path = plan->path;
+    one.dims = plan->dims;
+    Dims &D = one.dims;
+    D.B = D.H = D.BH = D.Hkv = D.G = 1;
+    simt_make_layout(&one);
+}
+
 }  // namespace
 }  // namespace darkattn
 
@@ -42,7 +53,11 @@ using namespace darkattn;
 
 extern "C" size_t darkattn_static_scratch_needed(darkattn_plan_t plan)
 {
-    return plan ? plan->simt.fwd_bytes : 0;
+    if (!plan) return 0;
+    if (plan->simt_fwd.bytes <= (size_t)DARKATTN_STATIC_SCRATCH_BYTES) return plan->simt_fwd.bytes;
+    darkattn_plan_s one;
+    single_pair(plan, one);
+    return one.simt_fwd.bytes;
 }
 
 extern "C" darkattn_status_t darkattn_forward_static(darkattn_plan_t plan, const void *Q, const void *K,
@@ -54,12 +69,24 @@ extern "C" darkattn_status_t darkattn_forward_static(darkattn_plan_t plan, const
     for (const void *p : ptrs)
         if (reinterpret_cast<uintptr_t>(p) & 15u) return DARKATTN_ERR_INVALID_ARG;
     // size check first: it needs no GPU, so a refusal never touches the device
-    if (plan->simt.fwd_bytes > (size_t)DARKATTN_STATIC_SCRATCH_BYTES) return DARKATTN_ERR_WORKSPACE;
+    if (darkattn_static_scratch_needed(plan) > (size_t)DARKATTN_STATIC_SCRATCH_BYTES) return DARKATTN_ERR_WORKSPACE;
     char *scratch = nullptr;
     darkattn_status_t s = scratch_for_current_device(&scratch);
     if (s != DARKATTN_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     // the array still holds the previous call's data: the first kernel clears the status word and the per-feature maxima,
     // every other region is written by this call before it is read
-    return simt_forward(plan, Q, K, V, M, W, O, scratch, st);
+    if (plan->simt_fwd.bytes <= (size_t)DARKATTN_STATIC_SCRATCH_BYTES) return simt_forward(plan, Q, K, V, M, W, O, scratch, st);
+    // pair by pair (heads are independent of one another)
+    darkattn_plan_s one;
+    single_pair(plan, one);
+    const Dims &D = plan->dims;
+    const size_t es = D.bf16 ? 2 : 4;
+    auto at = [&](const void *p, size_t elements) { return static_cast<const void *>(static_cast<const char *>(p) + elements * es); };
+    for (int bh = 0; bh < D.BH && s == DARKATTN_OK; ++bh) {
+        const size_t h = bh % D.H, kv = (size_t)(bh / D.H) * D.Hkv + h / D.G, N = D.N;
+        s = simt_forward(&one, at(Q, bh * N * D.d), at(K, kv * N * D.d), at(V, kv * N * D.dv), at(M, h * D.r * D.d),
+                         at(W, D.w_per_head ? h * D.m * D.r : 0), const_cast<void *>(at(O, bh * N * D.dv)), scratch, st);
+    }
+    return s;
 }

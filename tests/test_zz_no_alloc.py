@@ -73,3 +73,22 @@ def test_static_scratch_forward_matches_workspace_forward(binding, dtype, causal
         fro, mx = rel_errors(got.astype(np.float64), exact)          # and against the oracle, like every other entry point
         assert fro < TOL[dtype] and mx < TOL[dtype], ("oracle", call, fro, mx)
     plan.destroy()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_static_scratch_takes_the_heads_one_by_one(binding, dtype):
+    """A problem whose heads together need more than the array, each alone less: the same rows as with a workspace."""
+    wl = inputs.small(name="noalloc_heads", wid=42, B=3, H=4, N=1001, d=48, m=264, dv=40, dtype=dtype, causal=True, backward=False)
+    t = inputs.generate(wl)
+    dt = torch_dtype(dtype)
+    Q, K, V, M, W = (to_dev(x, dt) for x in (t.Q, t.K[:, ::2], t.V[:, ::2], t.M, t.W))       # two query heads per key/value head
+    plan = binding.darkattn_plan(3, 4, 1001, 48, 264, dv=40, dtype=binding.F32 if dtype == "f32" else binding.BF16, causal=True,
+                                 path=binding.PATH_SIMT, H_kv=2)
+    assert plan.workspace_bytes > binding.STATIC_SCRATCH_BYTES >= binding.darkattn_static_scratch_needed(plan)
+    want, got = (torch.full((3, 4, 1001, 40), float("nan"), dtype=dt, device="cuda") for _ in range(2))
+    binding.darkattn_forward(plan, Q, K, V, M, W, want, plan.alloc_workspace())
+    binding.darkattn_forward_static(plan, Q, K, V, M, W, got)
+    torch.cuda.synchronize()
+    assert torch.equal(got, want)
+    plan.destroy()
