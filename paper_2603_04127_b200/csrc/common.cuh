@@ -192,7 +192,7 @@ cudaError_t tensor_prologue(const darkattn_plan_s *plan, const void *K, const vo
 // dW from what the last backward call left in the workspace
 darkattn_status_t simt_backward_dw(const darkattn_plan_s *plan, float *dW, char *ws, cudaStream_t st);
 cudaError_t tensor_backward_nc_passes(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V, const void *dO,
-                                      const Stash &stash, void *dQ, void *dK, void *dV, bool per_head, char *ws, cudaStream_t st);
+                                      const Stash &stash, void *dQ, void *dK, void *dV, bool per_head, bool join, char *ws, cudaStream_t st);
 darkattn_status_t tensor_backward_dw(const darkattn_plan_s *plan, const void *M, float *dW, char *ws, cudaStream_t st);
 darkattn_status_t tensor_backward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
                                   const void *M, const void *W, const void *O, const void *dO, const void *saved,
@@ -212,6 +212,35 @@ inline int pick_splits(long long units, int T, double us_per_tile, double us_fix
     }
     return best_c;
 }
+
+// Dynamic shared memory a kernel may use (set once per kernel, size and device) and, the same for every kernel of the library, the
+// largest shared-memory share of an SM: kernels that overlap at their ends have to agree on it.
+cudaError_t allow_smem(const void *kernel, int bytes);
+
+// Launches a kernel that begins with griddepcontrol.wait (all its memory accesses come after that): it may start while the
+// kernel before it in the stream drains, so that its launch and its prologue cost nothing.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, int smem, cudaStream_t st, const Args &...args)
+{
+    cudaError_t e = allow_smem(reinterpret_cast<const void *>(k), smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, KArgs(args)...);
+}
+#ifdef __CUDACC__
+// Waits until the kernels before have completed; then lets the next one start its prologue.
+__device__ __forceinline__ void pdl_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+}
+#endif
 
 #define DARKATTN_CUDA_TRY(expr, where)                                   \
     do {                                                                 \

@@ -4,6 +4,7 @@
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
+#include <mutex>
 #include <new>
 
 namespace darkattn {
@@ -22,6 +23,24 @@ void timer_mark(const darkattn_plan_s *plan, cudaStream_t st, const char *name)
     t.name[t.n] = name;
     cudaEventRecord(t.ev[t.n], st);
     ++t.n;
+}
+
+cudaError_t allow_smem(const void *kernel, int bytes)
+{
+    struct Entry { const void *k; int dev, bytes; };
+    static std::mutex lock;
+    static Entry seen[256];
+    static int n = 0;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> guard(lock);
+    for (int i = 0; i < n; ++i)
+        if (seen[i].k == kernel && seen[i].dev == dev && seen[i].bytes >= bytes) return cudaSuccess;
+    if (bytes > 0) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess && n < 256) seen[n++] = {kernel, dev, bytes};
+    return e;
 }
 
 static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -96,7 +115,6 @@ darkattn_status_t darkattn_forward(darkattn_plan_t plan, const void *Q, const vo
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     darkattn_status_t rc;
     if (plan->path == DARKATTN_PATH_TENSOR) {
-        DARKATTN_CUDA_TRY(cudaMemsetAsync(workspace, 0, 256, st), "forward: clear status word");
         rc = tensor_forward(plan, Q, K, V, M, W, O, saved, static_cast<char *>(workspace), st, saved != nullptr);
     } else {
         timer_mark(plan, st, "simt_forward (all kernels)");
@@ -120,7 +138,6 @@ darkattn_status_t darkattn_backward(darkattn_plan_t plan, const void *Q, const v
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     darkattn_status_t rc;
     if (plan->path == DARKATTN_PATH_TENSOR) {
-        DARKATTN_CUDA_TRY(cudaMemsetAsync(workspace, 0, 256, st), "backward: clear status word");
         rc = tensor_backward(plan, Q, K, V, M, W, O, dO, saved, dQ, dK, dV, dM, static_cast<char *>(workspace), st);
     } else {
         timer_mark(plan, st, "simt_backward (all kernels)");

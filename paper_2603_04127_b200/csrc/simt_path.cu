@@ -10,7 +10,7 @@
 //              prefix over the chunks | output rows
 //   backward   the forward steps with the output rows turned into dO / den and -delta / den | dP and the reverse states |
 //              suffix over the chunks | E of both sides and dV | dx~ | dQ, dK and dM | sums over batch and token blocks
-// Each line's items between bars are one launch each; all but the first start while the one before drains
+// Each line's items between bars are one launch each; each starts while the one before drains
 // (programmatic dependent launch). Chunks are 128 tokens, a tile's rows, whatever chunk length the descriptor names (the
 // result does not depend on it).
 //
@@ -27,7 +27,6 @@
 
 namespace darkattn {
 
-using sg::launch_pdl;
 using sg::Mat;
 
 namespace {
@@ -192,20 +191,17 @@ struct Runner {
     const SimtLayout &Y;
     char *ws;
     cudaStream_t st;
-    bool dependent = false;         // a kernel of this call has been launched
     cudaError_t err = cudaSuccess;
     Mat Q, K, V, M, W;
 
     const Dims &D() const { return plan->dims; }
     float *f(size_t off) const { return reinterpret_cast<float *>(ws + off); }
-    void keep(cudaError_t e) { if (e != cudaSuccess && err == cudaSuccess) err = e; dependent = true; }
-    void gemms(sg::Launch &L) { L.status = reinterpret_cast<int *>(ws); keep(sg::run(L, st, dependent)); }
+    void keep(cudaError_t e) { if (e != cudaSuccess && err == cudaSuccess) err = e; }
+    void gemms(sg::Launch &L) { L.status = reinterpret_cast<int *>(ws); keep(sg::run(L, st)); }
     template <typename... KA, typename... A>
     void kernel(void (*k)(KA...), long long threads, const A &...args)
     {
-        // (the same division of the SM's memory as the products' kernel: a change between launches costs microseconds)
-        keep(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
-        keep(launch_pdl(k, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, st, dependent, args...));
+        keep(launch_pdl(k, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, st, args...));
     }
 
     // ---- matrices

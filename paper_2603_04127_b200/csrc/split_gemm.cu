@@ -627,14 +627,11 @@ void add(Launch &L, const Prob &q)
     L.total += p.blocks;
 }
 
-cudaError_t run(const Launch &L, cudaStream_t st, bool dependent)
+cudaError_t run(const Launch &L, cudaStream_t st)
 {
     static_assert(sizeof(Launch) <= 4000, "kernel parameter space");
     if (L.bad) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(split_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(split_gemm_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(split_gemm_kernel, dim3(L.total < 148 ? L.total : 148), dim3(kNT), kSmem, st, dependent, L);
+    return launch_pdl(split_gemm_kernel, dim3(L.total < 148 ? L.total : 148), dim3(kNT), kSmem, st, L);
 }
 
 }  // namespace sg

@@ -113,22 +113,7 @@ struct Launch {
 void set_operand(Launch &L, Prob &p, int i, const Op &o, bool hi_only = false);
 // Adds a product to a launch (fills in the derived fields).
 void add(Launch &L, const Prob &p);
-// Runs the launch; `dependent`: after a kernel of this library in the same stream, whose tail it may overlap.
-cudaError_t run(const Launch &L, cudaStream_t st, bool dependent);
-
-// Launches a kernel that starts with griddepcontrol.wait; `dependent` as above.
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool dependent, const Args &...args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = dependent ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k, KArgs(args)...);
-}
+cudaError_t run(const Launch &L, cudaStream_t st);
 
 }  // namespace sg
 }  // namespace darkattn

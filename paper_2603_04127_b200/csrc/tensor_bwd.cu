@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_q_kernel(const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_wait();
     const uint32_t tmem = *tmem_slot;
     int *status = p.status;
 
@@ -460,6 +461,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_k_kernel(const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_wait();
     const uint32_t tmem = *tmem_slot;
     int *status = p.status;
 
@@ -733,6 +735,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_finish_k_kernel(const __gr
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_wait();
     const uint32_t tmem = *tmem_slot;
     constexpr uint32_t C1 = 0, C2 = 128, C3 = 256;
     if (*abort_flag) { if (tid == 0) atomicExch(p.status, (int)DARKATTN_ERR_CUDA); }
@@ -866,6 +869,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_finish_k_kernel(const __gr
 // elements per thread.
 __global__ void group_sum_kernel(const __nv_bfloat16 *src, __nv_bfloat16 *out, int N, int w, int H, int Hkv, long long total8)
 {
+    pdl_wait();
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (t >= total8) return;
     const int per_row = w / 8, G = H / Hkv;
@@ -886,9 +890,17 @@ __global__ void group_sum_kernel(const __nv_bfloat16 *src, __nv_bfloat16 *out, i
     *reinterpret_cast<uint4 *>(out + t * 8) = pack8(pk);
 }
 
-// delta[row] = dO[row,:] . O[row,:]; dv/8 threads per row, 16 bytes of each tensor per thread.
-__global__ void delta_kernel(const __nv_bfloat16 *G, const __nv_bfloat16 *O, float *delta, long long rows, int dv)
+// delta[row] = dO[row,:] . O[row,:]; dv/8 threads per row, 16 bytes of each tensor per thread. The same threads clear what the
+// call's later kernels add into (each of these was a memset of its own before, with 4 us from one to the next) and the status
+// word (status may be null: the forward kernels of this call have cleared it).
+struct ZeroList { uint4 *p[6]; long long n[6]; int count; };
+__global__ void __launch_bounds__(256) delta_kernel(const __nv_bfloat16 *G, const __nv_bfloat16 *O, float *delta, long long rows, int dv, int *status,
+                                                    const __grid_constant__ ZeroList Z)
 {
+    pdl_wait();
+    if (status && blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
+    for (int k = 0; k < Z.count; ++k)
+        for (long long j = blockIdx.x * 256LL + threadIdx.x; j < Z.n[k]; j += gridDim.x * 256LL) Z.p[k][j] = make_uint4(0, 0, 0, 0);
     const int per_row = dv / 8;                       // 8 or 16: a power of two that divides the warp
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const long long row = i / per_row;
@@ -909,6 +921,7 @@ __global__ void delta_kernel(const __nv_bfloat16 *G, const __nv_bfloat16 *O, flo
 // blocks, because the kernel is bound by the latency of its loads.
 __global__ void dm_kernel(const __nv_bfloat16 *W, const float *Tacc, const float *dMn, float *dM, int m, int r, int d, int w_per_head, float s)
 {
+    pdl_wait();
     __shared__ float sw[64 * 8];
     const int a0 = blockIdx.x * 8, h = blockIdx.y, lb = blockIdx.z * 64, c = threadIdx.x;
     const __nv_bfloat16 *w = W + (size_t)(w_per_head ? h : 0) * m * r;
@@ -940,6 +953,7 @@ __global__ void dm_kernel(const __nv_bfloat16 *W, const float *Tacc, const float
 // dM += dMn (the norm term's part, when dm_kernel ran beside the kernel that produces it)
 __global__ void dm_add_kernel(float *dM, const float *dMn, int n)
 {
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) dM[i] += dMn[i];
 }
@@ -948,6 +962,7 @@ __global__ void dm_add_kernel(float *dM, const float *dMn, int n)
 // u_l = s w_l . (M x) the gradient of w_l is s M (sum_i E_il x_i). One block per row l (and head), one thread per a.
 __global__ void dw_kernel(const float *Tacc, const __nv_bfloat16 *M, float *dW, int H, int m, int r, int d, int w_per_head, float s)
 {
+    pdl_wait();
     const int l = blockIdx.x, a = threadIdx.x;
     const int h0 = w_per_head ? blockIdx.y : 0, h1 = w_per_head ? blockIdx.y + 1 : H;
     float acc = 0.f;
@@ -976,40 +991,28 @@ int sm_count()
 }
 
 template <int D, int DV>
-cudaError_t launch_scan(const darkattn_plan_s *plan, const BwdParams &P, int grid, cudaStream_t st)
+cudaError_t launch_scan(const darkattn_plan_s *plan, const BwdParams &P, int grid, bool join, cudaStream_t st)
 {
     using L = BwdSmem<D, DV>;
     static_assert(L::kTotal <= 232448, "shared memory budget of one CTA exceeded");
-    cudaError_t e = cudaFuncSetAttribute(tc_bwd_q_kernel<D, DV>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(tc_bwd_k_kernel<D, DV>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
-    if (e != cudaSuccess) return e;
     // the query-side kernel divides all chunks evenly over the SMs: groups of nslab CTAs, one group per piece
     long long groups = sm_count() / P.nslab;
     if (groups < 1) groups = 1;
     if (groups > (long long)P.BH * P.T) groups = (long long)P.BH * P.T;
     const int qgrid = (int)groups * P.nslab;
     timer_mark(plan, st, "tc_bwd_q_kernel");
-    tc_bwd_q_kernel<D, DV><<<qgrid, kThreads, L::kTotal, st>>>(P);
-    e = cudaGetLastError();
+    cudaError_t e = launch_pdl(tc_bwd_q_kernel<D, DV>, dim3(qgrid), dim3(kThreads), L::kTotal, st, P);
+    if (e == cudaSuccess && join) e = cudaStreamWaitEvent(st, plan->aux_join, 0);      // dK and dV have been zeroed
     if (e != cudaSuccess) return e;
-    if (P.add_kv) {
-        e = cudaStreamWaitEvent(st, plan->aux_join, 0);      // dK and dV have been zeroed
-        if (e != cudaSuccess) return e;
-    }
     timer_mark(plan, st, "tc_bwd_k_kernel");
-    tc_bwd_k_kernel<D, DV><<<grid, kThreads, L::kTotal, st>>>(P);
-    return cudaGetLastError();
+    return launch_pdl(tc_bwd_k_kernel<D, DV>, dim3(grid), dim3(kThreads), L::kTotal, st, P);
 }
 
 template <int D>
 cudaError_t launch_finish(FinishParams &P, int grid, cudaStream_t st)
 {
     constexpr int kTile = 128 * D * 2, smem_bytes = 4 * kTile + 32768 + 128;    // M, two K tiles, staging; w; barriers
-    cudaError_t e = cudaFuncSetAttribute(tc_bwd_finish_k_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-    if (e != cudaSuccess) return e;
-    tc_bwd_finish_k_kernel<D><<<grid, kThreads, smem_bytes, st>>>(P);
-    return cudaGetLastError();
+    return launch_pdl(tc_bwd_finish_k_kernel<D>, dim3(grid), dim3(kThreads), smem_bytes, st, P);
 }
 
 }  // namespace
@@ -1027,13 +1030,13 @@ darkattn_status_t tensor_backward(const darkattn_plan_s *plan, const void *Q, co
 
     cudaError_t e = cudaSuccess;
     auto keep = [&](cudaError_t x) { if (x != cudaSuccess && e == cudaSuccess) e = x; };
-    auto chk = [&]() { keep(cudaGetLastError()); };
 
     // The forward result and what the forward pass stashed (per-row normalisers, key norms, folded
     // projections, key shifts): taken from the caller when both are given, otherwise recomputed into the
     // workspace by running the forward kernels again.
     Stash stash;
-    if (!O || !saved) {
+    const bool recompute = !O || !saved;
+    if (recompute) {
         darkattn_status_t s = tensor_forward(plan, Q, K, V, M, W, bf(Y.Oscr), nullptr, ws, st, true);
         if (s != DARKATTN_OK) return s;
         O = bf(Y.Oscr);
@@ -1042,22 +1045,19 @@ darkattn_status_t tensor_backward(const darkattn_plan_s *plan, const void *Q, co
         stash = stash_in_saved(Y, const_cast<void *>(saved));
     }
 
-    const long long rows = (long long)BH * N;
-    timer_mark(plan, st, "delta_kernel");
-    delta_kernel<<<(unsigned)((rows * (D.dv / 8) + 255) / 256), 256, 0, st>>>((const __nv_bfloat16 *)dO, (const __nv_bfloat16 *)O, fl(Y.delta), rows, D.dv);
-    chk();
-    keep(cudaMemsetAsync(ws + Y.Tacc, 0, (size_t)D.H * D.m * D.d * 4, st));
-    keep(cudaMemsetAsync(ws + Y.dMn, 0, (size_t)D.H * D.r * D.d * 4, st));
     const size_t BHkv = (size_t)D.B * D.Hkv;
     // Grouped key/value heads: every query head's part of dK and dV goes to rows of its own in the workspace (so that an
     // element is rounded to bf16 as often as without groups), and a last kernel adds each group up in fp32.
     const bool per_head = D.G > 1;
     void *dKo = per_head ? (void *)bf(Y.dKh) : dK, *dVo = per_head ? (void *)bf(Y.dVh) : dV;
     const size_t BHo = per_head ? BH : BHkv;
+    // The slabs of a head add their parts into the gradients, which therefore start at zero. dQ is needed first and is
+    // cleared by the kernel that forms delta; dK and dV, where they are large (clearing 32 MB takes longer than the two events
+    // between the streams), on a side stream while the query-side scan runs: it leaves SMs and bandwidth free.
     const bool add_kv = Y.nslab > 1;
-    if (add_kv) {
-        // The slabs of a head add their parts into the gradients, which therefore start at zero. dQ is needed first; dK and
-        // dV are zeroed on a side stream while the query-side scan runs (it leaves SMs and bandwidth free).
+    const size_t kv_bytes = BHo * N * ((size_t)D.d + D.dv) * 2;
+    const bool beside_zero = add_kv && kv_bytes > (32u << 20);
+    if (beside_zero) {
         keep(ensure_aux(plan));
         if (e != cudaSuccess) { set_cuda_error(e, "tensor_backward: side stream"); return DARKATTN_ERR_CUDA; }
         keep(cudaEventRecord(plan->aux_fork, st));
@@ -1066,7 +1066,18 @@ darkattn_status_t tensor_backward(const darkattn_plan_s *plan, const void *Q, co
         keep(cudaMemsetAsync(dVo, 0, BHo * N * D.dv * 2, plan->aux_stream));
         keep(cudaEventRecord(plan->aux_join, plan->aux_stream));
     }
-    if (Y.nslab > 1) keep(cudaMemsetAsync(dQ, 0, BH * N * D.d * 2, st));
+    ZeroList Z;
+    Z.count = 0;
+    auto zero = [&](void *p, size_t bytes) { Z.p[Z.count] = static_cast<uint4 *>(p); Z.n[Z.count++] = (long long)(bytes / 16); };   // (all are multiples of 16 bytes)
+    zero(ws + Y.Tacc, (size_t)D.H * D.m * D.d * 4);
+    zero(ws + Y.dMn, (size_t)D.H * D.r * D.d * 4);
+    if (!D.causal) zero(ws + Y.Racc, (Y.rhot - Y.Racc) + BH * D.m * 4);      // R and rho sums (adjacent)
+    if (add_kv) zero(dQ, BH * N * D.d * 2);
+    if (add_kv && !beside_zero) { zero(dKo, BHo * N * D.d * 2); zero(dVo, BHo * N * D.dv * 2); }
+    const long long rows = (long long)BH * N;
+    timer_mark(plan, st, "delta_kernel");
+    keep(launch_pdl(delta_kernel, dim3((unsigned)((rows * (D.dv / 8) + 255) / 256)), dim3(256), 0, st, (const __nv_bfloat16 *)dO, (const __nv_bfloat16 *)O,
+                    fl(Y.delta), rows, D.dv, recompute ? (int *)nullptr : reinterpret_cast<int *>(ws + Y.status), Z));
 
     FinishParams F;
     memset(&F, 0, sizeof(F));
@@ -1092,12 +1103,12 @@ darkattn_status_t tensor_backward(const darkattn_plan_s *plan, const void *Q, co
         P.N = D.N; P.H = D.H; P.Hkv = D.Hkv; P.BH = D.BH; P.m = D.m; P.nslab = Y.nslab; P.T = Y.T; P.add_kv = add_kv ? 1 : 0;
         P.out_per_head = per_head ? 1 : 0;
         const int units = (int)(BH * Y.nslab);
-        if (D.d == 64 && D.dv == 64) keep(launch_scan<64, 64>(plan, P, units, st));
-        else if (D.d == 128 && D.dv == 128) keep(launch_scan<128, 128>(plan, P, units, st));
-        else if (D.d == 64 && D.dv == 128) keep(launch_scan<64, 128>(plan, P, units, st));
-        else keep(launch_scan<128, 64>(plan, P, units, st));
+        if (D.d == 64 && D.dv == 64) keep(launch_scan<64, 64>(plan, P, units, beside_zero, st));
+        else if (D.d == 128 && D.dv == 128) keep(launch_scan<128, 128>(plan, P, units, beside_zero, st));
+        else if (D.d == 64 && D.dv == 128) keep(launch_scan<64, 128>(plan, P, units, beside_zero, st));
+        else keep(launch_scan<128, 64>(plan, P, units, beside_zero, st));
     } else {
-        keep(tensor_backward_nc_passes(plan, Q, K, V, dO, stash, dQ, dKo, dVo, per_head, ws, st));
+        keep(tensor_backward_nc_passes(plan, Q, K, V, dO, stash, dQ, dKo, dVo, per_head, beside_zero, ws, st));
     }
 
     if (!make_map(&F.mapOut, dKo, BHo * N, D.d, 128)) { set_cuda_error(cudaErrorInvalidValue, "tensor_backward: tensor map encode"); return DARKATTN_ERR_CUDA; }
@@ -1114,8 +1125,7 @@ darkattn_status_t tensor_backward(const darkattn_plan_s *plan, const void *Q, co
         keep(cudaEventRecord(plan->aux_fork, st));
         keep(cudaStreamWaitEvent(plan->aux_stream, plan->aux_fork, 0));
         keep(cudaMemsetAsync(dM, 0, (size_t)D.H * D.r * D.d * 4, plan->aux_stream));
-        dm_kernel<<<dm_grid, D.d, 0, plan->aux_stream>>>((const __nv_bfloat16 *)W, fl(Y.Tacc), nullptr, dM, D.m, D.r, D.d, D.w_per_head, D.s);
-        chk();
+        keep(launch_pdl(dm_kernel, dm_grid, dim3(D.d), 0, plan->aux_stream, (const __nv_bfloat16 *)W, (const float *)fl(Y.Tacc), (const float *)nullptr, dM, D.m, D.r, D.d, D.w_per_head, D.s));
         keep(cudaEventRecord(plan->aux_join, plan->aux_stream));
     }
     timer_mark(plan, st, "tc_bwd_finish_k_kernel");
@@ -1125,22 +1135,18 @@ darkattn_status_t tensor_backward(const darkattn_plan_s *plan, const void *Q, co
     if (beside) {
         keep(cudaStreamWaitEvent(st, plan->aux_join, 0));
         const int n = D.H * D.r * D.d;
-        dm_add_kernel<<<(n + 255) / 256, 256, 0, st>>>(dM, fl(Y.dMn), n);
-        chk();
+        keep(launch_pdl(dm_add_kernel, dim3((n + 255) / 256), dim3(256), 0, st, dM, (const float *)fl(Y.dMn), n));
     } else {
         timer_mark(plan, st, "dm_kernel");
         keep(cudaMemsetAsync(dM, 0, (size_t)D.H * D.r * D.d * 4, st));
-        dm_kernel<<<dm_grid, D.d, 0, st>>>((const __nv_bfloat16 *)W, fl(Y.Tacc), fl(Y.dMn), dM, D.m, D.r, D.d, D.w_per_head, D.s);
-        chk();
+        keep(launch_pdl(dm_kernel, dm_grid, dim3(D.d), 0, st, (const __nv_bfloat16 *)W, (const float *)fl(Y.Tacc), (const float *)fl(Y.dMn), dM, D.m, D.r, D.d, D.w_per_head, D.s));
     }
     if (per_head) {
         const long long nk = (long long)BHkv * N * D.d / 8, nv = (long long)BHkv * N * D.dv / 8;
         timer_mark(plan, st, "group_sum_kernel (dK)");
-        group_sum_kernel<<<(unsigned)((nk + 255) / 256), 256, 0, st>>>(bf(Y.dKh), (__nv_bfloat16 *)dK, D.N, D.d, D.H, D.Hkv, nk);
-        chk();
+        keep(launch_pdl(group_sum_kernel, dim3((unsigned)((nk + 255) / 256)), dim3(256), 0, st, (const __nv_bfloat16 *)bf(Y.dKh), (__nv_bfloat16 *)dK, D.N, D.d, D.H, D.Hkv, nk));
         timer_mark(plan, st, "group_sum_kernel (dV)");
-        group_sum_kernel<<<(unsigned)((nv + 255) / 256), 256, 0, st>>>(bf(Y.dVh), (__nv_bfloat16 *)dV, D.N, D.dv, D.H, D.Hkv, nv);
-        chk();
+        keep(launch_pdl(group_sum_kernel, dim3((unsigned)((nv + 255) / 256)), dim3(256), 0, st, (const __nv_bfloat16 *)bf(Y.dVh), (__nv_bfloat16 *)dV, D.N, D.dv, D.H, D.Hkv, nv));
     }
     if (e != cudaSuccess) { set_cuda_error(e, "tensor_backward"); return DARKATTN_ERR_CUDA; }
     return DARKATTN_OK;
@@ -1151,9 +1157,8 @@ darkattn_status_t tensor_backward_dw(const darkattn_plan_s *plan, const void *M,
     const Dims &D = plan->dims;
     const TensorLayout &Y = plan->tensor;
     timer_mark(plan, st, "dw_kernel");
-    dw_kernel<<<dim3(D.m, D.w_per_head ? D.H : 1), D.r, 0, st>>>(reinterpret_cast<const float *>(ws + Y.Tacc), (const __nv_bfloat16 *)M, dW,
-                                                                D.H, D.m, D.r, D.d, D.w_per_head, D.s);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(dw_kernel, dim3(D.m, D.w_per_head ? D.H : 1), dim3(D.r), 0, st, reinterpret_cast<const float *>(ws + Y.Tacc), (const __nv_bfloat16 *)M, dW,
+                               D.H, D.m, D.r, D.d, D.w_per_head, D.s);
     if (e != cudaSuccess) { set_cuda_error(e, "tensor_backward_dw"); return DARKATTN_ERR_CUDA; }
     return DARKATTN_OK;
 }

@@ -100,6 +100,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_nc_kernel(const __grid_con
         *abort_flag = (smem_u32(smem) & 1023u) ? 1 : 0;
         fence_mbar_init();
     }
+    pdl_wait();
     if (tid < 128) sVec[tid] = (KEYS ? p.rhot : p.zt)[(size_t)bh * p.m + slab * 128 + tid];
     if (warp == kEpiWarps) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
     tc_fence_before();
@@ -331,6 +332,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_nc_kernel(const __grid_con
 // Rb = bf16(Racc): the operand of the key pass
 __global__ void nc_round_state_kernel(const float *R, __nv_bfloat16 *Rb, long long n)
 {
+    pdl_wait();
     for (long long i = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * 4; i < n; i += (long long)gridDim.x * blockDim.x * 4) {
         const float4 x = *reinterpret_cast<const float4 *>(R + i);
         *reinterpret_cast<uint2 *>(Rb + i) = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
@@ -343,35 +345,25 @@ cudaError_t launch_nc(const darkattn_plan_s *plan, const NcParams &PQ, const NcP
 {
     using L = NcSmem<D, DV>;
     static_assert(L::kTotal <= 232448, "shared memory budget of one CTA exceeded");
-    cudaError_t e = cudaFuncSetAttribute(tc_bwd_nc_kernel<D, DV, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(tc_bwd_nc_kernel<D, DV, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
-    if (e != cudaSuccess) return e;
     const int grid = PQ.BH * PQ.nslab * PQ.nsplit;
     timer_mark(plan, st, "tc_bwd_nc_q_kernel");
-    tc_bwd_nc_kernel<D, DV, false><<<grid, kThreads, L::kTotal, st>>>(PQ);
-    e = cudaGetLastError();
+    cudaError_t e = launch_pdl(tc_bwd_nc_kernel<D, DV, false>, dim3(grid), dim3(kThreads), L::kTotal, st, PQ);
     if (e != cudaSuccess) return e;
     timer_mark(plan, st, "nc_round_state_kernel");
-    nc_round_state_kernel<<<(unsigned)((nstate / 4 + 255) / 256), 256, 0, st>>>(Racc, Rb, nstate);
-    e = cudaGetLastError();
+    e = launch_pdl(nc_round_state_kernel, dim3((unsigned)((nstate / 4 + 255) / 256)), dim3(256), 0, st, Racc, Rb, nstate);
+    if (e == cudaSuccess && join) e = cudaStreamWaitEvent(st, plan->aux_join, 0);      // dK and dV have been zeroed
     if (e != cudaSuccess) return e;
-    if (join) {
-        e = cudaStreamWaitEvent(st, plan->aux_join, 0);      // dK and dV have been zeroed
-        if (e != cudaSuccess) return e;
-    }
     timer_mark(plan, st, "tc_bwd_nc_k_kernel");
-    tc_bwd_nc_kernel<D, DV, true><<<grid, kThreads, L::kTotal, st>>>(PK);
-    return cudaGetLastError();
+    return launch_pdl(tc_bwd_nc_kernel<D, DV, true>, dim3(grid), dim3(kThreads), L::kTotal, st, PK);
 }
 
 }  // namespace
 
-// The two passes of the non-causal backward. Expects delta computed, Tacc zeroed and (with several
-// slabs) dQ zeroed on `st`, dK and dV zeroed behind plan->aux_join. With `per_head`, dK and dV are the per-query-head
+// The two passes of the non-causal backward. Expects delta computed, Tacc, Racc, rhot and (with several
+// slabs) dQ, dK and dV zeroed on `st` (with `join` dK and dV behind plan->aux_join). With `per_head`, dK and dV are the per-query-head
 // buffers of grouped key/value heads ([BH, N, *]).
 cudaError_t tensor_backward_nc_passes(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V, const void *dO,
-                                      const Stash &stash, void *dQ, void *dK, void *dV, bool per_head, char *ws, cudaStream_t st)
+                                      const Stash &stash, void *dQ, void *dK, void *dV, bool per_head, bool join, char *ws, cudaStream_t st)
 {
     const Dims &D = plan->dims;
     const TensorLayout &Y = plan->tensor;
@@ -402,9 +394,6 @@ cudaError_t tensor_backward_nc_passes(const darkattn_plan_s *plan, const void *Q
     PK.mapOml = PQ.mapOml;
     PK.mapDV = PQ.mapDV;
     const long long nstate = (long long)BH * D.m * D.dv;
-    cudaError_t e = cudaMemsetAsync(ws + Y.Racc, 0, (Y.rhot - Y.Racc) + BH * D.m * 4, st);      // R and rho sums (adjacent)
-    if (e != cudaSuccess) return e;
-    const bool join = add_kv;
     if (D.d == 64 && D.dv == 64) return launch_nc<64, 64>(plan, PQ, PK, fl(Y.Racc), Rb, nstate, join, st);
     if (D.d == 128 && D.dv == 128) return launch_nc<128, 128>(plan, PQ, PK, fl(Y.Racc), Rb, nstate, join, st);
     if (D.d == 64 && D.dv == 128) return launch_nc<64, 128>(plan, PQ, PK, fl(Y.Racc), Rb, nstate, join, st);

@@ -41,14 +41,23 @@ constexpr float kShiftHeadroom = 64.f;
 // 4 d/32 products.
 template <int TC>
 __global__ void __launch_bounds__(128) fold_omega_kernel(const __nv_bfloat16 *W, const __nv_bfloat16 *M, __nv_bfloat16 *Om, __nv_bfloat16 *Oml,
-                                                         int m, int r, int w_per_head, float coef)
+                                                         int m, int r, int w_per_head, float coef, int *cs, int ncs, int *status, float4 *zero,
+                                                         long long nzero)
 {
     constexpr int R = 16, d = 32 * TC;
     __shared__ __align__(16) float sw[R][128];
     __shared__ float part[3][R * TC][32];           // the partial sums of warps 1..3
     const int h = blockIdx.y, l0 = blockIdx.x * R, lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
+    pdl_wait();
     const __nv_bfloat16 *w = W + ((size_t)(w_per_head ? h : 0) * m + l0) * r;
     for (int i = threadIdx.x; i < R * r; i += 128) sw[i / r][i % r] = __bfloat162float(w[i]);
+    {   // what the call's later kernels expect: a clear status word, the key shifts (which the prepass raises to the maximum over
+        // the keys) at the smallest order key, the sums of the non-causal state at zero
+        const int nb = gridDim.x * gridDim.y, b = blockIdx.y * gridDim.x + blockIdx.x;
+        if (b == 0 && threadIdx.x == 0) *status = 0;
+        for (int i = b * 128 + threadIdx.x; i < ncs; i += nb * 128) cs[i] = (int)0x80000000u;
+        for (long long i = b * 128 + threadIdx.x; i < nzero; i += nb * 128) zero[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     __syncthreads();
     const __nv_bfloat16 *Mh = M + (size_t)h * r * d + lane;
     float acc[R][TC];
@@ -90,13 +99,6 @@ __global__ void __launch_bounds__(128) fold_omega_kernel(const __nv_bfloat16 *W,
                 Oml[o] = __float2bfloat16_rn(om - __bfloat162float(hi));
             }
     }
-}
-
-// Start value of the key-side shifts, which tc_key_prepass_kernel raises to the maximum over the keys: the smallest order key.
-__global__ void shift_init_kernel(int *cs, int n)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) cs[i] = (int)0x80000000u;
 }
 
 // ------------------------------------------------------------------ key prepass: norms and key-side shifts in one pass over K
@@ -143,6 +145,7 @@ __global__ void __launch_bounds__(160, 1) tc_key_prepass_kernel(const __grid_con
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_wait();
     const uint32_t tmem = *tmem_slot;
     constexpr uint32_t kColX = 0, kColU = 128;      // x~ at 0, U of the two slabs at 128 and 256
     if (*abort_flag) { if (tid == 0) atomicExch(p.status, (int)DARKATTN_ERR_CUDA); }
@@ -375,6 +378,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_causal_kernel(const __grid
         *abort_flag = (smem_u32(smem) & 1023u) ? 1 : 0;
         fence_mbar_init();
     }
+    pdl_wait();
     if (tid < 128) sZ[tid] = fresh ? 0.f : p.zseg[((size_t)bh * p.nsplit + seg) * p.m + slab * 128 + tid];
     if (warp == kEpiWarps) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
     tc_fence_before();
@@ -697,6 +701,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_keys_kernel(const __grid_c
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_wait();
     const uint32_t tmem = *tmem_slot;
     int *status = p.status;
 
@@ -861,6 +866,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_queries_kernel(const __gri
         *abort_flag = (smem_u32(smem) & 1023u) ? 1 : 0;
         fence_mbar_init();
     }
+    pdl_wait();
     if (tid < 128) sZ[tid] = p.zacc[(size_t)bh * p.m + slab * 128 + tid];
     if (warp == kEpiWarps) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
     tc_fence_before();
@@ -974,6 +980,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_queries_kernel(const __gri
 // will look for it (zout == z when that is the workspace itself)
 __global__ void state_to_bf16_kernel(const float *S, __nv_bfloat16 *Sb, long long n, const float *z, float *zout, long long nz)
 {
+    pdl_wait();
     const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
     for (long long i = i0; i < n; i += step) Sb[i] = __float2bfloat16_rn(S[i]);
     if (zout != z)
@@ -984,6 +991,7 @@ __global__ void state_to_bf16_kernel(const float *S, __nv_bfloat16 *Sb, long lon
 // copy of the prefixed S. One thread per (bh, e).
 __global__ void segment_prefix_kernel(float *S, __nv_bfloat16 *Sb, float *z, int nseg, long long E, int m, long long total)
 {
+    pdl_wait();
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= total) return;
     const long long bh = i / E, e = i % E;
@@ -1014,6 +1022,7 @@ template <int NS>
 __global__ void combine_kernel(const __nv_bfloat16 *pnum, const float *pdr, __nv_bfloat16 *O, float2 *sv,
                                long long rows, int dv, int nslab_rt, int *status)
 {
+    pdl_wait();
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const int per_row = dv / 8;
     if (i >= rows * per_row) return;
@@ -1086,23 +1095,16 @@ cudaError_t launch_main(const MainParams &P, int grid, cudaStream_t st)
     if constexpr (MODE == MODE_CAUSAL) {
         using L = FwdCausalSmem<D, DV>;
         static_assert(L::kTotal <= 232448, "shared memory budget of one CTA exceeded");
-        cudaError_t e = cudaFuncSetAttribute(tc_fwd_causal_kernel<D, DV>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
-        if (e != cudaSuccess) return e;
-        tc_fwd_causal_kernel<D, DV><<<grid, kThreads, L::kTotal, st>>>(P);
+        return launch_pdl(tc_fwd_causal_kernel<D, DV>, dim3(grid), dim3(kThreads), L::kTotal, st, P);
     } else if constexpr (MODE == MODE_KEYS) {
         using L = FwdKeysSmem<D, DV>;
         static_assert(L::kTotal <= 232448, "shared memory budget of one CTA exceeded");
-        cudaError_t e = cudaFuncSetAttribute(tc_fwd_keys_kernel<D, DV>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
-        if (e != cudaSuccess) return e;
-        tc_fwd_keys_kernel<D, DV><<<grid, kThreads, L::kTotal, st>>>(P);
+        return launch_pdl(tc_fwd_keys_kernel<D, DV>, dim3(grid), dim3(kThreads), L::kTotal, st, P);
     } else {
         using L = FwdQueriesSmem<D, DV>;
         static_assert(L::kTotal <= 232448, "shared memory budget of one CTA exceeded");
-        cudaError_t e = cudaFuncSetAttribute(tc_fwd_queries_kernel<D, DV>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
-        if (e != cudaSuccess) return e;
-        tc_fwd_queries_kernel<D, DV><<<grid, kThreads, L::kTotal, st>>>(P);
+        return launch_pdl(tc_fwd_queries_kernel<D, DV>, dim3(grid), dim3(kThreads), L::kTotal, st, P);
     }
-    return cudaGetLastError();
 }
 
 template <int MODE>
@@ -1165,7 +1167,7 @@ void tensor_make_layout(darkattn_plan_s *plan)
     Y.Sb = take(off, BH * nstate * m * dv * 2);
     Y.sv = take(off, BH * N * 8);
     Y.zc = take(off, D.causal ? BH * (size_t)Y.T * m * 4 : 0);
-    plan->launches_fwd = D.causal ? (nsplit > 1 ? 7 : 5) : 7;
+    plan->launches_fwd = D.causal ? (nsplit > 1 ? 6 : 4) : 6;
     {
         size_t so = 0;
         Y.sv_sv = take(so, BH * N * 8);
@@ -1217,30 +1219,16 @@ cudaError_t tensor_prologue(const darkattn_plan_s *plan, const void *K, const vo
         !make_map(&PP.mapOm, out.Om, (size_t)D.H * D.m, D.d, 128))
         return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
-    auto chk = [&]() { cudaError_t x = cudaGetLastError(); if (x != cudaSuccess && e == cudaSuccess) e = x; };
-
-    // The two small kernels that read only M and W run on the plan's side stream (with per-kernel timing on,
-    // everything stays on one stream).
-    const bool beside = !plan->timer.on && ensure_aux(plan) == cudaSuccess;
-    cudaStream_t sp = beside ? plan->aux_stream : st;
-    if (beside) {
-        e = cudaEventRecord(plan->aux_fork, st);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(sp, plan->aux_fork, 0);
-    }
+    auto keep = [&](cudaError_t x) { if (x != cudaSuccess && e == cudaSuccess) e = x; };
     timer_mark(plan, st, "fold_omega_kernel");
-    if (D.d == 64)
-        fold_omega_kernel<2><<<dim3(D.m / 16, D.H), 128, 0, sp>>>((const __nv_bfloat16 *)W, (const __nv_bfloat16 *)M, out.Om, out.Oml, D.m, D.r,
-                                                               D.w_per_head, kLog2e * D.s);
-    else
-        fold_omega_kernel<4><<<dim3(D.m / 16, D.H), 128, 0, sp>>>((const __nv_bfloat16 *)W, (const __nv_bfloat16 *)M, out.Om, out.Oml, D.m, D.r,
-                                                               D.w_per_head, kLog2e * D.s);
-    chk();
-    timer_mark(plan, st, "shift_init_kernel");
-    shift_init_kernel<<<(unsigned)((BH * Y.nslab + 255) / 256), 256, 0, sp>>>(reinterpret_cast<int *>(out.cs), (int)(BH * Y.nslab));
-    chk();
-    if (beside && e == cudaSuccess) e = cudaEventRecord(plan->aux_join, sp);
-
-    if (beside && e == cudaSuccess) e = cudaStreamWaitEvent(st, plan->aux_join, 0);
+    // (S and z sums of the non-causal key pass: adjacent, multiples of 256 bytes)
+    float4 *zero = D.causal ? nullptr : reinterpret_cast<float4 *>(ws + Y.Sacc);
+    const long long nzero = D.causal ? 0 : (long long)((Y.Sb - Y.Sacc) / 16);
+    int *status = reinterpret_cast<int *>(ws + Y.status), *cs = reinterpret_cast<int *>(out.cs);
+    const int ncs = (int)(BH * Y.nslab);
+    const dim3 fold_grid(D.m / 16, D.H);
+    keep(launch_pdl(D.d == 64 ? fold_omega_kernel<2> : fold_omega_kernel<4>, fold_grid, dim3(128), 0, st, (const __nv_bfloat16 *)W, (const __nv_bfloat16 *)M,
+                    out.Om, out.Oml, D.m, D.r, D.w_per_head, kLog2e * D.s, cs, ncs, status, zero, nzero));
 
     // key norms and key-side shifts in one pass over K
     PP.nK = out.nK; PP.cs = reinterpret_cast<int *>(out.cs); PP.status = reinterpret_cast<int *>(ws + Y.status);
@@ -1250,14 +1238,7 @@ cudaError_t tensor_prologue(const darkattn_plan_s *plan, const void *K, const vo
     PP.nsplit = pick_splits((long long)BH * PP.npair, Y.T, 1.5, 3.0, 64, per_sm * 148);
     const int smem_bytes = 5 * 128 * D.d * 2 + 128;
     timer_mark(plan, st, "tc_key_prepass_kernel");
-    if (D.d == 64) {
-        cudaFuncSetAttribute(tc_key_prepass_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-        tc_key_prepass_kernel<64><<<(unsigned)(BH * PP.npair * PP.nsplit), 160, smem_bytes, st>>>(PP);
-    } else {
-        cudaFuncSetAttribute(tc_key_prepass_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-        tc_key_prepass_kernel<128><<<(unsigned)(BH * PP.npair * PP.nsplit), 160, smem_bytes, st>>>(PP);
-    }
-    chk();
+    keep(launch_pdl(D.d == 64 ? tc_key_prepass_kernel<64> : tc_key_prepass_kernel<128>, dim3((unsigned)(BH * PP.npair * PP.nsplit)), dim3(160), smem_bytes, st, PP));
     return e;
 }
 
@@ -1283,7 +1264,7 @@ darkattn_status_t tensor_forward(const darkattn_plan_s *plan, const void *Q, con
     if (!ok) { set_cuda_error(cudaErrorInvalidValue, "tensor_forward: tensor map encode"); return DARKATTN_ERR_CUDA; }
 
     cudaError_t e = tensor_prologue(plan, K, M, W, ws, stash, st);
-    auto chk = [&]() { cudaError_t x = cudaGetLastError(); if (x != cudaSuccess && e == cudaSuccess) e = x; };
+    auto keep = [&](cudaError_t x) { if (x != cudaSuccess && e == cudaSuccess) e = x; };
 
     P.nK = stash.nK; P.cs = stash.cs; P.zc = stash.zc; P.pdr = fl(Y.pdr); P.Sacc = fl(Y.Sacc); P.zacc = fl(Y.zacc);
     P.status = reinterpret_cast<int *>(ws + Y.status);
@@ -1298,39 +1279,28 @@ darkattn_status_t tensor_forward(const darkattn_plan_s *plan, const void *Q, con
         if (Y.nsplit > 1) {      // segment states, then their exclusive prefix
             P.Sseg = fl(Y.Sacc); P.zseg = fl(Y.zacc);
             timer_mark(plan, st, "tc_fwd_keys_kernel");
-            cudaError_t x = launch_main_shape<MODE_KEYS>(D.d, D.dv, P, units * Y.nsplit, st);
-            if (x != cudaSuccess && e == cudaSuccess) e = x;
+            keep(launch_main_shape<MODE_KEYS>(D.d, D.dv, P, units * Y.nsplit, st));
             const long long E = (long long)D.m * D.dv, total = (long long)BH * E;
             timer_mark(plan, st, "segment_prefix_kernel");
-            segment_prefix_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(fl(Y.Sacc), bf(Y.Sb), fl(Y.zacc), Y.nsplit, E, D.m, total);
-            chk();
+            keep(launch_pdl(segment_prefix_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, fl(Y.Sacc), bf(Y.Sb), fl(Y.zacc), Y.nsplit, E, D.m, total));
         }
         timer_mark(plan, st, "tc_fwd_causal_kernel");
-        cudaError_t x = launch_main_shape<MODE_CAUSAL>(D.d, D.dv, P, units * Y.nsplit, st);
-        if (x != cudaSuccess && e == cudaSuccess) e = x;
+        keep(launch_main_shape<MODE_CAUSAL>(D.d, D.dv, P, units * Y.nsplit, st));
     } else {
-        e = (e == cudaSuccess) ? cudaMemsetAsync(ws + Y.Sacc, 0, (Y.Sb - Y.Sacc), st) : e;   // S and z sums
         timer_mark(plan, st, "tc_fwd_keys_kernel");
-        cudaError_t x = launch_main_shape<MODE_KEYS>(D.d, D.dv, P, units * Y.nsplit, st);
-        if (x != cudaSuccess && e == cudaSuccess) e = x;
+        keep(launch_main_shape<MODE_KEYS>(D.d, D.dv, P, units * Y.nsplit, st));
         const long long n = (long long)BH * D.m * D.dv;
         timer_mark(plan, st, "state_to_bf16_kernel");
-        state_to_bf16_kernel<<<(unsigned)((n + 1023) / 1024), 256, 0, st>>>(fl(Y.Sacc), stash.Sb, n, fl(Y.zacc), stash.zt, (long long)BH * D.m);
-        chk();
+        keep(launch_pdl(state_to_bf16_kernel, dim3((unsigned)((n + 1023) / 1024)), dim3(256), 0, st, (const float *)fl(Y.Sacc), stash.Sb, n, (const float *)fl(Y.zacc), stash.zt, (long long)BH * D.m));
         timer_mark(plan, st, "tc_fwd_queries_kernel");
-        x = launch_main_shape<MODE_QUERIES>(D.d, D.dv, P, units * Y.nsplit, st);
-        if (x != cudaSuccess && e == cudaSuccess) e = x;
+        keep(launch_main_shape<MODE_QUERIES>(D.d, D.dv, P, units * Y.nsplit, st));
     }
     {
         const long long rows = (long long)BH * N, threads = rows * (D.dv / 8);
         timer_mark(plan, st, "combine_kernel");
         const unsigned grid = (unsigned)((threads + 255) / 256);
-        __nv_bfloat16 *Ob = (__nv_bfloat16 *)O;
-        if (Y.nslab == 1) combine_kernel<1><<<grid, 256, 0, st>>>(bf(Y.pnum), fl(Y.pdr), Ob, stash.sv, rows, D.dv, 1, P.status);
-        else if (Y.nslab == 2) combine_kernel<2><<<grid, 256, 0, st>>>(bf(Y.pnum), fl(Y.pdr), Ob, stash.sv, rows, D.dv, 2, P.status);
-        else if (Y.nslab == 4) combine_kernel<4><<<grid, 256, 0, st>>>(bf(Y.pnum), fl(Y.pdr), Ob, stash.sv, rows, D.dv, 4, P.status);
-        else combine_kernel<0><<<grid, 256, 0, st>>>(bf(Y.pnum), fl(Y.pdr), Ob, stash.sv, rows, D.dv, Y.nslab, P.status);
-        chk();
+        auto *combine = Y.nslab == 1 ? combine_kernel<1> : Y.nslab == 2 ? combine_kernel<2> : Y.nslab == 4 ? combine_kernel<4> : combine_kernel<0>;
+        keep(launch_pdl(combine, dim3(grid), dim3(256), 0, st, (const __nv_bfloat16 *)bf(Y.pnum), (const float *)fl(Y.pdr), (__nv_bfloat16 *)O, stash.sv, rows, D.dv, Y.nslab, P.status));
     }
     if (e != cudaSuccess) { set_cuda_error(e, "tensor_forward"); return DARKATTN_ERR_CUDA; }
     return DARKATTN_OK;
