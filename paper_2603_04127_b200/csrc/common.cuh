@@ -65,8 +65,8 @@ struct TensorLayout {
     size_t pnum;    // partial numerators, bf16 [nslab, BH, N, dv]
     size_t pdr;     // per slab and row: the partial normalisers of the four 32-column groups and the exponent the partial is
                     // scaled by, fp32 [nslab, BH, N, 8] (entries 0..3 and 4; 5..7 unused)
-    size_t Sacc;    // non-causal state sums, fp32 [BH, m, dv]
-    size_t zacc;    // fp32 [BH, m]
+    size_t Sacc;    // states of the key pass, fp32: non-causal [BH, m, dv], causal in segments [BH, npiece, m, dv]
+    size_t zacc;    // its z, fp32, four parts each
     size_t Sb;      // bf16 copy of the state, [BH, m, dv]
     size_t sv;      // per-row normaliser and the exponent it is scaled by, float2 [BH, N] (forward -> backward)
     // backward only
@@ -87,7 +87,9 @@ struct TensorLayout {
     // the forward -> backward stash (`saved`): per-row normalisers, key norms, folded projections, key shifts
     size_t sv_sv, sv_nK, sv_Om, sv_Oml, sv_cs, sv_zc, sv_Sb, sv_zt, sv_Sst, sv_Bphi, sv_bytes;
     size_t zc;      // workspace copy of the stash's per-chunk z (causal): sum_j phi(K)_jl over the chunks before t, fp32 [BH, T, m]
-    int nslab, T, nsplit;
+    size_t Sseg, zseg;   // causal, cut into segments: the state and z before each segment, fp32
+    size_t zq;      // non-causal: z of the whole sequence (workspace copy of the stash's)
+    int nslab, T, nsplit, npiece;     // npiece: pieces the key pass cuts the first nsplit - 1 segments into
 };
 
 // Where one call keeps what the prologue and the forward pass leave for the backward pass: in the
@@ -109,7 +111,7 @@ inline Stash stash_in_workspace(const TensorLayout &Y, char *ws)
                  reinterpret_cast<__nv_bfloat16 *>(ws + Y.Om), reinterpret_cast<__nv_bfloat16 *>(ws + Y.Oml),
                  reinterpret_cast<float *>(ws + Y.cs),
                  reinterpret_cast<float *>(ws + Y.zc), reinterpret_cast<__nv_bfloat16 *>(ws + Y.Sb),
-                 reinterpret_cast<float *>(ws + Y.zacc), reinterpret_cast<__nv_bfloat16 *>(ws + Y.Sst),
+                 reinterpret_cast<float *>(ws + Y.zq), reinterpret_cast<__nv_bfloat16 *>(ws + Y.Sst),
                  reinterpret_cast<__nv_bfloat16 *>(ws + Y.Bphi)};
 }
 inline Stash stash_in_saved(const TensorLayout &Y, void *saved)

@@ -26,7 +26,6 @@ using namespace tc;
 namespace {
 
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr int kMaxNsplit = 64;
 // The key features are scaled so that the largest one of a (batch, head, slab) is 2^kShiftHeadroom rather than 1: fp32 and
 // bf16 reach down to 2^-126, so keys up to 190 binary orders below the largest keep a nonzero feature (causal prefixes see
 // only some of the keys), while sums over 2^17 keys of products with values and query features (<= 1) stay far from 2^127.
@@ -263,12 +262,14 @@ struct MainParams {
     const float *nK;     // [BH, N]      key norms in log2 units
     const float *cs;     // [BH, nslab]  key-side shift per slab (log2 units)
     float *pdr;          // [nslab, BH*N, 8]  partial normalisers of the four column groups (0..3), exponent the partial is scaled by (4)
-    float *Sacc;         // [BH, m, DV]  fp32 state sums (non-causal key pass, atomics)
-    float *zacc;         // [BH, m]
-    // causal scan cut into nsplit segments of the sequence: the key pass stores one state per segment
-    // (Sseg [BH, nsplit, m, DV], zseg [BH, nsplit, m]) instead of adding into Sacc; after an exclusive prefix over the
-    // segments the causal kernel of segment s > 0 starts from Sseg[bh, s] (its bf16 copy comes through mapSb).
-    float *Sseg, *zseg;
+    // Key pass: sums over all keys, [BH, m, DV] and [BH, m, 4 parts]; with segments (npiece > 0) the states of the pieces,
+    // [BH, npiece, m, DV] and [BH, npiece, m, 4].
+    float *Sacc, *zacc;
+    const float *zq;     // [BH, m]  z for the query pass
+    // causal scan cut into nsplit segments of the sequence: the causal kernel of segment s > 0 starts from the state
+    // before it, Sseg[bh, s] and zseg[bh, s] ([BH, nsplit, ...]; the bf16 copy comes through mapSb).
+    const float *Sseg, *zseg;
+    int npiece;          // pieces the key pass cuts the nsplit - 1 segments of a (batch, head) into, 0 without segments
     float *zc;           // causal: z before chunk t for the backward pass, [BH, T, m] (row 0 not written)
     int *status;
     int N, H, Hkv, BH, m, nslab, T, nsplit;
@@ -646,56 +647,121 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_causal_kernel(const __grid
     if (warp == kEpiWarps) tmem_dealloc(tmem, 512);
 }
 
-// ------------------------------------------------------------------ non-causal, key pass: S = phi(K)^T V, z = phi(K)^T 1
+// ------------------------------------------------------------------ key pass: S = phi(K)^T V, z = phi(K)^T 1
+// Both passes below run one CTA per SM over a list of pieces (a run of tiles of one (batch, head, slab)); the roles (a warp
+// for TMA, a warp for the MMAs, the read-out warps) walk the list by themselves, so that one piece's end overlaps the next
+// one's start except where the slab's operands change. Key pass: the line of all (unit, tile) is cut evenly over the CTAs and
+// the pieces' states are added up by atomics; with segments (causal) the pieces are fixed and each stores its own state.
+struct Piece { int unit, t0, t1, dst; bool whole; };
+
+struct PieceList {
+    long long x, end;       // line: tiles [x, end); fixed pieces: index and count
+    int step;
+    __device__ __forceinline__ PieceList(const MainParams &p, int T)
+    {
+        if (p.npiece) { x = blockIdx.x; end = (long long)p.BH * p.nslab * p.npiece; step = gridDim.x; }
+        else {
+            const long long total = (long long)p.BH * p.nslab * T;
+            x = total * blockIdx.x / gridDim.x; end = total * (blockIdx.x + 1) / gridDim.x; step = 0;
+        }
+    }
+    __device__ __forceinline__ bool next(const MainParams &p, int T, Piece &c)
+    {
+        if (x >= end) return false;
+        if (step) {
+            const int per = p.npiece / (p.nsplit - 1);           // pieces of a segment; the last segment's state is not needed
+            c.unit = (int)(x / p.npiece); c.dst = (int)(x % p.npiece);
+            const int seg = c.dst / per, j = c.dst % per;
+            const int b0 = (int)((long long)T * seg / p.nsplit), len = (int)((long long)T * (seg + 1) / p.nsplit) - b0;
+            c.t0 = b0 + (int)((long long)len * j / per); c.t1 = b0 + (int)((long long)len * (j + 1) / per);
+            c.whole = true;
+            x += step;
+        } else {
+            c.unit = (int)(x / T); c.t0 = (int)(x % T); c.dst = 0;
+            c.t1 = (int)min((long long)T, c.t0 + (end - x));
+            c.whole = (c.t0 == 0 && c.t1 == T);
+            x += c.t1 - c.t0;
+        }
+        return true;
+    }
+};
+
+constexpr int kPassThreads = 576;       // 16 read-out warps, TMA warp, MMA warp; the key pass has a second TMA warp
+constexpr int kKeysThreads = 608;
+
+// (u0, u1) - (n0, n1) - (c, c)
+__device__ __forceinline__ void sub2(float &u0, float &u1, float n0, float n1, float c)
+{
+    asm("{\n\t.reg .b64 a, b, m, d;\n\t"
+        "mov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tmov.b64 d, {%4, %4};\n\tmov.b64 m, {%5, %5};\n\t"
+        "fma.rn.f32x2 a, b, m, a;\n\t"
+        "fma.rn.f32x2 a, d, m, a;\n\t"
+        "mov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(u0), "+f"(u1) : "f"(n0), "f"(n1), "f"(c), "f"(-1.f));
+}
+__device__ __forceinline__ void add2(float &a0, float &a1, float b0, float b1)
+{
+    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tadd.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(a0), "+f"(a1) : "f"(b0), "f"(b1));
+}
+__device__ __forceinline__ void fma2(float &a0, float &a1, float b0, float b1, float c0, float c1)
+{
+    asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tmov.b64 c, {%4, %5};\n\tfma.rn.f32x2 a, b, c, a;\n\tmov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(a0), "+f"(a1) : "f"(b0), "f"(b1), "f"(c0), "f"(c1));
+}
+// untiled copy of a multiple of 16 bytes (both addresses 16-byte aligned) into shared memory
+__device__ __forceinline__ void bulk_load(void *smem_dst, const void *src, uint32_t bytes, uint64_t *bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(smem_u32(smem_dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void red_add4(float *dst, float a, float b, float c, float d)
+{
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+
 template <int D, int DV>
 struct FwdKeysSmem {
-    // K and V tiles sit in rings of kStages buffers (4 where they are small enough), so that a tile's load is issued
-    // several tiles before its use; TMEM regions alternate between two, and so do the phi(K) tiles where two fit.
-    static constexpr int kFixed = 2 * 128 * D * 2 + 2048 + 256;       // both halves of the folded projections, ones, barriers
-    static constexpr int kStages = (kFixed + 4 * 128 * (D + DV) * 2 + 2 * 32768 <= 232448) ? 4 : 2;
-    static constexpr int kFKs = (kFixed + kStages * 128 * (D + DV) * 2 + 2 * 32768 <= 232448) ? 2 : 1;
+    static constexpr int kNormSlots = 8;       // see the loader: a slot is loaded again long after its tile has been read out
+    static constexpr int kFixed = 2 * 128 * D * 2 + kNormSlots * 512 + 512;
+    static constexpr int kStages = (kFixed + 4 * 128 * (D + DV) * 2 <= 232448) ? 4 : 2;
     static constexpr int kOm = 0;
     static constexpr int kOml = kOm + 128 * D * 2;
     static constexpr int kK = kOml + 128 * D * 2;
     static constexpr int kV = kK + kStages * 128 * D * 2;
-    static constexpr int kFK = kV + kStages * 128 * DV * 2;   // phi(K) tiles
-    static constexpr int kOnes = kFK + kFKs * 32768;
-    static constexpr int kBars = kOnes + 2048;
-    static constexpr int kTotal = kBars + 256;
+    static constexpr int kNorm = kV + kStages * 128 * DV * 2;
+    static constexpr int kBars = kNorm + kNormSlots * 512;
+    static constexpr int kTotal = kBars + 512;
 };
 
-// barriers of the key pass: Omega, K ring, V ring, then pairs (projection done, state update done, phi(K) written)
-enum KyBars { YB_OM = 0, YB_K0 = 1, YB_V0 = 5, YM2_0 = 9, YM2_1, YMS_0, YMS_1, YE1_0, YE1_1, YNBARS };
+// Omega loaded / free; K, V rings loaded / free; norms loaded; U ready / phi(K)^T written (three regions); state ready / read
+enum KyBars { YB_OM, YB_OMF, YB_K, YB_V = YB_K + 4, YB_KF = YB_V + 4, YB_VF = YB_KF + 4, YB_N = YB_VF + 4, YB_U = YB_N + 8, YB_S = YB_U + 3,
+              YB_E, YB_SR = YB_E + 3, YNBARS };
 
-// One CTA per (b, h, slab, token split); tiles alternate between two sets of buffers and two TMEM regions so that
-// the projection of tile i+1 runs while the epilogue warps exponentiate tile i.
+// The tile's exponents are formed transposed, U^T = Omega K^T: a lane of tensor memory is a feature, a column a token. Then
+// phi(K)^T, packed to bf16 in place by the warp that read it, is the A operand of S += phi(K)^T V straight from tensor memory
+// (no shared-memory tile, no proxy fence), z is a sum along a thread's own columns (no MMAs against ones), and what is left of
+// tensor memory holds three tiles: the projections run two tiles ahead and every warp goes from tile to tile without waiting
+// for any other. Bound by the exponentials (16384 per tile, 16 per clock and SM) at d = 64 and by MMA issue (24 per tile)
+// at d = 128. Encoder shape 8 x 12 heads, 4096 tokens, d 64, m 256: 101 -> 64 us; 4 x 16 heads, 8192 tokens, d 128: 138 -> 104 us.
 template <int D, int DV>
-__global__ void __launch_bounds__(kThreads, 1) tc_fwd_keys_kernel(const __grid_constant__ MainParams p)
+__global__ void __launch_bounds__(kKeysThreads, 1) tc_fwd_keys_kernel(const __grid_constant__ MainParams p)
 {
     using L = FwdKeysSmem<D, DV>;
     extern __shared__ __align__(1024) unsigned char smem[];
-    constexpr int kXT = 128 * D * 2, kVT = 128 * DV * 2;
-    unsigned char *sOm = smem + L::kOm, *sOml = smem + L::kOml, *sK = smem + L::kK, *sV = smem + L::kV, *sFK = smem + L::kFK, *sOnes = smem + L::kOnes;
-    constexpr int kFKstride = (L::kFKs == 2) ? 32768 : 0;     // one phi(K) tile: tile i + 1 is written once the state update of tile i is done
+    constexpr int kXT = 128 * D * 2, kVT = 128 * DV * 2, NST = L::kStages, NN = L::kNormSlots;
+    unsigned char *sOm = smem + L::kOm, *sOml = smem + L::kOml, *sK = smem + L::kK, *sV = smem + L::kV;
+    float *sNorm = reinterpret_cast<float *>(smem + L::kNorm);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L::kBars);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + YNBARS);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + YNBARS + 1);
-
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int unit = blockIdx.x / p.nsplit, split = blockIdx.x % p.nsplit;
-    const int bh = unit / p.nslab, slab = unit % p.nslab, h = bh % p.H;
-    const int t0 = (int)((long long)p.T * split / p.nsplit), t1 = (int)((long long)p.T * (split + 1) / p.nsplit);
-    const int n = t1 - t0, row0 = bh * p.N, rowk0 = kv_row0(bh, p.H, p.Hkv, p.N);
 
     if (tid == 0) {
-        for (int i = 0; i < YE1_0; ++i) mbar_init(bars + i, 1);
-        mbar_init(bars + YE1_0, kEpiWarps); mbar_init(bars + YE1_1, kEpiWarps);
+        for (int i = 0; i < YB_E; ++i) mbar_init(bars + i, 1);
+        for (int i = YB_E; i < YNBARS; ++i) mbar_init(bars + i, kEpiWarps);
         *abort_flag = (smem_u32(smem) & 1023u) ? 1 : 0;
         fence_mbar_init();
-    }
-    if (tid < 128) {
-        *reinterpret_cast<uint4 *>(sOnes + tid * 16) = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
-        fence_async_smem();
     }
     if (warp == kEpiWarps) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
     tc_fence_before();
@@ -704,117 +770,163 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_keys_kernel(const __grid_c
     pdl_wait();
     const uint32_t tmem = *tmem_slot;
     int *status = p.status;
+    PieceList list(p, p.T);
+    Piece c;
 
     if (*abort_flag) {
         if (tid == 0) atomicExch(status, (int)DARKATTN_ERR_CUDA);
-    } else if (n <= 0) {
-    } else if (warp == kEpiWarps) {
+    } else if (warp == kEpiWarps) {                     // ---- loads
         if ((tid & 31) == 0) {
-            constexpr int NST = L::kStages;
-            auto load_k = [&](int i) {
-                const int b = i % NST;
-                mbar_expect_tx(bars + YB_K0 + b, kXT);
-                for (int a = 0; a < D / 64; ++a) tma_load_2d(sK + b * kXT + a * 16384, &p.mapK, bars + YB_K0 + b, a * 64, rowk0 + (t0 + i) * 128);
-            };
-            auto load_v = [&](int i) {
-                const int b = i % NST;
-                mbar_expect_tx(bars + YB_V0 + b, kVT);
-                for (int a = 0; a < DV / 64; ++a) tma_load_2d(sV + b * kVT + a * 16384, &p.mapV, bars + YB_V0 + b, a * 64, rowk0 + (t0 + i) * 128);
-            };
-            const TileDesc tOm(sOm), tOml(sOml), tF0(sFK), tF1(sFK + kFKstride);
-            const uint64_t ones_desc = make_sdesc(smem_u32(sOnes), 16384, 1024);
-            const uint32_t id_kk = make_idesc(128, 128, 0, 0), id_s = make_idesc(128, DV, 1, 1), id_z = make_idesc(128, 16, 1, 1);
-
-            mbar_expect_tx(bars + YB_OM, 2 * 128 * D * 2);
-            for (int a = 0; a < D / 64; ++a) {
-                tma_load_2d(sOm + a * 16384, &p.mapOm, bars + YB_OM, a * 64, h * p.m + slab * 128);
-                tma_load_2d(sOml + a * 16384, &p.mapOml, bars + YB_OM, a * 64, h * p.m + slab * 128);
+            bool ok = true;
+            int it = 0;
+            for (int pc = 0; ok && list.next(p, p.T, c); ++pc) {
+                const int bh = c.unit / p.nslab, slab = c.unit % p.nslab, h = bh % p.H, rowk0 = kv_row0(bh, p.H, p.Hkv, p.N);
+                const float *nK = p.nK + (size_t)bh * p.N;
+                if (pc > 0) ok = wait_or_abort(bars + YB_OMF, (pc - 1) & 1, status, abort_flag);      // the piece before is projected
+                if (!ok) break;
+                mbar_expect_tx(bars + YB_OM, 2 * kXT);
+                for (int a = 0; a < D / 64; ++a) {
+                    tma_load_2d(sOm + a * 16384, &p.mapOm, bars + YB_OM, a * 64, h * p.m + slab * 128);
+                    tma_load_2d(sOml + a * 16384, &p.mapOml, bars + YB_OM, a * 64, h * p.m + slab * 128);
+                }
+                for (int t = c.t0; t < c.t1; ++t, ++it) {
+                    const int b = it % NST, y = rowk0 + t * 128;
+                    if (it >= NST) ok = wait_or_abort(bars + YB_KF + b, (it / NST - 1) & 1, status, abort_flag);
+                    if (!ok) break;
+                    mbar_expect_tx(bars + YB_K + b, kXT);
+                    for (int a = 0; a < D / 64; ++a) tma_load_2d(sK + b * kXT + a * 16384, &p.mapK, bars + YB_K + b, a * 64, y);
+                    // Here tile it - NST is projected, hence (the projections run two tiles ahead of the state) all warps are
+                    // done with tile it - NST - 3 and with the norms of tile it - 8.
+                    static_assert(NST + 3 <= NN, "a slot of norms would be loaded over");
+                    mbar_expect_tx(bars + YB_N + it % NN, 512);
+                    bulk_load(sNorm + (it % NN) * 128, nK + (size_t)t * 128, 512, bars + YB_N + it % NN);
+                    if (NST == 2 && t + 2 < c.t1)        // with a short ring the next loads come out of L2
+                        for (int a = 0; a < D / 64; ++a) tma_prefetch_l2_2d(&p.mapK, a * 64, y + 256);
+                }
             }
-            for (int i = 0; i < NST && i < n; ++i) { load_k(i); load_v(i); }
-            bool ok = wait_or_abort(bars + YB_OM, 0, status, abort_flag);
-            if (ok) ok = wait_or_abort(bars + YB_K0, 0, status, abort_flag);
-            if (ok) {
-                tc_fence_after();
-                const TileDesc tK0(sK);
-                issue_projection<D>(tmem + kColR1, tK0, tOm, tOml, id_kk);
-                mma_commit(bars + YM2_0);
+        }
+    } else if (warp == kEpiWarps + 2) {                 // ---- loads of V, whose tiles are held two steps longer than those of K
+        if ((tid & 31) == 0) {
+            bool ok = true;
+            int it = 0;
+            while (ok && list.next(p, p.T, c)) {
+                const int rowk0 = kv_row0(c.unit / p.nslab, p.H, p.Hkv, p.N);
+                for (int t = c.t0; t < c.t1; ++t, ++it) {
+                    const int b = it % NST, y = rowk0 + t * 128;
+                    if (it >= NST) ok = wait_or_abort(bars + YB_VF + b, (it / NST - 1) & 1, status, abort_flag);
+                    if (!ok) break;
+                    mbar_expect_tx(bars + YB_V + b, kVT);
+                    for (int a = 0; a < DV / 64; ++a) tma_load_2d(sV + b * kVT + a * 16384, &p.mapV, bars + YB_V + b, a * 64, y);
+                    if (NST == 2 && t + 2 < c.t1)
+                        for (int a = 0; a < DV / 64; ++a) tma_prefetch_l2_2d(&p.mapV, a * 64, y + 256);
+                }
             }
-            for (int i = 0; i < n && ok; ++i) {
-                const int b = i & 1;
-                const uint32_t phb = (i >> 1) & 1;
-                if (i + 1 < n) {       // projection of the next tile into the other region (read out two tiles ago)
-                    const int sn = (i + 1) % NST;
-                    ok = wait_or_abort(bars + YB_K0 + sn, ((i + 1) / NST) & 1, status, abort_flag);
+        }
+    } else if (warp == kEpiWarps + 1) {                 // ---- MMAs
+        if ((tid & 31) == 0) {
+            const TileDesc tOm(sOm), tOml(sOml);
+            const uint32_t id_u = make_idesc(128, 128, 0, 0), id_s = make_idesc(128, DV, 0, 1);
+            bool ok = true;
+            int base = 0;                               // tiles of the pieces before
+            for (int pc = 0; ok && list.next(p, p.T, c); ++pc) {
+                const int n = c.t1 - c.t0;
+                ok = wait_or_abort(bars + YB_OM, pc & 1, status, abort_flag);
+                auto project = [&](int i) {             // U^T of tile i into region i % 3 (the state MMAs that read it are ahead in the pipe)
+                    const int it = base + i, b = it % NST;
+                    ok = ok && wait_or_abort(bars + YB_K + b, (it / NST) & 1, status, abort_flag);
+                    if (!ok) return;
+                    tc_fence_after();
+                    const uint32_t dst = tmem + 128 + 128 * (it % 3);
+                    const TileDesc tK(sK + b * kXT);
+                    _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(dst, kdesc(tOm, k), kdesc(tK, k), id_u, k > 0);
+                    _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(dst, kdesc(tOml, k), kdesc(tK, k), id_u, 1);
+                    mma_commit(bars + YB_U + it % 3);
+                    mma_commit(bars + YB_KF + b);
+                    if (i + 1 == n) mma_commit(bars + YB_OMF);
+                };
+                project(0);
+                if (n > 1) project(1);
+                for (int i = 0; i < n && ok; ++i) {
+                    const int it = base + i, b = it % NST;
+                    if (i + 2 < n) project(i + 2);
+                    ok = ok && wait_or_abort(bars + YB_E + it % 3, (it / 3) & 1, status, abort_flag);
+                    ok = ok && wait_or_abort(bars + YB_V + b, (it / NST) & 1, status, abort_flag);
+                    if (ok && i == 0 && pc > 0) ok = wait_or_abort(bars + YB_SR, (pc - 1) & 1, status, abort_flag);   // the state before has been read out
                     if (!ok) break;
                     tc_fence_after();
-                    const TileDesc tKn(sK + sn * kXT);
-                    issue_projection<D>(tmem + (b ? kColR1 : kColR2), tKn, tOm, tOml, id_kk);
-                    mma_commit(bars + YM2_0 + (b ^ 1));
+                    const uint32_t src = tmem + 128 + 128 * (it % 3);
+                    const TileDesc tV(sV + b * kVT);
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(tmem, src + (k / 2) * 32 + (k % 2) * 8, mndesc(tV, k), id_s, i > 0 || k > 0);
+                    mma_commit(bars + YB_VF + b);
                 }
-                ok = wait_or_abort(bars + YE1_0 + b, phb, status, abort_flag);      // phi(K) of tile i in smem; its K tile is consumed
-                if (!ok) break;
-                if (i + NST < n) load_k(i + NST);
-                ok = wait_or_abort(bars + YB_V0 + i % NST, (i / NST) & 1, status, abort_flag);
+                if (ok) mma_commit(bars + YB_S);
+                base += n;
+            }
+        }
+    } else {                                            // ---- read-out
+        const int lane = tid & 31, q4 = warp & 3, g = warp >> 2, col0 = g * 32;
+        const int r = q4 * 32 + lane;                   // this thread's feature
+        const uint32_t lane_addr = tmem + ((uint32_t)(q4 * 32) << 16);
+        bool ok = true;
+        int it = 0;
+        for (int pc = 0; ok && list.next(p, p.T, c); ++pc) {
+            const int bh = c.unit / p.nslab, slab = c.unit % p.nslab;
+            const float cshift = load_key_shift(p.cs, bh * p.nslab + slab);
+            float z0 = 0.f, z1 = 0.f;
+            for (int t = c.t0; t < c.t1; ++t, ++it) {
+                const uint32_t addr = lane_addr + 128 + 128 * (it % 3) + col0;
+                ok = wait_or_abort(bars + YB_N + it % NN, (it / NN) & 1, status, abort_flag) &&
+                     wait_or_abort(bars + YB_U + it % 3, (it / 3) & 1, status, abort_flag);
+                ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
-                const TileDesc &tF = b ? tF1 : tF0;
-                const TileDesc tVb(sV + (i % NST) * kVT);
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColS, mndesc(tF, k), mndesc(tVb, k), id_s, i > 0 || k > 0);
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColZ, mndesc(tF, k), ones_desc, id_z, i > 0 || k > 0);
-                mma_commit(bars + YMS_0 + b);
-                ok = wait_or_abort(bars + YMS_0 + b, phb, status, abort_flag);
-                if (!ok) break;
-                if (i + NST < n) load_v(i + NST);
-            }
-        }
-    } else {
-        const int lane = tid & 31, q4 = warp & 3, g = warp >> 2, col0 = g * 32;
-        const int r = q4 * 32 + lane;
-        const uint32_t lane_addr = tmem + ((uint32_t)(q4 * 32) << 16);
-        const float cshift = load_key_shift(p.cs, bh * p.nslab + slab);
-        bool ok = true;
-        for (int i = 0; i < n && ok; ++i) {
-            const int b = i & 1;
-            const uint32_t phb = (i >> 1) & 1;
-            const float nk = p.nK[(size_t)row0 + (size_t)(t0 + i) * 128 + r] + cshift;
-            ok = __all_sync(0xffffffffu, wait_or_abort(bars + YM2_0 + b, phb, status, abort_flag));
-            if (!ok) break;
-            if (L::kFKs == 1 && i > 0) {       // the one phi(K) tile is free once the state update of the tile before is done
-                ok = __all_sync(0xffffffffu, wait_or_abort(bars + YMS_0 + (b ^ 1), ((i - 1) >> 1) & 1, status, abort_flag));
-                if (!ok) break;
-            }
-            tc_fence_after();
-            features_to_tile(lane_addr + (b ? kColR2 : kColR1) + col0, nk, sFK + b * kFKstride, r, col0);
-            fence_async_smem();
-            tc_fence_before();
-            mbar_arrive_warp(bars + YE1_0 + b);
-        }
-        if (ok) ok = __all_sync(0xffffffffu, wait_or_abort(bars + YMS_0 + ((n - 1) & 1), ((n - 1) >> 1) & 1, status, abort_flag));
-        if (ok) {        // add this CTA's state to the global sums, or store it as its segment's state
-            tc_fence_after();
-            const size_t srow = ((size_t)bh * p.nsplit + split) * p.m + slab * 128 + r;
-            if (col0 < DV) {
-                uint32_t v[32];
-                tmem_ld32(lane_addr + kColS + col0, v);
+                uint32_t v[32], pk[16];
+                tmem_ld32(addr, v);
+                const float4 *nrm = reinterpret_cast<const float4 *>(sNorm + (it % NN) * 128 + col0);
                 tmem_wait_ld();
-                if (p.Sseg) {
-                    float4 *dst = reinterpret_cast<float4 *>(p.Sseg + srow * DV + col0);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        dst[j] = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]), __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
-                } else {
-                    float *dst = p.Sacc + ((size_t)bh * p.m + slab * 128 + r) * DV + col0;
+                for (int j = 0; j < 8; ++j) {
+                    const float4 nk = nrm[j];
+                    float x[4];
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) atomicAdd(dst + j, __uint_as_float(v[j]));
+                    for (int k = 0; k < 4; ++k) x[k] = __uint_as_float(v[4 * j + k]);
+                    sub2(x[0], x[1], nk.x, nk.y, cshift);
+                    sub2(x[2], x[3], nk.z, nk.w, cshift);
+                    pk[2 * j] = pack_bf16(ex2f(x[0]), ex2f(x[1]));
+                    pk[2 * j + 1] = pack_bf16(ex2f(x[2]), ex2f(x[3]));
+                    // z sums what the MMA multiplies: the rounded features
+                    add2(z0, z1, __uint_as_float(pk[2 * j] << 16), __uint_as_float(pk[2 * j] & 0xffff0000u));
+                    add2(z0, z1, __uint_as_float(pk[2 * j + 1] << 16), __uint_as_float(pk[2 * j + 1] & 0xffff0000u));
+                }
+                tmem_st16(addr, pk);
+                tmem_wait_st();
+                tc_fence_before();
+                mbar_arrive_warp(bars + YB_E + it % 3);
+            }
+            if (!ok) break;
+            ok = __all_sync(0xffffffffu, wait_or_abort(bars + YB_S, pc & 1, status, abort_flag));
+            if (!ok) break;
+            tc_fence_after();
+            const size_t srow = ((size_t)bh * (p.npiece ? p.npiece : 1) + c.dst) * p.m + slab * 128 + r;
+            uint32_t v[32];
+            if (col0 < DV) {
+                tmem_ld32(lane_addr + col0, v);
+                tmem_wait_ld();
+            }
+            tc_fence_before();
+            mbar_arrive_warp(bars + YB_SR);
+            if (col0 < DV) {
+                float *dst = p.Sacc + srow * DV + col0;
+#pragma unroll
+                for (int j = 0; j < 32; j += 4) {
+                    const float a0 = __uint_as_float(v[j]), a1 = __uint_as_float(v[j + 1]), a2 = __uint_as_float(v[j + 2]), a3 = __uint_as_float(v[j + 3]);
+                    if (c.whole) *reinterpret_cast<float4 *>(dst + j) = make_float4(a0, a1, a2, a3);
+                    else red_add4(dst + j, a0, a1, a2, a3);
                 }
             }
-            if (g == 0) {
-                uint32_t v[16];
-                tmem_ld16(lane_addr + kColZ, v);
-                tmem_wait_ld();
-                if (p.Sseg) p.zseg[srow] = __uint_as_float(v[0]);
-                else atomicAdd(p.zacc + (size_t)bh * p.m + slab * 128 + r, __uint_as_float(v[0]));
-            }
+            // z: one part per column group, added up by the kernel that reads the state
+            if (c.whole) p.zacc[4 * srow + g] = z0 + z1;
+            else atomicAdd(p.zacc + 4 * srow + g, z0 + z1);
         }
     }
     if (*abort_flag) __nanosleep(200000);
@@ -826,149 +938,214 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_keys_kernel(const __grid_c
 // ------------------------------------------------------------------ non-causal, query pass: partial O = phi(Q) S, den = phi(Q) z
 template <int D, int DV>
 struct FwdQueriesSmem {
-    // ring of Q tiles: 4 where they fit beside both halves of the folded projections, else 3
-    static constexpr int kStages = (2 * 128 * D * 2 + 4 * 128 * D * 2 + 2 * 128 * DV * 2 + 512 + 2048 + 256 <= 232448) ? 4 : 3;
+    static constexpr int kGroups = DV == 64 ? 4 : 3;       // groups of four warps, each with a tile of its own in flight
+    static constexpr int kStg = kGroups * 4 * 4096;        // a warp's staging: 32 rows of 64 columns
+    static constexpr int kFixed = 2 * 128 * D * 2 + 128 * DV * 2 + kStg + 512 + 512;
+    static constexpr int kStages = (kFixed + 4 * 128 * D * 2 <= 232448) ? 4 : 2;
     static constexpr int kOm = 0;
     static constexpr int kOml = kOm + 128 * D * 2;
     static constexpr int kQ = kOml + 128 * D * 2;
     static constexpr int kSb = kQ + kStages * 128 * D * 2; // bf16 state of the slab [128 l, DV]
-    static constexpr int kStg = kSb + 128 * DV * 2;
-    static constexpr int kZ = kStg + 128 * DV * 2;
-    static constexpr int kRed = kZ + 512;
-    static constexpr int kBars = kRed + 2048;
-    static constexpr int kTotal = kBars + 256;
+    static constexpr int kStage = kSb + 128 * DV * 2;
+    static constexpr int kZ = kStage + kStg;
+    static constexpr int kBars = kZ + 512;
+    static constexpr int kTotal = kBars + 512;
 };
 
-enum QyBars { UB_OM = 0, UB_Q0 = 1, UM1_0 = 5, UM1_1, UM4_0, UM4_1, UE0_0, UE0_1, UE3_0, UE3_1, UNBARS };
+// operands of the slab loaded / free; Q ring loaded / free; U ready, O ready, phi(Q) written, O read (per group)
+enum QyBars { UB_OM, UB_OMF, UB_Q, UB_QF = UB_Q + 4, UB_U = UB_QF + 4, UB_O = UB_U + 4, UB_E = UB_O + 4, UB_R = UB_E + 4, UNBARS = UB_R + 4 };
 
-// TMEM: packed phi(Q) of the two tiles in flight at 0 and 64; R1, R2 hold U_Q and then the output tile.
+// A tile belongs to a group of four warps, a thread to a row: the row's maximum, its normaliser and its output row need no
+// exchange with another warp, and the groups work on different tiles (three or four in flight), so that one's exponentials
+// run under another's waits. Tensor memory: dv = 64: per group U (128 columns), phi(Q) packed into its first 64 in place, O into
+// the other 64; dv = 128: per group U and then O (128), phi(Q) in one of two 64-column slots. Bound like the key pass.
+// Encoder shape (see there) 103 -> 70 us; 4 x 16 heads, 8192 tokens, d 128: 170 -> 129 us.
 template <int D, int DV>
-__global__ void __launch_bounds__(kThreads, 1) tc_fwd_queries_kernel(const __grid_constant__ MainParams p)
+__global__ void __launch_bounds__(kPassThreads, 1) tc_fwd_queries_kernel(const __grid_constant__ MainParams p)
 {
     using L = FwdQueriesSmem<D, DV>;
     extern __shared__ __align__(1024) unsigned char smem[];
-    constexpr int kXT = 128 * D * 2;
-    unsigned char *sOm = smem + L::kOm, *sOml = smem + L::kOml, *sQ = smem + L::kQ, *sSb = smem + L::kSb, *sStg = smem + L::kStg;
-    float *sZ = reinterpret_cast<float *>(smem + L::kZ), *sRed = reinterpret_cast<float *>(smem + L::kRed);
+    constexpr int kXT = 128 * D * 2, NST = L::kStages, G = L::kGroups;
+    unsigned char *sOm = smem + L::kOm, *sOml = smem + L::kOml, *sQ = smem + L::kQ, *sSb = smem + L::kSb;
+    const float *sZ = reinterpret_cast<const float *>(smem + L::kZ);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L::kBars);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + UNBARS);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + UNBARS + 1);
-
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int unit = blockIdx.x / p.nsplit, split = blockIdx.x % p.nsplit;
-    const int bh = unit / p.nslab, slab = unit % p.nslab, h = bh % p.H;
-    const int t0 = (int)((long long)p.T * split / p.nsplit), t1 = (int)((long long)p.T * (split + 1) / p.nsplit);
-    const int n = t1 - t0, row0 = bh * p.N;
 
     if (tid == 0) {
-        for (int i = 0; i < UE0_0; ++i) mbar_init(bars + i, 1);
-        for (int i = UE0_0; i < UNBARS; ++i) mbar_init(bars + i, kEpiWarps);
+        for (int i = 0; i < UB_E; ++i) mbar_init(bars + i, 1);
+        for (int i = UB_E; i < UNBARS; ++i) mbar_init(bars + i, 4);
         *abort_flag = (smem_u32(smem) & 1023u) ? 1 : 0;
         fence_mbar_init();
     }
-    pdl_wait();
-    if (tid < 128) sZ[tid] = p.zacc[(size_t)bh * p.m + slab * 128 + tid];
     if (warp == kEpiWarps) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_wait();
     const uint32_t tmem = *tmem_slot;
     int *status = p.status;
+    PieceList list(p, p.T);
+    Piece c;
+    // tensor-memory columns of tile it: U; packed phi(Q); O
+    auto col_u = [](int it) { return (uint32_t)(128 * (it % G)); };
+    auto col_f = [&](int it) { return DV == 64 ? col_u(it) : (uint32_t)(384 + 64 * (it & 1)); };
+    auto col_o = [&](int it) { return DV == 64 ? col_u(it) + 64 : col_u(it); };
 
     if (*abort_flag) {
         if (tid == 0) atomicExch(status, (int)DARKATTN_ERR_CUDA);
-    } else if (n <= 0) {
-    } else if (warp == kEpiWarps) {
+    } else if (warp == kEpiWarps) {                     // ---- loads
         if ((tid & 31) == 0) {
-            constexpr int NST = L::kStages;
-            auto load_q = [&](int i) {
-                const int b = i % NST;
-                mbar_expect_tx(bars + UB_Q0 + b, kXT);
-                for (int a = 0; a < D / 64; ++a) tma_load_2d(sQ + b * kXT + a * 16384, &p.mapQ, bars + UB_Q0 + b, a * 64, row0 + (t0 + i) * 128);
-            };
-            const TileDesc tOm(sOm), tOml(sOml), tQ0(sQ), tSb(sSb);
-            const uint32_t id_kk = make_idesc(128, 128, 0, 0), id_o = make_idesc(128, DV, 0, 1);
-            mbar_expect_tx(bars + UB_OM, 2 * 128 * D * 2 + 128 * DV * 2);
-            for (int a = 0; a < D / 64; ++a) {
-                tma_load_2d(sOm + a * 16384, &p.mapOm, bars + UB_OM, a * 64, h * p.m + slab * 128);
-                tma_load_2d(sOml + a * 16384, &p.mapOml, bars + UB_OM, a * 64, h * p.m + slab * 128);
+            bool ok = true;
+            int it = 0;
+            for (int pc = 0; ok && list.next(p, p.T, c); ++pc) {
+                const int bh = c.unit / p.nslab, slab = c.unit % p.nslab, h = bh % p.H;
+                if (pc > 0) ok = wait_or_abort(bars + UB_OMF, (pc - 1) & 1, status, abort_flag);     // the piece before is done with its operands
+                if (!ok) break;
+                mbar_expect_tx(bars + UB_OM, 2 * kXT + 128 * DV * 2 + 512);
+                for (int a = 0; a < D / 64; ++a) {
+                    tma_load_2d(sOm + a * 16384, &p.mapOm, bars + UB_OM, a * 64, h * p.m + slab * 128);
+                    tma_load_2d(sOml + a * 16384, &p.mapOml, bars + UB_OM, a * 64, h * p.m + slab * 128);
+                }
+                for (int a = 0; a < DV / 64; ++a) tma_load_2d(sSb + a * 16384, &p.mapSb, bars + UB_OM, a * 64, bh * p.m + slab * 128);
+                bulk_load(smem + L::kZ, p.zq + (size_t)bh * p.m + slab * 128, 512, bars + UB_OM);
+                for (int t = c.t0; t < c.t1; ++t, ++it) {
+                    const int b = it % NST, y = bh * p.N + t * 128;
+                    if (it >= NST) ok = wait_or_abort(bars + UB_QF + b, (it / NST - 1) & 1, status, abort_flag);
+                    if (!ok) break;
+                    mbar_expect_tx(bars + UB_Q + b, kXT);
+                    for (int a = 0; a < D / 64; ++a) tma_load_2d(sQ + b * kXT + a * 16384, &p.mapQ, bars + UB_Q + b, a * 64, y);
+                    if (NST == 2 && t + 2 < c.t1)
+                        for (int a = 0; a < D / 64; ++a) tma_prefetch_l2_2d(&p.mapQ, a * 64, y + 256);
+                }
             }
-            for (int a = 0; a < DV / 64; ++a) tma_load_2d(sSb + a * 16384, &p.mapSb, bars + UB_OM, a * 64, bh * p.m + slab * 128);
-            for (int i = 0; i < NST && i < n; ++i) load_q(i);
-            bool ok = wait_or_abort(bars + UB_OM, 0, status, abort_flag);
-            if (ok) ok = wait_or_abort(bars + UB_Q0, 0, status, abort_flag);
-            if (ok) {
+        }
+    } else if (warp == kEpiWarps + 1) {                 // ---- MMAs
+        if ((tid & 31) == 0) {
+            const TileDesc tOm(sOm), tOml(sOml), tSb(sSb);
+            const uint32_t id_u = make_idesc(128, 128, 0, 0), id_o = make_idesc(128, DV, 0, 1);
+            bool ok = true;
+            int base = 0;
+            for (int pc = 0; ok && list.next(p, p.T, c); ++pc) {
+                const int n = c.t1 - c.t0;
+                ok = wait_or_abort(bars + UB_OM, pc & 1, status, abort_flag);
+                // projections run G - 1 tiles ahead of the outputs
+                for (int i = 0; i < n + G - 1 && ok; ++i) {
+                    if (i < n) {
+                        const int it = base + i, b = it % NST;
+                        ok = wait_or_abort(bars + UB_Q + b, (it / NST) & 1, status, abort_flag);
+                        if (ok && it >= G) ok = wait_or_abort(bars + UB_R + it % G, (it / G - 1) & 1, status, abort_flag);      // the group's last output has been read
+                        if (!ok) break;
+                        tc_fence_after();
+                        const TileDesc tQ(sQ + b * kXT);
+                        issue_projection<D>(tmem + col_u(it), tQ, tOm, tOml, id_u);
+                        mma_commit(bars + UB_U + it % G);
+                        mma_commit(bars + UB_QF + b);
+                    }
+                    if (i >= G - 1) {
+                        const int it = base + i - (G - 1);
+                        ok = wait_or_abort(bars + UB_E + it % G, (it / G) & 1, status, abort_flag);
+                        if (!ok) break;
+                        tc_fence_after();
+                        _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(tmem + col_o(it), tmem + col_f(it) + 8 * k, mndesc(tSb, k), id_o, k > 0);
+                        mma_commit(bars + UB_O + it % G);
+                    }
+                }
+                if (ok) mma_commit(bars + UB_OMF);
+                base += n;
+            }
+        }
+    } else if (warp < 4 * G) {                          // ---- read-out
+        const int lane = tid & 31, q4 = warp & 3, grp = warp >> 2;
+        const uint32_t lane_addr = tmem + ((uint32_t)(q4 * 32) << 16);
+        unsigned char *stage = smem + L::kStage + warp * 4096;
+        bool ok = true;
+        int it = 0;
+        for (int pc = 0; ok && list.next(p, p.T, c); ++pc) {
+            const int bh = c.unit / p.nslab, slab = c.unit % p.nslab;
+            const float cshift = load_key_shift(p.cs, bh * p.nslab + slab);
+            const size_t prow0 = ((size_t)slab * p.BH + bh) * p.N + q4 * 32;
+            bool fresh = true;
+            for (int t = c.t0; t < c.t1 && ok; ++t, ++it) {
+                if (it % G != grp) continue;
+                const uint32_t ph = (it / G) & 1;
+                ok = wait_or_abort(bars + UB_U + grp, ph, status, abort_flag);
+                if (ok && fresh) ok = wait_or_abort(bars + UB_OM, pc & 1, status, abort_flag);      // z is in place (the piece's first tile of this group)
+                fresh = false;
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
                 tc_fence_after();
-                issue_projection<D>(tmem + kColR1, tQ0, tOm, tOml, id_kk);
-                mma_commit(bars + UM1_0);
-            }
-            for (int i = 0; i < n && ok; ++i) {
-                const int b = i & 1;
-                const uint32_t phb = (i >> 1) & 1;
-                if (i + 1 < n) {       // projection of the next tile into the other region, once its last output tile was read
-                    ok = wait_or_abort(bars + UB_Q0 + (i + 1) % NST, ((i + 1) / NST) & 1, status, abort_flag);
-                    if (ok && i >= 1) ok = wait_or_abort(bars + UE3_0 + (b ^ 1), ((i - 1) >> 1) & 1, status, abort_flag);
+                const uint32_t U = lane_addr + col_u(it), F = lane_addr + col_f(it), O = lane_addr + col_o(it);
+                float rmax = -INFINITY;
+#pragma unroll
+                for (int c0 = 0; c0 < 128; c0 += 32) {
+                    uint32_t v[32];
+                    tmem_ld32(U + c0, v);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) rmax = fmaxf(rmax, __uint_as_float(v[j]));
+                }
+                if (DV == 128 && it >= 2) {            // the slot's last reader: the output MMAs of tile it - 2
+                    ok = __all_sync(0xffffffffu, wait_or_abort(bars + UB_O + (it - 2) % G, ((it - 2) / G) & 1, status, abort_flag));
                     if (!ok) break;
                     tc_fence_after();
-                    const TileDesc tQn(sQ + ((i + 1) % NST) * kXT);
-                    issue_projection<D>(tmem + (b ? kColR1 : kColR2), tQn, tOm, tOml, id_kk);
-                    mma_commit(bars + UM1_0 + (b ^ 1));
                 }
-                ok = wait_or_abort(bars + UE0_0 + b, phb, status, abort_flag);      // phi(Q) packed; U read; Q tile consumed
-                if (!ok) break;
-                if (i + NST < n) load_q(i + NST);
-                tc_fence_after();
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(tmem + (b ? kColR2 : kColR1), tmem + b * 64 + k * 8, mndesc(tSb, k), id_o, k > 0);
-                mma_commit(bars + UM4_0 + b);
-            }
-        }
-    } else {
-        const int lane = tid & 31, q4 = warp & 3, g = warp >> 2, col0 = g * 32;
-        const int r = q4 * 32 + lane;
-        const uint32_t lane_addr = tmem + ((uint32_t)(q4 * 32) << 16);
-        const float cshift = load_key_shift(p.cs, bh * p.nslab + slab);
-        const size_t prow0 = ((size_t)slab * p.BH + bh) * p.N;
-        bool ok = true;
-        // (a wait that gave up switches the warp to a dry run over the remaining tiles: see the causal kernel)
-        for (int i = 0; i < n; ++i) {
-            const int b = i & 1;
-            const uint32_t phb = (i >> 1) & 1;
-            const uint32_t R = lane_addr + (b ? kColR2 : kColR1);
-            float rmax;
-            ok = ok && __all_sync(0xffffffffu, wait_or_abort(bars + UM1_0 + b, phb, status, abort_flag));
-            tc_fence_after();
-            const float dz = query_features_to_tmem<true>(R, lane_addr + b * 64, sRed, sZ, q4, g, r, col0, rmax);
-            tc_fence_before();
-            mbar_arrive_warp(bars + UE0_0 + b);
-
-            ok = ok && __all_sync(0xffffffffu, wait_or_abort(bars + UM4_0 + b, phb, status, abort_flag));
-            tc_fence_after();
-            uint32_t v[32];
-            if (col0 < DV) {
-                tmem_ld32(R + col0, v);
-                tmem_wait_ld();
-            }
-            tc_fence_before();
-            mbar_arrive_warp(bars + UE3_0 + b);
-            if (tid == 0) tma_store_wait_read();       // the previous tile's store has left the staging tile
-            epi_sync();
-            if (col0 < DV) store_row_f32x32_bf16(v, sStg, r, col0);
-            sRed[g * 128 + r] = dz;
-            fence_async_smem();
-            epi_sync();
-            if (tid == 0) {
-                for (int a = 0; a < DV / 64; ++a) tma_store_2d(&p.mapPN, sStg + a * 16384, a * 64, (int)(prow0 + (size_t)(t0 + i) * 128));
-                tma_store_commit();
-            }
-            if (g == 0) {
-                const float den = sRed[r] + sRed[128 + r] + sRed[256 + r] + sRed[384 + r];
-                float *dst = p.pdr + 8 * (prow0 + (size_t)(t0 + i) * 128 + r);
-                *reinterpret_cast<float4 *>(dst) = make_float4(den, 0.f, 0.f, 0.f);
+                float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+                for (int c0 = 0; c0 < 128; c0 += 32) {
+                    uint32_t v[32], pk[16];
+                    tmem_ld32(U + c0, v);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4) {
+                        const float4 zz = *reinterpret_cast<const float4 *>(sZ + c0 + j);
+                        const float f0 = ex2f(__uint_as_float(v[j]) - rmax), f1 = ex2f(__uint_as_float(v[j + 1]) - rmax);
+                        const float f2 = ex2f(__uint_as_float(v[j + 2]) - rmax), f3 = ex2f(__uint_as_float(v[j + 3]) - rmax);
+                        fma2(d0, d1, f0, f1, zz.x, zz.y);
+                        fma2(d0, d1, f2, f3, zz.z, zz.w);
+                        pk[j / 2] = pack_bf16(f0, f1);
+                        pk[j / 2 + 1] = pack_bf16(f2, f3);
+                    }
+                    tmem_st16(F + c0 / 2, pk);
+                }
+                tmem_wait_st();
+                tc_fence_before();
+                mbar_arrive_warp(bars + UB_E + grp);
+                const size_t prow = prow0 + (size_t)t * 128;
+                float *dst = p.pdr + 8 * (prow + lane);
+                *reinterpret_cast<float4 *>(dst) = make_float4(d0 + d1, 0.f, 0.f, 0.f);
                 dst[4] = rmax + cshift;
+
+                ok = __all_sync(0xffffffffu, wait_or_abort(bars + UB_O + grp, ph, status, abort_flag));
+                if (!ok) break;
+                tc_fence_after();
+#pragma unroll
+                for (int a = 0; a < DV / 64; ++a) {
+                    if (lane == 0) tma_store_wait_read();       // what was staged before has left
+                    __syncwarp();
+#pragma unroll
+                    for (int half = 0; half < 2; ++half) {
+                        uint32_t v[32];
+                        tmem_ld32(O + 64 * a + 32 * half, v);
+                        tmem_wait_ld();
+                        if (a == DV / 64 - 1 && half == 1) {
+                            tc_fence_before();
+                            mbar_arrive_warp(bars + UB_R + grp);
+                        }
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) *reinterpret_cast<uint4 *>(stage + swz128(lane, 4 * half + q)) = pack8(v + 8 * q);
+                    }
+                    fence_async_smem();
+                    __syncwarp();
+                    if (lane == 0) {
+                        tma_store_2d(&p.mapPN, stage, a * 64, (int)prow);
+                        tma_store_commit();
+                    }
+                }
             }
-            quarter_sync(q4);
         }
-        if (tid == 0) tma_store_wait_all();
+        if (lane == 0) tma_store_wait_all();
     }
     if (*abort_flag) __nanosleep(200000);
     tc_fence_before();
@@ -976,40 +1153,53 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_queries_kernel(const __gri
     if (warp == kEpiWarps) tmem_dealloc(tmem, 512);
 }
 
-// Sb[bh,l,:] = bf16(Sacc[bh,l,:])  (operand of the query pass); z is copied beside it where the backward pass
-// will look for it (zout == z when that is the workspace itself)
-__global__ void state_to_bf16_kernel(const float *S, __nv_bfloat16 *Sb, long long n, const float *z, float *zout, long long nz)
+// Sb = bf16(S), the operand of the query pass, and z from its four parts, for that pass and for the backward pass
+__global__ void __launch_bounds__(256) state_to_bf16_kernel(const float *S, __nv_bfloat16 *Sb, long long n4, const float *zparts, float *z, long long nz)
 {
     pdl_wait();
-    const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
-    for (long long i = i0; i < n; i += step) Sb[i] = __float2bfloat16_rn(S[i]);
-    if (zout != z)
-        for (long long i = i0; i < nz; i += step) zout[i] = z[i];
+    const long long i = blockIdx.x * 256LL + threadIdx.x;
+    if (i < n4) {
+        const float4 x = reinterpret_cast<const float4 *>(S)[i];
+        reinterpret_cast<uint2 *>(Sb)[i] = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
+    }
+    if (i < nz) {
+        const float4 x = reinterpret_cast<const float4 *>(zparts)[i];
+        z[i] = (x.x + x.y) + (x.z + x.w);
+    }
 }
 
-// In-place exclusive prefix over the segments of S[bh, seg, e] (e over m*dv) and z[bh, seg, l]; Sb receives the bf16
-// copy of the prefixed S. One thread per (bh, e).
-__global__ void segment_prefix_kernel(float *S, __nv_bfloat16 *Sb, float *z, int nseg, long long E, int m, long long total)
+// The state before every segment but the first: Sseg[bh, s] = sum of the pieces of the segments before s (in fp32 and, as an
+// MMA operand, in bf16), the same for z. One thread per four elements of a (batch, head)'s state; a segment's pieces are
+// loaded together. (65536 tokens, 8 heads, m 512, d 64: 25 us when it prefixed in place, a load behind every store.)
+__global__ void __launch_bounds__(256) segment_prefix_kernel(const float *__restrict__ Spart, const float *__restrict__ zpart, float *__restrict__ Sseg,
+                                                             __nv_bfloat16 *__restrict__ Sb, float *__restrict__ zseg, int nseg, int npiece, int E4, int m, long long total)
 {
     pdl_wait();
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long i = blockIdx.x * 256LL + threadIdx.x;
     if (i >= total) return;
-    const long long bh = i / E, e = i % E;
-    float run = 0.f;
-    for (int s = 0; s < nseg; ++s) {
-        const long long at = (bh * nseg + s) * E + e;
-        const float v = S[at];
-        S[at] = run;
-        Sb[at] = __float2bfloat16_rn(run);
-        run += v;
+    const long long bh = i / E4;
+    const int e = (int)(i % E4), per = npiece / (nseg - 1);
+    float4 run = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s = 1; s < nseg; ++s) {
+        const float4 *src = reinterpret_cast<const float4 *>(Spart) + (bh * npiece + (s - 1) * per) * E4 + e;
+#pragma unroll 4
+        for (int j = 0; j < per; ++j) {
+            const float4 x = src[(long long)j * E4];
+            run.x += x.x; run.y += x.y; run.z += x.z; run.w += x.w;
+        }
+        const long long at = (bh * nseg + s) * E4 + e;
+        reinterpret_cast<float4 *>(Sseg)[at] = run;
+        reinterpret_cast<uint2 *>(Sb)[at] = make_uint2(pack_bf16(run.x, run.y), pack_bf16(run.z, run.w));
     }
     if (e < m) {
         float zr = 0.f;
-        for (int s = 0; s < nseg; ++s) {
-            const long long at = (bh * nseg + s) * m + e;
-            const float v = z[at];
-            z[at] = zr;
-            zr += v;
+        for (int s = 1; s < nseg; ++s) {
+#pragma unroll 4
+            for (int j = 0; j < per; ++j) {
+                const float4 x = reinterpret_cast<const float4 *>(zpart)[(bh * npiece + (s - 1) * per + j) * m + e];
+                zr += (x.x + x.y) + (x.z + x.w);
+            }
+            zseg[(bh * nseg + s) * m + e] = zr;
         }
     }
 }
@@ -1099,11 +1289,11 @@ cudaError_t launch_main(const MainParams &P, int grid, cudaStream_t st)
     } else if constexpr (MODE == MODE_KEYS) {
         using L = FwdKeysSmem<D, DV>;
         static_assert(L::kTotal <= 232448, "shared memory budget of one CTA exceeded");
-        return launch_pdl(tc_fwd_keys_kernel<D, DV>, dim3(grid), dim3(kThreads), L::kTotal, st, P);
+        return launch_pdl(tc_fwd_keys_kernel<D, DV>, dim3(grid), dim3(kKeysThreads), L::kTotal, st, P);
     } else {
         using L = FwdQueriesSmem<D, DV>;
         static_assert(L::kTotal <= 232448, "shared memory budget of one CTA exceeded");
-        return launch_pdl(tc_fwd_queries_kernel<D, DV>, dim3(grid), dim3(kThreads), L::kTotal, st, P);
+        return launch_pdl(tc_fwd_queries_kernel<D, DV>, dim3(grid), dim3(kPassThreads), L::kTotal, st, P);
     }
 }
 
@@ -1142,9 +1332,7 @@ void tensor_make_layout(darkattn_plan_s *plan)
     Y.T = D.N / 128;
     int nsplit = 1;
     const long long units = (long long)BH * Y.nslab;
-    if (!D.causal) {
-        nsplit = pick_splits(units, Y.T, 1.4, 5.0, kMaxNsplit);
-    } else if (units * 2 <= 148) {
+    if (D.causal && units * 2 <= 148) {
         // few long sequences: cut each into segments (a key pass computes the segment states, the causal
         // kernels of all segments then run side by side), as many as fill the SMs, at least 4 chunks each
         nsplit = (int)(148 / units);
@@ -1153,6 +1341,8 @@ void tensor_make_layout(darkattn_plan_s *plan)
         if (nsplit < 1) nsplit = 1;
     }
     Y.nsplit = nsplit;
+    // the key pass over all segments but the last, in pieces that fill the SMs (a tile takes 0.8 us, a piece's start and end 3)
+    Y.npiece = nsplit > 1 ? (nsplit - 1) * pick_splits(units * (nsplit - 1), Y.T / nsplit, 0.8, 3.0, 8) : 0;
     const size_t nstate = D.causal ? (size_t)nsplit : 1;
     size_t off = 0;
     Y.status = take(off, 256);
@@ -1162,9 +1352,13 @@ void tensor_make_layout(darkattn_plan_s *plan)
     Y.nK = take(off, BH * N * 4);
     Y.pnum = take(off, (size_t)Y.nslab * BH * N * dv * 2);
     Y.pdr = take(off, (size_t)Y.nslab * BH * N * 32);
-    Y.Sacc = take(off, BH * nstate * m * dv * 4);
-    Y.zacc = take(off, BH * nstate * m * 4);
+    // (states and z of the key pass: sums over all keys, or one per piece; what it adds into is cleared by one run of stores)
+    Y.Sacc = take(off, BH * (D.causal ? (size_t)Y.npiece : 1) * m * dv * 4);
+    Y.zacc = take(off, BH * (D.causal ? (size_t)Y.npiece : 1) * m * 16);
     Y.Sb = take(off, BH * nstate * m * dv * 2);
+    Y.Sseg = take(off, Y.npiece ? BH * nstate * m * dv * 4 : 0);
+    Y.zseg = take(off, Y.npiece ? BH * nstate * m * 4 : 0);
+    Y.zq = take(off, D.causal ? 0 : BH * m * 4);
     Y.sv = take(off, BH * N * 8);
     Y.zc = take(off, D.causal ? BH * (size_t)Y.T * m * 4 : 0);
     plan->launches_fwd = D.causal ? (nsplit > 1 ? 6 : 4) : 6;
@@ -1260,7 +1454,7 @@ darkattn_status_t tensor_forward(const darkattn_plan_s *plan, const void *Q, con
               make_map(&P.mapV, V, BHkv * N, D.dv, 128) && make_map(&P.mapOm, stash.Om, (size_t)D.H * D.m, D.d, 128) &&
               make_map(&P.mapOml, stash.Oml, (size_t)D.H * D.m, D.d, 128) &&
               make_map(&P.mapSb, D.causal ? bf(Y.Sb) : stash.Sb, BH * (D.causal ? Y.nsplit : 1) * D.m, D.dv, 128) &&
-              make_map(&P.mapPN, bf(Y.pnum), (size_t)Y.nslab * BH * N, D.dv, 128);
+              make_map(&P.mapPN, bf(Y.pnum), (size_t)Y.nslab * BH * N, D.dv, D.causal ? 128 : 32);     // (the query pass stores a warp's 32 rows)
     if (!ok) { set_cuda_error(cudaErrorInvalidValue, "tensor_forward: tensor map encode"); return DARKATTN_ERR_CUDA; }
 
     cudaError_t e = tensor_prologue(plan, K, M, W, ws, stash, st);
@@ -1277,23 +1471,28 @@ darkattn_status_t tensor_forward(const darkattn_plan_s *plan, const void *Q, con
     const int units = (int)(BH * Y.nslab);
     if (D.causal) {
         if (Y.nsplit > 1) {      // segment states, then their exclusive prefix
-            P.Sseg = fl(Y.Sacc); P.zseg = fl(Y.zacc);
+            P.npiece = Y.npiece; P.Sseg = fl(Y.Sseg); P.zseg = fl(Y.zseg);
+            const int pieces = units * Y.npiece, E4 = D.m * D.dv / 4;
             timer_mark(plan, st, "tc_fwd_keys_kernel");
-            keep(launch_main_shape<MODE_KEYS>(D.d, D.dv, P, units * Y.nsplit, st));
-            const long long E = (long long)D.m * D.dv, total = (long long)BH * E;
+            keep(launch_main_shape<MODE_KEYS>(D.d, D.dv, P, pieces < 148 ? pieces : 148, st));
+            const long long total = (long long)BH * E4;
             timer_mark(plan, st, "segment_prefix_kernel");
-            keep(launch_pdl(segment_prefix_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, fl(Y.Sacc), bf(Y.Sb), fl(Y.zacc), Y.nsplit, E, D.m, total));
+            keep(launch_pdl(segment_prefix_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, (const float *)fl(Y.Sacc), (const float *)fl(Y.zacc),
+                            fl(Y.Sseg), bf(Y.Sb), fl(Y.zseg), Y.nsplit, Y.npiece, E4, D.m, total));
         }
         timer_mark(plan, st, "tc_fwd_causal_kernel");
         keep(launch_main_shape<MODE_CAUSAL>(D.d, D.dv, P, units * Y.nsplit, st));
     } else {
+        // one CTA per SM; a problem of few tiles gets one CTA for each
+        const int grid = (long long)units * Y.T < 148 ? units * Y.T : 148;
         timer_mark(plan, st, "tc_fwd_keys_kernel");
-        keep(launch_main_shape<MODE_KEYS>(D.d, D.dv, P, units * Y.nsplit, st));
-        const long long n = (long long)BH * D.m * D.dv;
+        keep(launch_main_shape<MODE_KEYS>(D.d, D.dv, P, grid, st));
+        const long long n4 = (long long)BH * D.m * D.dv / 4;
         timer_mark(plan, st, "state_to_bf16_kernel");
-        keep(launch_pdl(state_to_bf16_kernel, dim3((unsigned)((n + 1023) / 1024)), dim3(256), 0, st, (const float *)fl(Y.Sacc), stash.Sb, n, (const float *)fl(Y.zacc), stash.zt, (long long)BH * D.m));
+        keep(launch_pdl(state_to_bf16_kernel, dim3((unsigned)((n4 + 255) / 256)), dim3(256), 0, st, (const float *)fl(Y.Sacc), stash.Sb, n4, (const float *)fl(Y.zacc), stash.zt, (long long)BH * D.m));
+        P.zq = stash.zt;
         timer_mark(plan, st, "tc_fwd_queries_kernel");
-        keep(launch_main_shape<MODE_QUERIES>(D.d, D.dv, P, units * Y.nsplit, st));
+        keep(launch_main_shape<MODE_QUERIES>(D.d, D.dv, P, grid, st));
     }
     {
         const long long rows = (long long)BH * N, threads = rows * (D.dv / 8);

@@ -401,6 +401,26 @@ def test_grouped_key_value_heads(binding, path, H, Hkv, kw, causal):
     _compare(got, want, TOL[dtype], f"grouped {path} H={H} H_kv={Hkv}")
 
 
+# The passes over keys and queries deal out the tiles of all (batch, head, slab) evenly: one tile in all; one tile per CTA;
+# CTAs whose run of tiles ends inside one and begins inside another, fewer tiles than the groups of a CTA; causal segments.
+PASS_EDGES = [
+    dict(B=1, H=1, N=128, d=64, m=128, causal=False),
+    dict(B=1, H=3, N=640, d=128, m=384, dv=64, causal=False),
+    dict(B=2, H=5, N=3968, d=64, m=256, causal=False),
+    dict(B=3, H=5, N=1152, d=128, m=256, causal=False),
+    dict(B=1, H=7, N=4224, d=64, m=256, dv=128, causal=False),
+    dict(B=1, H=2, N=4992, d=64, m=128, causal=True),
+    dict(B=1, H=3, N=1408, d=128, m=256, dv=128, causal=True),
+]
+
+
+@pytest.mark.parametrize("i", range(len(PASS_EDGES)))
+def test_passes_over_keys_and_queries_at_piece_edges(binding, i):
+    wl = inputs.small(name=f"pieces{i}", wid=430 + i, dtype="bf16", backward=False, **PASS_EDGES[i])
+    t = inputs.generate(wl)
+    _compare(run_gpu(binding, wl, t, path=binding.PATH_TENSOR), _oracle(t, wl), TOL["bf16"], f"pieces{i}")
+
+
 def test_tensor_path_is_deterministic(binding):
     """The scan kernels hand tiles between warps through shared and tensor memory; a missing wait shows up as rare,
     run-dependent errors of the size of the values themselves. O has a fixed summation order: repeated runs at the
