@@ -649,45 +649,49 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_causal_kernel(const __grid
 
 // ------------------------------------------------------------------ key pass: S = phi(K)^T V, z = phi(K)^T 1
 // Both passes below run one CTA per SM over a list of pieces (a run of tiles of one (batch, head, slab)); the roles (a warp
-// for TMA, a warp for the MMAs, the read-out warps) walk the list by themselves, so that one piece's end overlaps the next
-// one's start except where the slab's operands change. Key pass: the line of all (unit, tile) is cut evenly over the CTAs and
-// the pieces' states are added up by atomics; with segments (causal) the pieces are fixed and each stores its own state.
-struct Piece { int unit, t0, t1, dst; bool whole; };
+// for TMA, warps for the MMAs, the read-out warps) walk the list by themselves, so that one piece's end overlaps the next
+// one's start except where the slab's operands change. CTA i works on slab i % nslab, and the line of all (batch, head, tile)
+// is cut evenly over the CTAs of a slab: those of different slabs go through the same tiles at the same time and share them
+// through L2 (with the slabs one after the other in one line, K and V came from HBM once for each: 537 MB, 82 us of the 104
+// the key pass then took at 4 x 16 heads, 8192 tokens, d 128). The states of a line's pieces are added up by atomics; with
+// segments (causal) the pieces are fixed and each stores its own state.
+struct Piece { int bh, slab, t0, t1, dst; bool whole; };
 
 struct PieceList {
     long long x, end;       // line: tiles [x, end); fixed pieces: index and count
-    int step;
-    __device__ __forceinline__ PieceList(const MainParams &p, int T)
+    __device__ __forceinline__ explicit PieceList(const MainParams &p)
     {
-        if (p.npiece) { x = blockIdx.x; end = (long long)p.BH * p.nslab * p.npiece; step = gridDim.x; }
+        if (p.npiece) { x = blockIdx.x; end = (long long)p.BH * p.nslab * p.npiece; }
         else {
-            const long long total = (long long)p.BH * p.nslab * T;
-            x = total * blockIdx.x / gridDim.x; end = total * (blockIdx.x + 1) / gridDim.x; step = 0;
+            const int j = blockIdx.x / p.nslab, per = gridDim.x / p.nslab;
+            const long long total = (long long)p.BH * p.T;
+            x = total * j / per; end = total * (j + 1) / per;
         }
     }
-    __device__ __forceinline__ bool next(const MainParams &p, int T, Piece &c)
+    __device__ __forceinline__ bool next(const MainParams &p, Piece &c)
     {
         if (x >= end) return false;
-        if (step) {
+        if (p.npiece) {
             const int per = p.npiece / (p.nsplit - 1);           // pieces of a segment; the last segment's state is not needed
-            c.unit = (int)(x / p.npiece); c.dst = (int)(x % p.npiece);
+            c.slab = (int)(x % p.nslab); c.dst = (int)(x / p.nslab % p.npiece); c.bh = (int)(x / p.nslab / p.npiece);
             const int seg = c.dst / per, j = c.dst % per;
-            const int b0 = (int)((long long)T * seg / p.nsplit), len = (int)((long long)T * (seg + 1) / p.nsplit) - b0;
+            const int b0 = (int)((long long)p.T * seg / p.nsplit), len = (int)((long long)p.T * (seg + 1) / p.nsplit) - b0;
             c.t0 = b0 + (int)((long long)len * j / per); c.t1 = b0 + (int)((long long)len * (j + 1) / per);
             c.whole = true;
-            x += step;
+            x += gridDim.x;
         } else {
-            c.unit = (int)(x / T); c.t0 = (int)(x % T); c.dst = 0;
-            c.t1 = (int)min((long long)T, c.t0 + (end - x));
-            c.whole = (c.t0 == 0 && c.t1 == T);
+            c.slab = blockIdx.x % p.nslab; c.bh = (int)(x / p.T); c.t0 = (int)(x % p.T); c.dst = 0;
+            c.t1 = (int)min((long long)p.T, c.t0 + (end - x));
+            c.whole = (c.t0 == 0 && c.t1 == p.T);
             x += c.t1 - c.t0;
         }
         return true;
     }
 };
 
-constexpr int kPassThreads = 576;       // 16 read-out warps, TMA warp, MMA warp; the key pass has a second TMA warp
-constexpr int kKeysThreads = 608;
+// 16 read-out warps, TMA, MMAs of the projections, MMAs of the second product (a warp each: a thread that issues both kinds
+// spends its program order waiting for the one while the other is ready); the key pass has a second TMA warp
+constexpr int kPassThreads = 608, kKeysThreads = 640;
 
 // (u0, u1) - (n0, n1) - (c, c)
 __device__ __forceinline__ void sub2(float &u0, float &u1, float n0, float n1, float c)
@@ -734,15 +738,17 @@ struct FwdKeysSmem {
     static constexpr int kTotal = kBars + 512;
 };
 
-// Omega loaded / free; K, V rings loaded / free; norms loaded; U ready / phi(K)^T written (three regions); state ready / read
-enum KyBars { YB_OM, YB_OMF, YB_K, YB_V = YB_K + 4, YB_KF = YB_V + 4, YB_VF = YB_KF + 4, YB_N = YB_VF + 4, YB_U = YB_N + 8, YB_S = YB_U + 3,
+// Omega loaded / free; K, V rings loaded / free; norms loaded; U ready / state updated / phi(K)^T written (three regions);
+// piece's state ready / read
+enum KyBars { YB_OM, YB_OMF, YB_K, YB_V = YB_K + 4, YB_KF = YB_V + 4, YB_VF = YB_KF + 4, YB_N = YB_VF + 4, YB_U = YB_N + 8, YB_SD = YB_U + 3, YB_S = YB_SD + 3,
               YB_E, YB_SR = YB_E + 3, YNBARS };
 
 // The tile's exponents are formed transposed, U^T = Omega K^T: a lane of tensor memory is a feature, a column a token. Then
 // phi(K)^T, packed to bf16 in place by the warp that read it, is the A operand of S += phi(K)^T V straight from tensor memory
 // (no shared-memory tile, no proxy fence), z is a sum along a thread's own columns (no MMAs against ones), and what is left of
-// tensor memory holds three tiles: the projections run two tiles ahead and every warp goes from tile to tile without waiting
-// for any other. Bound by the exponentials (16384 per tile, 16 per clock and SM) at d = 64 and by MMA issue (24 per tile)
+// tensor memory holds three tiles: the projections run ahead and eight warps each work on the even and on the odd tiles, so
+// that the exponentials of one tile run under the waits, loads and stores of another (in lockstep on one tile a warp spent 1.0 k
+// of 2.3 k cycles on those). Bound by the exponentials (16384 per tile, 16 per clock and SM) at d = 64 and by MMA issue (24 per tile)
 // at d = 128. Encoder shape 8 x 12 heads, 4096 tokens, d 64, m 256: 101 -> 64 us; 4 x 16 heads, 8192 tokens, d 128: 138 -> 104 us.
 template <int D, int DV>
 __global__ void __launch_bounds__(kKeysThreads, 1) tc_fwd_keys_kernel(const __grid_constant__ MainParams p)
@@ -759,7 +765,8 @@ __global__ void __launch_bounds__(kKeysThreads, 1) tc_fwd_keys_kernel(const __gr
 
     if (tid == 0) {
         for (int i = 0; i < YB_E; ++i) mbar_init(bars + i, 1);
-        for (int i = YB_E; i < YNBARS; ++i) mbar_init(bars + i, kEpiWarps);
+        for (int i = YB_E; i < YB_SR; ++i) mbar_init(bars + i, kEpiWarps / 2);
+        mbar_init(bars + YB_SR, kEpiWarps);
         *abort_flag = (smem_u32(smem) & 1023u) ? 1 : 0;
         fence_mbar_init();
     }
@@ -770,7 +777,7 @@ __global__ void __launch_bounds__(kKeysThreads, 1) tc_fwd_keys_kernel(const __gr
     pdl_wait();
     const uint32_t tmem = *tmem_slot;
     int *status = p.status;
-    PieceList list(p, p.T);
+    PieceList list(p);
     Piece c;
 
     if (*abort_flag) {
@@ -779,8 +786,8 @@ __global__ void __launch_bounds__(kKeysThreads, 1) tc_fwd_keys_kernel(const __gr
         if ((tid & 31) == 0) {
             bool ok = true;
             int it = 0;
-            for (int pc = 0; ok && list.next(p, p.T, c); ++pc) {
-                const int bh = c.unit / p.nslab, slab = c.unit % p.nslab, h = bh % p.H, rowk0 = kv_row0(bh, p.H, p.Hkv, p.N);
+            for (int pc = 0; ok && list.next(p, c); ++pc) {
+                const int bh = c.bh, slab = c.slab, h = bh % p.H, rowk0 = kv_row0(bh, p.H, p.Hkv, p.N);
                 const float *nK = p.nK + (size_t)bh * p.N;
                 if (pc > 0) ok = wait_or_abort(bars + YB_OMF, (pc - 1) & 1, status, abort_flag);      // the piece before is projected
                 if (!ok) break;
@@ -795,8 +802,8 @@ __global__ void __launch_bounds__(kKeysThreads, 1) tc_fwd_keys_kernel(const __gr
                     if (!ok) break;
                     mbar_expect_tx(bars + YB_K + b, kXT);
                     for (int a = 0; a < D / 64; ++a) tma_load_2d(sK + b * kXT + a * 16384, &p.mapK, bars + YB_K + b, a * 64, y);
-                    // Here tile it - NST is projected, hence (the projections run two tiles ahead of the state) all warps are
-                    // done with tile it - NST - 3 and with the norms of tile it - 8.
+                    // Here tile it - NST is projected, so its region's tile before, it - NST - 3, has been read out, and with it
+                    // all tiles before, tile it - 8 (the last user of this slot of norms) among them.
                     static_assert(NST + 3 <= NN, "a slot of norms would be loaded over");
                     mbar_expect_tx(bars + YB_N + it % NN, 512);
                     bulk_load(sNorm + (it % NN) * 128, nK + (size_t)t * 128, 512, bars + YB_N + it % NN);
@@ -809,8 +816,8 @@ __global__ void __launch_bounds__(kKeysThreads, 1) tc_fwd_keys_kernel(const __gr
         if ((tid & 31) == 0) {
             bool ok = true;
             int it = 0;
-            while (ok && list.next(p, p.T, c)) {
-                const int rowk0 = kv_row0(c.unit / p.nslab, p.H, p.Hkv, p.N);
+            while (ok && list.next(p, c)) {
+                const int rowk0 = kv_row0(c.bh, p.H, p.Hkv, p.N);
                 for (int t = c.t0; t < c.t1; ++t, ++it) {
                     const int b = it % NST, y = rowk0 + t * 128;
                     if (it >= NST) ok = wait_or_abort(bars + YB_VF + b, (it / NST - 1) & 1, status, abort_flag);
@@ -822,83 +829,93 @@ __global__ void __launch_bounds__(kKeysThreads, 1) tc_fwd_keys_kernel(const __gr
                 }
             }
         }
-    } else if (warp == kEpiWarps + 1) {                 // ---- MMAs
+    } else if (warp == kEpiWarps + 1) {                 // ---- MMAs: U^T of tile it into region it % 3
         if ((tid & 31) == 0) {
             const TileDesc tOm(sOm), tOml(sOml);
-            const uint32_t id_u = make_idesc(128, 128, 0, 0), id_s = make_idesc(128, DV, 0, 1);
+            const uint32_t id_u = make_idesc(128, 128, 0, 0);
             bool ok = true;
-            int base = 0;                               // tiles of the pieces before
-            for (int pc = 0; ok && list.next(p, p.T, c); ++pc) {
-                const int n = c.t1 - c.t0;
+            int it = 0;
+            for (int pc = 0; ok && list.next(p, c); ++pc) {
                 ok = wait_or_abort(bars + YB_OM, pc & 1, status, abort_flag);
-                auto project = [&](int i) {             // U^T of tile i into region i % 3 (the state MMAs that read it are ahead in the pipe)
-                    const int it = base + i, b = it % NST;
+                for (int t = c.t0; t < c.t1; ++t, ++it) {
+                    const int b = it % NST, q = it % 3;
                     ok = ok && wait_or_abort(bars + YB_K + b, (it / NST) & 1, status, abort_flag);
-                    if (!ok) return;
+                    if (ok && it >= 3) ok = wait_or_abort(bars + YB_SD + q, (it / 3 - 1) & 1, status, abort_flag);      // the region's last reader is done
+                    if (!ok) break;
                     tc_fence_after();
-                    const uint32_t dst = tmem + 128 + 128 * (it % 3);
+                    const uint32_t dst = tmem + 128 + 128 * q;
                     const TileDesc tK(sK + b * kXT);
                     _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(dst, kdesc(tOm, k), kdesc(tK, k), id_u, k > 0);
                     _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(dst, kdesc(tOml, k), kdesc(tK, k), id_u, 1);
-                    mma_commit(bars + YB_U + it % 3);
+                    mma_commit(bars + YB_U + q);
                     mma_commit(bars + YB_KF + b);
-                    if (i + 1 == n) mma_commit(bars + YB_OMF);
-                };
-                project(0);
-                if (n > 1) project(1);
-                for (int i = 0; i < n && ok; ++i) {
-                    const int it = base + i, b = it % NST;
-                    if (i + 2 < n) project(i + 2);
-                    ok = ok && wait_or_abort(bars + YB_E + it % 3, (it / 3) & 1, status, abort_flag);
+                    if (t + 1 == c.t1) mma_commit(bars + YB_OMF);
+                }
+            }
+        }
+    } else if (warp == kEpiWarps + 3) {                 // ---- MMAs: S += phi(K)^T V
+        if ((tid & 31) == 0) {
+            const uint32_t id_s = make_idesc(128, DV, 0, 1);
+            bool ok = true;
+            int it = 0;
+            for (int pc = 0; ok && list.next(p, c); ++pc) {
+                if (pc > 0) ok = wait_or_abort(bars + YB_SR, (pc - 1) & 1, status, abort_flag);      // the state before has been read out
+                for (int t = c.t0; t < c.t1; ++t, ++it) {
+                    const int b = it % NST, q = it % 3;
                     ok = ok && wait_or_abort(bars + YB_V + b, (it / NST) & 1, status, abort_flag);
-                    if (ok && i == 0 && pc > 0) ok = wait_or_abort(bars + YB_SR, (pc - 1) & 1, status, abort_flag);   // the state before has been read out
+                    ok = ok && wait_or_abort(bars + YB_E + q, (it / 3) & 1, status, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t src = tmem + 128 + 128 * (it % 3);
+                    const uint32_t src = tmem + 128 + 128 * q;
                     const TileDesc tV(sV + b * kVT);
-                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(tmem, src + (k / 2) * 32 + (k % 2) * 8, mndesc(tV, k), id_s, i > 0 || k > 0);
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(tmem, src + (k / 2) * 32 + (k % 2) * 8, mndesc(tV, k), id_s, t > c.t0 || k > 0);
+                    mma_commit(bars + YB_SD + q);
                     mma_commit(bars + YB_VF + b);
                 }
                 if (ok) mma_commit(bars + YB_S);
-                base += n;
             }
         }
     } else {                                            // ---- read-out
         const int lane = tid & 31, q4 = warp & 3, g = warp >> 2, col0 = g * 32;
         const int r = q4 * 32 + lane;                   // this thread's feature
+        const int grp = warp >> 3, half = 64 * ((warp >> 2) & 1);     // even or odd tiles; which 64 tokens of the tile
         const uint32_t lane_addr = tmem + ((uint32_t)(q4 * 32) << 16);
         bool ok = true;
         int it = 0;
-        for (int pc = 0; ok && list.next(p, p.T, c); ++pc) {
-            const int bh = c.unit / p.nslab, slab = c.unit % p.nslab;
+        for (int pc = 0; ok && list.next(p, c); ++pc) {
+            const int bh = c.bh, slab = c.slab;
             const float cshift = load_key_shift(p.cs, bh * p.nslab + slab);
             float z0 = 0.f, z1 = 0.f;
             for (int t = c.t0; t < c.t1; ++t, ++it) {
-                const uint32_t addr = lane_addr + 128 + 128 * (it % 3) + col0;
+                if ((it & 1) != grp) continue;
+                const uint32_t addr = lane_addr + 128 + 128 * (it % 3) + half;
                 ok = wait_or_abort(bars + YB_N + it % NN, (it / NN) & 1, status, abort_flag) &&
                      wait_or_abort(bars + YB_U + it % 3, (it / 3) & 1, status, abort_flag);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
-                uint32_t v[32], pk[16];
-                tmem_ld32(addr, v);
-                const float4 *nrm = reinterpret_cast<const float4 *>(sNorm + (it % NN) * 128 + col0);
-                tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float4 nk = nrm[j];
-                    float x[4];
+                for (int c0 = 0; c0 < 64; c0 += 32) {
+                    uint32_t v[32], pk[16];
+                    tmem_ld32(addr + c0, v);
+                    const float4 *nrm = reinterpret_cast<const float4 *>(sNorm + (it % NN) * 128 + half + c0);
+                    tmem_wait_ld();
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) x[k] = __uint_as_float(v[4 * j + k]);
-                    sub2(x[0], x[1], nk.x, nk.y, cshift);
-                    sub2(x[2], x[3], nk.z, nk.w, cshift);
-                    pk[2 * j] = pack_bf16(ex2f(x[0]), ex2f(x[1]));
-                    pk[2 * j + 1] = pack_bf16(ex2f(x[2]), ex2f(x[3]));
-                    // z sums what the MMA multiplies: the rounded features
-                    add2(z0, z1, __uint_as_float(pk[2 * j] << 16), __uint_as_float(pk[2 * j] & 0xffff0000u));
-                    add2(z0, z1, __uint_as_float(pk[2 * j + 1] << 16), __uint_as_float(pk[2 * j + 1] & 0xffff0000u));
+                    for (int j = 0; j < 8; ++j) {
+                        const float4 nk = nrm[j];
+                        float x[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) x[k] = __uint_as_float(v[4 * j + k]);
+                        sub2(x[0], x[1], nk.x, nk.y, cshift);
+                        sub2(x[2], x[3], nk.z, nk.w, cshift);
+                        pk[2 * j] = pack_bf16(ex2f(x[0]), ex2f(x[1]));
+                        pk[2 * j + 1] = pack_bf16(ex2f(x[2]), ex2f(x[3]));
+                        // z sums what the MMA multiplies: the rounded features
+                        add2(z0, z1, __uint_as_float(pk[2 * j] << 16), __uint_as_float(pk[2 * j] & 0xffff0000u));
+                        add2(z0, z1, __uint_as_float(pk[2 * j + 1] << 16), __uint_as_float(pk[2 * j + 1] & 0xffff0000u));
+                    }
+                    tmem_st16(addr + c0, pk);
                 }
-                tmem_st16(addr, pk);
                 tmem_wait_st();
                 tc_fence_before();
                 mbar_arrive_warp(bars + YB_E + it % 3);
@@ -924,7 +941,7 @@ __global__ void __launch_bounds__(kKeysThreads, 1) tc_fwd_keys_kernel(const __gr
                     else red_add4(dst + j, a0, a1, a2, a3);
                 }
             }
-            // z: one part per column group, added up by the kernel that reads the state
+            // z: a part per (tile parity, token half), added up by the kernel that reads the state
             if (c.whole) p.zacc[4 * srow + g] = z0 + z1;
             else atomicAdd(p.zacc + 4 * srow + g, z0 + z1);
         }
@@ -986,7 +1003,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) tc_fwd_queries_kernel(const _
     pdl_wait();
     const uint32_t tmem = *tmem_slot;
     int *status = p.status;
-    PieceList list(p, p.T);
+    PieceList list(p);
     Piece c;
     // tensor-memory columns of tile it: U; packed phi(Q); O
     auto col_u = [](int it) { return (uint32_t)(128 * (it % G)); };
@@ -999,8 +1016,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) tc_fwd_queries_kernel(const _
         if ((tid & 31) == 0) {
             bool ok = true;
             int it = 0;
-            for (int pc = 0; ok && list.next(p, p.T, c); ++pc) {
-                const int bh = c.unit / p.nslab, slab = c.unit % p.nslab, h = bh % p.H;
+            for (int pc = 0; ok && list.next(p, c); ++pc) {
+                const int bh = c.bh, slab = c.slab, h = bh % p.H;
                 if (pc > 0) ok = wait_or_abort(bars + UB_OMF, (pc - 1) & 1, status, abort_flag);     // the piece before is done with its operands
                 if (!ok) break;
                 mbar_expect_tx(bars + UB_OM, 2 * kXT + 128 * DV * 2 + 512);
@@ -1021,39 +1038,43 @@ __global__ void __launch_bounds__(kPassThreads, 1) tc_fwd_queries_kernel(const _
                 }
             }
         }
-    } else if (warp == kEpiWarps + 1) {                 // ---- MMAs
+    } else if (warp == kEpiWarps + 1) {                 // ---- MMAs: U of a tile
         if ((tid & 31) == 0) {
-            const TileDesc tOm(sOm), tOml(sOml), tSb(sSb);
-            const uint32_t id_u = make_idesc(128, 128, 0, 0), id_o = make_idesc(128, DV, 0, 1);
+            const TileDesc tOm(sOm), tOml(sOml);
+            const uint32_t id_u = make_idesc(128, 128, 0, 0);
             bool ok = true;
-            int base = 0;
-            for (int pc = 0; ok && list.next(p, p.T, c); ++pc) {
-                const int n = c.t1 - c.t0;
+            int it = 0;
+            for (int pc = 0; ok && list.next(p, c); ++pc) {
                 ok = wait_or_abort(bars + UB_OM, pc & 1, status, abort_flag);
-                // projections run G - 1 tiles ahead of the outputs
-                for (int i = 0; i < n + G - 1 && ok; ++i) {
-                    if (i < n) {
-                        const int it = base + i, b = it % NST;
-                        ok = wait_or_abort(bars + UB_Q + b, (it / NST) & 1, status, abort_flag);
-                        if (ok && it >= G) ok = wait_or_abort(bars + UB_R + it % G, (it / G - 1) & 1, status, abort_flag);      // the group's last output has been read
-                        if (!ok) break;
-                        tc_fence_after();
-                        const TileDesc tQ(sQ + b * kXT);
-                        issue_projection<D>(tmem + col_u(it), tQ, tOm, tOml, id_u);
-                        mma_commit(bars + UB_U + it % G);
-                        mma_commit(bars + UB_QF + b);
-                    }
-                    if (i >= G - 1) {
-                        const int it = base + i - (G - 1);
-                        ok = wait_or_abort(bars + UB_E + it % G, (it / G) & 1, status, abort_flag);
-                        if (!ok) break;
-                        tc_fence_after();
-                        _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(tmem + col_o(it), tmem + col_f(it) + 8 * k, mndesc(tSb, k), id_o, k > 0);
-                        mma_commit(bars + UB_O + it % G);
-                    }
+                for (int t = c.t0; t < c.t1; ++t, ++it) {
+                    const int b = it % NST;
+                    ok = ok && wait_or_abort(bars + UB_Q + b, (it / NST) & 1, status, abort_flag);
+                    if (ok && it >= G) ok = wait_or_abort(bars + UB_R + it % G, (it / G - 1) & 1, status, abort_flag);      // the group's last output has been read
+                    if (!ok) break;
+                    tc_fence_after();
+                    const TileDesc tQ(sQ + b * kXT);
+                    issue_projection<D>(tmem + col_u(it), tQ, tOm, tOml, id_u);
+                    mma_commit(bars + UB_U + it % G);
+                    mma_commit(bars + UB_QF + b);
+                }
+            }
+        }
+    } else if (warp == kEpiWarps + 2) {                 // ---- MMAs: O = phi(Q) S
+        if ((tid & 31) == 0) {
+            const TileDesc tSb(sSb);
+            const uint32_t id_o = make_idesc(128, DV, 0, 1);
+            bool ok = true;
+            int it = 0;
+            for (int pc = 0; ok && list.next(p, c); ++pc) {
+                ok = wait_or_abort(bars + UB_OM, pc & 1, status, abort_flag);
+                for (int t = c.t0; t < c.t1; ++t, ++it) {
+                    ok = ok && wait_or_abort(bars + UB_E + it % G, (it / G) & 1, status, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(tmem + col_o(it), tmem + col_f(it) + 8 * k, mndesc(tSb, k), id_o, k > 0);
+                    mma_commit(bars + UB_O + it % G);
                 }
                 if (ok) mma_commit(bars + UB_OMF);
-                base += n;
             }
         }
     } else if (warp < 4 * G) {                          // ---- read-out
@@ -1062,8 +1083,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) tc_fwd_queries_kernel(const _
         unsigned char *stage = smem + L::kStage + warp * 4096;
         bool ok = true;
         int it = 0;
-        for (int pc = 0; ok && list.next(p, p.T, c); ++pc) {
-            const int bh = c.unit / p.nslab, slab = c.unit % p.nslab;
+        for (int pc = 0; ok && list.next(p, c); ++pc) {
+            const int bh = c.bh, slab = c.slab;
             const float cshift = load_key_shift(p.cs, bh * p.nslab + slab);
             const size_t prow0 = ((size_t)slab * p.BH + bh) * p.N + q4 * 32;
             bool fresh = true;
@@ -1483,8 +1504,10 @@ darkattn_status_t tensor_forward(const darkattn_plan_s *plan, const void *Q, con
         timer_mark(plan, st, "tc_fwd_causal_kernel");
         keep(launch_main_shape<MODE_CAUSAL>(D.d, D.dv, P, units * Y.nsplit, st));
     } else {
-        // one CTA per SM; a problem of few tiles gets one CTA for each
-        const int grid = (long long)units * Y.T < 148 ? units * Y.T : 148;
+        // one CTA per SM, the same number for every slab; a problem of few tiles gets one CTA for each
+        int per = 148 / Y.nslab;
+        if (per > (long long)BH * Y.T) per = (int)(BH * Y.T);
+        const int grid = Y.nslab * (per > 1 ? per : 1);
         timer_mark(plan, st, "tc_fwd_keys_kernel");
         keep(launch_main_shape<MODE_KEYS>(D.d, D.dv, P, grid, st));
         const long long n4 = (long long)BH * D.m * D.dv / 4;
