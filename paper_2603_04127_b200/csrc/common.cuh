@@ -89,6 +89,8 @@ struct TensorLayout {
     size_t zc;      // workspace copy of the stash's per-chunk z (causal): sum_j phi(K)_jl over the chunks before t, fp32 [BH, T, m]
     size_t Sseg, zseg;   // causal, cut into segments: the state and z before each segment, fp32
     size_t zq;      // non-causal: z of the whole sequence (workspace copy of the stash's)
+    size_t done;    // causal: slabs that have stored a tile's rows, int [BH, T]
+    int summers, cut;   // CTAs beside the causal scan that add up the slabs of the first `cut` chunks of every segment
     int nslab, T, nsplit, npiece;     // npiece: pieces the key pass cuts the first nsplit - 1 segments into
 };
 

@@ -273,6 +273,13 @@ struct MainParams {
     float *zc;           // causal: z before chunk t for the backward pass, [BH, T, m] (row 0 not written)
     int *status;
     int N, H, Hkv, BH, m, nslab, T, nsplit;
+    // Sum of the slabs beside the causal scan (done != null): slabs that have stored a tile's rows, [BH, T]; the CTAs from
+    // scan_ctas on add them up and normalise.
+    int *done;
+    int scan_ctas, cut;  // cut: chunks of each segment that are summed there (the kernel behind sums the rest)
+    const __nv_bfloat16 *pnum;
+    __nv_bfloat16 *O;
+    float2 *sv;
 };
 
 enum { MODE_CAUSAL = 0, MODE_KEYS = 1, MODE_QUERIES = 2 };
@@ -321,6 +328,145 @@ __device__ __forceinline__ float query_features_to_tmem(uint32_t u_addr, uint32_
     return dz;
 }
 
+// (u0, u1) - (n0, n1) - (c, c)
+__device__ __forceinline__ void sub2(float &u0, float &u1, float n0, float n1, float c)
+{
+    asm("{\n\t.reg .b64 a, b, m, d;\n\t"
+        "mov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tmov.b64 d, {%4, %4};\n\tmov.b64 m, {%5, %5};\n\t"
+        "fma.rn.f32x2 a, b, m, a;\n\t"
+        "fma.rn.f32x2 a, d, m, a;\n\t"
+        "mov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(u0), "+f"(u1) : "f"(n0), "f"(n1), "f"(c), "f"(-1.f));
+}
+__device__ __forceinline__ void add2(float &a0, float &a1, float b0, float b1)
+{
+    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tadd.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(a0), "+f"(a1) : "f"(b0), "f"(b1));
+}
+__device__ __forceinline__ void fma2(float &a0, float &a1, float b0, float b1, float c0, float c1)
+{
+    asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tmov.b64 c, {%4, %5};\n\tfma.rn.f32x2 a, b, c, a;\n\tmov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(a0), "+f"(a1) : "f"(b0), "f"(b1), "f"(c0), "f"(c1));
+}
+// 32 rows of the output by one warp: O[row,:] = sum_s num_s[row,:] 2^(rho_s - rho) / sum_s den_s 2^(rho_s - rho),
+// rho = max_s rho_s; den_s is the sum of the slab's four partial normalisers. Lane l forms row l's weights; DV / 8 lanes read a
+// row, 16 bytes each. The partial rows were written by other SMs a moment ago and come out of L2 (__ldcg: never from this SM's
+// L1); what bounds this is that latency, so all loads (up to 16 per lane) are issued before anything is used. The combined
+// normaliser and rho are also written to sv for the backward pass; a normaliser that is zero or not finite is reported.
+template <int DV, int NS>
+__device__ __forceinline__ void combine_rows32_n(const MainParams &p, long long row0, int lane)
+{
+    const long long rows = (long long)p.BH * p.N, own = row0 + lane;
+    constexpr int LPR = DV / 8, RI = 32 / LPR, NIT = 32 / RI;      // lanes of a row, rows and rounds
+    constexpr int KS = NS > 0 ? NS : 1, UN = NS > 0 ? (16 / KS < NIT ? 16 / KS : NIT) : 1;      // rounds in flight together
+    const int c0 = (lane % LPR) * 8, rl = lane / LPR;
+    const __nv_bfloat16 *src = p.pnum + (row0 + rl) * DV + c0;
+    __nv_bfloat16 *dst = p.O + (row0 + rl) * DV + c0;
+    float rho = -INFINITY, den = 0.f, w[KS];
+    float4 d4[KS];
+    if constexpr (NS > 0) {
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            const float *q = p.pdr + 8 * (s * rows + own);
+            d4[s] = __ldcg(reinterpret_cast<const float4 *>(q));
+            w[s] = __ldcg(q + 4);
+        }
+    }
+    for (int i0 = 0; i0 < NIT; i0 += UN) {
+        uint4 raw[UN][KS];
+        if constexpr (NS > 0) {
+#pragma unroll
+            for (int u = 0; u < UN; ++u)
+#pragma unroll
+                for (int s = 0; s < NS; ++s) raw[u][s] = __ldcg(reinterpret_cast<const uint4 *>(src + (s * rows + (i0 + u) * RI) * DV));
+        }
+        if (i0 == 0) {
+            if constexpr (NS > 0) {
+#pragma unroll
+                for (int s = 0; s < NS; ++s) rho = fmaxf(rho, w[s]);
+#pragma unroll
+                for (int s = 0; s < NS; ++s) {
+                    w[s] = exp2f(w[s] - rho);
+                    den = fmaf((d4[s].x + d4[s].y) + (d4[s].z + d4[s].w), w[s], den);
+                }
+            } else {
+                for (int s = 0; s < p.nslab; ++s) rho = fmaxf(rho, __ldcg(p.pdr + 8 * (s * rows + own) + 4));
+                for (int s = 0; s < p.nslab; ++s) {
+                    const float *q = p.pdr + 8 * (s * rows + own);
+                    const float4 x = __ldcg(reinterpret_cast<const float4 *>(q));
+                    den = fmaf((x.x + x.y) + (x.z + x.w), exp2f(__ldcg(q + 4) - rho), den);
+                }
+            }
+            p.sv[own] = make_float2(den, rho);
+            if (!(den > 0.f) || !isfinite(den)) atomicCAS(p.status, 0, (int)DARKATTN_ERR_NONFINITE);
+        }
+        const float inv = 1.f / den;
+#pragma unroll
+        for (int u = 0; u < UN; ++u) {
+            const int r = (i0 + u) * RI + rl;
+            const float ir = __shfl_sync(0xffffffffu, inv, r), rr = __shfl_sync(0xffffffffu, rho, r);
+            float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+            auto add = [&](const uint4 &x, float ws) {
+                float f[8];
+                unpack8(x, f);
+#pragma unroll
+                for (int k = 0; k < 8; k += 2) fma2(acc[k], acc[k + 1], f[k], f[k + 1], ws, ws);
+            };
+            if constexpr (NS > 0) {
+#pragma unroll
+                for (int s = 0; s < NS; ++s) add(raw[u][s], __shfl_sync(0xffffffffu, w[s], r));
+            } else {
+                for (int s = 0; s < p.nslab; ++s)
+                    add(__ldcg(reinterpret_cast<const uint4 *>(src + (s * rows + (i0 + u) * RI) * DV)), exp2f(__ldcg(p.pdr + 8 * (s * rows + row0 + r) + 4) - rr));
+            }
+            uint4 out;
+            out.x = pack_bf16(acc[0] * ir, acc[1] * ir); out.y = pack_bf16(acc[2] * ir, acc[3] * ir);
+            out.z = pack_bf16(acc[4] * ir, acc[5] * ir); out.w = pack_bf16(acc[6] * ir, acc[7] * ir);
+            *reinterpret_cast<uint4 *>(dst + (i0 + u) * RI * DV) = out;
+        }
+    }
+}
+template <int DV>
+__device__ __forceinline__ void combine_rows32(const MainParams &p, long long row0, int lane)
+{
+    if (p.nslab == 1) combine_rows32_n<DV, 1>(p, row0, lane);
+    else if (p.nslab == 2) combine_rows32_n<DV, 2>(p, row0, lane);
+    else if (p.nslab == 4) combine_rows32_n<DV, 4>(p, row0, lane);
+    else combine_rows32_n<DV, 0>(p, row0, lane);
+}
+// A CTA that adds up the slabs beside the scan: groups of four warps take the tiles in the order in which the scan reaches them
+// and wait for all slabs of a tile to be stored. (These CTAs come last in the grid and the scan never waits for them.) One SM
+// gets 45 GB/s of rows through this; a ring filled by bulk copies did not help (the copies alone, without the sums, ran at 35).
+template <int DV>
+__device__ void sum_tiles(const MainParams &p)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, quarter = warp & 3;
+    const int groups = (blockDim.x / 128) * (gridDim.x - p.scan_ctas), g0 = (blockIdx.x - p.scan_ctas) * (blockDim.x / 128) + warp / 4;
+    if (warp / 4 >= blockDim.x / 128) return;
+    const int lines = p.BH * p.nsplit;
+    for (long long k = g0; k < (long long)lines * p.cut; k += groups) {
+        const int i = (int)(k / lines), bh = (int)(k % lines) / p.nsplit, seg = (int)(k % lines) % p.nsplit;
+        const int t = (int)((long long)p.T * seg / p.nsplit) + i;
+        if (t >= (int)((long long)p.T * (seg + 1) / p.nsplit)) continue;
+        const int *flag = p.done + (size_t)bh * p.T + t;
+        bool ok = true;
+        const unsigned long long t0 = global_timer_ns();
+        for (;;) {
+            int v;
+            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
+            if (v >= p.nslab) break;
+            const int st = *reinterpret_cast<volatile int *>(p.status);
+            if (st == 5 /* DARKATTN_ERR_TIMEOUT */ || st == (int)DARKATTN_ERR_CUDA || global_timer_ns() - t0 > kWaitLimitNs) { ok = false; break; }
+            __nanosleep(500);
+        }
+        if (!__all_sync(0xffffffffu, ok)) {
+            if (lane == 0) atomicCAS(p.status, 0, 5 /* DARKATTN_ERR_TIMEOUT */);
+            return;
+        }
+        combine_rows32<DV>(p, (long long)bh * p.N + t * 128 + 32 * quarter, lane);
+    }
+}
+
 template <int D, int DV>
 struct FwdCausalSmem {
     static constexpr int kOm = 0;                          // folded projections of the slab, rounded    [128 l, D]
@@ -342,6 +488,9 @@ struct FwdCausalSmem {
 // R1 at 256, R2 at 384.
 constexpr uint32_t kColS = 0, kColZ = 128, kColFQ = 192, kColR1 = 256, kColR2 = 384;
 
+// 16 epilogue warps, the control warp, the warp that stores the output
+constexpr int kCausalThreads = 576;
+
 enum CBars { CB_OM, CB_Q, CB_K, CB_V, CB_ST, CM1, CM2, CM3, CMS, CM4, CE0, CE1, CE2, CE3, CE4, CNBARS };
 
 // Causal: one CTA per (b, h, slab) walks the chunks of the sequence.
@@ -350,9 +499,11 @@ enum CBars { CB_OM, CB_Q, CB_K, CB_V, CB_ST, CM1, CM2, CM3, CMS, CM4, CE0, CE1, 
 // The epilogue warps work in this order: phi(K) of chunk t; the bf16 copy of the state through chunk t - 1 (while P
 // runs); tril(P); the output tile and z; phi(Q) of chunk t + 1 (both projections of the next chunk are issued behind
 // the output MMAs and run while the output is read). The state tile's buffer doubles as the staging tile of the
-// output's TMA store: between the output MMAs of chunk t and the copy of the state through chunk t nobody reads it.
+// output's TMA store: between the output MMAs of chunk t and the copy of the state through chunk t nobody reads it. One thread
+// of another warp issues that store, so that waiting for it does not hold up the MMAs; where the slabs are summed beside the
+// scan (p.done) it then counts the tile.
 template <int D, int DV>
-__global__ void __launch_bounds__(kThreads, 1) tc_fwd_causal_kernel(const __grid_constant__ MainParams p)
+__global__ void __launch_bounds__(kCausalThreads, 1) tc_fwd_causal_kernel(const __grid_constant__ MainParams p)
 {
     using L = FwdCausalSmem<D, DV>;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -364,6 +515,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_causal_kernel(const __grid
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + CNBARS + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5;
+    if (blockIdx.x >= p.scan_ctas) {
+        pdl_wait();
+        sum_tiles<DV>(p);
+        return;
+    }
     const int unit = blockIdx.x / p.nsplit, seg = blockIdx.x % p.nsplit;
     const int bh = unit / p.nslab, slab = unit % p.nslab, h = bh % p.H;
     const int row0 = bh * p.N;
@@ -425,11 +581,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_causal_kernel(const __grid
                 const int base = (map == &p.mapQ) ? row0 : rowk0;
                 mbar_expect_tx(bar, 128 * width * 2);
                 for (int a = 0; a < width / 64; ++a) tma_load_2d(dst + a * 16384, map, bar, a * 64, base + t * 128);
-            };
-            const int prow0 = (slab * p.BH + bh) * p.N;
-            auto store_output = [&](int t) {       // this slab's part of the output rows of chunk t, staged in the state tile's buffer
-                for (int a = 0; a < DV / 64; ++a) tma_store_2d(&p.mapPN, sSb + a * 16384, a * 64, prow0 + t * 128);
-                tma_store_commit();
             };
             auto store_state = [&](int t) {        // the bf16 state before chunk t, for the backward pass
                 for (int a = 0; a < DV / 64; ++a) tma_store_2d(&p.mapSst, sSb + a * 16384, a * 64, (bh * p.T + t) * p.m + slab * 128);
@@ -510,14 +661,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_causal_kernel(const __grid
                 _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColS, mndesc(tFK, k), mndesc(tV, k), id_s, (!first) || k > 0);   // S += phi(K)^T V
                 mma_commit(bars + CMS);
                 CWAIT(CE3, ph); if (!ok) break;                                 // the output tile has been read out of R2 and staged
-                store_output(t);
                 if (!last) {
                     CWAIT(CB_K, ph ^ 1); if (!ok) break;
                     tc_fence_after();
                     issue_projection<D>(R2, tK, tOm, tOml, id_kk);                                                // U_K of the next chunk
                     mma_commit(bars + CM2);
                 }
-                if (!last || copy_last) { tma_store_wait_read(); mbar_arrive(bars + CB_ST); }     // the staged output has left the state tile's buffer
                 CWAIT(CMS, ph); if (!ok) break;                                 // V tile consumed
                 if (!last) {
                     load_tile(sV, &p.mapV, bars + CB_V, DV, t + 1);
@@ -530,6 +679,23 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_causal_kernel(const __grid
                 if (ok) store_state(tend);
             }
 #undef CWAIT
+            tma_store_wait_all();
+        }
+    } else if (warp == kEpiWarps + 1) {
+        if ((tid & 31) == 0) {
+            const int prow0 = (slab * p.BH + bh) * p.N;
+            for (int t = tbeg; t < tend; ++t) {     // this slab's part of the output rows of chunk t, staged in the state tile's buffer
+                if (!wait_or_abort(bars + CE3, (t - tbeg) & 1, status, abort_flag)) break;
+                for (int a = 0; a < DV / 64; ++a) tma_store_2d(&p.mapPN, sSb + a * 16384, a * 64, prow0 + t * 128);
+                tma_store_commit();
+                if (t + 1 < tend || copy_last) { tma_store_wait_read(); mbar_arrive(bars + CB_ST); }     // it has left the state tile's buffer
+                if (p.done && t - tbeg < p.cut) {       // the rows and (written before the arrivals on CE3) their normalisers are visible to who sees the count
+                    tma_store_wait_all();
+                    asm volatile("fence.proxy.async;" ::: "memory");
+                    __threadfence();
+                    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.done + (size_t)bh * p.T + t) : "memory");
+                }
+            }
             tma_store_wait_all();
         }
     } else {
@@ -626,11 +792,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_causal_kernel(const __grid
                 sZ[r] = zv;
                 p.zc[((size_t)bh * p.T + t + 1) * p.m + slab * 128 + r] = zv;
             }
+            p.pdr[8 * prow + g] = rowsum + dz;
+            if (g == 0) p.pdr[8 * prow + 4] = rmax + cshift;
             fence_async_smem();
             tc_fence_before();
             mbar_arrive_warp(bars + CE3);
-            p.pdr[8 * prow + g] = rowsum + dz;
-            if (g == 0) p.pdr[8 * prow + 4] = rmax + cshift;
             epi_sync();                             // every z is in place before anyone forms the next chunk's phi(Q)
 
             if (!last) {
@@ -693,26 +859,6 @@ struct PieceList {
 // spends its program order waiting for the one while the other is ready); the key pass has a second TMA warp
 constexpr int kPassThreads = 608, kKeysThreads = 640;
 
-// (u0, u1) - (n0, n1) - (c, c)
-__device__ __forceinline__ void sub2(float &u0, float &u1, float n0, float n1, float c)
-{
-    asm("{\n\t.reg .b64 a, b, m, d;\n\t"
-        "mov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tmov.b64 d, {%4, %4};\n\tmov.b64 m, {%5, %5};\n\t"
-        "fma.rn.f32x2 a, b, m, a;\n\t"
-        "fma.rn.f32x2 a, d, m, a;\n\t"
-        "mov.b64 {%0, %1}, a;\n\t}"
-        : "+f"(u0), "+f"(u1) : "f"(n0), "f"(n1), "f"(c), "f"(-1.f));
-}
-__device__ __forceinline__ void add2(float &a0, float &a1, float b0, float b1)
-{
-    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tadd.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
-        : "+f"(a0), "+f"(a1) : "f"(b0), "f"(b1));
-}
-__device__ __forceinline__ void fma2(float &a0, float &a1, float b0, float b1, float c0, float c1)
-{
-    asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tmov.b64 c, {%4, %5};\n\tfma.rn.f32x2 a, b, c, a;\n\tmov.b64 {%0, %1}, a;\n\t}"
-        : "+f"(a0), "+f"(a1) : "f"(b0), "f"(b1), "f"(c0), "f"(c1));
-}
 // untiled copy of a multiple of 16 bytes (both addresses 16-byte aligned) into shared memory
 __device__ __forceinline__ void bulk_load(void *smem_dst, const void *src, uint32_t bytes, uint64_t *bar)
 {
@@ -1231,13 +1377,15 @@ __global__ void __launch_bounds__(256) segment_prefix_kernel(const float *__rest
 // NS > 0: the number of slabs at compile time (all loads of a thread are issued before the first use).
 template <int NS>
 __global__ void combine_kernel(const __nv_bfloat16 *pnum, const float *pdr, __nv_bfloat16 *O, float2 *sv,
-                               long long rows, int dv, int nslab_rt, int *status)
+                               long long rows, int dv, int nslab_rt, int *status, int T, int nseg, int cut)
 {
     pdl_wait();
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const int per_row = dv / 8;
-    if (i >= rows * per_row) return;
-    const long long row = i / per_row;
+    const int per_row = dv / 8, seg = blockIdx.y % nseg;
+    // blockIdx.y: (batch, head) and segment of the sequence; the first `cut` chunks of a segment have been summed beside the scan
+    const int t0 = (int)((long long)T * seg / nseg) + cut, t1 = (int)((long long)T * (seg + 1) / nseg);
+    if (i >= (long long)(t1 - t0) * 128 * per_row) return;
+    const long long row = ((long long)(blockIdx.y / nseg) * T + t0) * 128 + i / per_row;
     const int c0 = (int)(i % per_row) * 8;
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0}, den = 0.f, rho = -INFINITY;
     auto slab_den = [](const float4 &d4) { return (d4.x + d4.y) + (d4.z + d4.w); };
@@ -1306,7 +1454,7 @@ cudaError_t launch_main(const MainParams &P, int grid, cudaStream_t st)
     if constexpr (MODE == MODE_CAUSAL) {
         using L = FwdCausalSmem<D, DV>;
         static_assert(L::kTotal <= 232448, "shared memory budget of one CTA exceeded");
-        return launch_pdl(tc_fwd_causal_kernel<D, DV>, dim3(grid), dim3(kThreads), L::kTotal, st, P);
+        return launch_pdl(tc_fwd_causal_kernel<D, DV>, dim3(grid), dim3(kCausalThreads), L::kTotal, st, P);
     } else if constexpr (MODE == MODE_KEYS) {
         using L = FwdKeysSmem<D, DV>;
         static_assert(L::kTotal <= 232448, "shared memory budget of one CTA exceeded");
@@ -1376,13 +1524,24 @@ void tensor_make_layout(darkattn_plan_s *plan)
     // (states and z of the key pass: sums over all keys, or one per piece; what it adds into is cleared by one run of stores)
     Y.Sacc = take(off, BH * (D.causal ? (size_t)Y.npiece : 1) * m * dv * 4);
     Y.zacc = take(off, BH * (D.causal ? (size_t)Y.npiece : 1) * m * 16);
+    Y.done = take(off, BH * (size_t)Y.T * 4);
     Y.Sb = take(off, BH * nstate * m * dv * 2);
     Y.Sseg = take(off, Y.npiece ? BH * nstate * m * dv * 4 : 0);
     Y.zseg = take(off, Y.npiece ? BH * nstate * m * 4 : 0);
     Y.zq = take(off, D.causal ? 0 : BH * m * 4);
     Y.sv = take(off, BH * N * 8);
     Y.zc = take(off, D.causal ? BH * (size_t)Y.T * m * 4 : 0);
-    plan->launches_fwd = D.causal ? (nsplit > 1 ? 6 : 4) : 6;
+    // The causal scan may leave SMs idle, which can add up the slabs meanwhile: 45 GB/s of rows read and written per SM, against
+    // 4.4 us (d 64) or 5.2 us (d 128) for a chunk of the scan; of every segment as many chunks as they manage in that time, less
+    // a tenth. Not for short scans, whose last tiles would be waited for, nor where they would sum less than a fifth.
+    const long long scan_ctas = units * nsplit, idle = 148 - scan_ctas;
+    Y.summers = Y.cut = 0;
+    if (D.causal && Y.T / nsplit >= 8 && idle > 0) {
+        const double part = 0.9 * idle * 45e3 * (d == 64 ? 4.4 : 5.2) / ((double)BH * nsplit * (Y.nslab + 1) * 256.0 * dv);
+        if (part >= 1.0) { Y.cut = (Y.T + nsplit - 1) / nsplit; Y.summers = (int)(idle / part) + 1; }
+        else if (part >= 0.2) { Y.cut = (int)(part * (Y.T / nsplit)); Y.summers = (int)idle; }
+    }
+    plan->launches_fwd = (D.causal ? (nsplit > 1 ? 6 : 4) : 6) - (Y.cut >= (Y.T + nsplit - 1) / nsplit ? 1 : 0);
     {
         size_t so = 0;
         Y.sv_sv = take(so, BH * N * 8);
@@ -1436,9 +1595,10 @@ cudaError_t tensor_prologue(const darkattn_plan_s *plan, const void *K, const vo
     cudaError_t e = cudaSuccess;
     auto keep = [&](cudaError_t x) { if (x != cudaSuccess && e == cudaSuccess) e = x; };
     timer_mark(plan, st, "fold_omega_kernel");
-    // (S and z sums of the non-causal key pass: adjacent, multiples of 256 bytes)
-    float4 *zero = D.causal ? nullptr : reinterpret_cast<float4 *>(ws + Y.Sacc);
-    const long long nzero = D.causal ? 0 : (long long)((Y.Sb - Y.Sacc) / 16);
+    // (S and z sums of the non-causal key pass and the counts of the tiles' slabs: adjacent, multiples of 256 bytes)
+    const size_t zero_at = D.causal ? Y.done : Y.Sacc;
+    float4 *zero = reinterpret_cast<float4 *>(ws + zero_at);
+    const long long nzero = (long long)((Y.Sb - zero_at) / 16);
     int *status = reinterpret_cast<int *>(ws + Y.status), *cs = reinterpret_cast<int *>(out.cs);
     const int ncs = (int)(BH * Y.nslab);
     const dim3 fold_grid(D.m / 16, D.H);
@@ -1502,7 +1662,10 @@ darkattn_status_t tensor_forward(const darkattn_plan_s *plan, const void *Q, con
                             fl(Y.Sseg), bf(Y.Sb), fl(Y.zseg), Y.nsplit, Y.npiece, E4, D.m, total));
         }
         timer_mark(plan, st, "tc_fwd_causal_kernel");
-        keep(launch_main_shape<MODE_CAUSAL>(D.d, D.dv, P, units * Y.nsplit, st));
+        P.cut = Y.cut;
+        P.done = Y.summers ? reinterpret_cast<int *>(ws + Y.done) : nullptr;
+        P.scan_ctas = units * Y.nsplit; P.pnum = bf(Y.pnum); P.O = (__nv_bfloat16 *)O; P.sv = stash.sv;
+        keep(launch_main_shape<MODE_CAUSAL>(D.d, D.dv, P, P.scan_ctas + Y.summers, st));
     } else {
         // one CTA per SM, the same number for every slab; a problem of few tiles gets one CTA for each
         int per = 148 / Y.nslab;
@@ -1517,12 +1680,17 @@ darkattn_status_t tensor_forward(const darkattn_plan_s *plan, const void *Q, con
         timer_mark(plan, st, "tc_fwd_queries_kernel");
         keep(launch_main_shape<MODE_QUERIES>(D.d, D.dv, P, grid, st));
     }
-    {
-        const long long rows = (long long)BH * N, threads = rows * (D.dv / 8);
+    const int longest = (Y.T + Y.nsplit - 1) / Y.nsplit;
+    if (Y.cut < longest) {
+        const long long rows = (long long)BH * N;
+        const int nseg = D.causal ? Y.nsplit : 1;
         timer_mark(plan, st, "combine_kernel");
-        const unsigned grid = (unsigned)((threads + 255) / 256);
         auto *combine = Y.nslab == 1 ? combine_kernel<1> : Y.nslab == 2 ? combine_kernel<2> : Y.nslab == 4 ? combine_kernel<4> : combine_kernel<0>;
-        keep(launch_pdl(combine, dim3(grid), dim3(256), 0, st, (const __nv_bfloat16 *)bf(Y.pnum), (const float *)fl(Y.pdr), (__nv_bfloat16 *)O, stash.sv, rows, D.dv, Y.nslab, P.status));
+        // (in the second dimension, which is limited to 65535, whole sequences where nothing has been summed yet)
+        const bool flat = Y.cut == 0;
+        const long long threads = flat ? rows * (D.dv / 8) : (long long)(longest - Y.cut) * 128 * (D.dv / 8);
+        keep(launch_pdl(combine, dim3((unsigned)((threads + 255) / 256), flat ? 1 : (unsigned)(BH * nseg)), dim3(256), 0, st, (const __nv_bfloat16 *)bf(Y.pnum),
+                        (const float *)fl(Y.pdr), (__nv_bfloat16 *)O, stash.sv, rows, D.dv, Y.nslab, P.status, flat ? (int)(rows / 128) : Y.T, flat ? 1 : nseg, Y.cut));
     }
     if (e != cudaSuccess) { set_cuda_error(e, "tensor_forward"); return DARKATTN_ERR_CUDA; }
     return DARKATTN_OK;

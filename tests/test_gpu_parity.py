@@ -411,6 +411,13 @@ PASS_EDGES = [
     dict(B=1, H=7, N=4224, d=64, m=256, dv=128, causal=False),
     dict(B=1, H=2, N=4992, d=64, m=128, causal=True),
     dict(B=1, H=3, N=1408, d=128, m=256, dv=128, causal=True),
+    # the slabs summed beside the scan: one, two, three, four slabs; some chunks only; uneven segments
+    dict(B=1, H=80, N=1024, d=64, m=128, causal=True),
+    dict(B=2, H=19, N=1152, d=128, m=256, dv=64, causal=True),
+    dict(B=1, H=26, N=1152, d=64, m=384, dv=128, causal=True),
+    dict(B=1, H=20, N=1152, d=64, m=512, causal=True),
+    dict(B=1, H=70, N=1152, d=64, m=256, causal=True),
+    dict(B=1, H=4, N=17792, d=64, m=256, causal=True),
 ]
 
 
