@@ -9,6 +9,7 @@
 #include "darkattn.h"
 
 namespace darkattn {
+namespace tc { struct ClearList; }
 
 // Resolved problem description (defaults filled in).
 struct Dims {
@@ -196,7 +197,7 @@ cudaError_t tensor_prologue(const darkattn_plan_s *plan, const void *K, const vo
 // dW from what the last backward call left in the workspace
 darkattn_status_t simt_backward_dw(const darkattn_plan_s *plan, float *dW, char *ws, cudaStream_t st);
 cudaError_t tensor_backward_nc_passes(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V, const void *dO,
-                                      const Stash &stash, void *dQ, void *dK, void *dV, bool per_head, bool join, char *ws, cudaStream_t st);
+                                      const Stash &stash, void *dQ, void *dK, void *dV, bool per_head, const tc::ClearList &clear, char *ws, cudaStream_t st);
 darkattn_status_t tensor_backward_dw(const darkattn_plan_s *plan, const void *M, float *dW, char *ws, cudaStream_t st);
 darkattn_status_t tensor_backward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
                                   const void *M, const void *W, const void *O, const void *dO, const void *saved,

@@ -366,6 +366,19 @@ __device__ __forceinline__ void issue_projection(uint32_t dst, const TileDesc &t
 // (grouped key/value heads: G = H / H_kv consecutive query heads share one).
 __device__ __forceinline__ int kv_row0(int bh, int H, int Hkv, int N) { return ((bh / H) * Hkv + (bh % H) / (H / Hkv)) * N; }
 
+// What a warp of a backward kernel clears beside the kernel's own work: the gradients that the next kernel adds into. (On a side
+// stream the two memsets, 24 us each at 4 x 16 heads, 8192 tokens, d 128, did not get onto the SMs beside a scan and ran after it.)
+constexpr int kClearThreads = kThreads + 32;       // with that warp
+struct ClearList { uint4 *p[2]; long long n[2]; };
+__device__ __forceinline__ void clear_share(const ClearList &c)
+{
+    const int lane = threadIdx.x & 31;
+    const long long step = (long long)gridDim.x * 32;
+    for (int k = 0; k < 2; ++k)
+#pragma unroll 4
+        for (long long i = blockIdx.x * 32LL + lane; i < c.n[k]; i += step) c.p[k][i] = make_uint4(0, 0, 0, 0);
+}
+
 // ---------------------------------------------------------------- host side: tensor maps
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,

@@ -53,6 +53,7 @@ struct BwdParams {
     int N, H, Hkv, BH, m, nslab, T;
     int add_kv;           // parts of dK and dV are added into the (zeroed) gradients: several slabs
     int out_per_head;     // grouped key/value heads: dK and dV rows are indexed by the query head (a later kernel sums each group)
+    ClearList clear;      // query side: dK and dV, where several slabs add into them
 };
 
 template <int D, int DV>
@@ -92,7 +93,7 @@ enum QBars { QB_OM, QB_Q, QB_B, QB_V, QB_G, QB_S, QB_X2, QM1, QM3, QM4, QM5, QM6
 // chunks are independent of one another here: the chunks of all (batch, head) pairs form one line that is cut evenly
 // over groups of nslab CTAs, and a CTA walks its piece run by run (a run = consecutive chunks of one (batch, head) pair).
 template <int D, int DV>
-__global__ void __launch_bounds__(kThreads, 1) tc_bwd_q_kernel(const __grid_constant__ BwdParams p)
+__global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_q_kernel(const __grid_constant__ BwdParams p)
 {
     using L = BwdSmem<D, DV>;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -127,6 +128,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_q_kernel(const __grid_cons
 
     if (*abort_flag) {
         if (tid == 0) atomicExch(status, (int)DARKATTN_ERR_CUDA);
+    } else if (warp == kEpiWarps + 1) {
+        clear_share(p.clear);
     } else if (warp == kEpiWarps) {
         if ((tid & 31) == 0) {
             const TileDesc tOm(sOm), tOml(sOml), tQA(sQA), tKB(sKB), tV(sV), tG(sG), tSt(sSt), tDel(sDelOp);
@@ -891,9 +894,9 @@ __global__ void group_sum_kernel(const __nv_bfloat16 *src, __nv_bfloat16 *out, i
 }
 
 // delta[row] = dO[row,:] . O[row,:]; dv/8 threads per row, 16 bytes of each tensor per thread. The same threads clear what the
-// call's later kernels add into (each of these was a memset of its own before, with 4 us from one to the next) and the status
+// call's first kernels add into (each of these was a memset of its own before, with 4 us from one to the next) and the status
 // word (status may be null: the forward kernels of this call have cleared it).
-struct ZeroList { uint4 *p[6]; long long n[6]; int count; };
+struct ZeroList { uint4 *p[4]; long long n[4]; int count; };
 __global__ void __launch_bounds__(256) delta_kernel(const __nv_bfloat16 *G, const __nv_bfloat16 *O, float *delta, long long rows, int dv, int *status,
                                                     const __grid_constant__ ZeroList Z)
 {
@@ -991,7 +994,7 @@ int sm_count()
 }
 
 template <int D, int DV>
-cudaError_t launch_scan(const darkattn_plan_s *plan, const BwdParams &P, int grid, bool join, cudaStream_t st)
+cudaError_t launch_scan(const darkattn_plan_s *plan, const BwdParams &P, int grid, cudaStream_t st)
 {
     using L = BwdSmem<D, DV>;
     static_assert(L::kTotal <= 232448, "shared memory budget of one CTA exceeded");
@@ -1001,8 +1004,7 @@ cudaError_t launch_scan(const darkattn_plan_s *plan, const BwdParams &P, int gri
     if (groups > (long long)P.BH * P.T) groups = (long long)P.BH * P.T;
     const int qgrid = (int)groups * P.nslab;
     timer_mark(plan, st, "tc_bwd_q_kernel");
-    cudaError_t e = launch_pdl(tc_bwd_q_kernel<D, DV>, dim3(qgrid), dim3(kThreads), L::kTotal, st, P);
-    if (e == cudaSuccess && join) e = cudaStreamWaitEvent(st, plan->aux_join, 0);      // dK and dV have been zeroed
+    cudaError_t e = launch_pdl(tc_bwd_q_kernel<D, DV>, dim3(qgrid), dim3(kClearThreads), L::kTotal, st, P);
     if (e != cudaSuccess) return e;
     timer_mark(plan, st, "tc_bwd_k_kernel");
     return launch_pdl(tc_bwd_k_kernel<D, DV>, dim3(grid), dim3(kThreads), L::kTotal, st, P);
@@ -1052,19 +1054,12 @@ darkattn_status_t tensor_backward(const darkattn_plan_s *plan, const void *Q, co
     void *dKo = per_head ? (void *)bf(Y.dKh) : dK, *dVo = per_head ? (void *)bf(Y.dVh) : dV;
     const size_t BHo = per_head ? BH : BHkv;
     // The slabs of a head add their parts into the gradients, which therefore start at zero. dQ is needed first and is
-    // cleared by the kernel that forms delta; dK and dV, where they are large (clearing 32 MB takes longer than the two events
-    // between the streams), on a side stream while the query-side scan runs: it leaves SMs and bandwidth free.
+    // cleared by the kernel that forms delta, dK and dV by a warp of the query-side kernel.
     const bool add_kv = Y.nslab > 1;
-    const size_t kv_bytes = BHo * N * ((size_t)D.d + D.dv) * 2;
-    const bool beside_zero = add_kv && kv_bytes > (32u << 20);
-    if (beside_zero) {
-        keep(ensure_aux(plan));
-        if (e != cudaSuccess) { set_cuda_error(e, "tensor_backward: side stream"); return DARKATTN_ERR_CUDA; }
-        keep(cudaEventRecord(plan->aux_fork, st));
-        keep(cudaStreamWaitEvent(plan->aux_stream, plan->aux_fork, 0));
-        keep(cudaMemsetAsync(dKo, 0, BHo * N * D.d * 2, plan->aux_stream));
-        keep(cudaMemsetAsync(dVo, 0, BHo * N * D.dv * 2, plan->aux_stream));
-        keep(cudaEventRecord(plan->aux_join, plan->aux_stream));
+    ClearList clear = {};
+    if (add_kv) {
+        clear.p[0] = static_cast<uint4 *>(dKo); clear.n[0] = (long long)(BHo * N * D.d * 2 / 16);
+        clear.p[1] = static_cast<uint4 *>(dVo); clear.n[1] = (long long)(BHo * N * D.dv * 2 / 16);
     }
     ZeroList Z;
     Z.count = 0;
@@ -1073,7 +1068,6 @@ darkattn_status_t tensor_backward(const darkattn_plan_s *plan, const void *Q, co
     zero(ws + Y.dMn, (size_t)D.H * D.r * D.d * 4);
     if (!D.causal) zero(ws + Y.Racc, (Y.rhot - Y.Racc) + BH * D.m * 4);      // R and rho sums (adjacent)
     if (add_kv) zero(dQ, BH * N * D.d * 2);
-    if (add_kv && !beside_zero) { zero(dKo, BHo * N * D.d * 2); zero(dVo, BHo * N * D.dv * 2); }
     const long long rows = (long long)BH * N;
     timer_mark(plan, st, "delta_kernel");
     keep(launch_pdl(delta_kernel, dim3((unsigned)((rows * (D.dv / 8) + 255) / 256)), dim3(256), 0, st, (const __nv_bfloat16 *)dO, (const __nv_bfloat16 *)O,
@@ -1102,13 +1096,14 @@ darkattn_status_t tensor_backward(const darkattn_plan_s *plan, const void *Q, co
         P.status = reinterpret_cast<int *>(ws + Y.status);
         P.N = D.N; P.H = D.H; P.Hkv = D.Hkv; P.BH = D.BH; P.m = D.m; P.nslab = Y.nslab; P.T = Y.T; P.add_kv = add_kv ? 1 : 0;
         P.out_per_head = per_head ? 1 : 0;
+        P.clear = clear;
         const int units = (int)(BH * Y.nslab);
-        if (D.d == 64 && D.dv == 64) keep(launch_scan<64, 64>(plan, P, units, beside_zero, st));
-        else if (D.d == 128 && D.dv == 128) keep(launch_scan<128, 128>(plan, P, units, beside_zero, st));
-        else if (D.d == 64 && D.dv == 128) keep(launch_scan<64, 128>(plan, P, units, beside_zero, st));
-        else keep(launch_scan<128, 64>(plan, P, units, beside_zero, st));
+        if (D.d == 64 && D.dv == 64) keep(launch_scan<64, 64>(plan, P, units, st));
+        else if (D.d == 128 && D.dv == 128) keep(launch_scan<128, 128>(plan, P, units, st));
+        else if (D.d == 64 && D.dv == 128) keep(launch_scan<64, 128>(plan, P, units, st));
+        else keep(launch_scan<128, 64>(plan, P, units, st));
     } else {
-        keep(tensor_backward_nc_passes(plan, Q, K, V, dO, stash, dQ, dKo, dVo, per_head, beside_zero, ws, st));
+        keep(tensor_backward_nc_passes(plan, Q, K, V, dO, stash, dQ, dKo, dVo, per_head, clear, ws, st));
     }
 
     if (!make_map(&F.mapOut, dKo, BHo * N, D.d, 128)) { set_cuda_error(cudaErrorInvalidValue, "tensor_backward: tensor map encode"); return DARKATTN_ERR_CUDA; }

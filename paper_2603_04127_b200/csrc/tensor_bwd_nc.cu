@@ -41,6 +41,7 @@ struct NcParams {
     int N, H, Hkv, BH, m, nslab, T, nsplit;
     int add_kv;           // parts of dK and dV are added into the (zeroed) gradients: several slabs
     int out_per_head;     // grouped key/value heads: dK and dV rows are indexed by the query head (a later kernel sums each group)
+    ClearList clear;      // query pass: dK and dV, where several slabs add into them
 };
 
 template <int D, int DV>
@@ -73,7 +74,7 @@ enum NBars { NB_OM, NB_X0, NB_X1, NB_Y, NM1, NMA, NM2, NM3, NE1, NE2, NE3, NNBAR
 //   R2: dO S^T | V R^T (independent of the features, issued at once) -> (E formed) -> E Omega -> (read, stored)
 // and the state updates R += A^^T dO, T += E^T X run behind them. KEYS selects the key pass.
 template <int D, int DV, bool KEYS>
-__global__ void __launch_bounds__(kThreads, 1) tc_bwd_nc_kernel(const __grid_constant__ NcParams p)
+__global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_nc_kernel(const __grid_constant__ NcParams p)
 {
     using L = NcSmem<D, DV>;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -111,6 +112,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_nc_kernel(const __grid_con
 
     if (*abort_flag) {
         if (tid == 0) atomicExch(status, (int)DARKATTN_ERR_CUDA);
+    } else if (warp == kEpiWarps + 1) {
+        clear_share(p.clear);
     } else if (nt <= 0) {
         // nothing to do for this piece
     } else if (warp == kEpiWarps) {
@@ -341,29 +344,28 @@ __global__ void nc_round_state_kernel(const float *R, __nv_bfloat16 *Rb, long lo
 
 template <int D, int DV>
 cudaError_t launch_nc(const darkattn_plan_s *plan, const NcParams &PQ, const NcParams &PK, const float *Racc, __nv_bfloat16 *Rb,
-                      long long nstate, bool join, cudaStream_t st)
+                      long long nstate, cudaStream_t st)
 {
     using L = NcSmem<D, DV>;
     static_assert(L::kTotal <= 232448, "shared memory budget of one CTA exceeded");
     const int grid = PQ.BH * PQ.nslab * PQ.nsplit;
     timer_mark(plan, st, "tc_bwd_nc_q_kernel");
-    cudaError_t e = launch_pdl(tc_bwd_nc_kernel<D, DV, false>, dim3(grid), dim3(kThreads), L::kTotal, st, PQ);
+    cudaError_t e = launch_pdl(tc_bwd_nc_kernel<D, DV, false>, dim3(grid), dim3(kClearThreads), L::kTotal, st, PQ);
     if (e != cudaSuccess) return e;
     timer_mark(plan, st, "nc_round_state_kernel");
     e = launch_pdl(nc_round_state_kernel, dim3((unsigned)((nstate / 4 + 255) / 256)), dim3(256), 0, st, Racc, Rb, nstate);
-    if (e == cudaSuccess && join) e = cudaStreamWaitEvent(st, plan->aux_join, 0);      // dK and dV have been zeroed
     if (e != cudaSuccess) return e;
     timer_mark(plan, st, "tc_bwd_nc_k_kernel");
-    return launch_pdl(tc_bwd_nc_kernel<D, DV, true>, dim3(grid), dim3(kThreads), L::kTotal, st, PK);
+    return launch_pdl(tc_bwd_nc_kernel<D, DV, true>, dim3(grid), dim3(kClearThreads), L::kTotal, st, PK);
 }
 
 }  // namespace
 
 // The two passes of the non-causal backward. Expects delta computed, Tacc, Racc, rhot and (with several
-// slabs) dQ, dK and dV zeroed on `st` (with `join` dK and dV behind plan->aux_join). With `per_head`, dK and dV are the per-query-head
+// slabs) dQ zeroed on `st`; `clear`: dK and dV, which the first pass clears. With `per_head`, dK and dV are the per-query-head
 // buffers of grouped key/value heads ([BH, N, *]).
 cudaError_t tensor_backward_nc_passes(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V, const void *dO,
-                                      const Stash &stash, void *dQ, void *dK, void *dV, bool per_head, bool join, char *ws, cudaStream_t st)
+                                      const Stash &stash, void *dQ, void *dK, void *dV, bool per_head, const ClearList &clear, char *ws, cudaStream_t st)
 {
     const Dims &D = plan->dims;
     const TensorLayout &Y = plan->tensor;
@@ -383,6 +385,7 @@ cudaError_t tensor_backward_nc_passes(const darkattn_plan_s *plan, const void *Q
     PQ.N = D.N; PQ.H = D.H; PQ.Hkv = D.Hkv; PQ.BH = D.BH; PQ.m = D.m; PQ.nslab = Y.nslab; PQ.T = Y.T; PQ.add_kv = add_kv ? 1 : 0;
     PQ.nsplit = pick_splits((long long)BH * Y.nslab, Y.T, 3.0, 6.0, 64);
     NcParams PK = PQ;
+    PQ.clear = clear;
     const bool ok = make_map(&PQ.mapX, Q, BH * N, D.d, 128) && make_map(&PQ.mapY, dO, BH * N, D.dv, 128) &&
                     make_map(&PQ.mapOm, stash.Om, (size_t)D.H * D.m, D.d, 128) && make_map(&PQ.mapOml, stash.Oml, (size_t)D.H * D.m, D.d, 128) &&
                     make_map(&PQ.mapSt, stash.Sb, BH * D.m, D.dv, 128) &&
@@ -394,10 +397,10 @@ cudaError_t tensor_backward_nc_passes(const darkattn_plan_s *plan, const void *Q
     PK.mapOml = PQ.mapOml;
     PK.mapDV = PQ.mapDV;
     const long long nstate = (long long)BH * D.m * D.dv;
-    if (D.d == 64 && D.dv == 64) return launch_nc<64, 64>(plan, PQ, PK, fl(Y.Racc), Rb, nstate, join, st);
-    if (D.d == 128 && D.dv == 128) return launch_nc<128, 128>(plan, PQ, PK, fl(Y.Racc), Rb, nstate, join, st);
-    if (D.d == 64 && D.dv == 128) return launch_nc<64, 128>(plan, PQ, PK, fl(Y.Racc), Rb, nstate, join, st);
-    return launch_nc<128, 64>(plan, PQ, PK, fl(Y.Racc), Rb, nstate, join, st);
+    if (D.d == 64 && D.dv == 64) return launch_nc<64, 64>(plan, PQ, PK, fl(Y.Racc), Rb, nstate, st);
+    if (D.d == 128 && D.dv == 128) return launch_nc<128, 128>(plan, PQ, PK, fl(Y.Racc), Rb, nstate, st);
+    if (D.d == 64 && D.dv == 128) return launch_nc<64, 128>(plan, PQ, PK, fl(Y.Racc), Rb, nstate, st);
+    return launch_nc<128, 64>(plan, PQ, PK, fl(Y.Racc), Rb, nstate, st);
 }
 
 }  // namespace darkattn
