@@ -436,7 +436,7 @@ __device__ __forceinline__ void combine_rows32(const MainParams &p, long long ro
 }
 // A CTA that adds up the slabs beside the scan: groups of four warps take the tiles in the order in which the scan reaches them
 // and wait for all slabs of a tile to be stored. (These CTAs come last in the grid and the scan never waits for them.) One SM
-// gets 45 GB/s of rows through this; a ring filled by bulk copies did not help (the copies alone, without the sums, ran at 35).
+// gets 47 GB/s of rows through this; a ring filled by bulk copies did not help (the copies alone, without the sums, ran at 35).
 template <int DV>
 __device__ void sum_tiles(const MainParams &p)
 {
@@ -1531,14 +1531,14 @@ void tensor_make_layout(darkattn_plan_s *plan)
     Y.zq = take(off, D.causal ? 0 : BH * m * 4);
     Y.sv = take(off, BH * N * 8);
     Y.zc = take(off, D.causal ? BH * (size_t)Y.T * m * 4 : 0);
-    // The causal scan may leave SMs idle, which can add up the slabs meanwhile: 45 GB/s of rows read and written per SM, against
-    // 4.4 us (d 64) or 5.2 us (d 128) for a chunk of the scan; of every segment as many chunks as they manage in that time, less
-    // a tenth. Not for short scans, whose last tiles would be waited for, nor where they would sum less than a fifth.
+    // The causal scan may leave SMs idle, which can add up the slabs meanwhile: 47 GB/s of rows read and written per SM, against
+    // 4.4 us (d 64) or 5.2 us (d 128) for a chunk of the scan; of every segment as many chunks as they manage in that time
+    // (4 x 16 heads, 8192 tokens, d 128: 465, 441, 430, 440 us with 0.53, 0.86, 1.0, 1.15 of that), and not many more CTAs than it takes. Not for short scans, whose last tiles would be waited for, nor where they would sum less than a fifth.
     const long long scan_ctas = units * nsplit, idle = 148 - scan_ctas;
     Y.summers = Y.cut = 0;
     if (D.causal && Y.T / nsplit >= 8 && idle > 0) {
-        const double part = 0.9 * idle * 45e3 * (d == 64 ? 4.4 : 5.2) / ((double)BH * nsplit * (Y.nslab + 1) * 256.0 * dv);
-        if (part >= 1.0) { Y.cut = (Y.T + nsplit - 1) / nsplit; Y.summers = (int)(idle / part) + 1; }
+        const double part = idle * 47e3 * (d == 64 ? 4.4 : 5.2) / ((double)BH * nsplit * (Y.nslab + 1) * 256.0 * dv);
+        if (part >= 1.0) { Y.cut = (Y.T + nsplit - 1) / nsplit; Y.summers = (int)(part > 1.6 ? idle * 1.6 / part : idle); if (Y.summers < 1) Y.summers = 1; }
         else if (part >= 0.2) { Y.cut = (int)(part * (Y.T / nsplit)); Y.summers = (int)idle; }
     }
     plan->launches_fwd = (D.causal ? (nsplit > 1 ? 6 : 4) : 6) - (Y.cut >= (Y.T + nsplit - 1) / nsplit ? 1 : 0);
