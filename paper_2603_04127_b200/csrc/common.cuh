@@ -17,9 +17,6 @@ struct Dims {
     int BH;          // B * H
     int Hkv, G;      // key/value heads and query heads per key/value head (H = Hkv * G)
     int C;           // causal chunk length
-    int nc;          // number of chunks = ceil(N / C)   (1 when not causal)
-    int Npad;        // nc * C when causal, else N
-    int dva;         // dv + 1: values with a ones column appended (its sums are the normaliser)
     int causal;
     int bf16;        // storage type of the tensors is bf16
     int w_per_head;

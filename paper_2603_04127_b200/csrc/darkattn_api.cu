@@ -78,9 +78,6 @@ darkattn_status_t darkattn_plan(const darkattn_desc_t *desc, darkattn_plan_t *ou
     D.Hkv = ds.H_kv; D.G = ds.H / ds.H_kv;
     D.causal = ds.causal ? 1 : 0;
     D.C = D.causal ? ds.chunk : ds.N;
-    D.nc = D.causal ? (ds.N + D.C - 1) / D.C : 1;
-    D.Npad = D.causal ? D.nc * D.C : ds.N;
-    D.dva = ds.dv + 1;
     D.bf16 = ds.dtype == DARKATTN_BF16;
     D.w_per_head = ds.w_per_head ? 1 : 0;
     D.s = sqrtf(ds.scale);
