@@ -151,7 +151,7 @@ __device__ __forceinline__ void apply(const Prob &P, const Tile &t, float (&acc)
         break;
     case EPI_COLMAX: {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) acc[j] = live ? acc[j] - rowv : -INFINITY;
+        for (int j = 0; j < 32; ++j) acc[j] = live ? fmaxf(acc[j] - rowv, -INFINITY) : -INFINITY;        // (NaN: a key that is not a number leaves the other keys' shift alone)
         // maxima over the warp's rows: halve the columns and the lanes that hold them in turn; lane l ends with column l
 #pragma unroll
         for (int o = 16; o; o >>= 1) {

@@ -88,6 +88,22 @@ def test_fp32_products_at_tile_edges(binding, i, dtype):
     _compare(got, want, TOL[dtype], f"split{i}")
 
 
+@pytest.mark.parametrize("m", [128, 200])
+@pytest.mark.parametrize("dtype,N", [("f32", 500), ("bf16", 500), ("bf16", 512)])
+def test_keys_that_are_not_numbers_leave_the_rows_before_them_alone(binding, dtype, N, m):
+    """A padded batch whose padding is uninitialised: with the causal mask no row before it depends on it. (Whole tiles of such
+    keys; the chunk of the first of them may mix in 0 * NaN.)"""
+    m = 256 if N % 128 == 0 and m % 128 else m      # (the tensor-core kernels' multiples)
+    wl = inputs.small(name="nanpad", wid=37, B=1, H=2, N=N, d=64, m=m, causal=True, dtype=dtype, backward=False)
+    t = inputs.generate(wl)
+    want = _oracle(t, wl)["O"][:, :, :256]
+    t.K[:, :, 256:] = np.nan
+    t.V[:, :, 256:] = np.nan
+    plan_path = binding.PATH_TENSOR if N % 128 == 0 else binding.PATH_SIMT
+    got = run_gpu(binding, wl, t, path=plan_path, want_ok=N % 128 != 0)["O"][:, :, :256]
+    assert_close(got, want, TOL[dtype], "nanpad")
+
+
 @pytest.mark.parametrize("chunk", [16, 64, 256])
 def test_chunk_length_does_not_change_the_result(binding, chunk):
     wl = inputs.small(name="chunks", wid=31, B=1, H=2, N=300, d=32, m=64, causal=True, dtype="f32")
