@@ -338,16 +338,6 @@ __device__ __forceinline__ void sub2(float &u0, float &u1, float n0, float n1, f
         "mov.b64 {%0, %1}, a;\n\t}"
         : "+f"(u0), "+f"(u1) : "f"(n0), "f"(n1), "f"(c), "f"(-1.f));
 }
-__device__ __forceinline__ void add2(float &a0, float &a1, float b0, float b1)
-{
-    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tadd.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
-        : "+f"(a0), "+f"(a1) : "f"(b0), "f"(b1));
-}
-__device__ __forceinline__ void fma2(float &a0, float &a1, float b0, float b1, float c0, float c1)
-{
-    asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tmov.b64 c, {%4, %5};\n\tfma.rn.f32x2 a, b, c, a;\n\tmov.b64 {%0, %1}, a;\n\t}"
-        : "+f"(a0), "+f"(a1) : "f"(b0), "f"(b1), "f"(c0), "f"(c1));
-}
 // 32 rows of the output by one warp: O[row,:] = sum_s num_s[row,:] 2^(rho_s - rho) / sum_s den_s 2^(rho_s - rho),
 // rho = max_s rho_s; den_s is the sum of the slab's four partial normalisers. Lane l forms row l's weights; DV / 8 lanes read a
 // row, 16 bytes each. The partial rows were written by other SMs a moment ago and come out of L2 (__ldcg: never from this SM's

@@ -143,6 +143,20 @@ def test_large_norm_inputs_stay_finite(binding, case):
     _compare(got, _oracle(t, wl), tol, case)
 
 
+@pytest.mark.parametrize("m", [64, 200])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_causal_prefixes_of_keys_far_below_the_largest(binding, dtype, m):
+    """The first keys' features lie up to 2^-150 below those of the sequence's largest keys, the shift's, and are all that the
+    first rows see. Forward and backward on the FP32 path; the bar of the large norms above (exponents 25 times larger)."""
+    wl = inputs.small(name="prefixes", wid=34, B=1, H=4, N=300, d=64, m=m, causal=True, dtype=dtype, backward=True)
+    t = inputs.generate(wl)
+    t.Q, t.K = t.Q * 5.0, t.K * 5.0
+    if dtype == "bf16":
+        t.Q, t.K = (inputs.round_to_bf16(x).astype(np.float64) for x in (t.Q, t.K))
+    got = run_gpu(binding, wl, t, path=binding.PATH_SIMT)
+    _compare(got, _oracle(t, wl), 5e-4 if dtype == "f32" else TOL[dtype], "prefixes")
+
+
 FULL = {
     # workload -> (b, h) pairs checked against the oracle at full sequence length
     "c2": [(0, 0), (3, 7), (7, 11)],
