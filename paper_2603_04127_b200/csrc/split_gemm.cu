@@ -227,10 +227,13 @@ __device__ __forceinline__ void apply(const Prob &P, const Tile &t, float (&acc)
         break;
     case EPI_DIVIDE: {
         const float inv = 1.f / den;
-        if (den > 1e-30f) {                         // quotients: the product with the reciprocal, corrected by the remainder
+        float f0 = 0.f, f1 = 0.f;
+#pragma unroll
+        for (int j = 0; j < 32; j += 2) fma2(f0, f1, acc[j], acc[j + 1], 0.f, 0.f);
+        if (den > 1e-30f && f0 + f1 == 0.f) {       // quotients: the product with the reciprocal, corrected by the remainder
 #pragma unroll
             for (int j = 0; j < 32; ++j) { const float q = acc[j] * inv; acc[j] = fmaf(fmaf(-q, den, acc[j]), inv, q); }
-        } else {                                    // (where the reciprocal may overflow)
+        } else {                                    // (where the reciprocal may overflow, or a numerator is infinite)
 #pragma unroll 1
             for (int j = 0; j < 32; ++j) {
                 const float q = acc[0] / den;
@@ -495,12 +498,14 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
                     tmem_ld32(taddr + (unit & 1) * 256, v);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) acc[j] += __uint_as_float(v[j]);
+                    for (int j = 0; j < 32; j += 2) add2(acc[j], acc[j + 1], __uint_as_float(v[j]), __uint_as_float(v[j + 1]));
                     if (small) {
                         tmem_ld32(taddr + (unit & 1) * 256 + 128, v);
                         tmem_wait_ld();
+                        // The parts of an infinite value are inf, NaN and NaN: where the large products are infinite they decide alone
+                        // (with the check kept to products of values 382 us at 2 x 16 heads of 2001 tokens, d 128, m 256, for all 379)
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) acc[j] += __uint_as_float(v[j]);
+                        for (int j = 0; j < 32; ++j) if (fabsf(acc[j]) < INFINITY) acc[j] += __uint_as_float(v[j]);
                     }
                 }
                 tc_fence_before();

@@ -143,6 +143,25 @@ def test_large_norm_inputs_stay_finite(binding, case):
     _compare(got, _oracle(t, wl), tol, case)
 
 
+@pytest.mark.parametrize("causal", [True, False], ids=["causal", "noncausal"])
+@pytest.mark.parametrize("dtype,m", [("f32", 64), ("f32", 200), ("bf16", 200)])
+def test_an_infinite_value_stays_infinite(binding, dtype, m, causal):
+    """One infinite element of V: its column of O is infinite in every row that attends to it, and nothing else changes."""
+    wl = inputs.small(name="infv", wid=38, B=1, H=2, N=300, d=64, m=m, causal=causal, dtype=dtype, backward=False)
+    t = inputs.generate(wl)
+    want = _oracle(t, wl)["O"]
+    t.V[:, :, 130, 3] = -np.inf
+    got = run_gpu(binding, wl, t, path=binding.PATH_SIMT)["O"]
+    first = 130 if causal else 0
+    assert (got[:, :, first:, 3] == -np.inf).all()
+    rest = np.ones(64, bool)
+    rest[3] = False
+    assert_close(got[..., rest], want[..., rest], TOL[dtype], "infv")
+    before = 128 if causal else 0                   # (the rows before it in its own chunk may mix in 0 * inf)
+    if before:
+        assert_close(got[:, :, :before, 3], want[:, :, :before, 3], TOL[dtype], "infv before")
+
+
 @pytest.mark.parametrize("m", [64, 200])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_causal_prefixes_of_keys_far_below_the_largest(binding, dtype, m):
