@@ -326,6 +326,47 @@ def test_gradient_of_the_projection_rows(binding, case):
     assert_close(got["dW"], want, TOL[wl.dtype], f"{case}: dW")
 
 
+def test_gradient_of_the_projection_rows_costs_a_step_what_it_costs_alone(binding):
+    """Behind the sums over grouped heads the kernel's blocks once crowded onto a few SMs and took 4.8 times as long there as
+    alone (measured 1.0 without; the bar lies between)."""
+    import torch
+    B, H, Hkv, N, d, m = 4, 16, 4, 2048, 64, 256
+    g = torch.Generator(device="cuda").manual_seed(3)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda").bfloat16()
+    Q, K, V, dO, M, W = rnd(B, H, N, d), rnd(B, Hkv, N, d), rnd(B, Hkv, N, d), rnd(B, H, N, d), 0.1 * rnd(H, d, d), rnd(m, d)
+    plan = binding.darkattn_plan(B, H, N, d, m, causal=True, H_kv=Hkv)
+    ws, saved = plan.alloc_workspace(), torch.empty(plan.saved_bytes, dtype=torch.uint8, device="cuda")
+    O, dQ, dK, dV = (torch.empty_like(x) for x in (Q, Q, K, V))
+    dM, dW = torch.empty(H, d, d, device="cuda"), torch.empty(m, d, device="cuda")
+
+    def step(with_dw):
+        binding.darkattn_forward(plan, Q, K, V, M, W, O, ws, saved=saved)
+        binding.darkattn_backward(plan, Q, K, V, M, W, O, dO, dQ, dK, dV, dM, ws, saved=saved)
+        if with_dw:
+            alone()
+
+    def alone():
+        binding.darkattn_backward_dw(plan, M, dW, ws)
+
+    def micros(f, n=30):
+        best = float("inf")
+        for _ in range(4):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(n):
+                f()
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1) * 1e3 / n)
+        return best
+
+    step(True)
+    extra, own = micros(lambda: step(True)) - micros(lambda: step(False)), micros(alone)
+    print(f"dW: {extra:.1f} us in a step, {own:.1f} us alone")
+    assert extra < 2.5 * own
+    plan.destroy()
+
+
 DECODE = [
     ("few_heads", dict(B=2, H=3, N=40, d=32, m=96, r=16, dv=64)),
     # several thousand (batch, head) pairs: more blocks than one wave of the GPU holds
