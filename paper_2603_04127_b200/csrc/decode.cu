@@ -24,6 +24,9 @@ namespace {
 
 constexpr int kNT = 256, kWarps = kNT / 32, kGroups = kNT / 8;      // kGroups: rows of M or W in work at a time, eight lanes each
 constexpr int kItems = 8, kSlots = 2;                               // 16-byte pieces per lane and slot, slots per warp
+constexpr int kRingBytes = kWarps * kSlots * kItems * 32 * 16, kMaxParts = 4, kMaxDv = 512;
+constexpr size_t kMaxVectors = 48 * 1024;                           // what a call may need for q, k, x~ and the features
+constexpr int kMaxSmem = kRingBytes + (int)kMaxVectors + kMaxParts * (kMaxDv + 2) * 4;
 
 template <typename T>
 __device__ __forceinline__ float ldf(const T *p, size_t i)
@@ -313,9 +316,10 @@ __global__ void __launch_bounds__(kNT, 3) decode_step_kernel(const __grid_consta
 template <typename T>
 cudaError_t launch_decode(const DecodeParams &P, int BH, cudaStream_t st)
 {
-    const size_t smem = ((size_t)kWarps * kSlots * kItems * 32 * 4 + 2 * P.d + 2 * P.r + 2 * P.mp + 2 * kWarps + (size_t)P.parts * (P.dv + 2)) * sizeof(float);
+    const size_t smem = kRingBytes + (2 * P.d + 2 * P.r + 2 * P.mp + 2 * kWarps + (size_t)P.parts * (P.dv + 2)) * sizeof(float);
     auto *k = P.dv <= 128 ? decode_step_kernel<T, 1> : P.dv <= 256 ? decode_step_kernel<T, 2> : decode_step_kernel<T, 4>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // One limit for all plans of a kernel, set once: another thread's plan must not lower it between this and the launch below.
+    const cudaError_t e = allow_smem(reinterpret_cast<const void *>(k), kMaxSmem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)BH * P.parts); cfg.blockDim = dim3(kNT); cfg.dynamicSmemBytes = smem; cfg.stream = st;
@@ -342,11 +346,11 @@ extern "C" darkattn_status_t darkattn_decode_step(darkattn_plan_t plan, const vo
     const Dims &D = plan->dims;
     if (!D.causal) return DARKATTN_ERR_UNSUPPORTED;          // the recurrent form is the causal one
     if (D.dv % 32) return DARKATTN_ERR_UNSUPPORTED;
-    if (D.dv > 512) return DARKATTN_ERR_UNSUPPORTED;
-    if ((size_t)(2 * D.d + 2 * D.r + 2 * D.m + 2048 + 16) * sizeof(float) > 48 * 1024) return DARKATTN_ERR_UNSUPPORTED;
+    if (D.dv > kMaxDv) return DARKATTN_ERR_UNSUPPORTED;
+    if ((size_t)(2 * D.d + 2 * D.r + 2 * D.m + 2048 + 16) * sizeof(float) > kMaxVectors) return DARKATTN_ERR_UNSUPPORTED;
     // CTAs per (batch, head): enough to give most SMs one while the pairs are few (64 pairs of m = 256, dv = 128: 10.2 us with
     // one CTA each, 8.3 with two, 10.5 with four, whose x~ is formed four times); at least 32 features each.
-    int parts = D.BH <= 37 ? 4 : D.BH < 148 ? 2 : 1;
+    int parts = D.BH <= 37 ? kMaxParts : D.BH < 148 ? 2 : 1;
     while (parts > 1 && D.m < 32 * parts) parts /= 2;
     DecodeParams P{q, k, v, M, W, S, z, o, D.H, D.Hkv, D.d, D.r, D.m, D.dv, D.w_per_head, 0, 0, D.s};
     P.mp = (D.m + parts - 1) / parts;

@@ -420,6 +420,53 @@ def test_decode_steps_in_parts(binding, name, kw, dtype):
     test_decode_steps_reproduce_the_causal_forward(binding, name, kw, dtype)
 
 
+def test_decode_steps_of_two_plans_in_two_threads(binding):
+    """Two host threads, each with a stream and a plan of its own whose kernel is the same and whose shared memory differs: no
+    step of one is refused because of the other, and the states come out as step by step in one thread."""
+    import sys
+    import threading
+    import torch
+    shapes, steps = ((1, 4, 64, 64, 64), (1, 4, 256, 2048, 128)), 6000
+    g = torch.Generator(device="cuda").manual_seed(4)
+    rnd = lambda *s: (0.3 * torch.randn(*s, generator=g, device="cuda")).bfloat16()
+    calls, want = [], []
+    for B, H, d, m, dv in shapes:
+        plan = binding.darkattn_plan(B, H, 1, d, m, dv=dv, causal=True)
+        args = [rnd(B, H, d), rnd(B, H, d), rnd(B, H, dv), rnd(H, d, d), rnd(m, d)]
+        state = [torch.zeros(B, H, m, dv, device="cuda"), torch.zeros(B, H, m, device="cuda"), torch.empty(B, H, dv, dtype=torch.bfloat16, device="cuda")]
+        for _ in range(steps):
+            binding.darkattn_decode_step(plan, *args, *state)
+        want.append([x.clone() for x in state])
+        for x in state:
+            x.zero_()
+        calls.append((plan, args, state, torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    errors = []
+
+    def work(plan, args, state, stream):
+        try:
+            for _ in range(steps):
+                binding.darkattn_decode_step(plan, *args, *state, stream=stream)
+        except Exception as e:
+            errors.append(e)
+
+    interval = sys.getswitchinterval()
+    sys.setswitchinterval(1e-5)
+    try:
+        threads = [threading.Thread(target=work, args=c) for c in calls]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+    finally:
+        sys.setswitchinterval(interval)
+    torch.cuda.synchronize()
+    assert not errors, errors
+    for (plan, _, state, _), w in zip(calls, want):
+        assert all(torch.equal(x, y) for x, y in zip(state, w))
+        plan.destroy()
+
+
 @pytest.mark.parametrize("name", ["headline", "headline_nc"])
 def test_headline_backward_sampled_heads(binding, name):
     """Forward + backward at the benchmark's full size; dQ, dK, dV of sampled (batch, head) pairs and
