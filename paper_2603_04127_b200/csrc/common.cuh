@@ -221,6 +221,8 @@ cudaError_t allow_smem(const void *kernel, int bytes);
 
 // Launches a kernel that begins with griddepcontrol.wait (all its memory accesses come after that): it may start while the
 // kernel before it in the stream drains, so that its launch and its prologue cost nothing.
+// A kernel that takes tensor memory has it before it lets its dependents start (pdl_wait): a dependent that got an SM's tensor
+// memory first would wait for this kernel's end while a block of this kernel waited, without a time limit, for that memory.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, int smem, cudaStream_t st, const Args &...args)
 {

@@ -101,12 +101,13 @@ __global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_nc_kernel(const __gri
         *abort_flag = (smem_u32(smem) & 1023u) ? 1 : 0;
         fence_mbar_init();
     }
-    pdl_wait();
-    if (tid < 128) sVec[tid] = (KEYS ? p.rhot : p.zt)[(size_t)bh * p.m + slab * 128 + tid];
     if (warp == kEpiWarps) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_wait();
+    if (tid < 128) sVec[tid] = (KEYS ? p.rhot : p.zt)[(size_t)bh * p.m + slab * 128 + tid];
+    __syncthreads();
     const uint32_t tmem = *tmem_slot;
     int *status = p.status;
 

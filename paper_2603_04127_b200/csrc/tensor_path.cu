@@ -430,6 +430,7 @@ __device__ __forceinline__ void combine_rows32(const MainParams &p, long long ro
 template <int DV>
 __device__ void sum_tiles(const MainParams &p)
 {
+    pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, quarter = warp & 3;
     const int groups = (blockDim.x / 128) * (gridDim.x - p.scan_ctas), g0 = (blockIdx.x - p.scan_ctas) * (blockDim.x / 128) + warp / 4;
     if (warp / 4 >= blockDim.x / 128) return;
@@ -505,8 +506,7 @@ __global__ void __launch_bounds__(kCausalThreads, 1) tc_fwd_causal_kernel(const 
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + CNBARS + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5;
-    if (blockIdx.x >= p.scan_ctas) {
-        pdl_wait();
+    if (blockIdx.x >= p.scan_ctas) {                // (takes no tensor memory)
         sum_tiles<DV>(p);
         return;
     }
@@ -525,13 +525,13 @@ __global__ void __launch_bounds__(kCausalThreads, 1) tc_fwd_causal_kernel(const 
         *abort_flag = (smem_u32(smem) & 1023u) ? 1 : 0;
         fence_mbar_init();
     }
-    pdl_wait();
-    if (tid < 128) sZ[tid] = fresh ? 0.f : p.zseg[((size_t)bh * p.nsplit + seg) * p.m + slab * 128 + tid];
     if (warp == kEpiWarps) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_wait();
     const uint32_t tmem = *tmem_slot;
+    if (tid < 128) sZ[tid] = fresh ? 0.f : p.zseg[((size_t)bh * p.nsplit + seg) * p.m + slab * 128 + tid];      // (read after the barrier below)
     int *status = p.status;
     if (!fresh && warp < kEpiWarps) {      // the segment's prefix state into the fp32 accumulators in TMEM
         const int lane = tid & 31, q4 = warp & 3, col0 = (warp >> 2) * 32, r = q4 * 32 + lane;
@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(kCausalThreads, 1) tc_fwd_causal_kernel(const 
         }
         {       // z: the prefix into the first partial sum, zero into the three others (one per column group's warp)
             uint32_t v[16];
-            const uint32_t zv = (col0 == 0) ? __float_as_uint(sZ[r]) : 0u;
+            const uint32_t zv = (col0 == 0) ? __float_as_uint(p.zseg[srow]) : 0u;
 #pragma unroll
             for (int j = 0; j < 16; ++j) v[j] = zv;
             tmem_st16(lane_addr + kColZ + (col0 / 32) * 16, v);
