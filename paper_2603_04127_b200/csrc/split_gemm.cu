@@ -593,6 +593,7 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
             }
         }
     }
+    if (__syncthreads_or(!ok)) __nanosleep(200000);         // error path only: let copies and MMAs in flight drain
     tc_fence_before();
     __syncthreads();
     if (warp == kMmaWarp) tmem_dealloc(tmem, 512);

@@ -42,3 +42,9 @@ def test_tensor_memory_is_taken_before_dependents_may_start(file, name, body):
     trigger = re.search(r"pdl_wait\w*\(\)|griddepcontrol\.launch_dependents", body)
     if trigger:
         assert re.search(r"tmem_alloc\(.*__syncthreads\(\)", body[:trigger.start()], re.S), f"{file}: {name}"
+
+
+@pytest.mark.parametrize("file,name,body", TENSOR_MEMORY, ids=[k[1] for k in TENSOR_MEMORY])
+def test_a_kernel_that_gave_up_waits_for_its_copies(file, name, body):
+    """After a wait ran into its limit, loads into the block's shared memory may still be in flight: it sleeps before it ends."""
+    assert re.search(r"__nanosleep\(200000\);(?!.*\bmbar_).*tmem_dealloc\(", body, re.S), f"{file}: {name}"
