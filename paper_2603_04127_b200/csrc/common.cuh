@@ -244,6 +244,14 @@ __device__ __forceinline__ void pdl_wait()
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
 }
+// The same where TMA reads what the kernels before wrote with ordinary stores (folded projections, states, parts of fp32 numbers):
+// the wait makes those writes visible to this grid, but TMA goes through the async proxy, for which the PTX manual asks for a
+// fence between the two; an ordinary launch would imply it.
+__device__ __forceinline__ void pdl_wait_tma()
+{
+    pdl_wait();
+    asm volatile("fence.proxy.async;" ::: "memory");
+}
 #endif
 
 #define DARKATTN_CUDA_TRY(expr, where)                                   \

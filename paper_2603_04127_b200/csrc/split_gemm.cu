@@ -310,9 +310,7 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
     // 2400 cycles) run under the kernel before
     Tile t;
     decode(L, blockIdx.x, t);
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
-    asm volatile("fence.proxy.async;" ::: "memory");       // (what the kernels before wrote is read by TMA)
+    pdl_wait_tma();
     if (L.init) {
         if (blockIdx.x == 0 && tid == 0) *L.status = 0;
         for (int i = blockIdx.x * kNT + tid; i < L.init_n; i += gridDim.x * kNT) L.init[i] = (int)0x80000000u;

@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_q_kernel(const __grid
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_wait();
+    pdl_wait_tma();
     const uint32_t tmem = *tmem_slot;
     int *status = p.status;
 
@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_k_kernel(const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_wait();
+    pdl_wait_tma();
     const uint32_t tmem = *tmem_slot;
     int *status = p.status;
 
@@ -738,7 +738,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_finish_k_kernel(const __gr
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_wait();
+    pdl_wait_tma();
     const uint32_t tmem = *tmem_slot;
     constexpr uint32_t C1 = 0, C2 = 128, C3 = 256;
     if (*abort_flag) { if (tid == 0) atomicExch(p.status, (int)DARKATTN_ERR_CUDA); }

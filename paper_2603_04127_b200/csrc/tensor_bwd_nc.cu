@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_nc_kernel(const __gri
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_wait();
+    pdl_wait_tma();
     if (tid < 128) sVec[tid] = (KEYS ? p.rhot : p.zt)[(size_t)bh * p.m + slab * 128 + tid];
     __syncthreads();
     const uint32_t tmem = *tmem_slot;

@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(160, 1) tc_key_prepass_kernel(const __grid_con
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_wait();
+    pdl_wait_tma();
     const uint32_t tmem = *tmem_slot;
     constexpr uint32_t kColX = 0, kColU = 128;      // x~ at 0, U of the two slabs at 128 and 256
     if (*abort_flag) { if (tid == 0) atomicExch(p.status, (int)DARKATTN_ERR_CUDA); }
@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(kCausalThreads, 1) tc_fwd_causal_kernel(const 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_wait();
+    pdl_wait_tma();
     const uint32_t tmem = *tmem_slot;
     if (tid < 128) sZ[tid] = fresh ? 0.f : p.zseg[((size_t)bh * p.nsplit + seg) * p.m + slab * 128 + tid];      // (read after the barrier below)
     int *status = p.status;
@@ -910,7 +910,7 @@ __global__ void __launch_bounds__(kKeysThreads, 1) tc_fwd_keys_kernel(const __gr
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_wait();
+    pdl_wait_tma();
     const uint32_t tmem = *tmem_slot;
     int *status = p.status;
     PieceList list(p);
@@ -1136,7 +1136,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) tc_fwd_queries_kernel(const _
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_wait();
+    pdl_wait_tma();
     const uint32_t tmem = *tmem_slot;
     int *status = p.status;
     PieceList list(p);

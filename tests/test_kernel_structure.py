@@ -48,3 +48,14 @@ def test_tensor_memory_is_taken_before_dependents_may_start(file, name, body):
 def test_a_kernel_that_gave_up_waits_for_its_copies(file, name, body):
     """After a wait ran into its limit, loads into the block's shared memory may still be in flight: it sleeps before it ends."""
     assert re.search(r"__nanosleep\(200000\);(?!.*\bmbar_).*tmem_dealloc\(", body, re.S), f"{file}: {name}"
+
+
+TMA = [k for k in KERNELS if re.search(r"tma_load_\w+\(|bulk_load\(", k[2])]
+
+
+@pytest.mark.parametrize("file,name,body", TMA, ids=[k[1] for k in TMA])
+def test_tma_reads_behind_a_proxy_fence(file, name, body):
+    """What a kernel before wrote with ordinary stores is read by TMA only behind the fence that goes with the early start."""
+    wait = re.search(r"pdl_wait_tma\(\)", body)
+    assert wait and wait.start() < re.search(r"tma_load_\w+\(|bulk_load\(", body).start(), f"{file}: {name}"
+    assert not re.search(r"pdl_wait\(\)|griddepcontrol", body), f"{file}: {name}"
