@@ -184,7 +184,8 @@ darkattn_status_t darkattn_selftest_wait_limit(int32_t *device_status, double *s
  *
  *  - The caller still passes Q, K, V, M, W (inputs) and O (output), laid out as for darkattn_forward.
  *  - darkattn_static_scratch_needed(plan) tells how much of the array a plan would use (when all
- *    heads of the batch together need more than the array, they are computed one after the other). A plan that
+ *    heads of the batch together need more than the array, they are computed one after the other, or where one
+ *    head alone needs more, by kernels that need less memory and take longer). A plan that
  *    needs more than DARKATTN_STATIC_SCRATCH_BYTES is refused with DARKATTN_ERR_WORKSPACE before
  *    anything touches the GPU; use darkattn_forward with a workspace of your own for it.
  *  - The first call on each device looks up the array's device address (with that device current).

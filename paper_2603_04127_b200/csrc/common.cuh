@@ -53,6 +53,23 @@ struct SimtLayout {
     int nsM, nsW, blkM, blkW;      // token blocks of the dM and dW products, tokens in each
 };
 
+// Offsets (bytes) into the scratch of the FFMA kernels' intermediates, all fp32.
+struct FfmaLayout {
+    int C, nc, Npad;               // chunk length, chunks, nc * C  (not causal: one chunk of N)
+    int dva;                       // dv + 1: values with a ones column appended (its sums are the normaliser)
+    size_t status;                 // device status word (first 256 bytes)
+    size_t Qf, Kf, Vf, Mf, Wf;     // fp32 copies of bf16 inputs, and of shared K and V per query head
+    size_t xtQ, xtK;               // x~            [BH, N, r]
+    size_t nK;                     // |x~_K|^2 / 2  [BH, N]
+    size_t fQ, fK;                 // exponents, then features  [BH, Npad, m]
+    size_t cK;                     // per-feature key shift     [BH, m]
+    size_t Va;                     // [V | 1]       [BH, Npad, dva]
+    size_t Sloc;                   // chunk states, then exclusive prefixes [BH, nc, m, dva]
+    size_t P;                      // masked intra-chunk kernel  [BH, nc, C, C]   (causal)
+    size_t num;                    // numerators and normaliser  [BH, Npad, dva]
+    size_t fwd_bytes;
+};
+
 // Offsets (bytes) into the workspace of the tensor-core forward path.
 struct TensorLayout {
     size_t status;
@@ -147,6 +164,7 @@ struct darkattn_plan_s {
     darkattn::Dims dims;
     int path;                      // resolved DARKATTN_PATH_*
     darkattn::SimtLayout simt, simt_fwd;   // with the backward pass; forward pass alone
+    darkattn::FfmaLayout ffma;
     darkattn::TensorLayout tensor;
     size_t workspace_bytes;
     size_t saved_bytes;
@@ -182,6 +200,11 @@ darkattn_status_t simt_forward(const darkattn_plan_s *plan, const void *Q, const
 darkattn_status_t simt_backward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
                                 const void *M, const void *W, const void *dO, void *dQ, void *dK,
                                 void *dV, float *dM, char *ws, cudaStream_t st);
+
+// FP32 kernels without matrix instructions
+void ffma_make_layout(darkattn_plan_s *plan);
+darkattn_status_t ffma_forward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
+                               const void *M, const void *W, void *O, char *ws, cudaStream_t st);
 
 // Tensor-core (tcgen05 / TMEM / TMA) path, bf16 operands with fp32 accumulation
 bool tensor_supported(const darkattn_plan_s *plan);

@@ -89,6 +89,7 @@ darkattn_status_t darkattn_plan(const darkattn_desc_t *desc, darkattn_plan_t *ou
     p->path = path;
 
     simt_make_layout(p);
+    ffma_make_layout(p);
     p->workspace_bytes = p->simt.bytes > p->simt_fwd.bytes ? p->simt.bytes : p->simt_fwd.bytes;
     p->saved_bytes = 0;
     simt_launches(p, p->launches_fwd, p->launches_bwd);

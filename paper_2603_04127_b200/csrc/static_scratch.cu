@@ -46,6 +46,24 @@ void single_pair(const darkattn_plan_s *plan, darkattn_plan_s &one)
     simt_make_layout(&one);
 }
 
+// How a plan is run: all pairs at once where their intermediates fit the array, else one pair after the other, else by the FFMA
+// kernels, whose intermediates take 4 bytes an element instead of 6 and which read fp32 inputs as they are (long sequences of wide
+// queries: 5090 tokens of width 429 take 34 MB for one pair, 8 MB here).
+enum Mode { ALL_PAIRS, PAIR_BY_PAIR, FFMA, REFUSED };
+Mode choose(const darkattn_plan_s *plan, size_t &bytes)
+{
+    constexpr size_t room = DARKATTN_STATIC_SCRATCH_BYTES;
+    bytes = plan->simt_fwd.bytes;
+    if (bytes <= room) return ALL_PAIRS;
+    darkattn_plan_s one;
+    single_pair(plan, one);
+    bytes = one.simt_fwd.bytes;
+    if (bytes <= room) return PAIR_BY_PAIR;
+    if (plan->ffma.fwd_bytes > room) return REFUSED;
+    bytes = plan->ffma.fwd_bytes;
+    return FFMA;
+}
+
 }  // namespace
 }  // namespace darkattn
 
@@ -54,10 +72,9 @@ using namespace darkattn;
 extern "C" size_t darkattn_static_scratch_needed(darkattn_plan_t plan)
 {
     if (!plan) return 0;
-    if (plan->simt_fwd.bytes <= (size_t)DARKATTN_STATIC_SCRATCH_BYTES) return plan->simt_fwd.bytes;
-    darkattn_plan_s one;
-    single_pair(plan, one);
-    return one.simt_fwd.bytes;
+    size_t bytes = 0;
+    choose(plan, bytes);
+    return bytes;
 }
 
 extern "C" darkattn_status_t darkattn_forward_static(darkattn_plan_t plan, const void *Q, const void *K,
@@ -69,14 +86,17 @@ extern "C" darkattn_status_t darkattn_forward_static(darkattn_plan_t plan, const
     for (const void *p : ptrs)
         if (reinterpret_cast<uintptr_t>(p) & 15u) return DARKATTN_ERR_INVALID_ARG;
     // size check first: it needs no GPU, so a refusal never touches the device
-    if (darkattn_static_scratch_needed(plan) > (size_t)DARKATTN_STATIC_SCRATCH_BYTES) return DARKATTN_ERR_WORKSPACE;
+    size_t bytes = 0;
+    const Mode mode = choose(plan, bytes);
+    if (mode == REFUSED) return DARKATTN_ERR_WORKSPACE;
     char *scratch = nullptr;
     darkattn_status_t s = scratch_for_current_device(&scratch);
     if (s != DARKATTN_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     // the array still holds the previous call's data: the first kernel clears the status word and the per-feature maxima,
     // every other region is written by this call before it is read
-    if (plan->simt_fwd.bytes <= (size_t)DARKATTN_STATIC_SCRATCH_BYTES) return simt_forward(plan, Q, K, V, M, W, O, scratch, st);
+    if (mode == ALL_PAIRS) return simt_forward(plan, Q, K, V, M, W, O, scratch, st);
+    if (mode == FFMA) return ffma_forward(plan, Q, K, V, M, W, O, scratch, st);
     // pair by pair (heads are independent of one another)
     darkattn_plan_s one;
     single_pair(plan, one);

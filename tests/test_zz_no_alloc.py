@@ -92,3 +92,41 @@ def test_static_scratch_takes_the_heads_one_by_one(binding, dtype):
     torch.cuda.synchronize()
     assert torch.equal(got, want)
     plan.destroy()
+
+
+LEAN = [
+    # one pair's bf16 parts (6 bytes an element, inputs among them) need more than the array, its fp32 intermediates less
+    dict(B=1, H=1, N=5090, d=429, r=21, m=63, dv=121, causal=False),
+    dict(B=1, H=2, N=6923, d=406, r=43, m=86, dv=10, causal=False),
+    dict(B=1, H=1, N=3571, d=373, r=106, m=357, dv=11, causal=True),
+    dict(B=1, H=1, N=10509, d=116, m=22, dv=9, causal=True, chunk=16),
+]
+
+
+@pytest.mark.skipif(not _have_library(), reason="neither libdarkattn.so nor nvcc to build it")
+@pytest.mark.parametrize("i", range(len(LEAN)))
+def test_long_sequences_of_wide_queries_are_accepted(binding, i):
+    kw = dict(LEAN[i])
+    B, H, N, d, m = (kw.pop(k) for k in ("B", "H", "N", "d", "m"))
+    plan = binding.darkattn_plan(B, H, N, d, m, dtype=binding.F32, **kw)
+    assert 0 < binding.darkattn_static_scratch_needed(plan) <= binding.STATIC_SCRATCH_BYTES // 2
+    plan.destroy()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("i", range(len(LEAN)))
+def test_static_scratch_forward_of_long_sequences(binding, i):
+    kw = dict(LEAN[i])
+    chunk = kw.pop("chunk", 0)
+    wl = inputs.small(name="noalloc_lean", wid=43 + i, dtype="f32", backward=False, **kw)
+    t = inputs.generate(wl)
+    Q, K, V, M, W = (to_dev(x, torch.float32) for x in (t.Q, t.K, t.V, t.M, t.W))
+    plan = binding.darkattn_plan(wl.B, wl.H, wl.N, wl.d, wl.m, r=wl.r, dv=wl.dv, dtype=binding.F32, causal=wl.causal, chunk=chunk)
+    got = torch.full((wl.B, wl.H, wl.N, wl.dv), float("nan"), device="cuda")
+    binding.darkattn_forward_static(plan, Q, K, V, M, W, got)
+    torch.cuda.synchronize()
+    from oracle import ref
+    want = ref.forward(t.Q, t.K, t.V, t.M, t.W, causal=wl.causal)
+    fro, mx = rel_errors(got.cpu().numpy().astype(np.float64), want)
+    assert fro < TOL["f32"] and mx < TOL["f32"], (fro, mx)
+    plan.destroy()
