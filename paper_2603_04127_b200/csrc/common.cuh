@@ -67,7 +67,19 @@ struct FfmaLayout {
     size_t Sloc;                   // chunk states, then exclusive prefixes [BH, nc, m, dva]
     size_t P;                      // masked intra-chunk kernel  [BH, nc, C, C]   (causal)
     size_t num;                    // numerators and normaliser  [BH, Npad, dva]
-    size_t fwd_bytes;
+    // backward only
+    size_t Gf;                     // fp32 copy of dO
+    size_t Ga;                     // [dO/den | -delta/den]      [BH, Npad, dva]
+    size_t dP;                     // [BH, nc, C, C]             (causal)
+    size_t Rloc;                   // reverse states             [BH, nc, m, dva]
+    size_t dA, dBf;                // feature gradients, then E  [BH, Npad, m]
+    size_t dVa;                    // [BH, Npad, dva]
+    size_t es;                     // rowsum(E) of one side      [BH, N]
+    size_t dxt;                    // dx~ of one side            [BH, N, r]
+    size_t dXf;                    // fp32 dX before the cast    [BH, N, d]
+    size_t dMp;                    // per-(b,h) dM               [BH, r, d]
+    size_t dWp;                    // per-(b,h) dW               [BH, m, r]
+    size_t fwd_bytes, total_bytes;
 };
 
 // Offsets (bytes) into the workspace of the tensor-core forward path.
@@ -165,6 +177,7 @@ struct darkattn_plan_s {
     int path;                      // resolved DARKATTN_PATH_*
     darkattn::SimtLayout simt, simt_fwd;   // with the backward pass; forward pass alone
     darkattn::FfmaLayout ffma;
+    bool ffma_fwd, ffma_bwd;       // which kernels an FP32 forward or backward call takes
     darkattn::TensorLayout tensor;
     size_t workspace_bytes;
     size_t saved_bytes;
@@ -194,6 +207,7 @@ void timer_mark(const darkattn_plan_s *plan, cudaStream_t st, const char *name);
 
 // FP32 path (products of split operands on the tensor cores)
 void simt_make_layout(darkattn_plan_s *plan);
+double simt_cost_us(const darkattn_plan_s *plan, bool backward);
 void simt_launches(const darkattn_plan_s *plan, int &fwd, int &bwd);     // kernels of a forward and of a backward call
 darkattn_status_t simt_forward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
                                const void *M, const void *W, void *O, char *ws, cudaStream_t st);
@@ -203,6 +217,12 @@ darkattn_status_t simt_backward(const darkattn_plan_s *plan, const void *Q, cons
 
 // FP32 kernels without matrix instructions
 void ffma_make_layout(darkattn_plan_s *plan);
+void ffma_launches(const darkattn_plan_s *plan, int &fwd, int &bwd);
+double ffma_cost_us(const darkattn_plan_s *plan, bool backward);
+darkattn_status_t ffma_backward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
+                                const void *M, const void *W, const void *dO, void *dQ, void *dK,
+                                void *dV, float *dM, char *ws, cudaStream_t st);
+darkattn_status_t ffma_backward_dw(const darkattn_plan_s *plan, float *dW, char *ws, cudaStream_t st);
 darkattn_status_t ffma_forward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
                                const void *M, const void *W, void *O, char *ws, cudaStream_t st);
 

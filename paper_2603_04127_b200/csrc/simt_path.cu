@@ -477,6 +477,30 @@ void simt_launches(const darkattn_plan_s *plan, int &fwd, int &bwd)
     bwd = fwd + 1 + scan + 4 + (D.G > 1 ? 2 : 0);
 }
 
+// Estimated time in us of a call that fills the SMs: launches one after the other, then per pair the 128 x 128 tiles of all products
+// (start and read-out, stages of 64 of the contraction; four fifths of a stage where the inputs are bf16). Fitted like ffma_cost_us.
+double simt_cost_us(const darkattn_plan_s *plan, bool backward)
+{
+    const Dims &D = plan->dims;
+    const double N = D.N, d = D.d, r = D.r, m = D.m, dv = D.dv, nb = tiles(D.N), more = nb > 1 ? 1 : 0;
+    double count = 0, stages = 0;
+    auto product = [&](double M, double Nn, double K, double times = 1) {
+        const double t = times * ceil(M / 128) * ceil(Nn / 128);
+        count += t;
+        stages += t * ceil(K / 64);
+    };
+    product(N, r, d, 2); product(N, m, r, 3 + (tiles(D.m) > 1 ? 1 : 0));
+    if (D.causal) { product(128, 128, m, nb); product(m, dv, 128, more * nb); product(128, dv, 128 + more * m, nb); }
+    else { product(m, dv, N); product(N, dv, m); }
+    if (backward) {
+        if (D.causal) { product(128, 128, dv, nb); product(m, dv, 128, more * nb); product(128, m, 128 + more * dv, 2 * nb); product(128, dv, 128 + more * m, nb); }
+        else { product(m, dv, N); product(N, m, dv, 2); product(N, dv, m); }
+        product(N, r, m, 2); product(N, d, r, 2); product(r, d, 2 * N);
+    }
+    const double parts = D.bf16 ? 0.8 : 1.0;
+    return backward ? 52 + D.BH * (9.2e-3 * count + 2.04e-2 * parts * stages) : 35 + D.BH * (1.7e-2 * count + 1.48e-2 * parts * stages);
+}
+
 darkattn_status_t simt_forward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
                                const void *M, const void *W, void *O, char *ws, cudaStream_t st)
 {

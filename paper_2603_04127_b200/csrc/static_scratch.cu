@@ -53,6 +53,8 @@ enum Mode { ALL_PAIRS, PAIR_BY_PAIR, FFMA, REFUSED };
 Mode choose(const darkattn_plan_s *plan, size_t &bytes)
 {
     constexpr size_t room = DARKATTN_STATIC_SCRATCH_BYTES;
+    bytes = plan->ffma.fwd_bytes;
+    if (plan->ffma_fwd && bytes <= room) return FFMA;
     bytes = plan->simt_fwd.bytes;
     if (bytes <= room) return ALL_PAIRS;
     darkattn_plan_s one;

@@ -104,6 +104,61 @@ def test_keys_that_are_not_numbers_leave_the_rows_before_them_alone(binding, dty
     assert_close(got, want, TOL[dtype], "nanpad")
 
 
+# Many short sequences, which the FFMA kernels take: one token, a last chunk of one, widths beside their 64-wide tiles, grouped heads.
+SHORT = [
+    dict(B=150, H=4, N=1, d=8, m=16, causal=False),
+    dict(B=150, H=4, N=9, d=16, m=24, r=12, dv=20, causal=False, Hkv=2),
+    dict(B=300, H=5, N=17, d=16, m=33, r=12, dv=20, causal=True),
+    dict(B=300, H=8, N=33, d=16, m=16, causal=True, chunk=16, Hkv=2),
+    dict(B=200, H=5, N=65, d=16, m=16, causal=False),
+]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("i", range(len(SHORT)))
+def test_many_short_sequences(binding, i, dtype):
+    kw = dict(SHORT[i])
+    chunk, Hkv = kw.pop("chunk", 0), kw.pop("Hkv", kw["H"])
+    plan = binding.darkattn_plan(kw["B"], kw["H"], kw["N"], kw["d"], kw["m"], r=kw.get("r", 0), dv=kw.get("dv", 0), causal=kw["causal"], chunk=chunk,
+                                 H_kv=Hkv, dtype=binding.F32 if dtype == "f32" else binding.BF16, path=binding.PATH_SIMT)
+    assert dtype == "bf16" or (plan.launches() >= 13 and plan.launches(True) >= 26)       # (the products on the tensor cores take 8 and 14 at most)
+    plan.destroy()
+    wl = inputs.small(name=f"short{i}", wid=460 + i, dtype=dtype, backward=True, **kw)
+    t = inputs.generate(wl)
+    G = wl.H // Hkv
+    t.K, t.V = np.ascontiguousarray(t.K[:, ::G]), np.ascontiguousarray(t.V[:, ::G])
+    got = run_gpu(binding, wl, t, path=binding.PATH_SIMT, chunk=chunk, want_dw=True)
+    want = _oracle(t, wl)
+    want["dW"] = ref.backward(t.Q, t.K, t.V, t.M, t.W, t.dO, causal=wl.causal)[4]
+    if wl.N == 1:               # O_0 = V_0 whatever Q, K, M and W are: those gradients are exactly zero (dM and dW sum 600 pairs' rounding)
+        for k in ("dQ", "dK", "dM", "dW"):
+            assert np.abs(want.pop(k)).max() < 1e-12 and np.abs(got[k]).max() < TOL[dtype]
+    _compare(got, want, TOL[dtype], f"short{i}")
+
+
+def test_a_short_sequence_costs_less_than_a_tile(binding):
+    """8192 pairs of 8 tokens take well under what as many of 128 take (0.3 of it; on tiles of 128 tokens they took 1.1 of it)."""
+    import torch
+    times = []
+    for N in (8, 128):
+        Q, K, V, W = (torch.randn(*s, device="cuda") for s in ((256, 32, N, 16), (256, 32, N, 16), (256, 32, N, 16), (16, 16)))
+        M, O = 0.3 * torch.randn(32, 16, 16, device="cuda"), torch.empty_like(V)
+        plan = binding.darkattn_plan(256, 32, N, 16, 16, dtype=binding.F32)
+        ws = plan.alloc_workspace()
+        best = float("inf")
+        for _ in range(4):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(10):
+                binding.darkattn_forward(plan, Q, K, V, M, W, O, ws)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        times.append(best)
+        plan.destroy()
+    assert times[0] < 0.6 * times[1], times
+
+
 @pytest.mark.parametrize("chunk", [16, 64, 256])
 def test_chunk_length_does_not_change_the_result(binding, chunk):
     wl = inputs.small(name="chunks", wid=31, B=1, H=2, N=300, d=32, m=64, causal=True, dtype="f32")
