@@ -57,7 +57,8 @@ typedef enum { DARKATTN_F32 = 0, DARKATTN_BF16 = 1 } darkattn_dtype_t;
  *   SIMT   : FP32 operands and FP32 accumulation (any shape; the only path that meets the 1e-4
  *            tolerance, because a single TF32/BF16 operand rounds the exponent's argument). Its
  *            products run on the tensor cores with every FP32 operand split exactly into three BF16
- *            parts, everything else on the FP32 pipes.
+ *            parts, everything else on the FP32 pipes (many short sequences: all on the FP32 pipes).
+ *            Elements below 1e-33 in magnitude lose digits, as their smallest part is below BF16's range.
  *   TENSOR : tcgen05 / TMEM / TMA kernels, BF16 operands, FP32 accumulation (BF16 dtype only;
  *            DARKATTN_ERR_UNSUPPORTED at plan time if the shape is not covered).               */
 typedef enum { DARKATTN_PATH_AUTO = 0, DARKATTN_PATH_SIMT = 1, DARKATTN_PATH_TENSOR = 2 } darkattn_path_t;
@@ -70,7 +71,9 @@ typedef struct {
     int32_t dv;           /* value width; 0 means dv = d                                           */
     int32_t dtype;        /* darkattn_dtype_t of Q,K,V,M,W,O,dO,dQ,dK,dV                            */
     int32_t causal;       /* 0: every key; 1: keys j <= i                                          */
-    int32_t chunk;        /* causal chunk length of the prefix scan; 0 means 128                   */
+    int32_t chunk;        /* causal chunk length of the prefix scan; 0 means 128. The result does not depend on it.
+                             The TENSOR path has chunks of 128 only; the FP32 path's products on the tensor cores
+                             always take 128, its FFMA kernels (many short sequences) the length given here   */
     float   scale;        /* multiplies q^T Sigma k; 0 means 1/sqrt(d) (Section 2 footnote: the
                              scaling is absorbed symmetrically, sqrt(scale) into Mq and into Mk)   */
     int32_t w_per_head;   /* 0: W [m,r] shared by all heads; 1: W [H,m,r]                          */
@@ -111,9 +114,9 @@ darkattn_status_t darkattn_forward(darkattn_plan_t plan, const void *Q, const vo
  * back-propagation, Section 4; the formulas follow from the chain rule through the definitions at
  * the top of this file, with every stabilising shift held constant, which is exact because O does
  * not depend on them). `O` is the forward result for the same inputs (may be NULL: recomputed).
- * On the tensor-core path part of the zeroing of dK and dV runs on a stream of the plan's own (created by the
- * first such call, non-blocking), forked from `cuda_stream` and joined back into it with events before the
- * call's later kernels: to the caller everything still happens in stream order on `cuda_stream`.           */
+ * On the tensor-core path the product that forms dM runs on a stream of the plan's own (created by the first such call,
+ * non-blocking) beside the kernel that finishes dK: forked from `cuda_stream` and joined back into it with events before the
+ * call's later kernels, so that to the caller everything still happens in stream order on `cuda_stream`.      */
 darkattn_status_t darkattn_backward(darkattn_plan_t plan, const void *Q, const void *K, const void *V,
                                     const void *M, const void *W, const void *O, const void *dO,
                                     const void *saved /* nullable */, void *dQ, void *dK, void *dV,

@@ -77,7 +77,7 @@ __device__ __forceinline__ float sum8(float v)
 // lanes share a row: lane `sub` of the eight takes every eighth 16-byte piece of it, so a warp's load covers four rows in
 // pieces of 128 contiguous bytes, and three shuffle steps add the eight parts up. put(row, d0, d1, nn) is called by all
 // eight lanes. PIECES > 0: rows of exactly 8 PIECES pieces; the lane's share of the vectors stays in registers and
-// the loads of 8 / PIECES rows are in flight together (a block is a chain of load latencies). PIECES = 0: any length, rows that
+// the loads of 8, 4 or (PIECES = 4: the registers) 1 rows are in flight together (a block is a chain of load latencies). PIECES = 0: any length, rows that
 // do not start on 16 bytes element by element.
 template <typename T, int PIECES, bool NORM, typename Put>
 __device__ __forceinline__ void rows_dots(const T *mat, int nrows, int n, const float *x0, const float *x1, int tid, Put put)
@@ -348,8 +348,10 @@ extern "C" darkattn_status_t darkattn_decode_step(darkattn_plan_t plan, const vo
     if (D.dv % 32) return DARKATTN_ERR_UNSUPPORTED;
     if (D.dv > kMaxDv) return DARKATTN_ERR_UNSUPPORTED;
     if ((size_t)(2 * D.d + 2 * D.r + 2 * D.m + 2048 + 16) * sizeof(float) > kMaxVectors) return DARKATTN_ERR_UNSUPPORTED;
-    // CTAs per (batch, head): enough to give most SMs one while the pairs are few (64 pairs of m = 256, dv = 128: 10.2 us with
-    // one CTA each, 8.3 with two, 10.5 with four, whose x~ is formed four times); at least 32 features each.
+    // CTAs per (batch, head): enough to give most SMs one while the pairs are few; at least 32 features each. In us with one, two and
+    // four, bf16, d = dv = 128: m = 256: 1 pair 9.8, 7.6, 6.7; 37 pairs 10.1, 8.2, 8.2; 64 pairs 10.3, 8.4, 10.6; 96 pairs 10.3, 10.4, 10.7; m = 1024:
+    // 64 pairs 25.2, 16.3, 19.9; 96 pairs 25.6, 23.5, 19.7; 147 pairs 33.6, 32.3, 36.6. From 75 pairs on two CTAs of some pairs share an SM,
+    // which pays for m = 1024 and not for less (m = 256, 147 pairs: 10.9, 13.9, 19.0; d = dv = 64, m = 128: 6.7, 8.3, 14.7); fp32 alike.
     int parts = D.BH <= 37 ? kMaxParts : D.BH < 148 ? 2 : 1;
     while (parts > 1 && D.m < 32 * parts) parts /= 2;
     DecodeParams P{q, k, v, M, W, S, z, o, D.H, D.Hkv, D.d, D.r, D.m, D.dv, D.w_per_head, 0, 0, D.s};

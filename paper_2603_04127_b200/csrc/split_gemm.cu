@@ -230,7 +230,8 @@ __device__ __forceinline__ void apply(const Prob &P, const Tile &t, float (&acc)
         float f0 = 0.f, f1 = 0.f;
 #pragma unroll
         for (int j = 0; j < 32; j += 2) fma2(f0, f1, acc[j], acc[j + 1], 0.f, 0.f);
-        if (den > 1e-30f && f0 + f1 == 0.f) {       // quotients: the product with the reciprocal, corrected by the remainder
+        if (den > 1e-30f && f0 + f1 == 0.f) {       // quotients: the product with the reciprocal, corrected once by the
+                                                    // remainder (Markstein, IBM J. Res. Dev. 34, 1990): within an ulp
 #pragma unroll
             for (int j = 0; j < 32; ++j) { const float q = acc[j] * inv; acc[j] = fmaf(fmaf(-q, den, acc[j]), inv, q); }
         } else {                                    // (where the reciprocal may overflow, or a numerator is infinite)
@@ -609,7 +610,8 @@ bool make_map4(CUtensorMap *map, const Mat &m, int box_rows, int box_planes)
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// n / d for n < 2^31 as (high word of n mul + n) >> shr
+// n / d for n < 2^31 as (high word of n mul + n) >> shr: division by an invariant with a rounded-up multiplier (Granlund and Montgomery,
+// PLDI 1994)
 FastDiv make_div(unsigned d)
 {
     FastDiv f;

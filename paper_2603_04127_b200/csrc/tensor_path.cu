@@ -284,11 +284,11 @@ struct MainParams {
 
 enum { MODE_CAUSAL = 0, MODE_KEYS = 1, MODE_QUERIES = 2 };
 
-// ------------------------------------------------------------------ forward scan kernels
-// All three use 16 epilogue warps (warp w: TMEM lanes 32 (w % 4) .. +31, columns 32 (w / 4) .. +31) and one
-// control warp whose first lane issues the TMA loads and the MMAs. phi(Q) and the masked kernel tile P are only
-// ever the A operand of an MMA whose rows are tokens, so they are packed to bf16 in tensor memory and read
-// by the MMA from there; phi(K) also serves transposed and as a B operand and goes to shared memory.
+// ------------------------------------------------------------------ causal forward kernel
+// 16 epilogue warps (warp w: TMEM lanes 32 (w % 4) .. +31, columns 32 (w / 4) .. +31), one control warp whose first lane issues
+// the TMA loads and the MMAs, and one that stores the output. phi(Q) and the masked kernel tile P are only ever the A operand of an
+// MMA whose rows are tokens, so they are packed to bf16 in tensor memory and read by the MMA from there; phi(K) also serves
+// transposed and as a B operand and goes to shared memory. (The passes over keys and queries further down have roles of their own.)
 
 __device__ __forceinline__ void store_row_f32x32_bf16(const uint32_t (&v)[32], unsigned char *tile, int row, int col0)
 {
@@ -298,8 +298,7 @@ __device__ __forceinline__ void store_row_f32x32_bf16(const uint32_t (&v)[32], u
 
 // phi(Q) of one row segment: row maximum over the slab's 128 features (exchanged with the three other warps
 // of the lane quarter through red[4][128]), 2^(u - max) packed to bf16 into TMEM columns fq + col0/2.
-// rmax receives the row maximum. WITH_Z: returns sum_l phi(Q)_l z_l over the segment (else 0).
-template <bool WITH_Z>
+// rmax receives the row maximum. Returns sum_l phi(Q)_l z_l over the segment.
 __device__ __forceinline__ float query_features_to_tmem(uint32_t u_addr, uint32_t fq_addr, float *red, const float *z, int q4,
                                                         int g, int r, int col0, float &rmax)
 {
@@ -316,11 +315,9 @@ __device__ __forceinline__ float query_features_to_tmem(uint32_t u_addr, uint32_
 #pragma unroll
     for (int j = 0; j < 32; j += 2) {
         const float f0 = ex2f(__uint_as_float(v[j]) - rmax), f1 = ex2f(__uint_as_float(v[j + 1]) - rmax);
-        if constexpr (WITH_Z) {
-            const float2 zz = *reinterpret_cast<const float2 *>(z + col0 + j);
-            dz = fmaf(f0, zz.x, dz);
-            dz = fmaf(f1, zz.y, dz);
-        }
+        const float2 zz = *reinterpret_cast<const float2 *>(z + col0 + j);
+        dz = fmaf(f0, zz.x, dz);
+        dz = fmaf(f1, zz.y, dz);
         pk[j / 2] = pack_bf16(f0, f1);
     }
     tmem_st16(fq_addr + col0 / 2, pk);
@@ -716,7 +713,7 @@ __global__ void __launch_bounds__(kCausalThreads, 1) tc_fwd_causal_kernel(const 
         float dz = 0.f;                             // phi(Q) z_prev over this thread's features, of the chunk whose phi(Q) was formed last
         auto query_features = [&]() {
             tc_fence_after();
-            dz = query_features_to_tmem<true>(R1, lane_addr + kColFQ, sRed, sZ, q4, g, r, col0, rmax);
+            dz = query_features_to_tmem(R1, lane_addr + kColFQ, sRed, sZ, q4, g, r, col0, rmax);
             tc_fence_before();
             mbar_arrive_warp(bars + CE0);
         };
@@ -885,7 +882,7 @@ enum KyBars { YB_OM, YB_OMF, YB_K, YB_V = YB_K + 4, YB_KF = YB_V + 4, YB_VF = YB
 // tensor memory holds three tiles: the projections run ahead and eight warps each work on the even and on the odd tiles, so
 // that the exponentials of one tile run under the waits, loads and stores of another (in lockstep on one tile a warp spent 1.0 k
 // of 2.3 k cycles on those). Bound by the exponentials (16384 per tile, 16 per clock and SM) at d = 64 and by MMA issue (24 per tile)
-// at d = 128. Encoder shape 8 x 12 heads, 4096 tokens, d 64, m 256: 101 -> 64 us; 4 x 16 heads, 8192 tokens, d 128: 138 -> 104 us.
+// at d = 128. Encoder shape 8 x 12 heads, 4096 tokens, d 64, m 256: 101 -> 51 us; 4 x 16 heads, 8192 tokens, d 128: 138 -> 88 us.
 template <int D, int DV>
 __global__ void __launch_bounds__(kKeysThreads, 1) tc_fwd_keys_kernel(const __grid_constant__ MainParams p)
 {
@@ -1112,7 +1109,7 @@ enum QyBars { UB_OM, UB_OMF, UB_Q, UB_QF = UB_Q + 4, UB_U = UB_QF + 4, UB_O = UB
 // exchange with another warp, and the groups work on different tiles (three or four in flight), so that one's exponentials
 // run under another's waits. Tensor memory: dv = 64: per group U (128 columns), phi(Q) packed into its first 64 in place, O into
 // the other 64; dv = 128: per group U and then O (128), phi(Q) in one of two 64-column slots. Bound like the key pass.
-// Encoder shape (see there) 103 -> 70 us; 4 x 16 heads, 8192 tokens, d 128: 170 -> 129 us.
+// Encoder shape (see there) 103 -> 53 us; 4 x 16 heads, 8192 tokens, d 128: 170 -> 117 us.
 template <int D, int DV>
 __global__ void __launch_bounds__(kPassThreads, 1) tc_fwd_queries_kernel(const __grid_constant__ MainParams p)
 {
@@ -1522,8 +1519,13 @@ void tensor_make_layout(darkattn_plan_s *plan)
     Y.sv = take(off, BH * N * 8);
     Y.zc = take(off, D.causal ? BH * (size_t)Y.T * m * 4 : 0);
     // The causal scan may leave SMs idle, which can add up the slabs meanwhile: 47 GB/s of rows read and written per SM, against
-    // 4.4 us (d 64) or 5.2 us (d 128) for a chunk of the scan; of every segment as many chunks as they manage in that time
-    // (4 x 16 heads, 8192 tokens, d 128: 465, 441, 430, 440 us with 0.53, 0.86, 1.0, 1.15 of that), and not many more CTAs than it takes. Not for short scans, whose last tiles would be waited for, nor where they would sum less than a fifth.
+    // 4.4 us (d 64) or 5.2 us (d 128) for a chunk of the scan; of every segment as many chunks as they manage in that time, and not
+    // many more CTAs than it takes (4 x 16 heads, 8192 tokens, d 128, no stash, one call's kernels alone: 465, 441, 430, 440 us
+    // with 0.53, 0.86, 1.0, 1.15 of that rate). Forward calls in a row, without -> with these sums: 504 -> 454 us at that
+    // shape, 146 -> 132 (2048 tokens), 818 -> 745 (8 heads, 65536 tokens, d 64, m 512), 193 -> 183 (48 heads, 4096 tokens, d 64); with a
+    // stash, whose stores slow the scan, 559 -> 535, 154 -> 141, 848 -> 784, 202 -> 189. The surplus of 1.6: the same as with all idle
+    // SMs, and with 1.0 the last tiles are waited for (745 -> 833, 183 -> 199). Not for scans of fewer than 8 chunks, nor where they would sum
+    // less than a fifth.
     const long long scan_ctas = units * nsplit, idle = 148 - scan_ctas;
     Y.summers = Y.cut = 0;
     if (D.causal && Y.T / nsplit >= 8 && idle > 0) {
@@ -1599,8 +1601,11 @@ cudaError_t tensor_prologue(const darkattn_plan_s *plan, const void *K, const vo
     PP.nK = out.nK; PP.cs = reinterpret_cast<int *>(out.cs); PP.status = reinterpret_cast<int *>(ws + Y.status);
     PP.N = D.N; PP.H = D.H; PP.Hkv = D.Hkv; PP.T = Y.T; PP.m = D.m; PP.r = D.r; PP.nslab = Y.nslab; PP.npair = (Y.nslab + 1) / 2;
     PP.coef = kLog2e * 0.5f * D.s * D.s;
-    const int per_sm = D.d == 64 ? 2 : 1;                           // CTAs of this kernel that fit one SM
-    PP.nsplit = pick_splits((long long)BH * PP.npair, Y.T, 1.5, 3.0, 64, per_sm * 148);
+    // Each CTA holds all of its SM's tensor memory, so they run one after the other; at d = 64, where two fit the shared memory, the
+    // second's start and first loads overlap the first's end. Pieces for 148 or for 296 CTAs at d = 64: the kernel 33.6 and 34.0 us
+    // (8 x 12 heads, 4096 tokens), 63.4 and 66.0 (8 heads, 65536 tokens, m 512), the calls around it 183.0 and 183.2, 795 and 744 (the
+    // CTAs of what follows land elsewhere), 108.8 and 101.4 (30 heads, 2048 tokens, m 512), 99.2 and 100.9 (32 heads, 8192 tokens, m 128).
+    PP.nsplit = pick_splits((long long)BH * PP.npair, Y.T, 1.5, 3.0, 64, D.d == 64 ? 296 : 148);
     const int smem_bytes = 5 * 128 * D.d * 2 + 128;
     timer_mark(plan, st, "tc_key_prepass_kernel");
     keep(launch_pdl(D.d == 64 ? tc_key_prepass_kernel<64> : tc_key_prepass_kernel<128>, dim3((unsigned)(BH * PP.npair * PP.nsplit)), dim3(160), smem_bytes, st, PP));

@@ -64,6 +64,19 @@ def test_tensor_path_refuses_f32(binding):
     assert e.value.status == binding.ERR_UNSUPPORTED
 
 
+def test_chunk_lengths_the_tensor_kernels_do_not_have(binding):
+    for chunk in (16, 64, 256):
+        with pytest.raises(binding.DarkAttnError) as e:
+            binding.darkattn_plan(1, 1, 256, 64, 256, causal=True, chunk=chunk, path=binding.PATH_TENSOR)
+        assert e.value.status == binding.ERR_UNSUPPORTED
+        plan = binding.darkattn_plan(1, 1, 256, 64, 256, causal=True, chunk=chunk)
+        assert plan.path == binding.PATH_SIMT
+        plan.destroy()
+    plan = binding.darkattn_plan(1, 1, 256, 64, 256, chunk=64)          # no mask: no chunks
+    assert plan.path == binding.PATH_TENSOR
+    plan.destroy()
+
+
 def test_null_and_misaligned_pointers_are_rejected_before_launch(binding):
     p = binding.darkattn_plan(1, 1, 128, 64, 64, dtype=binding.F32)
     vp = ctypes.c_void_p
