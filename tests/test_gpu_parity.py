@@ -166,6 +166,15 @@ def test_chunk_length_does_not_change_the_result(binding, chunk):
     _compare(run_gpu(binding, wl, t, chunk=chunk), _oracle(t, wl), TOL["f32"], f"chunk{chunk}")
 
 
+@pytest.mark.parametrize("chunk", [5, 16, 33, 64])
+def test_chunk_length_of_short_sequences(binding, chunk):
+    """The FFMA kernels, which many short sequences take, cut a sequence as the descriptor says (the products on the tensor cores
+    above have chunks of 128 whatever it says)."""
+    wl = inputs.small(name="short_chunks", wid=36, B=300, H=8, N=33, d=16, m=16, causal=True, dtype="f32")
+    t = inputs.generate(wl)
+    _compare(run_gpu(binding, wl, t, chunk=chunk), _oracle(t, wl), TOL["f32"], f"chunk{chunk}")
+
+
 def test_explicit_scale_and_per_head_projections(binding):
     wl = inputs.small(name="wph", wid=32, B=2, H=2, N=96, d=16, m=32, causal=True, dtype="f32")
     t = inputs.generate(wl)
@@ -618,6 +627,32 @@ def test_passes_over_keys_and_queries_at_piece_edges(binding, i):
     wl = inputs.small(name=f"pieces{i}", wid=430 + i, dtype="bf16", backward=False, **PASS_EDGES[i])
     t = inputs.generate(wl)
     _compare(run_gpu(binding, wl, t, path=binding.PATH_TENSOR), _oracle(t, wl), TOL["bf16"], f"pieces{i}")
+
+
+# The slabs summed beside the scan, with the backward pass that reads what the sums leave for it: all chunks summed there (no kernel
+# behind) of one, two, three and four slabs, some of them, and segments with their stash.
+SUMMED_BWD = [
+    dict(B=1, H=80, N=1024, d=64, m=128, causal=True),
+    dict(B=2, H=19, N=1152, d=128, m=256, dv=64, causal=True),
+    dict(B=1, H=26, N=1152, d=64, m=384, dv=128, causal=True),
+    dict(B=1, H=20, N=1152, d=64, m=512, causal=True),
+    dict(B=1, H=70, N=1152, d=64, m=256, causal=True),
+    dict(B=1, H=4, N=8960, d=64, m=256, causal=True),
+]
+
+
+@pytest.mark.parametrize("use_saved", [False, True], ids=["recompute", "saved"])
+@pytest.mark.parametrize("i", range(len(SUMMED_BWD)))
+def test_backward_behind_slabs_summed_beside_the_scan(binding, i, use_saved):
+    wl = inputs.small(name=f"summed{i}", wid=480 + i, dtype="bf16", backward=True, **SUMMED_BWD[i])
+    t = inputs.generate(wl)
+    got = run_gpu(binding, wl, t, path=binding.PATH_TENSOR, use_saved=use_saved)
+    for h in sorted({0, wl.H // 2, wl.H - 1}):      # (dM of a head sums over the batch: all entries of those heads)
+        sub = inputs.generate(wl, pairs=[(b, h) for b in range(wl.B)], as_batch=True)
+        want = _oracle(sub, wl)
+        for k in ("O", "dQ", "dK", "dV"):
+            assert_close(np.stack([got[k][b, h] for b in range(wl.B)])[:, None], want[k], TOL["bf16"], f"summed{i} head {h}: {k}")
+        assert_close(got["dM"][h], want["dM"][0], TOL["bf16"], f"summed{i} head {h}: dM")
 
 
 def test_tensor_path_is_deterministic(binding):
