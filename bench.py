@@ -68,7 +68,7 @@ def exps_per_token_head(m, causal, backward):
     return 2 * m + ((m if causal else 2 * m) if backward else 0)
 
 
-def kernel_work(d, r, m, dv, C, nslab, causal):
+def kernel_work(d, r, m, dv, C, nslab, causal, rows_summed=0.0):
     """Algorithmic work per (token, head) of each kernel of the tensor-core path: (flops, exps, bytes,
     bound). The scan kernels split the step's total of flops_per_token_head() between them: the causal
     query-side backward kernel is charged the query features' recompute (both backward kernels read the key features
@@ -89,8 +89,10 @@ def kernel_work(d, r, m, dv, C, nslab, causal):
         "tc_bwd_nc_k_kernel": (feat // 2 + 4 * m * dv + 2 * m * r + 4 * r * d, m, (2 * d + 2 * dv) * e, "tensor"),
         "tc_bwd_finish_k_kernel": (6 * r * d, 0, 3 * d * e, "hbm"),
         "tc_key_prepass_kernel": (2 * r * d + 2 * d * m, 0, d * e + 4, "hbm"),
-        "combine_kernel": (0, 0, (nslab * dv + dv) * e + nslab * 32, "hbm"),
-        "delta_kernel": (0, 0, 2 * dv * e + 4, "hbm"),
+        # (of the rows that the scan's own blocks have not summed)
+        "combine_kernel": (0, 0, (1.0 - rows_summed) * ((nslab * dv + dv) * e + nslab * 32), "hbm"),
+        # (it also clears dQ, where several slabs add into it)
+        "delta_kernel": (0, 0, 2 * dv * e + 4 + (d * e if nslab > 1 else 0), "hbm"),
     }
     return k
 
@@ -501,7 +503,7 @@ def main():
     # each kernel against the slowest of its three legs (tensor at the measured peak chosen above, ex2 at the
     # measured MUFU rate, bytes at the measured copy bandwidth)
     nslab = max(1, m // 128)
-    work = kernel_work(d, r, m, dv, 128, nslab, wl.causal)
+    work = kernel_work(d, r, m, dv, 128, nslab, wl.causal, plan.rows_summed())
     kernels = []
     for name, (tot_ms, cnt) in sorted(ktimes.items(), key=lambda kv: -kv[1][0]):
         entry = {"kernel": name, "launches_per_step": cnt / ksteps, "us_per_launch": 1e3 * tot_ms / max(cnt, 1),

@@ -17,6 +17,10 @@ extern "C" {
  * plan's current mode: with per-kernel timing on, the tensor-core backward launches one fewer.   */
 int32_t darkattn_plan_launches(darkattn_plan_t plan, int32_t which);
 
+/* Share of a forward call's rows whose slabs are added up beside the causal scan, by that kernel's own blocks; combine_kernel adds
+ * up the others. 0 without the mask and on the FP32 path.                                          */
+double darkattn_plan_rows_summed(darkattn_plan_t plan);
+
 /* Per-kernel device times, for benchmarks. While enabled, forward and backward record a CUDA event on
  * the call's stream in front of every kernel they launch and one behind the last (events are host
  * objects created by the first enabling call; no device memory is involved). Enabling also clears the

@@ -27,7 +27,7 @@ EXPORTS = [
     "darkattn_backward_dw", "darkattn_decode_step", "darkattn_selftest_wait_limit",
 ]
 # instruments of the benchmark, in a library of their own (include/darkattn_bench.h)
-BENCH_EXPORTS = ["darkattn_plan_launches", "darkattn_kernel_timing", "darkattn_kernel_times", "darkattn_measure_mma_cycles"]
+BENCH_EXPORTS = ["darkattn_plan_launches", "darkattn_plan_rows_summed", "darkattn_kernel_timing", "darkattn_kernel_times", "darkattn_measure_mma_cycles"]
 STATIC_SCRATCH_BYTES = 32 << 20
 
 
@@ -91,6 +91,8 @@ def benchlib():
         b = ctypes.CDLL(BENCH_LIB_PATH)
         b.darkattn_plan_launches.argtypes = [_vp, ctypes.c_int32]
         b.darkattn_plan_launches.restype = ctypes.c_int32
+        b.darkattn_plan_rows_summed.argtypes = [_vp]
+        b.darkattn_plan_rows_summed.restype = ctypes.c_double
         b.darkattn_measure_mma_cycles.argtypes = [ctypes.c_int32, ctypes.c_int32, ctypes.POINTER(ctypes.c_double),
                                                   ctypes.POINTER(ctypes.c_double), _vp]
         b.darkattn_measure_mma_cycles.restype = ctypes.c_int
@@ -137,6 +139,9 @@ class Plan:
 
     def launches(self, backward: bool = False) -> int:
         return int(benchlib().darkattn_plan_launches(self.handle, 1 if backward else 0))
+
+    def rows_summed(self) -> float:
+        return float(benchlib().darkattn_plan_rows_summed(self.handle))
 
     def alloc_workspace(self, device="cuda") -> torch.Tensor:
         return torch.empty(max(self.workspace_bytes, 256), dtype=torch.uint8, device=device)

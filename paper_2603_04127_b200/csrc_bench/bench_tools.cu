@@ -19,6 +19,18 @@ int32_t darkattn_plan_launches(darkattn_plan_t plan, int32_t which)
     return plan->launches_bwd - ((plan->path == DARKATTN_PATH_TENSOR && plan->timer.on) ? 1 : 0);
 }
 
+double darkattn_plan_rows_summed(darkattn_plan_t plan)
+{
+    if (!plan || plan->path != DARKATTN_PATH_TENSOR || !plan->tensor.cut) return 0;
+    const TensorLayout &Y = plan->tensor;
+    long long chunks = 0;
+    for (int s = 0; s < Y.nsplit; ++s) {
+        const int len = (int)((long long)Y.T * (s + 1) / Y.nsplit) - (int)((long long)Y.T * s / Y.nsplit);
+        chunks += len < Y.cut ? len : Y.cut;
+    }
+    return (double)chunks / Y.T;
+}
+
 darkattn_status_t darkattn_kernel_timing(darkattn_plan_t plan, int32_t enable)
 {
     if (!plan) return DARKATTN_ERR_INVALID_ARG;
