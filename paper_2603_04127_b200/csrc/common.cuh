@@ -289,11 +289,12 @@ __device__ __forceinline__ void pdl_wait()
 }
 // The same where TMA reads what the kernels before wrote with ordinary stores (folded projections, states, parts of fp32 numbers):
 // the wait makes those writes visible to this grid, but TMA goes through the async proxy, for which the PTX manual asks for a
-// fence between the two; an ordinary launch would imply it.
+// fence between the two (of global memory: with all state spaces 0.4 us a kernel, 606 -> 609.5 us for a training step of 8 x 12 heads of
+// 2048 tokens); an ordinary launch would imply it.
 __device__ __forceinline__ void pdl_wait_tma()
 {
     pdl_wait();
-    asm volatile("fence.proxy.async;" ::: "memory");
+    asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 #endif
 
