@@ -21,9 +21,13 @@
 // every second stage (every stage where the exponent's argument is formed) both are added to sums in registers, rounded to
 // nearest, and start from zero again: measured against float64 the path's results are closer than with a chain of fp32 FMAs.
 //
-// What bounds it: a stage of six products is 24 MMAs that take 99 cycles each (8 KB of shared memory per MMA beside 96 KB that
-// arrive per stage); a tile of features some 10 thousand cycles of its epilogue; a launch of few tiles the latencies of one:
-// parameters, loads, MMAs, epilogue, about 5 us.
+// What bounds it: a stage of six products is 24 MMAs that take 97 cycles each (8 KB of shared memory per MMA beside 96 KB that
+// arrive per stage; unrolled, so that each costs its thread less, they were issued in 75 and the calls took 4 % longer: the code no
+// longer fit the instruction caches); with all SMs busy the planes' way through L2, 5 to 6 TB/s in the launches of features and output rows; a
+// launch of few tiles the latencies of one: parameters, loads, MMAs, epilogue, about 5 us. All roles' code passes through every SM's
+// instruction cache, so its size counts (162 -> 101 KB: waits, x and the plain output as small loops), and so do reads of the launch's
+// parameters (kept in shared memory). 2 x 16 heads of 2001 tokens, d 128, m 256: 380 -> 352 us; training step of 2 x 8 heads, 1000 tokens,
+// d 64, fp32: 291 -> 264 us, mostly by the coalesced loads of x in the backward products.
 #include "split_gemm.cuh"
 #include "tc_common.cuh"
 
@@ -43,8 +47,12 @@ constexpr int kMaxStages = 6;
 constexpr int kStg = kRing * kPlane;                // 2 KB per epilogue warp: what is on its way out
 constexpr int kDot = kStg + 2 * kPlane;             // float[2][128]: the rows' dot products
 constexpr int kWt = kDot + 1024;                    // float[64]: the vector's part of a stage; float[128]: half of the MN-major sums
-constexpr int kBar = kWt + 1024;                    // (the row maxima's parts, float[4][128], are exchanged in kDot and kWt, which have no other use then)
-constexpr int kSmem = kBar + 256;
+constexpr int kBar = kWt + 768;
+// The products' descriptions: a tile's steps read some forty fields of them, chosen by the tile's product, and an indexed read of
+// the launch's parameters takes well over 100 cycles (it misses the constant cache that all roles share).
+constexpr int kBody = kBar + 176;
+constexpr int kSmem = (kBody + kMaxProbs * (int)sizeof(ProbBody) + 15) / 16 * 16;
+static_assert(sizeof(ProbBody) % 8 == 0, "read as words from 8-byte aligned places");
 static_assert(kSmem <= 232448, "shared memory budget of one CTA exceeded");
 constexpr float kLog2e = 1.4426950408889634f;
 // Key features are kept 2^24 times too large (a common factor, it cancels). A causal prefix may hold only keys far below the sequence's
@@ -59,12 +67,12 @@ struct Tile { int pb, z, pair, blk, h, hk, m0, n0, tn, Mlim, Nlim, K0, K1, total
 
 __device__ __forceinline__ uint32_t fast_div(uint32_t n, const FastDiv &d) { return (__umulhi(n, d.mul) + n) >> d.shr; }
 
-__device__ __forceinline__ void decode(const Launch &L, uint32_t w, Tile &t)
+__device__ __forceinline__ void decode(const Launch &L, const ProbBody *body, uint32_t w, Tile &t)
 {
     if (w >= L.total) return;
     int pb = 0;
-    while (pb + 1 < L.n && w >= L.p[pb].blocks) { w -= L.p[pb].blocks; ++pb; }
-    const Prob &P = L.p[pb];
+    while (pb + 1 < L.n && w >= body[pb].blocks) { w -= body[pb].blocks; ++pb; }
+    const ProbBody &P = body[pb];
     const uint32_t z = fast_div(w, P.dTiles), tl = w - z * P.dTiles.d, tm = fast_div(tl, P.dTilesN), pair = fast_div(z, P.dBlk), b = fast_div(pair, P.dH);
     t.pb = pb;
     t.z = (int)z;
@@ -116,32 +124,72 @@ __device__ __forceinline__ float tok_value(const TokVec &t, long long at)
 __device__ __forceinline__ void epi_all_sync() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
 __device__ __forceinline__ void dot_sync() { asm volatile("bar.sync 2, 64;" ::: "memory"); }
 
-// four neighbouring elements of x (n of them exist)
-__device__ __forceinline__ void load_x4(const Prob &P, long long at, int n, float (&y)[4])
+// Sixteen columns of x from `col` on for the warp's 32 rows (`row0`: the first one's token, `rows` of them and `n` columns exist): y gets
+// this lane's row. Neighbouring lanes load neighbouring pieces of a row and hand them over through the warp's 2 KB: a row per
+// lane, 8 bytes at a time, took 13 k cycles a tile where this takes 3 k. Rows that do not start on 16 bytes go element by element.
+__device__ __forceinline__ void load_x16(const ProbBody &P, long long row0, int rows, int col, int n, unsigned char *mine, int lane, float (&y)[16])
 {
-    y[0] = y[1] = y[2] = y[3] = 0.f;
-    if (n <= 0) return;
-    if (P.xkind == X_PLANES) {                      // rows are padded to a multiple of 8: all four are there
-        const __nv_bfloat16 *p = static_cast<const __nv_bfloat16 *>(P.x) + at;
+    const int es = P.xkind == X_F32 ? 4 : 2;
+    const char *base = static_cast<const char *>(P.x) + (row0 * P.xld + col) * es;
+    const long long ldb = (long long)P.xld * es;
+    auto at = [&](int r, int q) { return reinterpret_cast<uint4 *>(mine + r * 64 + ((q ^ ((r >> 1) & 3)) << 4)); };
+    __syncwarp();
+    if (((reinterpret_cast<uintptr_t>(P.x) | (uintptr_t)ldb) & 15) == 0) {
+        const uint4 zero = make_uint4(0, 0, 0, 0);
+        if (P.xkind == X_F32) {
+            uint4 u[4];
 #pragma unroll
-        for (int i = 2; i >= 0; --i) {              // (small parts first; the sum of the three is exact)
-            const uint2 u = *reinterpret_cast<const uint2 *>(p + i * P.xps);
-            y[0] += __uint_as_float(u.x << 16); y[1] += __uint_as_float(u.x & 0xffff0000u);
-            y[2] += __uint_as_float(u.y << 16); y[3] += __uint_as_float(u.y & 0xffff0000u);
+            for (int it = 0; it < 4; ++it) {
+                const int r = it * 8 + (lane >> 2), q = lane & 3;
+                u[it] = r < rows && 4 * q < n ? __ldg(reinterpret_cast<const uint4 *>(base + r * ldb) + q) : zero;
+            }
+#pragma unroll
+            for (int it = 0; it < 4; ++it) *at(it * 8 + (lane >> 2), lane & 3) = u[it];
+        } else {
+            const int planes = P.xkind == X_PLANES ? 3 : 1;
+            uint4 u[2][3];
+#pragma unroll
+            for (int it = 0; it < 2; ++it)
+#pragma unroll
+                for (int pl = 0; pl < 3; ++pl) {
+                    const int r = it * 16 + (lane >> 1), q = lane & 1;
+                    u[it][pl] = pl < planes && r < rows && 8 * q < n ? __ldg(reinterpret_cast<const uint4 *>(base + r * ldb + pl * P.xps * 2) + q) : zero;
+                }
+#pragma unroll
+            for (int it = 0; it < 2; ++it) {
+                float f[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) f[j] = 0.f;
+#pragma unroll
+                for (int pl = 2; pl >= 0; --pl) {   // (small parts first; the sum of the three is exact)
+                    const uint32_t v[4] = {u[it][pl].x, u[it][pl].y, u[it][pl].z, u[it][pl].w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) add2(f[2 * j], f[2 * j + 1], __uint_as_float(v[j] << 16), __uint_as_float(v[j] & 0xffff0000u));
+                }
+                const int r = it * 16 + (lane >> 1), q = lane & 1;
+                *reinterpret_cast<float4 *>(at(r, 2 * q)) = make_float4(f[0], f[1], f[2], f[3]);
+                *reinterpret_cast<float4 *>(at(r, 2 * q + 1)) = make_float4(f[4], f[5], f[6], f[7]);
+            }
         }
-    } else if (P.xkind == X_F32) {
-        const float *p = static_cast<const float *>(P.x) + at;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) if (j < n) y[j] = p[j];
     } else {
-        const unsigned short *p = static_cast<const unsigned short *>(P.x) + at;
+        const char *p = base + lane * ldb;          // (never planes: those are the path's own)
+#pragma unroll 1
+        for (int j = 0; j < 16; ++j) {
+            float v = 0.f;
+            if (lane < rows && j < n) v = es == 4 ? reinterpret_cast<const float *>(p)[j] : __uint_as_float((uint32_t)reinterpret_cast<const unsigned short *>(p)[j] << 16);
+            reinterpret_cast<float *>(at(lane, j >> 2))[j & 3] = v;
+        }
+    }
+    __syncwarp();
 #pragma unroll
-        for (int j = 0; j < 4; ++j) if (j < n) y[j] = __uint_as_float((uint32_t)p[j] << 16);
+    for (int q = 0; q < 4; ++q) {
+        const float4 v = *reinterpret_cast<const float4 *>(at(lane, q));
+        y[4 * q] = v.x; y[4 * q + 1] = v.y; y[4 * q + 2] = v.z; y[4 * q + 3] = v.w;
     }
 }
 
 // What the path does to a row's 32 columns: acc (this lane's row, columns n0 + 32 g .. + 31) in place. mine: the warp's staging.
-__device__ __forceinline__ void apply(const Prob &P, const Tile &t, float (&acc)[32], float den, float rowv, float *xch, unsigned char *mine, int g, int rl)
+__device__ __forceinline__ void apply(const ProbBody &P, const Tile &t, float (&acc)[32], float den, float rowv, unsigned char *mine, int g, int rl)
 {
     const int col0 = t.n0 + g * 32, row = t.m0 + rl, lane = rl & 31;
     const bool live = row < t.Mlim;
@@ -180,17 +228,23 @@ __device__ __forceinline__ void apply(const Prob &P, const Tile &t, float (&acc)
         skey[lane] = col0 + lane < t.Nlim ? float_from_order_key(__ldg(P.colmax + (long long)t.pair * P.colkey_ld + col0 + lane)) : 0.f;
         __syncwarp();
         if (P.epi == EPI_PHI_K) {
+            float low = 0.f;
 #pragma unroll
             for (int j = 0; j < 32; j += 2) {
                 const float2 k = *reinterpret_cast<const float2 *>(skey + j);
                 add2(acc[j], acc[j + 1], -rowv, -rowv);
                 add2(acc[j], acc[j + 1], -k.x, -k.y);
                 mul2(acc[j], acc[j + 1], kLog2e, kLog2e);
-                const bool low0 = acc[j] < kKeyScaleLine, low1 = acc[j + 1] < kKeyScaleLine;
-                acc[j] = ex2f(low0 ? acc[j] + kKeyScaleLog2 : acc[j]); acc[j + 1] = ex2f(low1 ? acc[j + 1] + kKeyScaleLog2 : acc[j + 1]);
-                mul2(acc[j], acc[j + 1], low0 ? 1.f : kKeyScale, low1 ? 1.f : kKeyScale);
+                low = fminf(low, fminf(acc[j], acc[j + 1]));
             }
             __syncwarp();
+            if (low < kKeyScaleLine) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) { const bool l = acc[j] < kKeyScaleLine; acc[j] = ex2f(l ? acc[j] + kKeyScaleLog2 : acc[j]) * (l ? 1.f : kKeyScale); }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 32; j += 2) { acc[j] = ex2f(acc[j]); acc[j + 1] = ex2f(acc[j + 1]); mul2(acc[j], acc[j + 1], kKeyScale, kKeyScale); }
+            }
             break;
         }
         const int n = t.Nlim - col0;
@@ -212,9 +266,11 @@ __device__ __forceinline__ void apply(const Prob &P, const Tile &t, float (&acc)
         if (P.epi == EPI_ROWMAX) break;
         if (P.row.p) mx = rowv;
         else {                                      // the row is whole in this tile: its other parts' maxima
-            xch[g * 128 + rl] = mx;
+            float *xch = reinterpret_cast<float *>(mine) + 32 + lane;       // (behind the shifts)
+            *xch = mx;
             epi_all_sync();
-            mx = fmaxf(fmaxf(xch[rl], xch[128 + rl]), fmaxf(xch[256 + rl], xch[384 + rl]));
+            xch -= g * 2048;                        // the other parts: every fourth warp's, 2 KB to a warp
+            mx = fmaxf(fmaxf(xch[0], xch[2048]), fmaxf(xch[2 * 2048], xch[3 * 2048]));
             epi_all_sync();
         }
 #pragma unroll
@@ -245,44 +301,37 @@ __device__ __forceinline__ void apply(const Prob &P, const Tile &t, float (&acc)
         }
         break;
     }
-    case EPI_GRAD: {
-        const float inv = 1.f / den;
-#pragma unroll
-        for (int j = 0; j < 32; j += 4) {
-            float y[4];
-            load_x4(P, tok * P.xld + col0 + j, live ? t.Nlim - col0 - j : 0, y);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { part = fmaf(y[i], acc[j + i] * inv, part); acc[j + i] = y[i] * inv; }
-        }
-        part *= -inv;
-        break;
-    }
-    case EPI_RANK1: {
+    case EPI_GRAD:
+    case EPI_RANK1:
+    case EPI_SUBX: {
+        if (P.xkind == X_NONE) break;
+        const float inv = 1.f / den, v = P.epi == EPI_SUBX || P.row.p ? rowv : 1.f;     // (den: 1 where there is no dot product)
         const float *f = P.colvec + t.pair * P.vec_pair + t.blk * P.vec_blk + col0;     // (padded to a multiple of four)
-        const float v = P.row.p ? rowv : 1.f;
 #pragma unroll
-        for (int j = 0; j < 32; j += 4) {
-            const int n = t.Nlim - col0 - j;
-            float y[4];
-            load_x4(P, tok * P.xld + col0 + j, live ? n : 0, y);
-            const float4 c = n > 0 && P.colvec ? __ldg(reinterpret_cast<const float4 *>(f + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            acc[j] = y[0] * fmaf(v, c.x, acc[j]); acc[j + 1] = n > 1 ? y[1] * fmaf(v, c.y, acc[j + 1]) : 0.f;
-            acc[j + 2] = n > 2 ? y[2] * fmaf(v, c.z, acc[j + 2]) : 0.f; acc[j + 3] = n > 3 ? y[3] * fmaf(v, c.w, acc[j + 3]) : 0.f;
-            part += (acc[j] + acc[j + 1]) + (acc[j + 2] + acc[j + 3]);
-        }
-        break;
-    }
-    case EPI_SUBX:
-        if (P.xkind != X_NONE) {
+        for (int j0 = 0; j0 < 32; j0 += 16) {
+            float y[16];
+            const int n = t.Nlim - col0 - j0;
+            load_x16(P, tok - lane, t.Mlim - row + lane, col0 + j0, n, mine, lane, y);
+            float *a = acc + j0;
+            if (P.epi == EPI_GRAD) {
 #pragma unroll
-            for (int j = 0; j < 32; j += 4) {
-                float y[4];
-                load_x4(P, tok * P.xld + col0 + j, live ? t.Nlim - col0 - j : 0, y);
+                for (int i = 0; i < 16; ++i) { part = fmaf(y[i], a[i] * inv, part); a[i] = y[i] * inv; }
+            } else if (P.epi == EPI_SUBX) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[j + i] = fmaf(-rowv, y[i], acc[j + i]);
+                for (int i = 0; i < 16; ++i) a[i] = fmaf(-v, y[i], a[i]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 16; i += 4) {
+                    const float4 c = i < n && P.colvec ? __ldg(reinterpret_cast<const float4 *>(f + j0 + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    a[i] = y[i] * fmaf(v, c.x, a[i]); a[i + 1] = i + 1 < n ? y[i + 1] * fmaf(v, c.y, a[i + 1]) : 0.f;
+                    a[i + 2] = i + 2 < n ? y[i + 2] * fmaf(v, c.z, a[i + 2]) : 0.f; a[i + 3] = i + 3 < n ? y[i + 3] * fmaf(v, c.w, a[i + 3]) : 0.f;
+                    part += (a[i] + a[i + 1]) + (a[i + 2] + a[i + 3]);
+                }
             }
         }
+        if (P.epi == EPI_GRAD) part *= -inv;
         break;
+    }
     }
     if (P.sums && live) P.sums[(long long)(t.tn * 4 + g) * P.batch * P.ntok + tok] = part;
 }
@@ -297,6 +346,11 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int stages = min(kMaxStages, kRing / L.stage_planes), stage_bytes = L.stage_planes * kPlane;
 
+    ProbBody *body = reinterpret_cast<ProbBody *>(smem + kBody);
+    for (int i = tid; i < L.n * (int)(sizeof(ProbBody) / 4); i += kNT) {
+        const int pb = i / (int)(sizeof(ProbBody) / 4), k = i % (int)(sizeof(ProbBody) / 4);
+        reinterpret_cast<int *>(body + pb)[k] = reinterpret_cast<const int *>(static_cast<const ProbBody *>(&L.p[pb]))[k];
+    }
     if (tid == 0) {
         for (int i = 0; i < kMaxStages; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, 1 + kDots); }
         for (int i = 0; i < 2; ++i) { mbar_init(accfull + i, 1); mbar_init(accfree + i, kEpi); mbar_init(dotfull + i, kDots); mbar_init(dotfree + i, kEpi); }
@@ -307,10 +361,9 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    // the first tile's place is worked out before the wait: its reads of the launch's parameters (none is in a cache yet: some
-    // 2400 cycles) run under the kernel before
+    // (the reads of the parameters, none of which is in a cache yet, and the first tile's place run under the kernel before)
     Tile t;
-    decode(L, blockIdx.x, t);
+    decode(L, body, blockIdx.x, t);
     pdl_wait_tma();
     if (L.init) {
         if (blockIdx.x == 0 && tid == 0) *L.status = 0;
@@ -326,8 +379,8 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
     if (warp == kLoadWarp) {
         // ---------------------------------------------------------------- load
         if (lane == 0) {
-            for (uint32_t w = blockIdx.x; w < L.total; w += gridDim.x, decode(L, w, t)) {
-                const Prob &P = L.p[t.pb];
+            for (uint32_t w = blockIdx.x; w < L.total; w += gridDim.x, decode(L, body, w, t)) {
+                const ProbBody &P = body[t.pb];
                 for (int i = 0; i < t.total && ok; ++i) {
                     const int s = i >= t.n0st, k0 = (i - (s ? t.n0st : 0)) * 64;
                     wait(empty + st, sph ^ 1);
@@ -342,8 +395,8 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
                         else
                             for (int hh = 0; hh < halves; ++hh) tma_load_4d(d + hh * o.planes * (kPlane / 2), map, full + st, mn0 + hh * 64, rb + k0, bt, 0);
                     };
-                    load(a, &P.map[2 * s], dst, t.m0, 2);
-                    load(b, &P.map[2 * s + 1], dst + a.planes * kPlane, t.n0, bhalves);
+                    load(a, &L.p[t.pb].map[2 * s], dst, t.m0, 2);
+                    load(b, &L.p[t.pb].map[2 * s + 1], dst + a.planes * kPlane, t.n0, bhalves);
                     next_stage();
                 }
             }
@@ -352,8 +405,8 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
         // ---------------------------------------------------------------- multiply
         if (lane == 0) {
             uint32_t unit = 0;
-            for (uint32_t w = blockIdx.x; w < L.total; w += gridDim.x, decode(L, w, t)) {
-                const Prob &P = L.p[t.pb];
+            for (uint32_t w = blockIdx.x; w < L.total; w += gridDim.x, decode(L, body, w, t)) {
+                const ProbBody &P = body[t.pb];
                 const int nw = (min(t.Nlim - t.n0, 128) + 15) & ~15;                    // columns of this tile, in the MMA's granularity
                 for (int i = 0; i < t.total && ok; ++unit) {
                     const uint32_t big = tmem + (unit & 1) * 256, sml = big + 128;
@@ -391,8 +444,8 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
         // ---------------------------------------------------------------- dot products of A's rows
         const int dt = tid - kDotWarp * 32;         // 0..63
         uint32_t nd = 0;
-        for (uint32_t w = blockIdx.x; w < L.total; w += gridDim.x, decode(L, w, t)) {
-            const Prob &P = L.p[t.pb];
+        for (uint32_t w = blockIdx.x; w < L.total; w += gridDim.x, decode(L, body, w, t)) {
+            const ProbBody &P = body[t.pb];
             // K-major A: rd[0..3] of row dt, rd[4..7] of row dt + 64; MN-major A: the eight rows of chunk dt % 16, every fourth index
             float rd[8];
 #pragma unroll
@@ -476,8 +529,8 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
         const uint32_t taddr = tmem + ((uint32_t)(q4 * 32) << 16) + g * 32;
         unsigned char *mine = smem + kStg + warp * 2048;
         uint32_t unit = 0, nd = 0;
-        for (uint32_t w = blockIdx.x; w < L.total; w += gridDim.x, decode(L, w, t)) {
-            const Prob &P = L.p[t.pb];
+        for (uint32_t w = blockIdx.x; w < L.total; w += gridDim.x, decode(L, body, w, t)) {
+            const ProbBody &P = body[t.pb];
             const int row = t.m0 + rl, cols = t.Nlim - t.n0 - g * 32;                   // this warp's columns (may be negative or above 32)
             float rowv = 0.f;
             if (P.row.p && row < t.Mlim) {
@@ -487,9 +540,9 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
             float acc[32];
 #pragma unroll
             for (int j = 0; j < 32; ++j) acc[j] = 0.f;
-            for (int i = 0; i < t.total; i += P.chain, ++unit) {
-                bool small = false;
-                for (int c = i; c < i + P.chain && c < t.total; ++c) { const int s = c >= t.n0st; small |= P.op[2 * s].planes + P.op[2 * s + 1].planes > 2; }
+            const int chain = P.chain, n0 = P.small[0] ? t.n0st : 0, n1 = P.small[1] ? t.n0st : t.total;       // small products: stages below n0 and from n1 on
+            for (int i = 0; i < t.total; i += chain, ++unit) {
+                const bool small = i < n0 || min(i + chain, t.total) > n1;
                 ok = ok && __all_sync(0xffffffffu, mbar_wait(accfull + (unit & 1), (unit >> 1) & 1, L.status));
                 tc_fence_after();
                 if (cols > 0) {
@@ -503,8 +556,16 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
                         tmem_wait_ld();
                         // The parts of an infinite value are inf, NaN and NaN: where the large products are infinite they decide alone
                         // (with the check kept to products of values 382 us at 2 x 16 heads of 2001 tokens, d 128, m 256, for all 379)
+                        float top = 0.f;
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) if (fabsf(acc[j]) < INFINITY) acc[j] += __uint_as_float(v[j]);
+                        for (int j = 0; j < 32; ++j) top = fmaxf(top, fabsf(acc[j]));
+                        if (top < INFINITY) {
+#pragma unroll
+                            for (int j = 0; j < 32; j += 2) add2(acc[j], acc[j + 1], __uint_as_float(v[j]), __uint_as_float(v[j + 1]));
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) if (fabsf(acc[j]) < INFINITY) acc[j] += __uint_as_float(v[j]);
+                        }
                     }
                 }
                 tc_fence_before();
@@ -522,7 +583,7 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
                 mbar_arrive_warp(dotfree + (nd & 1));
                 ++nd;
             }
-            apply(P, t, acc, den, rowv, sDot, mine, g, rl);
+            apply(P, t, acc, den, rowv, mine, g, rl);
             if (P.okind == OUT_NONE) continue;
             if (P.okind == OUT_PLANES) {
                 // plane by plane through the warp's 2 KB: four lanes per row's 64 bytes, eight rows per store (rows are padded to
@@ -568,7 +629,7 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
                     for (int q = 0; q < 4; ++q)
                         *reinterpret_cast<float4 *>(mine + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4)) = make_float4(acc[c * 16 + 4 * q], acc[c * 16 + 4 * q + 1], acc[c * 16 + 4 * q + 2], acc[c * 16 + 4 * q + 3]);
                     __syncwarp();
-#pragma unroll
+#pragma unroll 1
                     for (int it = 0; it < 4; ++it) {
                         const int r2 = it * 8 + (lane >> 2), q = lane & 3, orow = t.m0 + q4 * 32 + r2, oc = t.n0 + g * 32 + c * 16 + q * 4, n = t.Nlim - oc;
                         const float4 x = *reinterpret_cast<const float4 *>(mine + r2 * 64 + ((q ^ ((r2 >> 1) & 3)) << 4));
@@ -627,7 +688,7 @@ void set_operand(Launch &L, Prob &p, int i, const Op &o, bool hi_only)
 {
     const int planes = hi_only ? 1 : o.m.planes;
     if (!make_map4(&p.map[i], o.m, o.mn ? 64 : 128, planes)) L.bad = 1;
-    p.op[i] = {planes, o.mn, o.batch, o.tok};
+    p.op[i] = {(unsigned char)planes, (unsigned char)o.mn, (unsigned char)o.batch, (unsigned char)o.tok};
 }
 
 void add(Launch &L, const Prob &q)
@@ -639,6 +700,7 @@ void add(Launch &L, const Prob &q)
     p.blocks = (unsigned)p.batch * p.nblk * tilesM * tilesN;
     p.dTiles = make_div(tilesM * tilesN); p.dTilesN = make_div(tilesN);
     p.dBlk = make_div((unsigned)p.nblk); p.dH = make_div((unsigned)p.H); p.dG = make_div((unsigned)p.G);
+    for (int s = 0; s < 2; ++s) p.small[s] = p.op[2 * s].planes + p.op[2 * s + 1].planes > 2;
     for (int s = 0; s < 2; ++s)
         if (p.K[s] > 0 && p.op[2 * s].planes + p.op[2 * s + 1].planes > L.stage_planes) L.stage_planes = p.op[2 * s].planes + p.op[2 * s + 1].planes;
     L.total += p.blocks;

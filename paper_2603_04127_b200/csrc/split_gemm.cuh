@@ -63,14 +63,13 @@ enum Epi {
 enum OutKind { OUT_NONE = 0, OUT_PLANES, OUT_F32, OUT_BF16 };
 enum XKind { X_NONE = 0, X_PLANES, X_F32, X_BF16 };
 
-struct Opnd { int planes, mn, batch, tok; };
+struct Opnd { unsigned char planes, mn, batch, tok; };
 
 // C = A[0] B[0] (+ A[1] B[1]) for every (batch, head, token block) and what is done with it on the way out; K = 0: no product.
 // Dimensions marked as tokens end with the block: their size is min(block, ntok - index * block). Blocks are multiples of 64
 // tokens, of 128 where a tile's rows are tokens of a block.
-struct Prob {
-    CUtensorMap map[4];             // A0, B0, A1, B1
-    Opnd op[4];
+struct ProbBody {
+    Opnd op[4];                     // A0, B0, A1, B1
     int K[2] = {0, 0}, ktok[2] = {0, 0};
     int M = 0, N = 0, mtok = 0, ntok_dim = 0;
     int skip2 = -1;                 // the second product is left out for this token block (its state is zero)
@@ -94,8 +93,12 @@ struct Prob {
     void *out = nullptr;            // element (row, col) at out + pair * os_pair + block * os_blk + row * old_ + col
     long long os_pair = 0, os_blk = 0, ops = 0;     // ops: from plane to plane
     // derived
+    int small[2] = {0, 0};          // whether the products have small parts
     unsigned blocks = 0;
     FastDiv dTiles, dTilesN, dBlk, dH, dG;
+};
+struct Prob : ProbBody {
+    CUtensorMap map[4];             // of the operands
 };
 
 constexpr int kMaxProbs = 3;
