@@ -213,6 +213,20 @@ __device__ __forceinline__ uint64_t make_sdesc(uint32_t saddr, uint32_t lbo_byte
     return d;
 }
 
+// MMAs are issued by one lane. The warp around it runs its code as a whole (all lanes wait at the barriers together) and enters
+// `if (elect_one())` for each batch: then the compiler knows addresses and descriptors to be the same in all lanes and keeps them in
+// uniform registers, where the instruction wants them: one instruction an MMA, where code that a single lane runs by itself took
+// six and more, most of them moves into those registers, and was as long as the MMAs of 64 columns and less.
+// The same lane is elected every time (its TMA stores, commits and waits belong together).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+// A value that is the same in all lanes (a warp's number, an address read from shared memory), in a form that shows it.
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+
 // D[tmem] (+)= A[smem] * B[smem]; issued by ONE thread. accumulate = 0 overwrites D.
 __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
 {
@@ -285,6 +299,11 @@ __device__ __forceinline__ float load_key_shift(const float *cs, int i) { return
 __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, int *status, volatile int *abort_flag)
 {
     return mbar_wait_limited(bar, parity, status, abort_flag);
+}
+// The same by a whole warp, with one answer.
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, int *status, volatile int *abort_flag)
+{
+    return __all_sync(0xffffffffu, wait_or_abort(bar, parity, status, abort_flag));
 }
 
 // ---------------------------------------------------------------- tiles, epilogue layout, descriptors

@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_q_kernel(const __grid
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + QNBARS);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + QNBARS + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5);
     const int T = p.T;
     // CTAs work in groups of nslab (one per slab of the head) on the same piece of the line of (batch, head, chunk)
     // items, so that the Q, V, dO tiles a group reads are fetched from HBM once
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_q_kernel(const __grid
     __syncthreads();
     tc_fence_after();
     pdl_wait_tma();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = uniform(*tmem_slot);
     int *status = p.status;
 
     if (*abort_flag) {
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_q_kernel(const __grid
     } else if (warp == kEpiWarps + 1) {
         clear_share(p.clear);
     } else if (warp == kEpiWarps) {
-        if ((tid & 31) == 0) {
+        {
             const TileDesc tOm(sOm), tOml(sOml), tQA(sQA), tKB(sKB), tV(sV), tG(sG), tSt(sSt), tDel(sDelOp);
             const uint32_t id_kk = make_idesc(128, 128, 0, 0);
             const uint32_t id_vec = make_idesc(128, 16, 1, 0);
@@ -172,31 +172,40 @@ __global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_q_kernel(const __grid
                     mbar_expect_tx(bars + QB_S, 128 * DV * 2);
                     for (int a = 0; a < DV / 64; ++a) tma_load_2d(dst + a * 16384, &p.mapSst, bars + QB_S, a * 64, (bh * T + t) * p.m + slab * 128);
                 };
-                tma_store_wait_read();      // the last dQ tile of the run before has left its buffer
-                mbar_expect_tx(bars + QB_OM, 2 * 128 * D * 2);
-                for (int a = 0; a < D / 64; ++a) {
-                    tma_load_2d(sOm + a * 16384, &p.mapOm, bars + QB_OM, a * 64, h * p.m + slab * 128);
-                    tma_load_2d(sOml + a * 16384, &p.mapOml, bars + QB_OM, a * 64, h * p.m + slab * 128);
+                if (elect_one()) {
+                    tma_store_wait_read();      // the last dQ tile of the run before has left its buffer
+                    mbar_expect_tx(bars + QB_OM, 2 * 128 * D * 2);
                 }
-                load_tile((it & 1) ? sSt : sQA, &p.mapQ, bars + QB_Q, D, t0);
-                load_tile(sV, &p.mapV, bars + QB_V, DV, t0);
-                load_tile(sG, &p.mapG, bars + QB_G, DV, t0);
-                load_key_features(t0);
-                load_state((it & 1) ? sQA : sSt, t0);
-                ok = wait_or_abort(bars + QB_OM, run & 1, status, abort_flag);
-                if (ok) ok = wait_or_abort(bars + QB_Q, it & 1, status, abort_flag);
+                if (elect_one())
+                    for (int a = 0; a < D / 64; ++a) {
+                        tma_load_2d(sOm + a * 16384, &p.mapOm, bars + QB_OM, a * 64, h * p.m + slab * 128);
+                        tma_load_2d(sOml + a * 16384, &p.mapOml, bars + QB_OM, a * 64, h * p.m + slab * 128);
+                    }
+                if (elect_one()) {
+                    load_tile((it & 1) ? sSt : sQA, &p.mapQ, bars + QB_Q, D, t0);
+                    load_tile(sV, &p.mapV, bars + QB_V, DV, t0);
+                    load_tile(sG, &p.mapG, bars + QB_G, DV, t0);
+                    load_key_features(t0);
+                    load_state((it & 1) ? sQA : sSt, t0);
+                }
+                ok = warp_wait(bars + QB_OM, run & 1, status, abort_flag);
+                if (ok) ok = warp_wait(bars + QB_Q, it & 1, status, abort_flag);
                 if (ok) {
                     tc_fence_after();
                     const TileDesc &tX0 = (it & 1) ? tSt : tQA;
-                    issue_projection<D>(R3, tX0, tOm, tOml, id_kk);                                              // U_Q of the run's first chunk
-                    mma_commit(bars + QM1);
-                    ok = wait_or_abort(bars + QB_V, it & 1, status, abort_flag);
-                    if (ok) ok = wait_or_abort(bars + QB_G, it & 1, status, abort_flag);
+                    if (elect_one()) {
+                        issue_projection<D>(R3, tX0, tOm, tOml, id_kk);                                              // U_Q of the run's first chunk
+                        mma_commit(bars + QM1);
+                    }
+                    ok = warp_wait(bars + QB_V, it & 1, status, abort_flag);
+                    if (ok) ok = warp_wait(bars + QB_G, it & 1, status, abort_flag);
                 }
                 if (ok) {
                     tc_fence_after();
-                    _Pragma("unroll") for (int k = 0; k < DV / 16; ++k) mma_ss(R2, kdesc(tG, k), kdesc(tV, k), id_kk, k > 0);     // dO V^T of the run's first chunk
-                    mma_commit(bars + QM3);
+                    if (elect_one()) {
+                        _Pragma("unroll") for (int k = 0; k < DV / 16; ++k) mma_ss(R2, kdesc(tG, k), kdesc(tV, k), id_kk, k > 0);     // dO V^T of the run's first chunk
+                        mma_commit(bars + QM3);
+                    }
                 }
                 for (int c = 0; c < nrun && ok; ++c, ++it) {
                     const int t = t0 + c;
@@ -204,75 +213,92 @@ __global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_q_kernel(const __grid
                     const bool first = (t == 0), last = (c + 1 == nrun);
                     unsigned char *bX = ph ? sSt : sQA, *bS = ph ? sQA : sSt;
                     const TileDesc &tX = ph ? tSt : tQA, &tS = ph ? tQA : tSt;
-#define QWAIT(b) do { ok = wait_or_abort(bars + (b), ph, status, abort_flag); } while (0)
+#define QWAIT(b) do { ok = warp_wait(bars + (b), ph, status, abort_flag); } while (0)
                     QWAIT(QE1); if (!ok) break;                                                                  // A^ in X, R3 read, -delta operand written
-                    tma_store_2d(&p.mapAh, bX, slab * 128, row0 + t * 128);                                      // A^ kept for the key-side kernel
-                    tma_store_2d(&p.mapAh, bX + 16384, slab * 128 + 64, row0 + t * 128);
-                    tma_store_commit();
+                    if (elect_one()) {
+                        tma_store_2d(&p.mapAh, bX, slab * 128, row0 + t * 128);                                      // A^ kept for the key-side kernel
+                        tma_store_2d(&p.mapAh, bX + 16384, slab * 128 + 64, row0 + t * 128);
+                        tma_store_commit();
+                    }
                     QWAIT(QE2A); if (!ok) break;                                                                 // dO V^T read out of R2: V is done with
-                    if (!last) load_tile(sV, &p.mapV, bars + QB_V, DV, t + 1);
+                    if (!last && elect_one()) load_tile(sV, &p.mapV, bars + QB_V, DV, t + 1);
                     tc_fence_after();
-                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R2 + 64, mndesc(tX, k), vecdesc(tDel, k), id_vec, k > 0);  // rho_c = -A^^T delta (columns 0, 1)
+                    if (elect_one()) _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R2 + 64, mndesc(tX, k), vecdesc(tDel, k), id_vec, k > 0);  // rho_c = -A^^T delta (columns 0, 1)
                     QWAIT(QE2); if (!ok) break;                                                                  // dP packed in R2
                     QWAIT(QB_B); if (!ok) break;
                     tc_fence_after();
-                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(R1, R2 + k * 8, mndesc(tKB, k), id_tm, k > 0);           // dP Bf
+                    if (elect_one()) _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(R1, R2 + k * 8, mndesc(tKB, k), id_tm, k > 0);           // dP Bf
                     QWAIT(QB_S); if (!ok) break;                                                                 // (for the first chunk the tile is loaded but not used)
                     if (!first) {
                         tc_fence_after();
-                        _Pragma("unroll") for (int k = 0; k < DV / 16; ++k) mma_ss(R1, kdesc(tG, k), kdesc(tS, k), id_kk, 1);     // + dO S_prev^T
+                        if (elect_one()) _Pragma("unroll") for (int k = 0; k < DV / 16; ++k) mma_ss(R1, kdesc(tG, k), kdesc(tS, k), id_kk, 1);     // + dO S_prev^T
                     }
-                    tma_store_wait_read();      // the A^ tile has left shared memory: E may overwrite it
-                    mma_commit(bars + QM4);
+                    if (elect_one()) {
+                        tma_store_wait_read();      // the A^ tile has left shared memory: E may overwrite it
+                        mma_commit(bars + QM4);
+                    }
                     QWAIT(QM4); if (!ok) break;                                                                  // Bf, dO and S of this chunk are done with
-                    load_tile(sKB, &p.mapQ, bars + QB_X2, D, t);                                                // Q again, for T, where Bf was
+                    if (elect_one()) load_tile(sKB, &p.mapQ, bars + QB_X2, D, t);                                                // Q again, for T, where Bf was
                     if (!last) {
-                        load_tile(sG, &p.mapG, bars + QB_G, DV, t + 1);
-                        load_tile(bS, &p.mapQ, bars + QB_Q, D, t + 1);                                          // the state tile is done with: the next chunk's Q
-                        for (int a = 0; a < DV / 64; ++a)                                                        // into L2 now: the next state's load can only be issued at the chunk's very end
-                            tma_prefetch_l2_2d(&p.mapSst, a * 64, (bh * T + t + 1) * p.m + slab * 128);
+                        if (elect_one()) {
+                            load_tile(sG, &p.mapG, bars + QB_G, DV, t + 1);
+                            load_tile(bS, &p.mapQ, bars + QB_Q, D, t + 1);                                          // the state tile is done with: the next chunk's Q
+                            for (int a = 0; a < DV / 64; ++a)                                                        // into L2 now: the next state's load can only be issued at the chunk's very end
+                                tma_prefetch_l2_2d(&p.mapSst, a * 64, (bh * T + t + 1) * p.m + slab * 128);
+                        }
                     }
                     QWAIT(QE3); if (!ok) break;
                     tc_fence_after();
-                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R1, kdesc(tX, k), mndesc(tOm, k), id_dx, k > 0);         // E Omega
-                    mma_commit(bars + QM5);
+                    if (elect_one()) {
+                        _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R1, kdesc(tX, k), mndesc(tOm, k), id_dx, k > 0);         // E Omega
+                        mma_commit(bars + QM5);
+                    }
                     QWAIT(QB_X2); if (!ok) break;
                     if (c == 0 && run > 0) {                                                                     // T of the previous run has been read out
-                        ok = wait_or_abort(bars + QET, (run - 1) & 1, status, abort_flag);
+                        ok = warp_wait(bars + QET, (run - 1) & 1, status, abort_flag);
                         if (!ok) break;
                     }
                     tc_fence_after();
-                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColT, mndesc(tX, k), mndesc(tKB, k), id_t, (c > 0) || k > 0);   // T += E^T Q
-                    mma_commit(bars + QM6);
+                    if (elect_one()) {
+                        _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColT, mndesc(tX, k), mndesc(tKB, k), id_t, (c > 0) || k > 0);   // T += E^T Q
+                        mma_commit(bars + QM6);
+                    }
                     if (!last) {
-                        ok = wait_or_abort(bars + QB_Q, ph ^ 1, status, abort_flag);
+                        ok = warp_wait(bars + QB_Q, ph ^ 1, status, abort_flag);
                         if (!ok) break;
                         tc_fence_after();
-                        issue_projection<D>(R3, tS, tOm, tOml, id_kk);                                           // U_Q of the next chunk (its Q sits in S)
-                        mma_commit(bars + QM1);
-                        ok = wait_or_abort(bars + QB_V, ph ^ 1, status, abort_flag);
-                        if (ok) ok = wait_or_abort(bars + QB_G, ph ^ 1, status, abort_flag);
+                        if (elect_one()) {
+                            issue_projection<D>(R3, tS, tOm, tOml, id_kk);                                           // U_Q of the next chunk (its Q sits in S)
+                            mma_commit(bars + QM1);
+                        }
+                        ok = warp_wait(bars + QB_V, ph ^ 1, status, abort_flag);
+                        if (ok) ok = warp_wait(bars + QB_G, ph ^ 1, status, abort_flag);
                         if (!ok) break;
                         tc_fence_after();
-                        _Pragma("unroll") for (int k = 0; k < DV / 16; ++k) mma_ss(R2, kdesc(tG, k), kdesc(tV, k), id_kk, k > 0); // dO V^T of the next chunk
-                        mma_commit(bars + QM3);
+                        if (elect_one()) {
+                            _Pragma("unroll") for (int k = 0; k < DV / 16; ++k) mma_ss(R2, kdesc(tG, k), kdesc(tV, k), id_kk, k > 0); // dO V^T of the next chunk
+                            mma_commit(bars + QM3);
+                        }
                     }
                     QWAIT(QM6); if (!ok) break;                                                                  // the Q tile is done with:
-                    if (!last) load_key_features(t + 1);                                                         // the next chunk's Bf
+                    if (!last && elect_one()) load_key_features(t + 1);                                                         // the next chunk's Bf
                     QWAIT(QE4); if (!ok) break;                                                                  // this slab's part of dQ is staged where E was
-                    for (int a = 0; a < D / 64; ++a) {
-                        if (p.nslab > 1) tma_reduce_add_2d(&p.mapDQ, bX + a * 16384, a * 64, row0 + t * 128);
-                        else tma_store_2d(&p.mapDQ, bX + a * 16384, a * 64, row0 + t * 128);
-                    }
-                    tma_store_commit();
+                    if (elect_one())
+                        for (int a = 0; a < D / 64; ++a) {
+                            if (p.nslab > 1) tma_reduce_add_2d(&p.mapDQ, bX + a * 16384, a * 64, row0 + t * 128);
+                            else tma_store_2d(&p.mapDQ, bX + a * 16384, a * 64, row0 + t * 128);
+                        }
+                    if (elect_one()) tma_store_commit();
                     if (!last) {
-                        tma_store_wait_read();
-                        load_state(bX, t + 1);                                                                   // the next chunk's state
+                        if (elect_one()) {
+                            tma_store_wait_read();
+                            load_state(bX, t + 1);                                                                   // the next chunk's state
+                        }
                     }
 #undef QWAIT
                 }
             }
-            tma_store_wait_all();
+            if (elect_one()) tma_store_wait_all();
         }
     } else {
         // ============================== epilogue threads (see kEpiWarps)
@@ -448,7 +474,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_k_kernel(const __grid_cons
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + KNBARS);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + KNBARS + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5);
     const int bh = blockIdx.x / p.nslab, slab = blockIdx.x % p.nslab, h = bh % p.H;
     const int row0 = bh * p.N, rowk0 = kv_row0(bh, p.H, p.Hkv, p.N), T = p.T;      // rowk0: K and V may be shared by a group of query heads
     const int rowo0 = p.out_per_head ? row0 : rowk0;                                 // rows of dK and dV
@@ -465,13 +491,13 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_k_kernel(const __grid_cons
     __syncthreads();
     tc_fence_after();
     pdl_wait_tma();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = uniform(*tmem_slot);
     int *status = p.status;
 
     if (*abort_flag) {
         if (tid == 0) atomicExch(status, (int)DARKATTN_ERR_CUDA);
     } else if (warp == kEpiWarps) {
-        if ((tid & 31) == 0) {
+        {
             auto load_tile = [&](unsigned char *dst, const CUtensorMap *map, uint64_t *bar, int width, int t) {
                 mbar_expect_tx(bar, 128 * width * 2);
                 const int base = (map == &p.mapG) ? row0 : rowk0;
@@ -495,12 +521,14 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_k_kernel(const __grid_cons
             const uint32_t id_t = make_idesc(128, D, 1, 1);
             const uint32_t R1 = tmem + kColR1, R2 = tmem + kColR2;
 
-            mbar_expect_tx(bars + KB_OM, 128 * D * 2);
-            for (int a = 0; a < D / 64; ++a) tma_load_2d(sOm + a * 16384, &p.mapOm, bars + KB_OM, a * 64, h * p.m + slab * 128);
-            load_tile(sV, &p.mapV, bars + KB_V, DV, T - 1);
-            load_tile(sG, &p.mapG, bars + KB_G, DV, T - 1);
-            load_features(sQA, &p.mapAh, bars + KB_A, T - 1);
-            load_features(sKB, &p.mapBf, bars + KB_B, T - 1);
+            if (elect_one()) {
+                mbar_expect_tx(bars + KB_OM, 128 * D * 2);
+                for (int a = 0; a < D / 64; ++a) tma_load_2d(sOm + a * 16384, &p.mapOm, bars + KB_OM, a * 64, h * p.m + slab * 128);
+                load_tile(sV, &p.mapV, bars + KB_V, DV, T - 1);
+                load_tile(sG, &p.mapG, bars + KB_G, DV, T - 1);
+                load_features(sQA, &p.mapAh, bars + KB_A, T - 1);
+                load_features(sKB, &p.mapBf, bars + KB_B, T - 1);
+            }
 
             // Schedule of one chunk. A^ comes from the query-side kernel through the workspace, Bf from the forward pass
             // through the stash; V dO^T of the next chunk is issued in the tail of the current one.
@@ -515,71 +543,87 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_k_kernel(const __grid_cons
                 }
                 tma_store_commit();
             };
-            bool ok = wait_or_abort(bars + KB_OM, 0, status, abort_flag);
-            if (ok) ok = wait_or_abort(bars + KB_V, 0, status, abort_flag);
-            if (ok) ok = wait_or_abort(bars + KB_G, 0, status, abort_flag);
+            bool ok = warp_wait(bars + KB_OM, 0, status, abort_flag);
+            if (ok) ok = warp_wait(bars + KB_V, 0, status, abort_flag);
+            if (ok) ok = warp_wait(bars + KB_G, 0, status, abort_flag);
             if (ok) {
                 tc_fence_after();
-                _Pragma("unroll") for (int k = 0; k < DV / 16; ++k) mma_ss(R1, kdesc(tV, k), kdesc(tG, k), id_kk, k > 0);         // V dO^T of the last chunk
-                mma_commit(bars + KM3);
+                if (elect_one()) {
+                    _Pragma("unroll") for (int k = 0; k < DV / 16; ++k) mma_ss(R1, kdesc(tV, k), kdesc(tG, k), id_kk, k > 0);         // V dO^T of the last chunk
+                    mma_commit(bars + KM3);
+                }
             }
             for (int it = 0; it < T && ok; ++it) {
                 const int t = T - 1 - it;
                 const uint32_t ph = it & 1;
                 const bool first = (it == 0), last = (it + 1 == T);
-#define KWAIT(b) do { ok = wait_or_abort(bars + (b), ph, status, abort_flag); } while (0)
+#define KWAIT(b) do { ok = warp_wait(bars + (b), ph, status, abort_flag); } while (0)
                 KWAIT(KB_A); if (!ok) break;
                 KWAIT(KB_B); if (!ok) break;
                 tc_fence_after();
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R2, kdesc(tKB, k), kdesc(tQA, k), id_kk, k > 0);             // P^^T = Bf A^^T
-                mma_commit(bars + KM4);
-                if (!last) prefetch_features(&p.mapBf, t - 1);      // into L2 now: its load can only be issued late in the chunk
+                if (elect_one()) {
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R2, kdesc(tKB, k), kdesc(tQA, k), id_kk, k > 0);             // P^^T = Bf A^^T
+                    mma_commit(bars + KM4);
+                    if (!last) prefetch_features(&p.mapBf, t - 1);      // into L2 now: its load can only be issued late in the chunk
+                }
                 KWAIT(KE2); if (!ok) break;                                                                      // dP^T and P^^T packed in R1
                 tc_fence_after();
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(R2, R1 + 64 + k * 8, mndesc(tG, k), id_dv_t, k > 0);         // P^^T dO
-                if (!first)
-                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R2, kdesc(tKB, k), mndesc(tSt, k), id_dv_t, 1);          // + Bf R_next
-                tma_store_wait_read();      // the dK tile of the chunk before has left the spare tile: dV may be staged there
-                mma_commit(bars + KM6);
-                // the state update is not on the chunk's critical path: it runs while dV is read out
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColState, mndesc(tQA, k), mndesc(tG, k), id_state, (!first) || k > 0);   // R += A^^T dO
-                mma_commit(bars + KM5);
+                if (elect_one()) {
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(R2, R1 + 64 + k * 8, mndesc(tG, k), id_dv_t, k > 0);         // P^^T dO
+                    if (!first)
+                        _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R2, kdesc(tKB, k), mndesc(tSt, k), id_dv_t, 1);          // + Bf R_next
+                    tma_store_wait_read();      // the dK tile of the chunk before has left the spare tile: dV may be staged there
+                    mma_commit(bars + KM6);
+                    // the state update is not on the chunk's critical path: it runs while dV is read out
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColState, mndesc(tQA, k), mndesc(tG, k), id_state, (!first) || k > 0);   // R += A^^T dO
+                    mma_commit(bars + KM5);
+                }
                 KWAIT(KE3); if (!ok) break;                                                                      // dV read out of R2 and staged
-                store_out(&p.mapDV, DV, t);
+                if (elect_one()) store_out(&p.mapDV, DV, t);
                 tc_fence_after();
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(R2, R1 + k * 8, mndesc(tQA, k), id_tm, k > 0);               // dP^T A^
-                if (!first)
-                    _Pragma("unroll") for (int k = 0; k < DV / 16; ++k) mma_ss(R2, kdesc(tV, k), kdesc(tSt, k), id_kk, 1);        // + V R_next^T
-                mma_commit(bars + KM7);
+                if (elect_one()) {
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(R2, R1 + k * 8, mndesc(tQA, k), id_tm, k > 0);               // dP^T A^
+                    if (!first)
+                        _Pragma("unroll") for (int k = 0; k < DV / 16; ++k) mma_ss(R2, kdesc(tV, k), kdesc(tSt, k), id_kk, 1);        // + V R_next^T
+                    mma_commit(bars + KM7);
+                }
                 KWAIT(KM7); if (!ok) break;                                                                      // A^, V and dO of this chunk are done with
-                tma_store_wait_read();                                                                           // the staged dV has left the spare tile:
-                load_tile(sStg, &p.mapK, bars + KB_X2, D, t);                                                   // the K tile, for T
+                if (elect_one()) {
+                    tma_store_wait_read();                                                                           // the staged dV has left the spare tile:
+                    load_tile(sStg, &p.mapK, bars + KB_X2, D, t);                                                   // the K tile, for T
+                }
                 if (!last) {
-                    load_features(sQA, &p.mapAh, bars + KB_A, t - 1);
-                    load_tile(sV, &p.mapV, bars + KB_V, DV, t - 1);
-                    load_tile(sG, &p.mapG, bars + KB_G, DV, t - 1);
+                    if (elect_one()) {
+                        load_features(sQA, &p.mapAh, bars + KB_A, t - 1);
+                        load_tile(sV, &p.mapV, bars + KB_V, DV, t - 1);
+                        load_tile(sG, &p.mapG, bars + KB_G, DV, t - 1);
+                    }
                 }
                 KWAIT(KE4); if (!ok) break;                                                                      // E in smem, R2 read
                 KWAIT(KB_X2); if (!ok) break;
                 tc_fence_after();
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColT, mndesc(tKB, k), mndesc(tStg, k), id_t, (!first) || k > 0);   // T += E^T K
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R2, kdesc(tKB, k), mndesc(tOm, k), id_dx, k > 0);            // E Omega
-                mma_commit(bars + KM8);
+                if (elect_one()) {
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColT, mndesc(tKB, k), mndesc(tStg, k), id_t, (!first) || k > 0);   // T += E^T K
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R2, kdesc(tKB, k), mndesc(tOm, k), id_dx, k > 0);            // E Omega
+                    mma_commit(bars + KM8);
+                }
                 if (!last) {
-                    ok = wait_or_abort(bars + KB_V, ph ^ 1, status, abort_flag);
-                    if (ok) ok = wait_or_abort(bars + KB_G, ph ^ 1, status, abort_flag);
+                    ok = warp_wait(bars + KB_V, ph ^ 1, status, abort_flag);
+                    if (ok) ok = warp_wait(bars + KB_G, ph ^ 1, status, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    _Pragma("unroll") for (int k = 0; k < DV / 16; ++k) mma_ss(R1, kdesc(tV, k), kdesc(tG, k), id_kk, k > 0);     // V dO^T of the next chunk
-                    mma_commit(bars + KM3);
+                    if (elect_one()) {
+                        _Pragma("unroll") for (int k = 0; k < DV / 16; ++k) mma_ss(R1, kdesc(tV, k), kdesc(tG, k), id_kk, k > 0);     // V dO^T of the next chunk
+                        mma_commit(bars + KM3);
+                    }
                 }
                 KWAIT(KM8); if (!ok) break;                                                                      // E and the K tile are done with
-                if (!last) load_features(sKB, &p.mapBf, bars + KB_B, t - 1);
+                if (!last && elect_one()) load_features(sKB, &p.mapBf, bars + KB_B, t - 1);
                 KWAIT(KE5); if (!ok) break;                                                                      // dK read out of R2 and staged; bf16 copy of R in place
-                store_out(&p.mapDK, D, t);
+                if (elect_one()) store_out(&p.mapDK, D, t);
 #undef KWAIT
             }
-            tma_store_wait_all();
+            if (elect_one()) tma_store_wait_all();
         }
     } else {
         const int lane = tid & 31, q4 = warp & 3, g = warp >> 2, col0 = g * 32;
@@ -722,7 +766,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_finish_k_kernel(const __gr
     uint64_t *e1 = bars + 7, *e2 = bars + 8;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 10);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + 11);
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5);
     const int bh = blockIdx.x / p.nsplit, split = blockIdx.x % p.nsplit, h = bh % p.H;
     const int t0 = (int)((long long)p.T * split / p.nsplit), t1 = (int)((long long)p.T * (split + 1) / p.nsplit);
     const size_t rows = (size_t)p.BH * p.N;
@@ -739,55 +783,63 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_finish_k_kernel(const __gr
     __syncthreads();
     tc_fence_after();
     pdl_wait_tma();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = uniform(*tmem_slot);
     constexpr uint32_t C1 = 0, C2 = 128, C3 = 256;
     if (*abort_flag) { if (tid == 0) atomicExch(p.status, (int)DARKATTN_ERR_CUDA); }
     else if (t1 <= t0) {}
     else if (warp == kEpiWarps) {
-        if ((tid & 31) == 0) {
+        {
             const TileDesc tM(sM), tW(sW), tK0(sK0), tK1(sK0 + kTile);
             auto load_k = [&](int t) {
                 const int b = (t - t0) & 1;
                 mbar_expect_tx(bar_k + b, kTile);
                 for (int a = 0; a < D / 64; ++a) tma_load_2d(sK0 + b * kTile + a * 16384, &p.mapK, bar_k + b, a * 64, kv_row0(bh, p.H, p.Hkv, p.N) + t * 128);
             };
-            mbar_expect_tx(bar_m, kTile);
-            for (int a = 0; a < D / 64; ++a) tma_load_2d(sM + a * 16384, &p.mapM, bar_m, a * 64, h * p.r);
-            load_k(t0);
+            if (elect_one()) {
+                mbar_expect_tx(bar_m, kTile);
+                for (int a = 0; a < D / 64; ++a) tma_load_2d(sM + a * 16384, &p.mapM, bar_m, a * 64, h * p.r);
+                load_k(t0);
+            }
             const uint32_t id_x = make_idesc(128, p.r, 0, 0), id_d = make_idesc(128, D, 0, 1), id_t = make_idesc(128, D, 1, 1);
             // K M^T of tile i+1 is issued right behind the two products of tile i, so that it runs while the epilogue
             // warps still write tile i out.
-            bool ok = wait_or_abort(bar_m, 0, p.status, abort_flag);
-            if (t0 + 1 < t1) load_k(t0 + 1);
-            if (ok) ok = wait_or_abort(bar_k, 0, p.status, abort_flag);
+            bool ok = warp_wait(bar_m, 0, p.status, abort_flag);
+            if (t0 + 1 < t1 && elect_one()) load_k(t0 + 1);
+            if (ok) ok = warp_wait(bar_k, 0, p.status, abort_flag);
             if (ok) {
                 tc_fence_after();
-                _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(tmem + C1, kdesc(tK0, k), kdesc(tM, k), id_x, k > 0);
-                mma_commit(m1);
+                if (elect_one()) {
+                    _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(tmem + C1, kdesc(tK0, k), kdesc(tM, k), id_x, k > 0);
+                    mma_commit(m1);
+                }
             }
             for (int t = t0; t < t1 && ok; ++t) {
                 const int i = t - t0, b = i & 1;
                 const uint32_t ph = i & 1;
                 const TileDesc &tK = b ? tK1 : tK0;
-                ok = wait_or_abort(e1, ph, p.status, abort_flag);
+                ok = warp_wait(e1, ph, p.status, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
-                for (int k = 0; k < p.r / 16; ++k) mma_ss(tmem + C2, kdesc(tW, k), mndesc(tM, k), id_d, k > 0);
-                mma_commit(m2);
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + C3, mndesc(tW, k), mndesc(tK, k), id_t, (t > t0) || k > 0);
-                mma_commit(m3);
+                if (elect_one()) {
+                    for (int k = 0; k < p.r / 16; ++k) mma_ss(tmem + C2, kdesc(tW, k), mndesc(tM, k), id_d, k > 0);
+                    mma_commit(m2);
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + C3, mndesc(tW, k), mndesc(tK, k), id_t, (t > t0) || k > 0);
+                    mma_commit(m3);
+                }
                 if (t + 1 < t1) {
-                    ok = wait_or_abort(bar_k + (b ^ 1), ((i + 1) >> 1) & 1, p.status, abort_flag);
+                    ok = warp_wait(bar_k + (b ^ 1), ((i + 1) >> 1) & 1, p.status, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
                     const TileDesc &tKn = b ? tK0 : tK1;
-                    _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(tmem + C1, kdesc(tKn, k), kdesc(tM, k), id_x, k > 0);
-                    mma_commit(m1);
+                    if (elect_one()) {
+                        _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(tmem + C1, kdesc(tKn, k), kdesc(tM, k), id_x, k > 0);
+                        mma_commit(m1);
+                    }
                 }
-                ok = wait_or_abort(m3, ph, p.status, abort_flag);
+                ok = warp_wait(m3, ph, p.status, abort_flag);
                 if (!ok) break;
-                if (t + 2 < t1) load_k(t + 2);          // this tile's K buffer has been read by both of its products
-                ok = wait_or_abort(e2, ph, p.status, abort_flag);
+                if (t + 2 < t1 && elect_one()) load_k(t + 2);          // this tile's K buffer has been read by both of its products
+                ok = warp_wait(e2, ph, p.status, abort_flag);
             }
         }
     } else {

@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_nc_kernel(const __gri
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + NNBARS);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + NNBARS + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5);
     const int unit = blockIdx.x / p.nsplit, piece = blockIdx.x % p.nsplit;
     const int bh = unit / p.nslab, slab = unit % p.nslab, h = bh % p.H;
     const int row0 = bh * p.N;
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_nc_kernel(const __gri
     pdl_wait_tma();
     if (tid < 128) sVec[tid] = (KEYS ? p.rhot : p.zt)[(size_t)bh * p.m + slab * 128 + tid];
     __syncthreads();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = uniform(*tmem_slot);
     int *status = p.status;
 
     if (*abort_flag) {
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_nc_kernel(const __gri
     } else if (nt <= 0) {
         // nothing to do for this piece
     } else if (warp == kEpiWarps) {
-        if ((tid & 31) == 0) {
+        {
             auto load_tile = [&](unsigned char *dst, const CUtensorMap *map, uint64_t *bar, int width, int t) {
                 mbar_expect_tx(bar, 128 * width * 2);
                 const int base = (map == &p.mapX) ? rowx0 : rowy0;
@@ -133,28 +133,33 @@ __global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_nc_kernel(const __gri
             const uint32_t id_t = make_idesc(128, D, 1, 1);
             const uint32_t R1 = tmem + kColR1, R2 = tmem + kColR2;
 
-            mbar_expect_tx(bars + NB_OM, 2 * 128 * D * 2 + 128 * DV * 2);
-            for (int a = 0; a < D / 64; ++a) {
-                tma_load_2d(sOm + a * 16384, &p.mapOm, bars + NB_OM, a * 64, h * p.m + slab * 128);
-                tma_load_2d(sOml + a * 16384, &p.mapOml, bars + NB_OM, a * 64, h * p.m + slab * 128);
+            if (elect_one()) mbar_expect_tx(bars + NB_OM, 2 * 128 * D * 2 + 128 * DV * 2);
+            if (elect_one())
+                for (int a = 0; a < D / 64; ++a) {
+                    tma_load_2d(sOm + a * 16384, &p.mapOm, bars + NB_OM, a * 64, h * p.m + slab * 128);
+                    tma_load_2d(sOml + a * 16384, &p.mapOml, bars + NB_OM, a * 64, h * p.m + slab * 128);
+                }
+            if (elect_one()) {
+                for (int a = 0; a < DV / 64; ++a) tma_load_2d(sSt + a * 16384, &p.mapSt, bars + NB_OM, a * 64, bh * p.m + slab * 128);
+                load_tile(sX, &p.mapX, bars + NB_X0, D, tbeg);
+                load_tile(sY, &p.mapY, bars + NB_Y, DV, tbeg);
             }
-            for (int a = 0; a < DV / 64; ++a) tma_load_2d(sSt + a * 16384, &p.mapSt, bars + NB_OM, a * 64, bh * p.m + slab * 128);
-            load_tile(sX, &p.mapX, bars + NB_X0, D, tbeg);
-            load_tile(sY, &p.mapY, bars + NB_Y, DV, tbeg);
 
-            bool ok = wait_or_abort(bars + NB_OM, 0, status, abort_flag);
-            if (ok) ok = wait_or_abort(bars + NB_X0, 0, status, abort_flag);
+            bool ok = warp_wait(bars + NB_OM, 0, status, abort_flag);
+            if (ok) ok = warp_wait(bars + NB_X0, 0, status, abort_flag);
             if (ok) {
                 tc_fence_after();
-                issue_projection<D>(R1, tX0, tOm, tOml, id_kk);                                                  // U of the first tile
-                mma_commit(bars + NM1);
+                if (elect_one()) {
+                    issue_projection<D>(R1, tX0, tOm, tOml, id_kk);                                                  // U of the first tile
+                    mma_commit(bars + NM1);
+                }
             }
             for (int it = 0; it < nt && ok; ++it) {
                 const int t = tbeg + it;
                 const uint32_t ph = it & 1;
                 const bool first = (it == 0), last = (it + 1 == nt);
                 const TileDesc &tX = (it & 1) ? tX1 : tX0;
-#define NWAIT(b, q) do { ok = wait_or_abort(bars + (b), (q), status, abort_flag); } while (0)
+#define NWAIT(b, q) do { ok = warp_wait(bars + (b), (q), status, abort_flag); } while (0)
                 auto store_out = [&](const CUtensorMap *map, unsigned char *src, int width, int tt) {     // (adds into the gradient when the head has several slabs)
                     const bool add = KEYS ? (p.add_kv != 0) : (p.nslab > 1);
                     for (int a = 0; a < width / 64; ++a) {
@@ -166,44 +171,54 @@ __global__ void __launch_bounds__(kClearThreads, 1) tc_bwd_nc_kernel(const __gri
                 NWAIT(NB_Y, ph); if (!ok) break;
                 if (!first) {                                                       // the tile before: R2 read out, its part of dQ | dK staged in its X buffer
                     NWAIT(NE3, ph ^ 1); if (!ok) break;
-                    store_out(&p.mapOut, sX + ((it + 1) & 1) * 128 * D * 2, D, t - 1);
+                    if (elect_one()) store_out(&p.mapOut, sX + ((it + 1) & 1) * 128 * D * 2, D, t - 1);
                 }
                 tc_fence_after();
-                _Pragma("unroll") for (int k = 0; k < DV / 16; ++k) mma_ss(R2, kdesc(tY, k), kdesc(tSt, k), id_kk, k > 0);      // dO S^T | V R^T
-                mma_commit(bars + NMA);
-                if (!first) tma_store_wait_read();                                  // the staged tile has left the X buffer
-                if (!last) load_tile(sX + ((it + 1) & 1) * 128 * D * 2, &p.mapX, bars + NB_X0 + ((it + 1) & 1), D, t + 1);
+                if (elect_one()) {
+                    _Pragma("unroll") for (int k = 0; k < DV / 16; ++k) mma_ss(R2, kdesc(tY, k), kdesc(tSt, k), id_kk, k > 0);      // dO S^T | V R^T
+                    mma_commit(bars + NMA);
+                    if (!first) tma_store_wait_read();                                  // the staged tile has left the X buffer
+                    if (!last) load_tile(sX + ((it + 1) & 1) * 128 * D * 2, &p.mapX, bars + NB_X0 + ((it + 1) & 1), D, t + 1);
+                }
                 NWAIT(NE1, ph); if (!ok) break;                                     // features in smem, R1 read
                 tc_fence_after();
                 if (KEYS) {
-                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R1, kdesc(tA, k), mndesc(tSt, k), id_dv, k > 0);        // dV = Bf R
+                    if (elect_one()) _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R1, kdesc(tA, k), mndesc(tSt, k), id_dv, k > 0);        // dV = Bf R
                 } else {
-                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R1, mndesc(tA, k), vecdesc(tDel, k), id_vec, k > 0);   // rho_c = -A^^T delta (columns 0, 1)
-                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColState, mndesc(tA, k), mndesc(tY, k), id_state, (!first) || k > 0);   // R += A^^T dO
+                    if (elect_one()) {
+                        _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R1, mndesc(tA, k), vecdesc(tDel, k), id_vec, k > 0);   // rho_c = -A^^T delta (columns 0, 1)
+                        _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColState, mndesc(tA, k), mndesc(tY, k), id_state, (!first) || k > 0);   // R += A^^T dO
+                    }
                 }
-                mma_commit(bars + NM2);
+                if (elect_one()) mma_commit(bars + NM2);
                 NWAIT(NE2, ph); if (!ok) break;                                     // E in smem; R1 and R2 read; key pass: dV staged over the V tile
-                if (KEYS) store_out(&p.mapDV, sY, DV, t);
-                else if (!last) load_tile(sY, &p.mapY, bars + NB_Y, DV, t + 1);
+                if (elect_one()) {
+                    if (KEYS) store_out(&p.mapDV, sY, DV, t);
+                    else if (!last) load_tile(sY, &p.mapY, bars + NB_Y, DV, t + 1);
+                }
                 tc_fence_after();
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R2, kdesc(tA, k), mndesc(tOm, k), id_dx, k > 0);            // E Omega
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColT, mndesc(tA, k), mndesc(tX, k), id_t, (!first) || k > 0);   // T += E^T X
-                mma_commit(bars + NM3);
+                if (elect_one()) {
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(R2, kdesc(tA, k), mndesc(tOm, k), id_dx, k > 0);            // E Omega
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColT, mndesc(tA, k), mndesc(tX, k), id_t, (!first) || k > 0);   // T += E^T X
+                    mma_commit(bars + NM3);
+                }
                 if (!last) {       // U of the next tile behind them (R1 has been read): its features can be formed at once
                     NWAIT(NB_X0 + ((it + 1) & 1), ((it + 1) >> 1) & 1); if (!ok) break;
                     tc_fence_after();
                     const TileDesc &tXn = ((it + 1) & 1) ? tX1 : tX0;
-                    issue_projection<D>(R1, tXn, tOm, tOml, id_kk);
-                    mma_commit(bars + NM1);
+                    if (elect_one()) {
+                        issue_projection<D>(R1, tXn, tOm, tOml, id_kk);
+                        mma_commit(bars + NM1);
+                    }
                 }
-                if (KEYS && !last) { tma_store_wait_read(); load_tile(sY, &p.mapY, bars + NB_Y, DV, t + 1); }     // the staged dV has left the V tile's buffer
+                if (KEYS && !last && elect_one()) { tma_store_wait_read(); load_tile(sY, &p.mapY, bars + NB_Y, DV, t + 1); }     // the staged dV has left the V tile's buffer
                 if (last) {        // the last tile's part of dQ | dK
                     NWAIT(NE3, ph); if (!ok) break;
-                    store_out(&p.mapOut, sX + (it & 1) * 128 * D * 2, D, t);
+                    if (elect_one()) store_out(&p.mapOut, sX + (it & 1) * 128 * D * 2, D, t);
                 }
 #undef NWAIT
             }
-            tma_store_wait_all();
+            if (elect_one()) tma_store_wait_all();
         }
     } else {
         const int lane = tid & 31, q4 = warp & 3, g = warp >> 2, col0 = g * 32;

@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(160, 1) tc_key_prepass_kernel(const __grid_con
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + 5 * kTile);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + PNBARS);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + PNBARS + 1);
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5);
     const int unit = blockIdx.x / p.nsplit, split = blockIdx.x % p.nsplit;
     const int bh = unit / p.npair, pair = unit % p.npair, h = bh % p.H;
     const int slab0 = 2 * pair, ns = (slab0 + 1 < p.nslab) ? 2 : 1;           // this CTA's one or two slabs
@@ -145,46 +145,52 @@ __global__ void __launch_bounds__(160, 1) tc_key_prepass_kernel(const __grid_con
     __syncthreads();
     tc_fence_after();
     pdl_wait_tma();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = uniform(*tmem_slot);
     constexpr uint32_t kColX = 0, kColU = 128;      // x~ at 0, U of the two slabs at 128 and 256
     if (*abort_flag) { if (tid == 0) atomicExch(p.status, (int)DARKATTN_ERR_CUDA); }
     else if (warp == 4) {
-        if ((tid & 31) == 0 && t1 > t0) {
+        if (t1 > t0) {
             auto load_k = [&](int t) {
                 const int b = (t - t0) & 1;
                 mbar_expect_tx(bars + PB_K0 + b, kTile);
                 for (int a = 0; a < D / 64; ++a) tma_load_2d(sK + b * kTile + a * 16384, &p.mapK, bars + PB_K0 + b, a * 64, rowk0 + t * 128);
             };
-            mbar_expect_tx(bars + PB_M, kTile * (1 + ns));
-            for (int a = 0; a < D / 64; ++a) {
-                tma_load_2d(sM + a * 16384, &p.mapM, bars + PB_M, a * 64, h * p.r);
-                for (int s = 0; s < ns; ++s) tma_load_2d(sOm + s * kTile + a * 16384, &p.mapOm, bars + PB_M, a * 64, h * p.m + (slab0 + s) * 128);
+            if (elect_one()) {
+                mbar_expect_tx(bars + PB_M, kTile * (1 + ns));
+                for (int a = 0; a < D / 64; ++a) {
+                    tma_load_2d(sM + a * 16384, &p.mapM, bars + PB_M, a * 64, h * p.r);
+                    for (int s = 0; s < ns; ++s) tma_load_2d(sOm + s * kTile + a * 16384, &p.mapOm, bars + PB_M, a * 64, h * p.m + (slab0 + s) * 128);
+                }
+                load_k(t0);
+                if (t0 + 1 < t1) load_k(t0 + 1);
             }
-            load_k(t0);
-            if (t0 + 1 < t1) load_k(t0 + 1);
             const TileDesc tM(sM), tOm0(sOm), tOm1(sOm + kTile), tK0(sK), tK1(sK + kTile);
             const uint32_t id_x = make_idesc(128, p.r, 0, 0), id_u = make_idesc(128, 128, 0, 0);
-            bool ok = wait_or_abort(bars + PB_M, 0, p.status, abort_flag);
+            bool ok = warp_wait(bars + PB_M, 0, p.status, abort_flag);
             for (int t = t0; t < t1 && ok; ++t) {
                 const int i = t - t0, b = i & 1;
                 const uint32_t ph = i & 1, phk = (i >> 1) & 1;
                 const TileDesc &tK = b ? tK1 : tK0;
-                ok = wait_or_abort(bars + PB_K0 + b, phk, p.status, abort_flag);
-                if (ok && i > 0) ok = wait_or_abort(bars + PEX, ph ^ 1, p.status, abort_flag);       // x~ of the tile before has been read
+                ok = warp_wait(bars + PB_K0 + b, phk, p.status, abort_flag);
+                if (ok && i > 0) ok = warp_wait(bars + PEX, ph ^ 1, p.status, abort_flag);       // x~ of the tile before has been read
                 if (!ok) break;
                 tc_fence_after();
-                _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(tmem + kColX, kdesc(tK, k), kdesc(tM, k), id_x, k > 0);
-                mma_commit(bars + PMX);
-                if (i > 0) { ok = wait_or_abort(bars + PEU, ph ^ 1, p.status, abort_flag); if (!ok) break; }      // U of the tile before has been read
+                if (elect_one()) {
+                    _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(tmem + kColX, kdesc(tK, k), kdesc(tM, k), id_x, k > 0);
+                    mma_commit(bars + PMX);
+                }
+                if (i > 0) { ok = warp_wait(bars + PEU, ph ^ 1, p.status, abort_flag); if (!ok) break; }      // U of the tile before has been read
                 tc_fence_after();
-                _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(tmem + kColU, kdesc(tK, k), kdesc(tOm0, k), id_u, k > 0);
-                if (ns == 2)
-                    _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(tmem + kColU + 128, kdesc(tK, k), kdesc(tOm1, k), id_u, k > 0);
-                mma_commit(bars + PMU);
+                if (elect_one()) {
+                    _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(tmem + kColU, kdesc(tK, k), kdesc(tOm0, k), id_u, k > 0);
+                    if (ns == 2)
+                        _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(tmem + kColU + 128, kdesc(tK, k), kdesc(tOm1, k), id_u, k > 0);
+                    mma_commit(bars + PMU);
+                }
                 if (t + 2 < t1) {       // this tile's buffer is free once its MMAs are done
-                    ok = wait_or_abort(bars + PMU, ph, p.status, abort_flag);
+                    ok = warp_wait(bars + PMU, ph, p.status, abort_flag);
                     if (!ok) break;
-                    load_k(t + 2);
+                    if (elect_one()) load_k(t + 2);
                 }
             }
         }
@@ -502,7 +508,7 @@ __global__ void __launch_bounds__(kCausalThreads, 1) tc_fwd_causal_kernel(const 
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + CNBARS);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + CNBARS + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5);
     if (blockIdx.x >= p.scan_ctas) {                // (takes no tensor memory)
         sum_tiles<DV>(p);
         return;
@@ -527,7 +533,7 @@ __global__ void __launch_bounds__(kCausalThreads, 1) tc_fwd_causal_kernel(const 
     __syncthreads();
     tc_fence_after();
     pdl_wait_tma();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = uniform(*tmem_slot);
     if (tid < 128) sZ[tid] = fresh ? 0.f : p.zseg[((size_t)bh * p.nsplit + seg) * p.m + slab * 128 + tid];      // (read after the barrier below)
     int *status = p.status;
     if (!fresh && warp < kEpiWarps) {      // the segment's prefix state into the fp32 accumulators in TMEM
@@ -562,16 +568,20 @@ __global__ void __launch_bounds__(kCausalThreads, 1) tc_fwd_causal_kernel(const 
         if (tid == 0) atomicExch(status, (int)DARKATTN_ERR_CUDA);
     } else if (tend <= tbeg) {
     } else if (warp == kEpiWarps) {
-        if ((tid & 31) == 0) {
+        {
             const int rowk0 = kv_row0(bh, p.H, p.Hkv, p.N);       // K and V may be shared by a group of query heads
             auto load_tile = [&](unsigned char *dst, const CUtensorMap *map, uint64_t *bar, int width, int t) {
                 const int base = (map == &p.mapQ) ? row0 : rowk0;
-                mbar_expect_tx(bar, 128 * width * 2);
-                for (int a = 0; a < width / 64; ++a) tma_load_2d(dst + a * 16384, map, bar, a * 64, base + t * 128);
+                if (elect_one()) {
+                    mbar_expect_tx(bar, 128 * width * 2);
+                    for (int a = 0; a < width / 64; ++a) tma_load_2d(dst + a * 16384, map, bar, a * 64, base + t * 128);
+                }
             };
             auto store_state = [&](int t) {        // the bf16 state before chunk t, for the backward pass
-                for (int a = 0; a < DV / 64; ++a) tma_store_2d(&p.mapSst, sSb + a * 16384, a * 64, (bh * p.T + t) * p.m + slab * 128);
-                tma_store_commit();
+                if (elect_one()) {
+                    for (int a = 0; a < DV / 64; ++a) tma_store_2d(&p.mapSst, sSb + a * 16384, a * 64, (bh * p.T + t) * p.m + slab * 128);
+                    tma_store_commit();
+                }
             };
             const TileDesc tOm(sOm), tOml(sOml), tQ(sQ), tK(sK), tV(sV), tFK(sFK), tSb(sSb);
             const uint64_t ones_desc = make_sdesc(smem_u32(sRed), 16384, 1024);
@@ -581,32 +591,38 @@ __global__ void __launch_bounds__(kCausalThreads, 1) tc_fwd_causal_kernel(const 
             const uint32_t id_z = make_idesc(128, 16, 1, 1);
             const uint32_t R1 = tmem + kColR1, R2 = tmem + kColR2, FQ = tmem + kColFQ;
 
-            mbar_expect_tx(bars + CB_OM, 2 * 128 * D * 2 + (fresh ? 0 : 128 * DV * 2));
-            for (int a = 0; a < D / 64; ++a) {
-                tma_load_2d(sOm + a * 16384, &p.mapOm, bars + CB_OM, a * 64, h * p.m + slab * 128);
-                tma_load_2d(sOml + a * 16384, &p.mapOml, bars + CB_OM, a * 64, h * p.m + slab * 128);
+            if (elect_one()) {
+                mbar_expect_tx(bars + CB_OM, 2 * 128 * D * 2 + (fresh ? 0 : 128 * DV * 2));
+                for (int a = 0; a < D / 64; ++a) {
+                    tma_load_2d(sOm + a * 16384, &p.mapOm, bars + CB_OM, a * 64, h * p.m + slab * 128);
+                    tma_load_2d(sOml + a * 16384, &p.mapOml, bars + CB_OM, a * 64, h * p.m + slab * 128);
+                }
+                if (!fresh)     // bf16 copy of the segment's prefix state
+                    for (int a = 0; a < DV / 64; ++a)
+                        tma_load_2d(sSb + a * 16384, &p.mapSb, bars + CB_OM, a * 64, (bh * p.nsplit + seg) * p.m + slab * 128);
             }
-            if (!fresh)     // bf16 copy of the segment's prefix state
-                for (int a = 0; a < DV / 64; ++a)
-                    tma_load_2d(sSb + a * 16384, &p.mapSb, bars + CB_OM, a * 64, (bh * p.nsplit + seg) * p.m + slab * 128);
             load_tile(sQ, &p.mapQ, bars + CB_Q, D, tbeg);
             load_tile(sK, &p.mapK, bars + CB_K, D, tbeg);
             load_tile(sV, &p.mapV, bars + CB_V, DV, tbeg);
 
-#define CWAIT(b, q) do { ok = wait_or_abort(bars + (b), (q), status, abort_flag); } while (0)
+#define CWAIT(b, q) do { ok = warp_wait(bars + (b), (q), status, abort_flag); } while (0)
             bool ok = true;
             CWAIT(CB_OM, 0);
             if (ok) CWAIT(CB_Q, 0);
             if (ok) {
                 tc_fence_after();
-                issue_projection<D>(R1, tQ, tOm, tOml, id_kk);                                                    // U_Q of the first chunk
-                mma_commit(bars + CM1);
+                if (elect_one()) {
+                    issue_projection<D>(R1, tQ, tOm, tOml, id_kk);                                                // U_Q of the first chunk
+                    mma_commit(bars + CM1);
+                }
                 CWAIT(CB_K, 0);
             }
             if (ok) {
                 tc_fence_after();
-                issue_projection<D>(R2, tK, tOm, tOml, id_kk);                                                    // U_K of the first chunk
-                mma_commit(bars + CM2);
+                if (elect_one()) {
+                    issue_projection<D>(R2, tK, tOm, tOml, id_kk);                                                // U_K of the first chunk
+                    mma_commit(bars + CM2);
+                }
                 CWAIT(CE0, 0);                                                  // phi(Q) packed, Q tile consumed
             }
             if (ok && tbeg + 1 < tend) load_tile(sQ, &p.mapQ, bars + CB_Q, D, tbeg + 1);
@@ -615,44 +631,56 @@ __global__ void __launch_bounds__(kCausalThreads, 1) tc_fwd_causal_kernel(const 
                 const bool first = (t == tbeg) && fresh, last = (t + 1 == tend);
                 CWAIT(CE1, ph); if (!ok) break;                                 // phi(K) and the ones in smem, R2 read, K tile consumed
                 if (!last) load_tile(sK, &p.mapK, bars + CB_K, D, t + 1);
-                if (p.stash_S) {        // the backward kernels read the key features back instead of forming them again
+                if (p.stash_S && elect_one()) {         // the backward kernels read the key features back instead of forming them again
                     tma_store_2d(&p.mapBf, sFK, slab * 128, row0 + t * 128);
                     tma_store_2d(&p.mapBf, sFK + 16384, slab * 128 + 64, row0 + t * 128);
                     tma_store_commit();
                 }
                 tc_fence_after();
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(R1, FQ + k * 8, kdesc(tFK, k), id_kk, k > 0);                // P = phi(Q) phi(K)^T
-                mma_commit(bars + CM3);
+                if (elect_one()) {
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(R1, FQ + k * 8, kdesc(tFK, k), id_kk, k > 0);            // P = phi(Q) phi(K)^T
+                    mma_commit(bars + CM3);
+                }
                 if (!first) {
                     if (t > tbeg) {                                             // the bf16 state through chunk t - 1 is in smem
                         CWAIT(CE4, ph ^ 1); if (!ok) break;
                         if (p.stash_S) store_state(t);
                     }
-                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(R2, FQ + k * 8, mndesc(tSb, k), id_o, k > 0);            // O = phi(Q) S_prev
+                    if (elect_one())
+                        _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(R2, FQ + k * 8, mndesc(tSb, k), id_o, k > 0);        // O = phi(Q) S_prev
                 }
-                _Pragma("unroll") for (int k = 0; k < 8; ++k)                                                                     // z += phi(K)^T 1
-                    mma_ss(tmem + kColZ + 16 * (k & 3), mndesc(tFK, k), ones_desc, id_z, (!first) || k >= 4);
+                if (elect_one())
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k)                                                                 // z += phi(K)^T 1
+                        mma_ss(tmem + kColZ + 16 * (k & 3), mndesc(tFK, k), ones_desc, id_z, (!first) || k >= 4);
                 CWAIT(CB_V, ph); if (!ok) break;
                 CWAIT(CE2, ph); if (!ok) break;                                 // tril(P) packed in R1
                 tc_fence_after();
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(R2, R1 + k * 8, mndesc(tV, k), id_o, (!first) || k > 0);     // O += P V
-                if (p.stash_S) tma_store_wait_read();       // the stash copies of the state before this chunk and of phi(K) have left their tiles: the output may be
+                if (elect_one()) {
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(R2, R1 + k * 8, mndesc(tV, k), id_o, (!first) || k > 0); // O += P V
+                    if (p.stash_S) tma_store_wait_read();   // the stash copies of the state before this chunk and of phi(K) have left their tiles: the output may be
                                                             // staged in the first, the next phi(K) written to the second
-                mma_commit(bars + CM4);
+                    mma_commit(bars + CM4);
+                }
                 if (!last) {        // U_Q of the next chunk, while the epilogue warps read the output tile out
                     CWAIT(CB_Q, ph ^ 1); if (!ok) break;
                     tc_fence_after();
-                    issue_projection<D>(R1, tQ, tOm, tOml, id_kk);
-                    mma_commit(bars + CM1);
+                    if (elect_one()) {
+                        issue_projection<D>(R1, tQ, tOm, tOml, id_kk);
+                        mma_commit(bars + CM1);
+                    }
                 }
-                _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColS, mndesc(tFK, k), mndesc(tV, k), id_s, (!first) || k > 0);   // S += phi(K)^T V
-                mma_commit(bars + CMS);
+                if (elect_one()) {
+                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ss(tmem + kColS, mndesc(tFK, k), mndesc(tV, k), id_s, (!first) || k > 0);   // S += phi(K)^T V
+                    mma_commit(bars + CMS);
+                }
                 CWAIT(CE3, ph); if (!ok) break;                                 // the output tile has been read out of R2 and staged
                 if (!last) {
                     CWAIT(CB_K, ph ^ 1); if (!ok) break;
                     tc_fence_after();
-                    issue_projection<D>(R2, tK, tOm, tOml, id_kk);                                                // U_K of the next chunk
-                    mma_commit(bars + CM2);
+                    if (elect_one()) {
+                        issue_projection<D>(R2, tK, tOm, tOml, id_kk);                                            // U_K of the next chunk
+                        mma_commit(bars + CM2);
+                    }
                 }
                 CWAIT(CMS, ph); if (!ok) break;                                 // V tile consumed
                 if (!last) {
@@ -666,7 +694,7 @@ __global__ void __launch_bounds__(kCausalThreads, 1) tc_fwd_causal_kernel(const 
                 if (ok) store_state(tend);
             }
 #undef CWAIT
-            tma_store_wait_all();
+            if (elect_one()) tma_store_wait_all();
         }
     } else if (warp == kEpiWarps + 1) {
         if ((tid & 31) == 0) {
@@ -894,7 +922,7 @@ __global__ void __launch_bounds__(kKeysThreads, 1) tc_fwd_keys_kernel(const __gr
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L::kBars);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + YNBARS);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + YNBARS + 1);
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5);
 
     if (tid == 0) {
         for (int i = 0; i < YB_E; ++i) mbar_init(bars + i, 1);
@@ -908,7 +936,7 @@ __global__ void __launch_bounds__(kKeysThreads, 1) tc_fwd_keys_kernel(const __gr
     __syncthreads();
     tc_fence_after();
     pdl_wait_tma();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = uniform(*tmem_slot);
     int *status = p.status;
     PieceList list(p);
     Piece c;
@@ -916,96 +944,105 @@ __global__ void __launch_bounds__(kKeysThreads, 1) tc_fwd_keys_kernel(const __gr
     if (*abort_flag) {
         if (tid == 0) atomicExch(status, (int)DARKATTN_ERR_CUDA);
     } else if (warp == kEpiWarps) {                     // ---- loads
-        if ((tid & 31) == 0) {
+        {
             bool ok = true;
             int it = 0;
             for (int pc = 0; ok && list.next(p, c); ++pc) {
                 const int bh = c.bh, slab = c.slab, h = bh % p.H, rowk0 = kv_row0(bh, p.H, p.Hkv, p.N);
                 const float *nK = p.nK + (size_t)bh * p.N;
-                if (pc > 0) ok = wait_or_abort(bars + YB_OMF, (pc - 1) & 1, status, abort_flag);      // the piece before is projected
+                if (pc > 0) ok = warp_wait(bars + YB_OMF, (pc - 1) & 1, status, abort_flag);      // the piece before is projected
                 if (!ok) break;
-                mbar_expect_tx(bars + YB_OM, 2 * kXT);
-                for (int a = 0; a < D / 64; ++a) {
-                    tma_load_2d(sOm + a * 16384, &p.mapOm, bars + YB_OM, a * 64, h * p.m + slab * 128);
-                    tma_load_2d(sOml + a * 16384, &p.mapOml, bars + YB_OM, a * 64, h * p.m + slab * 128);
-                }
+                if (elect_one()) mbar_expect_tx(bars + YB_OM, 2 * kXT);
+                if (elect_one())
+                    for (int a = 0; a < D / 64; ++a) {
+                        tma_load_2d(sOm + a * 16384, &p.mapOm, bars + YB_OM, a * 64, h * p.m + slab * 128);
+                        tma_load_2d(sOml + a * 16384, &p.mapOml, bars + YB_OM, a * 64, h * p.m + slab * 128);
+                    }
                 for (int t = c.t0; t < c.t1; ++t, ++it) {
                     const int b = it % NST, y = rowk0 + t * 128;
-                    if (it >= NST) ok = wait_or_abort(bars + YB_KF + b, (it / NST - 1) & 1, status, abort_flag);
+                    if (it >= NST) ok = warp_wait(bars + YB_KF + b, (it / NST - 1) & 1, status, abort_flag);
                     if (!ok) break;
-                    mbar_expect_tx(bars + YB_K + b, kXT);
-                    for (int a = 0; a < D / 64; ++a) tma_load_2d(sK + b * kXT + a * 16384, &p.mapK, bars + YB_K + b, a * 64, y);
-                    // Here tile it - NST is projected, so its region's tile before, it - NST - 3, has been read out, and with it
-                    // all tiles before, tile it - 8 (the last user of this slot of norms) among them.
-                    static_assert(NST + 3 <= NN, "a slot of norms would be loaded over");
-                    mbar_expect_tx(bars + YB_N + it % NN, 512);
-                    bulk_load(sNorm + (it % NN) * 128, nK + (size_t)t * 128, 512, bars + YB_N + it % NN);
-                    if (NST == 2 && t + 2 < c.t1)        // with a short ring the next loads come out of L2
-                        for (int a = 0; a < D / 64; ++a) tma_prefetch_l2_2d(&p.mapK, a * 64, y + 256);
+                    if (elect_one()) {
+                        mbar_expect_tx(bars + YB_K + b, kXT);
+                        for (int a = 0; a < D / 64; ++a) tma_load_2d(sK + b * kXT + a * 16384, &p.mapK, bars + YB_K + b, a * 64, y);
+                        // Here tile it - NST is projected, so its region's tile before, it - NST - 3, has been read out, and with it
+                        // all tiles before, tile it - 8 (the last user of this slot of norms) among them.
+                        static_assert(NST + 3 <= NN, "a slot of norms would be loaded over");
+                        mbar_expect_tx(bars + YB_N + it % NN, 512);
+                        bulk_load(sNorm + (it % NN) * 128, nK + (size_t)t * 128, 512, bars + YB_N + it % NN);
+                        if (NST == 2 && t + 2 < c.t1)        // with a short ring the next loads come out of L2
+                            for (int a = 0; a < D / 64; ++a) tma_prefetch_l2_2d(&p.mapK, a * 64, y + 256);
+                    }
                 }
             }
         }
     } else if (warp == kEpiWarps + 2) {                 // ---- loads of V, whose tiles are held two steps longer than those of K
-        if ((tid & 31) == 0) {
+        {
             bool ok = true;
             int it = 0;
             while (ok && list.next(p, c)) {
                 const int rowk0 = kv_row0(c.bh, p.H, p.Hkv, p.N);
                 for (int t = c.t0; t < c.t1; ++t, ++it) {
                     const int b = it % NST, y = rowk0 + t * 128;
-                    if (it >= NST) ok = wait_or_abort(bars + YB_VF + b, (it / NST - 1) & 1, status, abort_flag);
+                    if (it >= NST) ok = warp_wait(bars + YB_VF + b, (it / NST - 1) & 1, status, abort_flag);
                     if (!ok) break;
-                    mbar_expect_tx(bars + YB_V + b, kVT);
-                    for (int a = 0; a < DV / 64; ++a) tma_load_2d(sV + b * kVT + a * 16384, &p.mapV, bars + YB_V + b, a * 64, y);
-                    if (NST == 2 && t + 2 < c.t1)
-                        for (int a = 0; a < DV / 64; ++a) tma_prefetch_l2_2d(&p.mapV, a * 64, y + 256);
+                    if (elect_one()) {
+                        mbar_expect_tx(bars + YB_V + b, kVT);
+                        for (int a = 0; a < DV / 64; ++a) tma_load_2d(sV + b * kVT + a * 16384, &p.mapV, bars + YB_V + b, a * 64, y);
+                        if (NST == 2 && t + 2 < c.t1)
+                            for (int a = 0; a < DV / 64; ++a) tma_prefetch_l2_2d(&p.mapV, a * 64, y + 256);
+                    }
                 }
             }
         }
     } else if (warp == kEpiWarps + 1) {                 // ---- MMAs: U^T of tile it into region it % 3
-        if ((tid & 31) == 0) {
+        {
             const TileDesc tOm(sOm), tOml(sOml);
             const uint32_t id_u = make_idesc(128, 128, 0, 0);
             bool ok = true;
             int it = 0;
             for (int pc = 0; ok && list.next(p, c); ++pc) {
-                ok = wait_or_abort(bars + YB_OM, pc & 1, status, abort_flag);
+                ok = warp_wait(bars + YB_OM, pc & 1, status, abort_flag);
                 for (int t = c.t0; t < c.t1; ++t, ++it) {
                     const int b = it % NST, q = it % 3;
-                    ok = ok && wait_or_abort(bars + YB_K + b, (it / NST) & 1, status, abort_flag);
-                    if (ok && it >= 3) ok = wait_or_abort(bars + YB_SD + q, (it / 3 - 1) & 1, status, abort_flag);      // the region's last reader is done
+                    ok = ok && warp_wait(bars + YB_K + b, (it / NST) & 1, status, abort_flag);
+                    if (ok && it >= 3) ok = warp_wait(bars + YB_SD + q, (it / 3 - 1) & 1, status, abort_flag);      // the region's last reader is done
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t dst = tmem + 128 + 128 * q;
                     const TileDesc tK(sK + b * kXT);
-                    _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(dst, kdesc(tOm, k), kdesc(tK, k), id_u, k > 0);
-                    _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(dst, kdesc(tOml, k), kdesc(tK, k), id_u, 1);
-                    mma_commit(bars + YB_U + q);
-                    mma_commit(bars + YB_KF + b);
-                    if (t + 1 == c.t1) mma_commit(bars + YB_OMF);
+                    if (elect_one()) {
+                        _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(dst, kdesc(tOm, k), kdesc(tK, k), id_u, k > 0);
+                        _Pragma("unroll") for (int k = 0; k < D / 16; ++k) mma_ss(dst, kdesc(tOml, k), kdesc(tK, k), id_u, 1);
+                        mma_commit(bars + YB_U + q);
+                        mma_commit(bars + YB_KF + b);
+                        if (t + 1 == c.t1) mma_commit(bars + YB_OMF);
+                    }
                 }
             }
         }
     } else if (warp == kEpiWarps + 3) {                 // ---- MMAs: S += phi(K)^T V
-        if ((tid & 31) == 0) {
+        {
             const uint32_t id_s = make_idesc(128, DV, 0, 1);
             bool ok = true;
             int it = 0;
             for (int pc = 0; ok && list.next(p, c); ++pc) {
-                if (pc > 0) ok = wait_or_abort(bars + YB_SR, (pc - 1) & 1, status, abort_flag);      // the state before has been read out
+                if (pc > 0) ok = warp_wait(bars + YB_SR, (pc - 1) & 1, status, abort_flag);      // the state before has been read out
                 for (int t = c.t0; t < c.t1; ++t, ++it) {
                     const int b = it % NST, q = it % 3;
-                    ok = ok && wait_or_abort(bars + YB_V + b, (it / NST) & 1, status, abort_flag);
-                    ok = ok && wait_or_abort(bars + YB_E + q, (it / 3) & 1, status, abort_flag);
+                    ok = ok && warp_wait(bars + YB_V + b, (it / NST) & 1, status, abort_flag);
+                    ok = ok && warp_wait(bars + YB_E + q, (it / 3) & 1, status, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t src = tmem + 128 + 128 * q;
                     const TileDesc tV(sV + b * kVT);
-                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(tmem, src + (k / 2) * 32 + (k % 2) * 8, mndesc(tV, k), id_s, t > c.t0 || k > 0);
-                    mma_commit(bars + YB_SD + q);
-                    mma_commit(bars + YB_VF + b);
+                    if (elect_one()) {
+                        _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(tmem, src + (k / 2) * 32 + (k % 2) * 8, mndesc(tV, k), id_s, t > c.t0 || k > 0);
+                        mma_commit(bars + YB_SD + q);
+                        mma_commit(bars + YB_VF + b);
+                    }
                 }
-                if (ok) mma_commit(bars + YB_S);
+                if (ok && elect_one()) mma_commit(bars + YB_S);
             }
         }
     } else {                                            // ---- read-out
@@ -1121,7 +1158,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) tc_fwd_queries_kernel(const _
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L::kBars);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + UNBARS);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + UNBARS + 1);
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5);
 
     if (tid == 0) {
         for (int i = 0; i < UB_E; ++i) mbar_init(bars + i, 1);
@@ -1134,7 +1171,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) tc_fwd_queries_kernel(const _
     __syncthreads();
     tc_fence_after();
     pdl_wait_tma();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = uniform(*tmem_slot);
     int *status = p.status;
     PieceList list(p);
     Piece c;
@@ -1146,68 +1183,77 @@ __global__ void __launch_bounds__(kPassThreads, 1) tc_fwd_queries_kernel(const _
     if (*abort_flag) {
         if (tid == 0) atomicExch(status, (int)DARKATTN_ERR_CUDA);
     } else if (warp == kEpiWarps) {                     // ---- loads
-        if ((tid & 31) == 0) {
+        {
             bool ok = true;
             int it = 0;
             for (int pc = 0; ok && list.next(p, c); ++pc) {
                 const int bh = c.bh, slab = c.slab, h = bh % p.H;
-                if (pc > 0) ok = wait_or_abort(bars + UB_OMF, (pc - 1) & 1, status, abort_flag);     // the piece before is done with its operands
+                if (pc > 0) ok = warp_wait(bars + UB_OMF, (pc - 1) & 1, status, abort_flag);     // the piece before is done with its operands
                 if (!ok) break;
-                mbar_expect_tx(bars + UB_OM, 2 * kXT + 128 * DV * 2 + 512);
-                for (int a = 0; a < D / 64; ++a) {
-                    tma_load_2d(sOm + a * 16384, &p.mapOm, bars + UB_OM, a * 64, h * p.m + slab * 128);
-                    tma_load_2d(sOml + a * 16384, &p.mapOml, bars + UB_OM, a * 64, h * p.m + slab * 128);
+                if (elect_one()) mbar_expect_tx(bars + UB_OM, 2 * kXT + 128 * DV * 2 + 512);
+                if (elect_one())
+                    for (int a = 0; a < D / 64; ++a) {
+                        tma_load_2d(sOm + a * 16384, &p.mapOm, bars + UB_OM, a * 64, h * p.m + slab * 128);
+                        tma_load_2d(sOml + a * 16384, &p.mapOml, bars + UB_OM, a * 64, h * p.m + slab * 128);
+                    }
+                if (elect_one()) {
+                    for (int a = 0; a < DV / 64; ++a) tma_load_2d(sSb + a * 16384, &p.mapSb, bars + UB_OM, a * 64, bh * p.m + slab * 128);
+                    bulk_load(smem + L::kZ, p.zq + (size_t)bh * p.m + slab * 128, 512, bars + UB_OM);
                 }
-                for (int a = 0; a < DV / 64; ++a) tma_load_2d(sSb + a * 16384, &p.mapSb, bars + UB_OM, a * 64, bh * p.m + slab * 128);
-                bulk_load(smem + L::kZ, p.zq + (size_t)bh * p.m + slab * 128, 512, bars + UB_OM);
                 for (int t = c.t0; t < c.t1; ++t, ++it) {
                     const int b = it % NST, y = bh * p.N + t * 128;
-                    if (it >= NST) ok = wait_or_abort(bars + UB_QF + b, (it / NST - 1) & 1, status, abort_flag);
+                    if (it >= NST) ok = warp_wait(bars + UB_QF + b, (it / NST - 1) & 1, status, abort_flag);
                     if (!ok) break;
-                    mbar_expect_tx(bars + UB_Q + b, kXT);
-                    for (int a = 0; a < D / 64; ++a) tma_load_2d(sQ + b * kXT + a * 16384, &p.mapQ, bars + UB_Q + b, a * 64, y);
-                    if (NST == 2 && t + 2 < c.t1)
-                        for (int a = 0; a < D / 64; ++a) tma_prefetch_l2_2d(&p.mapQ, a * 64, y + 256);
+                    if (elect_one()) {
+                        mbar_expect_tx(bars + UB_Q + b, kXT);
+                        for (int a = 0; a < D / 64; ++a) tma_load_2d(sQ + b * kXT + a * 16384, &p.mapQ, bars + UB_Q + b, a * 64, y);
+                        if (NST == 2 && t + 2 < c.t1)
+                            for (int a = 0; a < D / 64; ++a) tma_prefetch_l2_2d(&p.mapQ, a * 64, y + 256);
+                    }
                 }
             }
         }
     } else if (warp == kEpiWarps + 1) {                 // ---- MMAs: U of a tile
-        if ((tid & 31) == 0) {
+        {
             const TileDesc tOm(sOm), tOml(sOml);
             const uint32_t id_u = make_idesc(128, 128, 0, 0);
             bool ok = true;
             int it = 0;
             for (int pc = 0; ok && list.next(p, c); ++pc) {
-                ok = wait_or_abort(bars + UB_OM, pc & 1, status, abort_flag);
+                ok = warp_wait(bars + UB_OM, pc & 1, status, abort_flag);
                 for (int t = c.t0; t < c.t1; ++t, ++it) {
                     const int b = it % NST;
-                    ok = ok && wait_or_abort(bars + UB_Q + b, (it / NST) & 1, status, abort_flag);
-                    if (ok && it >= G) ok = wait_or_abort(bars + UB_R + it % G, (it / G - 1) & 1, status, abort_flag);      // the group's last output has been read
+                    ok = ok && warp_wait(bars + UB_Q + b, (it / NST) & 1, status, abort_flag);
+                    if (ok && it >= G) ok = warp_wait(bars + UB_R + it % G, (it / G - 1) & 1, status, abort_flag);      // the group's last output has been read
                     if (!ok) break;
                     tc_fence_after();
                     const TileDesc tQ(sQ + b * kXT);
-                    issue_projection<D>(tmem + col_u(it), tQ, tOm, tOml, id_u);
-                    mma_commit(bars + UB_U + it % G);
-                    mma_commit(bars + UB_QF + b);
+                    if (elect_one()) {
+                        issue_projection<D>(tmem + col_u(it), tQ, tOm, tOml, id_u);
+                        mma_commit(bars + UB_U + it % G);
+                        mma_commit(bars + UB_QF + b);
+                    }
                 }
             }
         }
     } else if (warp == kEpiWarps + 2) {                 // ---- MMAs: O = phi(Q) S
-        if ((tid & 31) == 0) {
+        {
             const TileDesc tSb(sSb);
             const uint32_t id_o = make_idesc(128, DV, 0, 1);
             bool ok = true;
             int it = 0;
             for (int pc = 0; ok && list.next(p, c); ++pc) {
-                ok = wait_or_abort(bars + UB_OM, pc & 1, status, abort_flag);
+                ok = warp_wait(bars + UB_OM, pc & 1, status, abort_flag);
                 for (int t = c.t0; t < c.t1; ++t, ++it) {
-                    ok = ok && wait_or_abort(bars + UB_E + it % G, (it / G) & 1, status, abort_flag);
+                    ok = ok && warp_wait(bars + UB_E + it % G, (it / G) & 1, status, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(tmem + col_o(it), tmem + col_f(it) + 8 * k, mndesc(tSb, k), id_o, k > 0);
-                    mma_commit(bars + UB_O + it % G);
+                    if (elect_one()) {
+                        _Pragma("unroll") for (int k = 0; k < 8; ++k) mma_ts(tmem + col_o(it), tmem + col_f(it) + 8 * k, mndesc(tSb, k), id_o, k > 0);
+                        mma_commit(bars + UB_O + it % G);
+                    }
                 }
-                if (ok) mma_commit(bars + UB_OMF);
+                if (ok && elect_one()) mma_commit(bars + UB_OMF);
             }
         }
     } else if (warp < 4 * G) {                          // ---- read-out
@@ -1519,7 +1565,7 @@ void tensor_make_layout(darkattn_plan_s *plan)
     Y.sv = take(off, BH * N * 8);
     Y.zc = take(off, D.causal ? BH * (size_t)Y.T * m * 4 : 0);
     // The causal scan may leave SMs idle, which can add up the slabs meanwhile: 47 GB/s of rows read and written per SM, against
-    // 4.4 us (d 64) or 5.2 us (d 128) for a chunk of the scan; of every segment as many chunks as they manage in that time, and not
+    // 3.6 us (d 64) or 4.2 us (d 128) for a chunk of the scan; of every segment as many chunks as they manage in that time, and not
     // many more CTAs than it takes (4 x 16 heads, 8192 tokens, d 128, no stash, one call's kernels alone: 465, 441, 430, 440 us
     // with 0.53, 0.86, 1.0, 1.15 of that rate). Forward calls in a row, without -> with these sums: 504 -> 454 us at that
     // shape, 146 -> 132 (2048 tokens), 818 -> 745 (8 heads, 65536 tokens, d 64, m 512), 193 -> 183 (48 heads, 4096 tokens, d 64); with a
@@ -1529,7 +1575,7 @@ void tensor_make_layout(darkattn_plan_s *plan)
     const long long scan_ctas = units * nsplit, idle = 148 - scan_ctas;
     Y.summers = Y.cut = 0;
     if (D.causal && Y.T / nsplit >= 8 && idle > 0) {
-        const double part = idle * 47e3 * (d == 64 ? 4.4 : 5.2) / ((double)BH * nsplit * (Y.nslab + 1) * 256.0 * dv);
+        const double part = idle * 47e3 * (d == 64 ? 3.6 : 4.2) / ((double)BH * nsplit * (Y.nslab + 1) * 256.0 * dv);
         if (part >= 1.0) { Y.cut = (Y.T + nsplit - 1) / nsplit; Y.summers = (int)(part > 1.6 ? idle * 1.6 / part : idle); if (Y.summers < 1) Y.summers = 1; }
         else if (part >= 0.2) { Y.cut = (int)(part * (Y.T / nsplit)); Y.summers = (int)idle; }
     }
