@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
     uint64_t *accfull = empty + kMaxStages, *accfree = accfull + 2, *dotfull = accfree + 2, *dotfree = dotfull + 2;     // two of each
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(dotfree + 2);
     float *sDot = reinterpret_cast<float *>(smem + kDot), *sWt = reinterpret_cast<float *>(smem + kWt);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
     const int stages = min(kMaxStages, kRing / L.stage_planes), stage_bytes = L.stage_planes * kPlane;
 
     ProbBody *body = reinterpret_cast<ProbBody *>(smem + kBody);
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = uniform(*tmem_slot);
     // (the reads of the parameters, none of which is in a cache yet, and the first tile's place run under the kernel before)
     Tile t;
     decode(L, body, blockIdx.x, t);
@@ -373,6 +373,7 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
     // ok: false once a wait gave up: later waits are skipped, the loops run dry (the status word says so)
     bool ok = true;
     auto wait = [&](uint64_t *bar, uint32_t parity) { ok = ok && mbar_wait(bar, parity & 1, L.status); };
+    auto warp_wait = [&](uint64_t *bar, uint32_t parity) { wait(bar, parity); ok = __all_sync(0xffffffffu, ok); };       // one answer for the warp
     uint32_t st = 0, sph = 0;       // slot and parity of the next stage
     auto next_stage = [&]() { if (++st == (uint32_t)stages) { st = 0; sph ^= 1; } };
 
@@ -403,41 +404,48 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
         }
     } else if (warp == kMmaWarp) {
         // ---------------------------------------------------------------- multiply
-        if (lane == 0) {
-            uint32_t unit = 0;
-            for (uint32_t w = blockIdx.x; w < L.total; w += gridDim.x, decode(L, body, w, t)) {
-                const ProbBody &P = body[t.pb];
-                const int nw = (min(t.Nlim - t.n0, 128) + 15) & ~15;                    // columns of this tile, in the MMA's granularity
-                for (int i = 0; i < t.total && ok; ++unit) {
-                    const uint32_t big = tmem + (unit & 1) * 256, sml = big + 128;
-                    wait(accfree + (unit & 1), (unit >> 1) ^ 1);
-                    bool small = false;
-                    for (int c = 0; c < P.chain && i < t.total && ok; ++c, ++i) {
-                        const int s = i >= t.n0st;
-                        const Opnd &a = P.op[2 * s], &b = P.op[2 * s + 1];
-                        const uint32_t base = smem_u32(smem) + st * stage_bytes, baseB = base + a.planes * kPlane;
-                        const uint32_t idesc = make_idesc(128, nw, a.mn, b.mn);
-                        const uint64_t dA = a.mn ? make_sdesc(base, a.planes * 8192, 1024) : make_sdesc(base, 16, 1024);
-                        const uint64_t dB = b.mn ? make_sdesc(baseB, b.planes * 8192, 1024) : make_sdesc(baseB, 16, 1024);
-                        const uint64_t kA = (a.mn ? 2048 : 32) >> 4, kB = (b.mn ? 2048 : 32) >> 4, pA = (a.mn ? 8192 : kPlane) >> 4, pB = (b.mn ? 8192 : kPlane) >> 4;
-                        wait(full + st, sph);
-                        if (!ok) break;
-                        tc_fence_after();
-                        for (int x = 0; x < a.planes; ++x)
-                            for (int y = 0; y < b.planes && x + y < 3; ++y) {
+        uint32_t unit = 0;
+        for (uint32_t w = blockIdx.x; w < L.total; w += gridDim.x, decode(L, body, w, t)) {
+            const ProbBody &P = body[t.pb];
+            const int nw = uniform((min(t.Nlim - t.n0, 128) + 15) & ~15);               // columns of this tile, in the MMA's granularity
+            const int total = uniform(t.total), n0st = uniform(t.n0st), chain = uniform(P.chain);
+            const uint32_t planesA0 = uniform(P.op[0].planes), planesB0 = uniform(P.op[1].planes), mnA0 = uniform(P.op[0].mn), mnB0 = uniform(P.op[1].mn);
+            const uint32_t planesA1 = uniform(P.op[2].planes), planesB1 = uniform(P.op[3].planes), mnA1 = uniform(P.op[2].mn), mnB1 = uniform(P.op[3].mn);
+            for (int i = 0; i < total && ok; ++unit) {
+                const uint32_t big = tmem + (unit & 1) * 256, sml = big + 128;
+                warp_wait(accfree + (unit & 1), (unit >> 1) ^ 1);
+                bool small = false;
+                for (int c = 0; c < chain && i < total && ok; ++c, ++i) {
+                    const bool s = i >= n0st;
+                    const uint32_t planesA = s ? planesA1 : planesA0, planesB = s ? planesB1 : planesB0, mnA = s ? mnA1 : mnA0, mnB = s ? mnB1 : mnB0;
+                    const uint32_t base = smem_u32(smem) + st * stage_bytes, baseB = base + planesA * kPlane;
+                    const uint32_t idesc = make_idesc(128, nw, mnA, mnB);
+                    const uint64_t dA = mnA ? make_sdesc(base, planesA * 8192, 1024) : make_sdesc(base, 16, 1024);
+                    const uint64_t dB = mnB ? make_sdesc(baseB, planesB * 8192, 1024) : make_sdesc(baseB, 16, 1024);
+                    const uint32_t kA = (mnA ? 2048 : 32) >> 4, kB = (mnB ? 2048 : 32) >> 4, pA = (mnA ? 8192 : kPlane) >> 4, pB = (mnB ? 8192 : kPlane) >> 4;
+                    warp_wait(full + st, sph);
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        bool acc = small;
+#pragma unroll 1
+                        for (uint32_t x = 0; x < planesA; ++x)
+#pragma unroll 1
+                            for (uint32_t y = 0; y < planesB && x + y < 3; ++y) {
                                 const uint32_t d = x + y ? sml : big;
                                 const uint64_t a0 = dA + x * pA, b0 = dB + y * pB;
-                                mma_ss(d, a0, b0, idesc, x + y ? small : c > 0);
+                                mma_ss(d, a0, b0, idesc, x + y ? acc : c > 0);
                                 mma_ss(d, a0 + kA, b0 + kB, idesc, 1);
                                 mma_ss(d, a0 + 2 * kA, b0 + 2 * kB, idesc, 1);
                                 mma_ss(d, a0 + 3 * kA, b0 + 3 * kB, idesc, 1);
-                                small |= x + y > 0;
+                                acc |= x + y > 0;
                             }
                         mma_commit(empty + st);
-                        next_stage();
                     }
-                    if (ok) mma_commit(accfull + (unit & 1));
+                    small |= planesA + planesB > 2;
+                    next_stage();
                 }
+                if (ok && elect_one()) mma_commit(accfull + (unit & 1));
             }
         }
     } else if (warp >= kDotWarp) {
