@@ -15,6 +15,7 @@
 // 14.3 -> 8.3 us, 1024 pairs (134 MB of state) 90.7 -> 62 us, 4.3 TB/s; there the features' arithmetic, 27 thousand warp
 // instructions a pair, is what keeps it from the copy bandwidth.
 #include "common.cuh"
+#include "tc_common.cuh"
 
 #include <math.h>
 
@@ -102,20 +103,20 @@ __device__ __forceinline__ void rows_dots(const T *mat, int nrows, int n, const 
 #pragma unroll
             for (int k = 0; k < RB; ++k) {
                 if (r0 + k * kGroups >= nrows) break;
-                float d0 = 0.f, d1 = 0.f, nn = 0.f;
+                float d0 = 0.f, d1 = 0.f, nn = 0.f, e0 = 0.f, e1 = 0.f, en = 0.f;      // sums over even and odd elements, two to an instruction
 #pragma unroll
                 for (int i = 0; i < PIECES; ++i) {
                     float w[V];
                     unpack16<T>(raw[k][i], w);
 #pragma unroll
-                    for (int j = 0; j < V; ++j) {
-                        d0 = fmaf(w[j], a[i][j], d0);
-                        d1 = fmaf(w[j], b[i][j], d1);
-                        if (NORM) nn = fmaf(w[j], w[j], nn);
+                    for (int j = 0; j < V; j += 2) {
+                        tc::fma2(d0, e0, w[j], w[j + 1], a[i][j], a[i][j + 1]);
+                        tc::fma2(d1, e1, w[j], w[j + 1], b[i][j], b[i][j + 1]);
+                        if (NORM) tc::fma2(nn, en, w[j], w[j + 1], w[j], w[j + 1]);
                     }
                 }
-                d0 = sum8(d0); d1 = sum8(d1);
-                if (NORM) nn = sum8(nn);
+                d0 = sum8(d0 + e0); d1 = sum8(d1 + e1);
+                if (NORM) nn = sum8(nn + en);
                 const int row = r0 + k * kGroups + grp;
                 if (row < nrows) put(row, d0, d1, nn);
             }
@@ -264,10 +265,13 @@ __global__ void __launch_bounds__(kNT, 3) decode_step_kernel(const __grid_consta
                 const float4 x = src[j * 32], v4 = vv[b];
                 const float2 fg = fkq[row0 + n * step];
                 const float f = fg.x, g = fg.y;
-                const float4 sn = make_float4(fmaf(f, v4.x, x.x), fmaf(f, v4.y, x.y), fmaf(f, v4.z, x.z), fmaf(f, v4.w, x.w));
+                float4 sn = x;
+                tc::fma2(sn.x, sn.y, f, f, v4.x, v4.y);
+                tc::fma2(sn.z, sn.w, f, f, v4.z, v4.w);
                 *reinterpret_cast<float4 *>(Sb + n * rstride + 128 * b) = sn;
                 float4 &nm = num[b];
-                nm.x = fmaf(g, sn.x, nm.x); nm.y = fmaf(g, sn.y, nm.y); nm.z = fmaf(g, sn.z, nm.z); nm.w = fmaf(g, sn.w, nm.w);
+                tc::fma2(nm.x, nm.y, g, g, sn.x, sn.y);
+                tc::fma2(nm.z, nm.w, g, g, sn.z, sn.w);
             }
         }
         if (slot + kSlots < nslots) start_slot(slot + kSlots);
