@@ -53,6 +53,15 @@ struct SimtLayout {
     int nsM, nsW, blkM, blkW;      // token blocks of the dM and dW products, tokens in each
 };
 
+// Offsets (bytes) into `saved` of what the FP32 path's forward pass (products on the tensor cores) leaves for the backward pass.
+struct SimtSaved {
+    size_t fQ, fK;                 // features      planes [BH, N, m]
+    size_t P;                      // masked intra-chunk kernel  planes [BH, nb, 128, 128]   (causal)
+    size_t Sp, zloc;               // state before every chunk, or the sum over all  planes [BH, nb or 1, m, dv], [BH, nb, m4]
+    size_t O, den;                 // output and normaliser, fp32  [BH, N, dv], [BH, N]
+    size_t bytes;
+};
+
 // Offsets (bytes) into the scratch of the FFMA kernels' intermediates, all fp32.
 struct FfmaLayout {
     int C, nc, Npad;               // chunk length, chunks, nc * C  (not causal: one chunk of N)
@@ -176,6 +185,7 @@ struct darkattn_plan_s {
     darkattn::Dims dims;
     int path;                      // resolved DARKATTN_PATH_*
     darkattn::SimtLayout simt, simt_fwd;   // with the backward pass; forward pass alone
+    darkattn::SimtSaved simt_saved;
     darkattn::FfmaLayout ffma;
     bool ffma_fwd, ffma_bwd;       // which kernels an FP32 forward or backward call takes
     darkattn::TensorLayout tensor;
@@ -208,11 +218,11 @@ void timer_mark(const darkattn_plan_s *plan, cudaStream_t st, const char *name);
 // FP32 path (products of split operands on the tensor cores)
 void simt_make_layout(darkattn_plan_s *plan);
 double simt_cost_us(const darkattn_plan_s *plan, bool backward);
-void simt_launches(const darkattn_plan_s *plan, int &fwd, int &bwd);     // kernels of a forward and of a backward call
+void simt_launches(const darkattn_plan_s *plan, bool saved, int &fwd, int &bwd);     // kernels of a forward and of a backward call (with a stash or without)
 darkattn_status_t simt_forward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
-                               const void *M, const void *W, void *O, char *ws, cudaStream_t st);
+                               const void *M, const void *W, void *O, char *saved, char *ws, cudaStream_t st);
 darkattn_status_t simt_backward(const darkattn_plan_s *plan, const void *Q, const void *K, const void *V,
-                                const void *M, const void *W, const void *dO, void *dQ, void *dK,
+                                const void *M, const void *W, const void *dO, const char *saved, void *dQ, void *dK,
                                 void *dV, float *dM, char *ws, cudaStream_t st);
 
 // FP32 kernels without matrix instructions

@@ -104,9 +104,10 @@ darkattn_status_t darkattn_plan(const darkattn_desc_t *desc, darkattn_plan_t *ou
     p->ffma_bwd = ffma_is_faster(p, true);
     const size_t bytes_fwd = p->ffma_fwd ? p->ffma.fwd_bytes : p->simt_fwd.bytes, bytes_bwd = p->ffma_bwd ? p->ffma.total_bytes : p->simt.bytes;
     p->workspace_bytes = bytes_fwd > bytes_bwd ? bytes_fwd : bytes_bwd;
-    p->saved_bytes = 0;
+    // (the FFMA kernels keep nothing: where either pass takes them there is no stash)
+    p->saved_bytes = p->ffma_fwd || p->ffma_bwd ? 0 : p->simt_saved.bytes;
     int fwd, bwd;
-    simt_launches(p, p->launches_fwd, p->launches_bwd);
+    simt_launches(p, p->saved_bytes > 0, p->launches_fwd, p->launches_bwd);
     ffma_launches(p, fwd, bwd);
     if (p->ffma_fwd) p->launches_fwd = fwd;
     if (p->ffma_bwd) p->launches_bwd = bwd;
@@ -133,7 +134,8 @@ darkattn_status_t darkattn_forward(darkattn_plan_t plan, const void *Q, const vo
         rc = tensor_forward(plan, Q, K, V, M, W, O, saved, static_cast<char *>(workspace), st, saved != nullptr);
     } else {
         timer_mark(plan, st, "simt_forward (all kernels)");
-        rc = (plan->ffma_fwd ? ffma_forward : simt_forward)(plan, Q, K, V, M, W, O, static_cast<char *>(workspace), st);
+        char *ws = static_cast<char *>(workspace), *keep = plan->saved_bytes ? static_cast<char *>(saved) : nullptr;
+        rc = plan->ffma_fwd ? ffma_forward(plan, Q, K, V, M, W, O, ws, st) : simt_forward(plan, Q, K, V, M, W, O, keep, ws, st);
     }
     timer_mark(plan, st, nullptr);
     return rc;
@@ -156,7 +158,9 @@ darkattn_status_t darkattn_backward(darkattn_plan_t plan, const void *Q, const v
         rc = tensor_backward(plan, Q, K, V, M, W, O, dO, saved, dQ, dK, dV, dM, static_cast<char *>(workspace), st);
     } else {
         timer_mark(plan, st, "simt_backward (all kernels)");
-        rc = (plan->ffma_bwd ? ffma_backward : simt_backward)(plan, Q, K, V, M, W, dO, dQ, dK, dV, dM, static_cast<char *>(workspace), st);
+        char *ws = static_cast<char *>(workspace);
+        const char *kept = plan->saved_bytes ? static_cast<const char *>(saved) : nullptr;
+        rc = plan->ffma_bwd ? ffma_backward(plan, Q, K, V, M, W, dO, dQ, dK, dV, dM, ws, st) : simt_backward(plan, Q, K, V, M, W, dO, kept, dQ, dK, dV, dM, ws, st);
     }
     timer_mark(plan, st, nullptr);
     return rc;

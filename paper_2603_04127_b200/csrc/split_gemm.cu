@@ -588,6 +588,7 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
             if (P.epi == EPI_DIVIDE || P.epi == EPI_GRAD) {
                 ok = ok && __all_sync(0xffffffffu, mbar_wait(dotfull + (nd & 1), (nd >> 1) & 1, L.status));
                 den = sDot[(nd & 1) * 128 + rl];
+                if (P.den_out && t.tn == 0 && g == 0 && t.m0 + rl < t.Mlim) P.den_out[(long long)t.pair * P.ntok + (long long)t.blk * P.block + t.m0 + rl] = den;
                 mbar_arrive_warp(dotfree + (nd & 1));
                 ++nd;
             }
@@ -624,36 +625,40 @@ __global__ void __launch_bounds__(kNT, 1) split_gemm_kernel(const __grid_constan
                 }
             } else {
                 // rows of any width and alignment: 16 columns at a time through the warp's 2 KB, eight rows of 64 bytes per store
-                const bool bf = P.okind == OUT_BF16;
-                const int es = bf ? 2 : 4;
-                char *out = static_cast<char *>(P.out) + (t.pair * P.os_pair + t.blk * P.os_blk) * es;
-                const long long ldb = (long long)P.old_ * es;
-                const bool vec = ((reinterpret_cast<uintptr_t>(out) | (uintptr_t)ldb) & (4 * es - 1)) == 0;
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    if (c * 16 >= cols) break;
-                    __syncwarp();
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        *reinterpret_cast<float4 *>(mine + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4)) = make_float4(acc[c * 16 + 4 * q], acc[c * 16 + 4 * q + 1], acc[c * 16 + 4 * q + 2], acc[c * 16 + 4 * q + 3]);
-                    __syncwarp();
 #pragma unroll 1
-                    for (int it = 0; it < 4; ++it) {
-                        const int r2 = it * 8 + (lane >> 2), q = lane & 3, orow = t.m0 + q4 * 32 + r2, oc = t.n0 + g * 32 + c * 16 + q * 4, n = t.Nlim - oc;
-                        const float4 x = *reinterpret_cast<const float4 *>(mine + r2 * 64 + ((q ^ ((r2 >> 1) & 3)) << 4));
-                        if (orow >= t.Mlim || n <= 0) continue;
-                        char *d = out + orow * ldb + (long long)oc * es;
-                        if (vec && n >= 4) {
-                            if (bf) *reinterpret_cast<uint2 *>(d) = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
-                            else *reinterpret_cast<float4 *>(d) = x;
-                        } else {
-                            const float xs[4] = {x.x, x.y, x.z, x.w};
+                for (int o = 0; o < 2; ++o) {       // (o = 1: the fp32 copy)
+                    if (o && !P.out2) break;
+                    const bool bf = !o && P.okind == OUT_BF16;
+                    const int es = bf ? 2 : 4;
+                    char *out = (o ? reinterpret_cast<char *>(P.out2) : static_cast<char *>(P.out)) + (t.pair * P.os_pair + t.blk * P.os_blk) * es;
+                    const long long ldb = (long long)P.old_ * es;
+                    const bool vec = ((reinterpret_cast<uintptr_t>(out) | (uintptr_t)ldb) & (4 * es - 1)) == 0;
 #pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                if (j < n) {
-                                    if (bf) reinterpret_cast<__nv_bfloat16 *>(d)[j] = __float2bfloat16_rn(xs[j]);
-                                    else reinterpret_cast<float *>(d)[j] = xs[j];
-                                }
+                    for (int c = 0; c < 2; ++c) {
+                        if (c * 16 >= cols) break;
+                        __syncwarp();
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            *reinterpret_cast<float4 *>(mine + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4)) = make_float4(acc[c * 16 + 4 * q], acc[c * 16 + 4 * q + 1], acc[c * 16 + 4 * q + 2], acc[c * 16 + 4 * q + 3]);
+                        __syncwarp();
+#pragma unroll 1
+                        for (int it = 0; it < 4; ++it) {
+                            const int r2 = it * 8 + (lane >> 2), q = lane & 3, orow = t.m0 + q4 * 32 + r2, oc = t.n0 + g * 32 + c * 16 + q * 4, n = t.Nlim - oc;
+                            const float4 x = *reinterpret_cast<const float4 *>(mine + r2 * 64 + ((q ^ ((r2 >> 1) & 3)) << 4));
+                            if (orow >= t.Mlim || n <= 0) continue;
+                            char *d = out + orow * ldb + (long long)oc * es;
+                            if (vec && n >= 4) {
+                                if (bf) *reinterpret_cast<uint2 *>(d) = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
+                                else *reinterpret_cast<float4 *>(d) = x;
+                            } else {
+                                const float xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                                for (int j = 0; j < 4; ++j)
+                                    if (j < n) {
+                                        if (bf) reinterpret_cast<__nv_bfloat16 *>(d)[j] = __float2bfloat16_rn(xs[j]);
+                                        else reinterpret_cast<float *>(d)[j] = xs[j];
+                                    }
+                            }
                         }
                     }
                 }

@@ -92,6 +92,7 @@ struct ProbBody {
     int okind = OUT_NONE, old_ = 0;
     void *out = nullptr;            // element (row, col) at out + pair * os_pair + block * os_blk + row * old_ + col
     long long os_pair = 0, os_blk = 0, ops = 0;     // ops: from plane to plane
+    float *out2 = nullptr, *den_out = nullptr;      // EPI_DIVIDE (if given): the quotients in fp32 as well, laid out like `out`; the rows' dot products, [pair][token]
     // derived
     int small[2] = {0, 0};          // whether the products have small parts
     unsigned blocks = 0;

@@ -97,7 +97,7 @@ extern "C" darkattn_status_t darkattn_forward_static(darkattn_plan_t plan, const
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     // the array still holds the previous call's data: the first kernel clears the status word and the per-feature maxima,
     // every other region is written by this call before it is read
-    if (mode == ALL_PAIRS) return simt_forward(plan, Q, K, V, M, W, O, scratch, st);
+    if (mode == ALL_PAIRS) return simt_forward(plan, Q, K, V, M, W, O, nullptr, scratch, st);
     if (mode == FFMA) return ffma_forward(plan, Q, K, V, M, W, O, scratch, st);
     // pair by pair (heads are independent of one another)
     darkattn_plan_s one;
@@ -108,7 +108,7 @@ extern "C" darkattn_status_t darkattn_forward_static(darkattn_plan_t plan, const
     for (int bh = 0; bh < D.BH && s == DARKATTN_OK; ++bh) {
         const size_t h = bh % D.H, kv = (size_t)(bh / D.H) * D.Hkv + h / D.G, N = D.N;
         s = simt_forward(&one, at(Q, bh * N * D.d), at(K, kv * N * D.d), at(V, kv * N * D.dv), at(M, h * D.r * D.d),
-                         at(W, D.w_per_head ? h * D.m * D.r : 0), const_cast<void *>(at(O, bh * N * D.dv)), scratch, st);
+                         at(W, D.w_per_head ? h * D.m * D.r : 0), const_cast<void *>(at(O, bh * N * D.dv)), nullptr, scratch, st);
     }
     return s;
 }

@@ -88,6 +88,26 @@ def test_fp32_products_at_tile_edges(binding, i, dtype):
     _compare(got, want, TOL[dtype], f"split{i}")
 
 
+# Backward from the forward pass's stash: the same shapes, one chunk (no states), one and several token blocks without a mask.
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("kw", [SPLIT_EDGES[0], SPLIT_EDGES[1], SPLIT_EDGES[2], SPLIT_EDGES[5], dict(B=1, H=2, N=100, d=64, m=64, dv=64, causal=True),
+                                dict(B=1, H=2, N=700, d=32, m=40, dv=24, causal=False)], ids=str)
+def test_fp32_backward_from_the_stash(binding, kw, dtype):
+    wl = inputs.small(name="stash", wid=430, dtype=dtype, backward=True, **kw)
+    t = inputs.generate(wl)
+    plan = binding.darkattn_plan(wl.B, wl.H, wl.N, wl.d, wl.m, r=wl.r, dv=wl.dv, dtype=binding.F32 if dtype == "f32" else binding.BF16,
+                                 causal=wl.causal, path=binding.PATH_SIMT)
+    assert plan.saved_bytes > 0
+    plan.destroy()
+    want = _oracle(t, wl)
+    want["dW"] = ref.backward(t.Q, t.K, t.V, t.M, t.W, t.dO, causal=wl.causal)[4]
+    got = run_gpu(binding, wl, t, path=binding.PATH_SIMT, use_saved=True, want_dw=True)
+    _compare(got, want, TOL[dtype], "stash")
+    # the same intermediates as without it, but for the order of the sums dO . O: to fp32 rounding, and bf16 results within one of theirs
+    plain = run_gpu(binding, wl, t, path=binding.PATH_SIMT, want_dw=True)
+    _compare(got, plain, 1e-5 if dtype == "f32" else 2.0 ** -7, "stash against none")
+
+
 @pytest.mark.parametrize("m", [128, 200])
 @pytest.mark.parametrize("dtype,N", [("f32", 500), ("bf16", 500), ("bf16", 512)])
 def test_keys_that_are_not_numbers_leave_the_rows_before_them_alone(binding, dtype, N, m):
