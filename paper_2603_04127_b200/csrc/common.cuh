@@ -55,6 +55,7 @@ struct SimtLayout {
 
 // Offsets (bytes) into `saved` of what the FP32 path's forward pass (products on the tensor cores) leaves for the backward pass.
 struct SimtSaved {
+    size_t in[5];                  // Q, K, V, M, W as planes (one plane when bf16), where they cannot be read as they are
     size_t fQ, fK;                 // features      planes [BH, N, m]
     size_t P;                      // masked intra-chunk kernel  planes [BH, nb, 128, 128]   (causal)
     size_t Sp, zloc;               // state before every chunk, or the sum over all  planes [BH, nb or 1, m, dv], [BH, nb, m4]

@@ -155,20 +155,36 @@ __global__ void __launch_bounds__(256) chunk_scan_kernel(const float *S, float *
 }
 
 // out[o, e] = sum of src over `n1` outer and `n2` inner slices: src[(i1 * stride1 + o) * n2 + i2, e]. dM sums over the batch
-// and the token blocks (o = head), dW also over the heads where they share W (o = 0).
+// and the token blocks (o = head), dW also over the heads where they share W (o = 0). SPLIT: eight warps of a block take every eighth slice
+// of the same 32 elements, for few elements and many slices, where a thread for each that adds them up alone is a chain of load latencies
+// (dW of m x r = 128 x 64 from 128 slices: 19 us). From 64 k elements on there are threads enough.
+template <bool SPLIT>
 __global__ void __launch_bounds__(256) reduce_kernel(const float *src, float *out, int n1, long long stride1, int n2, long long E, long long total)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const long long t = blockIdx.x * 256LL + threadIdx.x;
-    if (t >= total) return;
-    const long long o = t / E, e = t % E;
+    __shared__ float part[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, n = n1 * n2;      // (SPLIT)
+    const long long t = SPLIT ? blockIdx.x * 32LL + lane : blockIdx.x * 256LL + threadIdx.x;
     float acc = 0.f;
-    for (int i1 = 0; i1 < n1; ++i1) {
-        const float *p = src + (i1 * stride1 + o) * n2 * E + e;
+    if (t < total) {
+        const long long o = t / E, e = t % E;
+        if constexpr (SPLIT) {
+#pragma unroll 4
+            for (int k = w; k < n; k += 8) acc += src[(((k / n2) * stride1 + o) * n2 + k % n2) * E + e];
+        } else
+            for (int i1 = 0; i1 < n1; ++i1) {
+                const float *p = src + (i1 * stride1 + o) * n2 * E + e;
 #pragma unroll 8
-        for (int i2 = 0; i2 < n2; ++i2) acc += p[i2 * E];
+                for (int i2 = 0; i2 < n2; ++i2) acc += p[i2 * E];
+            }
     }
-    out[t] = acc;
+    if constexpr (SPLIT) {
+        part[w][lane] = acc;
+        __syncthreads();
+        if (w) return;
+        acc = ((part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane])) + ((part[4][lane] + part[5][lane]) + (part[6][lane] + part[7][lane]));
+    }
+    if (t < total) out[t] = acc;
 }
 
 // Grouped key/value heads: out[(b,hk), e] = sum_g src[(b, hk G + g), e]: the gradient of a shared key or value row
@@ -306,6 +322,11 @@ struct Runner {
         if (D().dv % 4 == 0) kernel(chunk_scan_kernel<4>, BH * (E / 4 + D().m), (const float *)f(S), f(z), out, Y.nb, D().m, D().dv, ld, m4, BH, mode);
         else kernel(chunk_scan_kernel<1>, BH * (E + D().m), (const float *)f(S), f(z), out, Y.nb, D().m, D().dv, ld, m4, BH, mode);
     }
+    void sum_slices(size_t src, float *out, int n1, long long stride1, int n2, long long E, long long total)
+    {
+        if (total < 65536) kernel(reduce_kernel<true>, 8 * total, (const float *)f(src), out, n1, stride1, n2, E, total);
+        else kernel(reduce_kernel<false>, total, (const float *)f(src), out, n1, stride1, n2, E, total);
+    }
     Mat state_planes(size_t off) const { return planes(off, (long long)D().BH * (D().causal ? Y.nb : 1), D().m, D().dv); }
 };
 
@@ -313,12 +334,13 @@ struct Runner {
 SimtLayout with_saved(const SimtLayout &Y, const SimtSaved &S)
 {
     SimtLayout y = Y;
+    for (int i = 0; i < 5; ++i) y.in[i] = kInSaved | S.in[i];
     y.fQ = kInSaved | S.fQ; y.fK = kInSaved | S.fK; y.P = kInSaved | S.P; y.Sp = kInSaved | S.Sp; y.zloc = kInSaved | S.zloc;
     return y;
 }
 
-// Inputs into parts and x~, the first two launches of either pass.
-void run_projections(Runner &R, const void *Q, const void *K, const void *V, const void *M, const void *W)
+// Inputs into parts (unless they are, in `saved`) and x~, the first two launches of either pass.
+void run_projections(Runner &R, const void *Q, const void *K, const void *V, const void *M, const void *W, bool parts_kept)
 {
     const Dims &D = R.D();
     const SimtLayout &Y = R.Y;
@@ -331,7 +353,7 @@ void run_projections(Runner &R, const void *Q, const void *K, const void *V, con
     SplitJobs J;
     J.n = 0; J.total = 0;
     for (int i = 0; i < 5; ++i)
-        if (Y.conv[i]) {
+        if (Y.conv[i] && !parts_kept) {
             const Mat &x = *in[i];
             J.j[J.n++] = {src[i], x.p, x.w, x.ld, x.w % 8 == 0, x.rows * x.batch, J.total};
             J.total += x.rows * x.batch * (x.ld / 8);
@@ -366,7 +388,7 @@ void run_forward_stages(Runner &R, const void *Q, const void *K, const void *V, 
     const SimtLayout &Y = R.Y;
     const int N = D.N, r = D.r, m = D.m, dv = D.dv, nb = Y.nb, m4 = up4(m);
     const long long BH = D.BH;
-    run_projections(R, Q, K, V, M, W);
+    run_projections(R, Q, K, V, M, W, false);
     const Mat xt[2] = {R.tokens(Y.xtQ, r), R.tokens(Y.xtK, r)}, phi[2] = {R.tokens(Y.fQ, m), R.tokens(Y.fK, m)};
     int *cK = reinterpret_cast<int *>(R.f(Y.cK));
     const sg::TokVec norm = {R.f(Y.nK), BH * N, 4 * tiles(r), 0.5f}, rmax = {R.f(Y.rmax), BH * N, 4 * tiles(m), 1.f};
@@ -461,10 +483,19 @@ void cut_tokens(int N, long long units, int most, int &nblk, int &blk)
     nblk = (N + blk - 1) / blk;
 }
 
+// the inputs Q, K, V, M, W: width of a row, bytes as planes
+int input_width(const Dims &D, int i) { return i == 2 ? D.dv : i == 4 ? D.r : D.d; }
+size_t input_bytes(const Dims &D, int i)
+{
+    const size_t tokens = (size_t)D.N * (i == 0 ? D.BH : D.B * D.Hkv);
+    const size_t rows = i < 3 ? tokens : i == 3 ? (size_t)D.H * D.r : (size_t)(D.w_per_head ? D.H : 1) * D.m;
+    return (D.bf16 ? 1 : 3) * rows * up8(input_width(D, i)) * 2;
+}
+
 SimtLayout make_layout(const Dims &D, bool backward)
 {
     SimtLayout Y = {};
-    const size_t BH = D.BH, N = D.N, m = D.m, dv = D.dv, m4 = up4(D.m), BHkv = (size_t)D.B * D.Hkv;
+    const size_t BH = D.BH, N = D.N, m = D.m, dv = D.dv, m4 = up4(D.m);
     if (D.causal) {
         Y.blk = 128;
         Y.nb = tiles(D.N);
@@ -477,10 +508,8 @@ SimtLayout make_layout(const Dims &D, bool backward)
     size_t off = 0;
     Y.status = take(off, 256);
     Y.cK = take(off, BH * m4 * 4);
-    const int widths[5] = {D.d, D.d, D.dv, D.d, D.r};
-    const size_t rows[5] = {BH * N, BHkv * N, BHkv * N, (size_t)D.H * D.r, (size_t)(D.w_per_head ? D.H : 1) * m};
-    for (int i = 0; i < 5; ++i) Y.conv[i] = !D.bf16 || widths[i] % 8;
-    auto take_in = [&](int i) { if (Y.conv[i]) Y.in[i] = take(off, (D.bf16 ? 1 : 3) * rows[i] * up8(widths[i]) * 2); };
+    for (int i = 0; i < 5; ++i) Y.conv[i] = !D.bf16 || input_width(D, i) % 8;
+    auto take_in = [&](int i) { if (Y.conv[i]) Y.in[i] = take(off, input_bytes(D, i)); };
     take_in(2);
     Y.fQ = take(off, planes(BH * N, D.m)); Y.fK = take(off, planes(BH * N, D.m));
     // What is done with once the features are formed, unless the backward pass needs it again; there the states and kernel
@@ -530,6 +559,7 @@ void simt_make_layout(darkattn_plan_s *plan)
     auto planes = [](size_t rows, int w) { return 3 * rows * up8(w) * 2; };
     const bool states = !D.causal || nb > 1;
     size_t off = 0;
+    for (int i = 0; i < 5; ++i) S.in[i] = Y.conv[i] ? take(off, input_bytes(D, i)) : 0;
     S.fQ = take(off, planes(BH * N, D.m)); S.fK = take(off, planes(BH * N, D.m));
     S.P = take(off, D.causal ? planes(BH * nb * 128, 128) : 0);
     S.Sp = take(off, states ? planes(BH * (D.causal ? nb : 1) * D.m, D.dv) : 0);
@@ -546,7 +576,7 @@ void simt_launches(const darkattn_plan_s *plan, bool saved, int &fwd, int &bwd)
     for (bool c : Y.conv) conv = conv || c;
     const int scan = Y.nb > 1;
     fwd = (conv ? 1 : 0) + 5 + (tiles(D.m) > 1 ? 1 : 0) + scan;
-    bwd = (saved ? (conv ? 1 : 0) + 2 : fwd) + 1 + scan + 4 + (D.G > 1 ? 2 : 0);
+    bwd = (saved ? 2 : fwd) + 1 + scan + 4 + (D.G > 1 ? 2 : 0);
 }
 
 // Estimated time in us of a call that fills the SMs: launches one after the other, then per pair the 128 x 128 tiles of all products
@@ -597,7 +627,7 @@ darkattn_status_t simt_backward(const darkattn_plan_s *plan, const void *Q, cons
     // backward: fp32, 2 x 8 heads of 1000 tokens, d 64, m 128, with dW 240 -> 197 us; bf16, 12 heads of 1500 tokens, d 64, m 256 306 -> 230;
     // 8 heads of 3001 tokens on 4, d 128, m 256 522 -> 398; no mask, fp32, 2 x 8 heads of 1000 tokens 184 -> 150.
     if (saved) {
-        run_projections(R, Q, K, V, M, W);
+        run_projections(R, Q, K, V, M, W, true);
         const Mat ga = R.tokens(Y.Ga, dv);
         const float *O = R.f(kInSaved | plan->simt_saved.O), *den = R.f(kInSaved | plan->simt_saved.den);
         if (D.bf16) R.kernel(grad_rows_kernel<__nv_bfloat16>, BH * N * 32, (const __nv_bfloat16 *)dO, O, den, ga.p, R.f(Y.gd), dv, ga.ld, ga.ps(), BH * N);
@@ -694,7 +724,7 @@ darkattn_status_t simt_backward(const darkattn_plan_s *plan, const void *Q, cons
         R.gemms(L);
     }
     const long long Em = (long long)r * d;
-    R.kernel(reduce_kernel, D.H * Em, (const float *)R.f(Y.dMp), dM, D.B, (long long)D.H, Y.nsM, Em, D.H * Em);
+    R.sum_slices(Y.dMp, dM, D.B, D.H, Y.nsM, Em, D.H * Em);
     if (grouped) {
         const long long BHkv = (long long)D.B * D.Hkv, nv = BHkv * N * dv, nk = BHkv * N * d;
         auto threads = [](long long n) { return n < 148LL * 16 * 256 ? n : 148LL * 16 * 256; };
@@ -726,8 +756,8 @@ darkattn_status_t simt_backward_dw(const darkattn_plan_s *plan, float *dW, char 
     sg::add(L, p);
     R.gemms(L);
     const long long E = (long long)D.m * D.r;
-    if (D.w_per_head) R.kernel(reduce_kernel, D.H * E, (const float *)R.f(Y.dWp), dW, D.B, (long long)D.H, Y.nsW, E, D.H * E);
-    else R.kernel(reduce_kernel, E, (const float *)R.f(Y.dWp), dW, D.BH, 1LL, Y.nsW, E, E);
+    if (D.w_per_head) R.sum_slices(Y.dWp, dW, D.B, D.H, Y.nsW, E, D.H * E);
+    else R.sum_slices(Y.dWp, dW, D.BH, 1, Y.nsW, E, E);
     if (R.err != cudaSuccess) { set_cuda_error(R.err, "simt_backward_dw"); return DARKATTN_ERR_CUDA; }
     return DARKATTN_OK;
 }
