@@ -12,7 +12,7 @@
 // synchronised), and the features are formed while they are on their way. The features of a pair are cut over the CTAs of
 // a cluster: each forms x~, then the exponents of its own features, updates its own rows of the state and sends its partial
 // numerators and normaliser, scaled by its own maximum, to the first CTA. Measured (m = 256, dv = 128, bf16): 64 pairs
-// 14.3 -> 8.3 us, 1024 pairs (134 MB of state) 90.7 -> 62 us, 4.3 TB/s; there the features' arithmetic, 27 thousand warp
+// 14.3 -> 8.1 us, 1024 pairs (134 MB of state) 90.7 -> 63 us, 4.3 TB/s; there the features' arithmetic, 27 thousand warp
 // instructions a pair, is what keeps it from the copy bandwidth.
 #include "common.cuh"
 #include "tc_common.cuh"
@@ -84,6 +84,9 @@ template <typename T, int PIECES, bool NORM, typename Put>
 __device__ __forceinline__ void rows_dots(const T *mat, int nrows, int n, const float *x0, const float *x1, int tid, Put put)
 {
     constexpr int V = 16 / (int)sizeof(T);          // elements per 16-byte load
+    // Two products to an instruction for bf16 (64 pairs, d = dv = 128, m 256: 8.28 -> 8.13 us). Not for fp32, whose 16 bytes hold four
+    // elements: there the two halves of each sum only add registers (8.29 -> 8.89 us).
+    constexpr bool PAIRS = sizeof(T) == 2;
     const int sub = tid & 7, grp = tid >> 3;
     if constexpr (PIECES > 0) {
         constexpr int RB = PIECES == 4 ? 1 : 8 / PIECES;
@@ -110,9 +113,15 @@ __device__ __forceinline__ void rows_dots(const T *mat, int nrows, int n, const 
                     unpack16<T>(raw[k][i], w);
 #pragma unroll
                     for (int j = 0; j < V; j += 2) {
-                        tc::fma2(d0, e0, w[j], w[j + 1], a[i][j], a[i][j + 1]);
-                        tc::fma2(d1, e1, w[j], w[j + 1], b[i][j], b[i][j + 1]);
-                        if (NORM) tc::fma2(nn, en, w[j], w[j + 1], w[j], w[j + 1]);
+                        if constexpr (PAIRS) {
+                            tc::fma2(d0, e0, w[j], w[j + 1], a[i][j], a[i][j + 1]);
+                            tc::fma2(d1, e1, w[j], w[j + 1], b[i][j], b[i][j + 1]);
+                            if (NORM) tc::fma2(nn, en, w[j], w[j + 1], w[j], w[j + 1]);
+                        } else {
+                            d0 = fmaf(w[j + 1], a[i][j + 1], fmaf(w[j], a[i][j], d0));
+                            d1 = fmaf(w[j + 1], b[i][j + 1], fmaf(w[j], b[i][j], d1));
+                            if (NORM) nn = fmaf(w[j + 1], w[j + 1], fmaf(w[j], w[j], nn));
+                        }
                     }
                 }
                 d0 = sum8(d0 + e0); d1 = sum8(d1 + e1);
