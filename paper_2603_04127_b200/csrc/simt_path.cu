@@ -9,7 +9,8 @@
 //              (several tiles of features) | features phi = exp(x~ W^T ...) | chunk states and masked kernel tiles |
 //              prefix over the chunks | output rows
 //   backward   the forward steps with the output rows turned into dO / den and -delta / den | dP and the reverse states |
-//              suffix over the chunks | E of both sides and dV | dx~ | dQ, dK and dM | sums over batch and token blocks
+//              suffix over the chunks | E of both sides and dV | dx~ | dQ, dK and dM | sums over batch and token blocks;
+//              with `saved` of the forward pass only x~ is formed again of its steps, and a launch makes the rows from O and the normaliser
 // Each line's items between bars are one launch each; each starts while the one before drains
 // (programmatic dependent launch). Chunks are 128 tokens, a tile's rows, whatever chunk length the descriptor names (the
 // result does not depend on it).

@@ -58,7 +58,7 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint64_t *bar, uint32_t parity
     return ok;
 }
 // One small loop, not unrolled: with two loops a wait, unrolled by the compiler, the waits were most of the kernels' code (causal
-// scan 285 KB, product kernel of the FP32 path 162 KB; now 119 and 101), more than the instruction caches hold.
+// scan 285 KB, product kernel of the FP32 path 162 KB; now 108 and 88), more than the instruction caches hold.
 // Returns false (after setting *status) if the phase did not complete within kWaitLimitNs, or (abort_flag given) another thread gave up.
 __device__ __forceinline__ bool mbar_wait_limited(uint64_t *bar, uint32_t parity, int *status, volatile int *abort_flag)
 {
