@@ -722,7 +722,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_k_kernel(const __grid_cons
             mbar_arrive_warp(bars + KE5);
 #undef EWAIT
         }
-        ok = ok && wait_or_abort(bars + KM8, (T - 1) & 1, status, abort_flag);
+        ok = ok && warp_wait(bars + KM8, (T - 1) & 1, status, abort_flag);
         if (ok && col0 < D) {
             tc_fence_after();
             float *dst = p.Tacc + ((size_t)h * p.m + slab * 128 + r) * D + col0;
@@ -900,7 +900,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_finish_k_kernel(const __gr
             mbar_arrive_warp(e2);
         }
         if (tid == 0) tma_store_wait_all();
-        if (ok) ok = wait_or_abort(m3, (t1 - 1 - t0) & 1, p.status, abort_flag);
+        ok = ok && warp_wait(m3, (t1 - 1 - t0) & 1, p.status, abort_flag);
         if (ok && q4 * 32 < p.r && col0 < D) {      // whole warps: the tensor-memory load is a warp-wide instruction
             tc_fence_after();
             float *dst = p.dMn + ((size_t)h * p.r + r) * D + col0;

@@ -59,3 +59,14 @@ def test_tma_reads_behind_a_proxy_fence(file, name, body):
     wait = re.search(r"pdl_wait_tma\(\)", body)
     assert wait and wait.start() < re.search(r"tma_load_\w+\(|bulk_load\(", body).start(), f"{file}: {name}"
     assert not re.search(r"pdl_wait\(\)|griddepcontrol", body), f"{file}: {name}"
+
+
+@pytest.mark.parametrize("file,name,body", TENSOR_MEMORY, ids=[k[1] for k in TENSOR_MEMORY])
+def test_a_wait_has_one_answer_before_tensor_memory_is_read(file, name, body):
+    """Tensor-memory loads and stores are instructions of a whole warp: where the lanes of a warp could leave a wait with different
+    answers, half of it would enter one. The warp votes in between."""
+    for wait in re.finditer(r"(?<!__all_sync\(0xffffffffu, )\b(?:wait_or_abort|mbar_wait)\(", body):
+        access = re.search(r"\btmem_(?:ld|st|row_to_tile)\w*\(", body[wait.end():])
+        if access:
+            between = body[wait.end():wait.end() + access.start()]
+            assert "__all_sync(" in between or "warp_wait(" in between, f"{file}: {name}: {body[wait.start():wait.start() + 60]}"
