@@ -100,7 +100,7 @@ size_t darkattn_workspace_bytes(darkattn_plan_t plan);
  * projections, the key-side shifts and the key-side sums: z before every chunk when causal, S and
  * z of the whole sequence otherwise; on the FP32 path the features, the masked kernel tiles, the states, the output in
  * fp32, the normalisers and the parts of fp32 inputs: some 12 m + 4 dv + 800 bytes per token and head, more than on the tensor-core
- * path). 0 means there is none (the FFMA kernels: `saved` is not used then). `saved` may always be NULL in both
+ * path). 0 means there is none (where the FFMA kernels take the backward pass: `saved` is not used then). `saved` may always be NULL in both
  * calls: backward then recomputes what it needs, at the cost of running the forward kernels again. */
 size_t darkattn_saved_bytes(darkattn_plan_t plan);
 

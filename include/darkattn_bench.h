@@ -13,7 +13,7 @@ extern "C" {
 #endif
 
 /* Number of kernel launches one forward (which = 0) or one backward (which = 1) call enqueues
- * (backward: when it is given O and `saved`; otherwise the forward launches come on top), in the
+ * (forward: without `saved`; backward: when it is given O and `saved`; otherwise the forward launches come on top), in the
  * plan's current mode: with per-kernel timing on, the tensor-core backward launches one fewer.   */
 int32_t darkattn_plan_launches(darkattn_plan_t plan, int32_t which);
 

@@ -44,9 +44,10 @@ cudaError_t allow_smem(const void *kernel, int bytes)
 }
 
 // Many short sequences go to the FFMA kernels where their estimate is 5 % lower. 8192 pairs of 8 tokens, d = m = 16, no mask: forward
-// 480 us against 1808 by the products on the tensor cores, training 2214 against 7932; 2048 pairs, d = m = 64: 487 against 494 at 32 tokens,
-// the other way round from 64 on. Fewer pairs than SMs, or more than 256 tokens, are outside what the estimates were
-// fitted to, and the tensor cores were faster wherever it was tried.
+// 481 us against 1575 by the products on the tensor cores, backward 1354 against 2883; 2048 pairs, d = m = 64: forward 407 against 418 at
+// 16 tokens, 486 against 428 at 32. Fewer pairs than SMs, or more than 256 tokens, are outside what the estimates were
+// fitted to, and the tensor cores were faster wherever it was tried. The products have become a fifth faster since the fit, so FFMA is kept
+// somewhat past the line: of 2389 plans in its range 3 % of the forward and 6 % of the backward calls take over 10 % longer by it.
 static bool ffma_is_faster(const darkattn_plan_s *plan, bool backward)
 {
     const Dims &D = plan->dims;
@@ -104,8 +105,10 @@ darkattn_status_t darkattn_plan(const darkattn_desc_t *desc, darkattn_plan_t *ou
     p->ffma_bwd = ffma_is_faster(p, true);
     const size_t bytes_fwd = p->ffma_fwd ? p->ffma.fwd_bytes : p->simt_fwd.bytes, bytes_bwd = p->ffma_bwd ? p->ffma.total_bytes : p->simt.bytes;
     p->workspace_bytes = bytes_fwd > bytes_bwd ? bytes_fwd : bytes_bwd;
-    // (the FFMA kernels keep nothing: where either pass takes them there is no stash)
-    p->saved_bytes = p->ffma_fwd || p->ffma_bwd ? 0 : p->simt_saved.bytes;
+    // The FFMA kernels' backward pass keeps its own intermediates, which backward_dw reads: no stash. Where that pass is the products', a
+    // forward call with a stash takes them too: 240 plans whose forward pass alone is FFMA took 0.68 to 0.84 of their step by it (5th to 95th
+    // percentile), none above 0.87; 4096 pairs of 64 tokens, d 32, m 64, no mask, fp32: 2655 -> 2218 us.
+    p->saved_bytes = p->ffma_bwd ? 0 : p->simt_saved.bytes;
     int fwd, bwd;
     simt_launches(p, p->saved_bytes > 0, p->launches_fwd, p->launches_bwd);
     ffma_launches(p, fwd, bwd);
@@ -135,7 +138,7 @@ darkattn_status_t darkattn_forward(darkattn_plan_t plan, const void *Q, const vo
     } else {
         timer_mark(plan, st, "simt_forward (all kernels)");
         char *ws = static_cast<char *>(workspace), *keep = plan->saved_bytes ? static_cast<char *>(saved) : nullptr;
-        rc = plan->ffma_fwd ? ffma_forward(plan, Q, K, V, M, W, O, ws, st) : simt_forward(plan, Q, K, V, M, W, O, keep, ws, st);
+        rc = plan->ffma_fwd && !keep ? ffma_forward(plan, Q, K, V, M, W, O, ws, st) : simt_forward(plan, Q, K, V, M, W, O, keep, ws, st);
     }
     timer_mark(plan, st, nullptr);
     return rc;

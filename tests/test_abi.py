@@ -58,6 +58,17 @@ def test_plan_rejects_bad_descriptors(binding, kw):
     assert e.value.status == binding.ERR_INVALID_ARG
 
 
+# The FFMA kernels take: the forward pass alone, both passes, neither.
+@pytest.mark.parametrize("kw,ffma_fwd,stash", [(dict(B=75, H=4, N=129, d=16, m=33), True, True), (dict(B=150, H=4, N=40, d=16, m=33, causal=True), True, True),
+                                               (dict(B=256, H=32, N=8, d=16, m=16), True, False), (dict(B=2, H=2, N=64, d=16, m=33), False, True)])
+def test_a_stash_wherever_the_products_take_the_backward_pass(binding, kw, ffma_fwd, stash):
+    args = dict(kw)
+    B, H, N, d, m = (args.pop(k) for k in ("B", "H", "N", "d", "m"))
+    plan = binding.darkattn_plan(B, H, N, d, m, dtype=binding.F32, **args)
+    assert (plan.launches() >= 13) == ffma_fwd and (plan.saved_bytes > 0) == stash        # (the products take 8 launches at most)
+    plan.destroy()
+
+
 def test_tensor_path_refuses_f32(binding):
     with pytest.raises(binding.DarkAttnError) as e:
         binding.darkattn_plan(1, 1, 256, 64, 256, dtype=binding.F32, path=binding.PATH_TENSOR)

@@ -108,6 +108,20 @@ def test_fp32_backward_from_the_stash(binding, kw, dtype):
     _compare(got, plain, 1e-5 if dtype == "f32" else 2.0 ** -7, "stash against none")
 
 
+@pytest.mark.parametrize("kw", [dict(B=75, H=4, N=129, d=16, m=33, causal=False), dict(B=150, H=4, N=40, d=16, m=33, causal=True)], ids=str)
+def test_short_sequences_with_a_stash(binding, kw):
+    """Plans whose forward pass is the FFMA kernels' and whose backward pass is not: with a stash both are the products."""
+    wl = inputs.small(name="shortstash", wid=431, dtype="f32", backward=True, **kw)
+    t = inputs.generate(wl)
+    plan = binding.darkattn_plan(wl.B, wl.H, wl.N, wl.d, wl.m, dtype=binding.F32, causal=wl.causal)
+    assert plan.launches() >= 13 and plan.saved_bytes > 0
+    plan.destroy()
+    want = _oracle(t, wl)
+    want["dW"] = ref.backward(t.Q, t.K, t.V, t.M, t.W, t.dO, causal=wl.causal)[4]
+    for use_saved in (True, False):
+        _compare(run_gpu(binding, wl, t, use_saved=use_saved, want_dw=True), want, TOL["f32"], f"stash={use_saved}")
+
+
 @pytest.mark.parametrize("m", [128, 200])
 @pytest.mark.parametrize("dtype,N", [("f32", 500), ("bf16", 500), ("bf16", 512)])
 def test_keys_that_are_not_numbers_leave_the_rows_before_them_alone(binding, dtype, N, m):
