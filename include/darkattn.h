@@ -95,6 +95,11 @@ darkattn_status_t darkattn_plan(const darkattn_desc_t *desc, darkattn_plan_t *ou
  * the two needs). Contents need not be preserved between calls.                                  */
 size_t darkattn_workspace_bytes(darkattn_plan_t plan);
 
+/* The same for a caller that passes `saved` to every forward and backward call: what the stash holds needs no room in
+ * the workspace then (FP32 path; on the tensor-core path the same number). A call without `saved` needs
+ * darkattn_workspace_bytes.                                                                       */
+size_t darkattn_workspace_bytes_with_saved(darkattn_plan_t plan);
+
 /* Bytes of the forward->backward stash (`saved`): what the forward pass computed and the backward
  * pass needs again (on the tensor-core path the per-row normalisers, the key norms, the folded
  * projections, the key-side shifts and the key-side sums: z before every chunk when causal, S and

@@ -20,7 +20,7 @@ F32, BF16 = 0, 1
 PATH_AUTO, PATH_SIMT, PATH_TENSOR = 0, 1, 2
 
 EXPORTS = [
-    "darkattn_plan", "darkattn_workspace_bytes", "darkattn_saved_bytes", "darkattn_plan_path",
+    "darkattn_plan", "darkattn_workspace_bytes", "darkattn_workspace_bytes_with_saved", "darkattn_saved_bytes", "darkattn_plan_path",
     "darkattn_forward", "darkattn_backward", "darkattn_last_device_status",
     "darkattn_destroy", "darkattn_status_string", "darkattn_last_cuda_error", "darkattn_measure_alu_peak",
     "darkattn_static_scratch_needed", "darkattn_forward_static",
@@ -48,6 +48,8 @@ lib.darkattn_plan.argtypes = [ctypes.POINTER(Desc), ctypes.POINTER(_vp)]
 lib.darkattn_plan.restype = ctypes.c_int
 lib.darkattn_workspace_bytes.argtypes = [_vp]
 lib.darkattn_workspace_bytes.restype = ctypes.c_size_t
+lib.darkattn_workspace_bytes_with_saved.argtypes = [_vp]
+lib.darkattn_workspace_bytes_with_saved.restype = ctypes.c_size_t
 lib.darkattn_saved_bytes.argtypes = [_vp]
 lib.darkattn_saved_bytes.restype = ctypes.c_size_t
 lib.darkattn_plan_path.argtypes = [_vp]
@@ -130,6 +132,10 @@ class Plan:
         return int(lib.darkattn_workspace_bytes(self.handle))
 
     @property
+    def workspace_bytes_with_saved(self) -> int:
+        return int(lib.darkattn_workspace_bytes_with_saved(self.handle))
+
+    @property
     def saved_bytes(self) -> int:
         return int(lib.darkattn_saved_bytes(self.handle))
 
@@ -143,8 +149,10 @@ class Plan:
     def rows_summed(self) -> float:
         return float(benchlib().darkattn_plan_rows_summed(self.handle))
 
-    def alloc_workspace(self, device="cuda") -> torch.Tensor:
-        return torch.empty(max(self.workspace_bytes, 256), dtype=torch.uint8, device=device)
+    def alloc_workspace(self, device="cuda", with_saved=False) -> torch.Tensor:
+        """``with_saved``: for a caller that passes ``saved`` to every forward and backward call."""
+        need = self.workspace_bytes_with_saved if with_saved else self.workspace_bytes
+        return torch.empty(max(need, 256), dtype=torch.uint8, device=device)
 
     def destroy(self):
         if self.handle:

@@ -185,12 +185,13 @@ struct darkattn_plan_s {
     darkattn_desc_t desc;
     darkattn::Dims dims;
     int path;                      // resolved DARKATTN_PATH_*
-    darkattn::SimtLayout simt, simt_fwd;   // with the backward pass; forward pass alone
+    darkattn::SimtLayout simt, simt_fwd;               // with the backward pass; forward pass alone
+    darkattn::SimtLayout simt_stash, simt_fwd_stash;   // the same for calls that are given `saved`
     darkattn::SimtSaved simt_saved;
     darkattn::FfmaLayout ffma;
     bool ffma_fwd, ffma_bwd;       // which kernels an FP32 forward or backward call takes
     darkattn::TensorLayout tensor;
-    size_t workspace_bytes;
+    size_t workspace_bytes, workspace_saved_bytes;     // of any call; of calls that are given `saved`
     size_t saved_bytes;
     int launches_fwd, launches_bwd;
     mutable darkattn::KernelTimer timer;

@@ -109,17 +109,22 @@ darkattn_status_t darkattn_plan(const darkattn_desc_t *desc, darkattn_plan_t *ou
     // forward call with a stash takes them too: 240 plans whose forward pass alone is FFMA took 0.68 to 0.84 of their step by it (5th to 95th
     // percentile), none above 0.87; 4096 pairs of 64 tokens, d 32, m 64, no mask, fp32: 2655 -> 2218 us.
     p->saved_bytes = p->ffma_bwd ? 0 : p->simt_saved.bytes;
+    p->workspace_saved_bytes = !p->saved_bytes ? p->workspace_bytes : p->simt_stash.bytes > p->simt_fwd_stash.bytes ? p->simt_stash.bytes : p->simt_fwd_stash.bytes;
     int fwd, bwd;
     simt_launches(p, p->saved_bytes > 0, p->launches_fwd, p->launches_bwd);
     ffma_launches(p, fwd, bwd);
     if (p->ffma_fwd) p->launches_fwd = fwd;
     if (p->ffma_bwd) p->launches_bwd = bwd;
-    if (path == DARKATTN_PATH_TENSOR) tensor_make_layout(p);
+    if (path == DARKATTN_PATH_TENSOR) {
+        tensor_make_layout(p);
+        p->workspace_saved_bytes = p->workspace_bytes;
+    }
     *out = p;
     return DARKATTN_OK;
 }
 
 size_t darkattn_workspace_bytes(darkattn_plan_t plan) { return plan ? plan->workspace_bytes : 0; }
+size_t darkattn_workspace_bytes_with_saved(darkattn_plan_t plan) { return plan ? plan->workspace_saved_bytes : 0; }
 size_t darkattn_saved_bytes(darkattn_plan_t plan) { return plan ? plan->saved_bytes : 0; }
 int32_t darkattn_plan_path(darkattn_plan_t plan) { return plan ? plan->path : -1; }
 darkattn_status_t darkattn_forward(darkattn_plan_t plan, const void *Q, const void *K, const void *V,

@@ -58,6 +58,17 @@ def test_plan_rejects_bad_descriptors(binding, kw):
     assert e.value.status == binding.ERR_INVALID_ARG
 
 
+def test_a_step_with_a_stash_takes_no_more_memory_than_one_without(binding):
+    """bf16, causal, d = dv = 128, m = 256; without `saved` the workspace is what it was."""
+    for dtype in (binding.BF16, binding.F32):
+        plan = binding.darkattn_plan(2, 16, 2048, 128, 256, dtype=dtype, causal=True, path=binding.PATH_SIMT)
+        assert 0 < plan.workspace_bytes_with_saved and plan.workspace_bytes_with_saved + plan.saved_bytes <= plan.workspace_bytes
+        plan.destroy()
+    plan = binding.darkattn_plan(2, 16, 2048, 128, 256, causal=True)
+    assert plan.path == binding.PATH_TENSOR and plan.workspace_bytes_with_saved == plan.workspace_bytes
+    plan.destroy()
+
+
 # The FFMA kernels take: the forward pass alone, both passes, neither.
 @pytest.mark.parametrize("kw,ffma_fwd,stash", [(dict(B=75, H=4, N=129, d=16, m=33), True, True), (dict(B=150, H=4, N=40, d=16, m=33, causal=True), True, True),
                                                (dict(B=256, H=32, N=8, d=16, m=16), True, False), (dict(B=2, H=2, N=64, d=16, m=33), False, True)])

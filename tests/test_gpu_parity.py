@@ -108,6 +108,19 @@ def test_fp32_backward_from_the_stash(binding, kw, dtype):
     _compare(got, plain, 1e-5 if dtype == "f32" else 2.0 ** -7, "stash against none")
 
 
+# A step in the workspace of calls with a stash, between whose forward and backward call another user of that workspace may run.
+@pytest.mark.parametrize("use_saved", [True, False], ids=["stash", "none"])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("kw", [SPLIT_EDGES[0], SPLIT_EDGES[2], SPLIT_EDGES[5], dict(B=1, H=2, N=100, d=64, m=64, dv=64, causal=True),
+                                dict(B=1, H=2, N=700, d=32, m=40, dv=24, causal=False)], ids=str)
+def test_fp32_step_in_a_workspace_used_by_others(binding, kw, dtype, use_saved):
+    wl = inputs.small(name="wsreuse", wid=432, dtype=dtype, backward=True, **kw)
+    t = inputs.generate(wl)
+    want = _oracle(t, wl)
+    want["dW"] = ref.backward(t.Q, t.K, t.V, t.M, t.W, t.dO, causal=wl.causal)[4]
+    _compare(run_gpu(binding, wl, t, path=binding.PATH_SIMT, use_saved=use_saved, want_dw=True, poison=True), want, TOL[dtype], "wsreuse")
+
+
 @pytest.mark.parametrize("kw", [dict(B=75, H=4, N=129, d=16, m=33, causal=False), dict(B=150, H=4, N=40, d=16, m=33, causal=True)], ids=str)
 def test_short_sequences_with_a_stash(binding, kw):
     """Plans whose forward pass is the FFMA kernels' and whose backward pass is not: with a stash both are the products."""
