@@ -121,6 +121,59 @@ def test_fp32_step_in_a_workspace_used_by_others(binding, kw, dtype, use_saved):
     _compare(run_gpu(binding, wl, t, path=binding.PATH_SIMT, use_saved=use_saved, want_dw=True, poison=True), want, TOL[dtype], "wsreuse")
 
 
+# The same with projections per head, with grouped heads, and on the tensor-core path.
+@pytest.mark.parametrize("use_saved", [True, False], ids=["stash", "none"])
+@pytest.mark.parametrize("case", ["simt_f32_wph", "simt_bf16_wph", "simt_bf16_grouped", "simt_bf16_grouped_nc", "tensor", "tensor_nc", "tensor_grouped"])
+def test_step_in_a_workspace_used_by_others(binding, case, use_saved):
+    dtype, tensor = "f32" if "f32" in case else "bf16", "tensor" in case
+    kw = dict(B=2, H=4, N=384, d=64, m=256) if tensor else dict(B=2, H=4, N=333, d=48, m=140, r=24, dv=40)
+    wl = inputs.small(name="wsreuse2", wid=433, dtype=dtype, backward=True, causal=not case.endswith("_nc"), **kw)
+    t = inputs.generate(wl)
+    if "wph" in case:
+        g = np.random.default_rng(7)
+        t.W = g.standard_normal((wl.H, wl.m, wl.r))
+        if dtype == "bf16":
+            t.W = inputs.round_to_bf16(t.W).astype(np.float64)
+    if "grouped" in case:
+        t.K, t.V = np.ascontiguousarray(t.K[:, ::2]), np.ascontiguousarray(t.V[:, ::2])
+    want = _oracle(t, wl)
+    want["dW"] = ref.backward(t.Q, t.K, t.V, t.M, t.W, t.dO, causal=wl.causal)[4]
+    got = run_gpu(binding, wl, t, path=binding.PATH_TENSOR if tensor else binding.PATH_SIMT, use_saved=use_saved, want_dw=True, poison=True,
+                  w_per_head="wph" in case)
+    _compare(got, want, TOL[dtype], case)
+
+
+@pytest.mark.parametrize("m", [64, 200])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_stash_of_causal_prefixes_far_below_the_largest(binding, dtype, m):
+    """The tiny normalisers of test_causal_prefixes_of_keys_far_below_the_largest, kept in the stash; its bar."""
+    wl = inputs.small(name="prefixes", wid=34, B=1, H=4, N=300, d=64, m=m, causal=True, dtype=dtype, backward=True)
+    t = inputs.generate(wl)
+    t.Q, t.K = t.Q * 5.0, t.K * 5.0
+    if dtype == "bf16":
+        t.Q, t.K = (inputs.round_to_bf16(x).astype(np.float64) for x in (t.Q, t.K))
+    got = run_gpu(binding, wl, t, path=binding.PATH_SIMT, use_saved=True, poison=True)
+    _compare(got, _oracle(t, wl), 5e-4 if dtype == "f32" else TOL[dtype], "prefixes")
+
+
+@pytest.mark.parametrize("value", [np.inf, np.nan])
+@pytest.mark.parametrize("causal", [True, False], ids=["causal", "noncausal"])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_stash_of_a_value_that_is_not_finite(binding, dtype, causal, value):
+    """What it spoils is the same with the stash as without, and the rest agrees: to fp32 rounding, bf16 results within one of theirs."""
+    wl = inputs.small(name="infstash", wid=38, B=1, H=2, N=300, d=64, m=72, causal=causal, dtype=dtype, backward=True)
+    t = inputs.generate(wl)
+    t.V[:, 0, 140, 3] = value
+    kept, plain = (run_gpu(binding, wl, t, path=binding.PATH_SIMT, use_saved=s, want_dw=True) for s in (True, False))
+    for k in plain:
+        fine = np.isfinite(plain[k])
+        assert (np.isfinite(kept[k]) == fine).all(), k
+        assert fine.all() if k == "dV" else not fine.all(), k           # (dV does not depend on V)
+        assert k == "dW" or fine.any(), k                               # (dW sums over both heads)
+        if fine.any():
+            assert_close(kept[k][fine], plain[k][fine], 1e-5 if dtype == "f32" else 2.0 ** -7, k)
+
+
 @pytest.mark.parametrize("kw", [dict(B=75, H=4, N=129, d=16, m=33, causal=False), dict(B=150, H=4, N=40, d=16, m=33, causal=True)], ids=str)
 def test_short_sequences_with_a_stash(binding, kw):
     """Plans whose forward pass is the FFMA kernels' and whose backward pass is not: with a stash both are the products."""
