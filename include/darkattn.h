@@ -103,9 +103,12 @@ size_t darkattn_workspace_bytes_with_saved(darkattn_plan_t plan);
 /* Bytes of the forward->backward stash (`saved`): what the forward pass computed and the backward
  * pass needs again (on the tensor-core path the per-row normalisers, the key norms, the folded
  * projections, the key-side shifts and the key-side sums: z before every chunk when causal, S and
- * z of the whole sequence otherwise; on the FP32 path the features, the masked kernel tiles, the states, the output in
- * fp32, the normalisers and the parts of fp32 inputs: some 12 m + 4 dv + 800 bytes per token and head, more than on the tensor-core
- * path). 0 means there is none (where the FFMA kernels take the backward pass: `saved` is not used then). `saved` may always be NULL in both
+ * z of the whole sequence otherwise; on the FP32 path the features, the masked kernel tiles, the
+ * states, the output in fp32, the normalisers and the parts of fp32 inputs: 12 m + 4 dv bytes per
+ * token and head, with the causal mask 768 + 6 m dv / 128 more, and 6 for every element of fp32
+ * inputs; 5.9 KB (bf16) and 8.2 KB (fp32) at d = dv = 128, m = 256, causal, several times what it is
+ * on the tensor-core path). 0 means there is none (where the FFMA kernels take the backward pass:
+ * `saved` is not used then). `saved` may always be NULL in both
  * calls: backward then recomputes what it needs, at the cost of running the forward kernels again. */
 size_t darkattn_saved_bytes(darkattn_plan_t plan);
 
