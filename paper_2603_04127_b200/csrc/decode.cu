@@ -12,8 +12,10 @@
 // synchronised), and the features are formed while they are on their way. The features of a pair are cut over the CTAs of
 // a cluster: each forms x~, then the exponents of its own features, updates its own rows of the state and sends its partial
 // numerators and normaliser, scaled by its own maximum, to the first CTA. Measured (m = 256, dv = 128, bf16): 64 pairs
-// 14.3 -> 8.1 us, 1024 pairs (134 MB of state) 90.7 -> 63 us, 4.3 TB/s; there the features' arithmetic, 27 thousand warp
-// instructions a pair, is what keeps it from the copy bandwidth.
+// 14.3 -> 8.1 us, 1024 pairs (134 MB of state) 90.7 -> 63 us, 4.3 TB/s. There seven pairs an SM go through three resident blocks, and a block
+// loads the first half of its state, forms features while nothing else of it moves, then streams the rest: not the features' instructions
+// (cut by the paired products below: 62.2 -> 61.6 us) but these phases keep it from the copy bandwidth. With few pairs the loads of M and of W stand
+// behind the barriers that follow q, k and x~, by the order of this program: their addresses depend on neither.
 #include "common.cuh"
 #include "tc_common.cuh"
 
@@ -84,8 +86,9 @@ template <typename T, int PIECES, bool NORM, typename Put>
 __device__ __forceinline__ void rows_dots(const T *mat, int nrows, int n, const float *x0, const float *x1, int tid, Put put)
 {
     constexpr int V = 16 / (int)sizeof(T);          // elements per 16-byte load
-    // Two products to an instruction for bf16 (64 pairs, d = dv = 128, m 256: 8.28 -> 8.13 us). Not for fp32, whose 16 bytes hold four
-    // elements: there the two halves of each sum only add registers (8.29 -> 8.89 us).
+    // Two products to an instruction for bf16: with those of the state update, steps in one graph, d = dv = 128, m 256, five runs a side that differ
+    // by 0.01 us: 1 pair 6.08 -> 5.94 us, 32: 7.17 -> 7.06, 64: 7.79 -> 7.63, 128: 13.7 -> 13.3, 256: 17.9 -> 17.4, 512: 26.9 -> 26.3. Not for
+    // fp32, whose 16 bytes hold four elements: there the two halves of each sum only add registers (8.29 -> 8.89 us).
     constexpr bool PAIRS = sizeof(T) == 2;
     const int sub = tid & 7, grp = tid >> 3;
     if constexpr (PIECES > 0) {

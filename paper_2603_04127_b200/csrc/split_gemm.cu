@@ -21,11 +21,13 @@
 // every second stage (every stage where the exponent's argument is formed) both are added to sums in registers, rounded to
 // nearest, and start from zero again: measured against float64 the path's results are closer than with a chain of fp32 FMAs.
 //
-// What bounds it: with all SMs busy the planes' way through L2, 5 to 6 TB/s in the launches of features and output rows; a launch of
-// few tiles the latencies of one: parameters, loads, MMAs, epilogue, about 5 us. The MMA warp runs converged (tc::elect_one): by a
-// lane of its own the 24 MMAs of a stage of six products took 97 cycles each, whatever their width. All roles' code passes through
-// every SM's instruction cache, so its size counts (162 -> 88 KB: waits, x and the plain output as small loops, the issue), and so do reads of
-// the launch's parameters (kept in shared memory). With all of this 2 x 16 heads of 2001 tokens, d 128, m 256: 380 -> 337 us; training
+// What bounds it: a launch of few tiles the latencies of one: parameters, loads, MMAs, epilogue, about 5 us. With all SMs busy no unit by
+// the counters (2 x 16 heads of 2001 tokens, d 128, m 256, the six launches of a forward call): tensor pipe 5 to 21 % of the time, L2 5 to 8 TB/s in the four
+// long ones, which is 21 to 30 % of its peak, DRAM up to 54 %, an instruction issued in 31 to 45 % of the cycles; the sixteen read-out warps mostly
+// wait for memory, tensor memory and barriers. The MMA warp runs converged (tc::elect_one): by a lane of its own the 24 MMAs of a stage of six
+// products took 97 cycles each, whatever their width. All roles' code passes through every SM's instruction cache, so its size counts (162 -> 136 KB
+// by the waits' small loop, 101 by small loops for x and the plain output, 90 by the issue), and so do reads of the launch's parameters (kept in shared
+// memory). With all of this 2 x 16 heads of 2001 tokens, d 128, m 256: 380 -> 337 us; training
 // step of 2 x 8 heads, 1000 tokens, d 64, fp32: 291 -> 242 us (191 with the stash), mostly by the coalesced loads of x in the backward products.
 #include "split_gemm.cuh"
 #include "tc_common.cuh"

@@ -57,8 +57,9 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint64_t *bar, uint32_t parity
         : "memory");
     return ok;
 }
-// One small loop, not unrolled: with two loops a wait, unrolled by the compiler, the waits were most of the kernels' code (causal
-// scan 285 KB, product kernel of the FP32 path 162 KB; now 108 and 88), more than the instruction caches hold.
+// One small loop, not unrolled: with two loops a wait, unrolled by the compiler, the waits were most of the kernels' code, more than
+// the instruction caches hold. By this loop alone the causal scan went from 285 to 119 KB, the query-side backward kernel from 234 to 83,
+// the product kernel of the FP32 path from 162 to 136.
 // Returns false (after setting *status) if the phase did not complete within kWaitLimitNs, or (abort_flag given) another thread gave up.
 __device__ __forceinline__ bool mbar_wait_limited(uint64_t *bar, uint32_t parity, int *status, volatile int *abort_flag)
 {
@@ -214,9 +215,9 @@ __device__ __forceinline__ uint64_t make_sdesc(uint32_t saddr, uint32_t lbo_byte
 }
 
 // MMAs are issued by one lane. The warp around it runs its code as a whole (all lanes wait at the barriers together) and enters
-// `if (elect_one())` for each batch: then the compiler knows addresses and descriptors to be the same in all lanes and keeps them in
-// uniform registers, where the instruction wants them: one instruction an MMA, where code that a single lane runs by itself took
-// six and more, most of them moves into those registers, and was as long as the MMAs of 64 columns and less.
+// `if (elect_one())` for each batch: so the compiler can see that addresses and descriptors are the same in all lanes. Issued by a lane
+// that ran by itself an MMA of the FP32 path's kernel took 97 cycles (clock64) whatever its width; forward calls of 12 heads of 4096 tokens, d 128,
+// m 512: 131 -> 119 us, training steps of 8 x 12 heads of 2048 tokens, d 64: 588 -> 522.
 // The same lane is elected every time (its TMA stores, commits and waits belong together).
 __device__ __forceinline__ bool elect_one()
 {

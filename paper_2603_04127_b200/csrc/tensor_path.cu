@@ -1566,12 +1566,11 @@ void tensor_make_layout(darkattn_plan_s *plan)
     Y.zc = take(off, D.causal ? BH * (size_t)Y.T * m * 4 : 0);
     // The causal scan may leave SMs idle, which can add up the slabs meanwhile: 47 GB/s of rows read and written per SM, against
     // 3.6 us (d 64) or 4.2 us (d 128) for a chunk of the scan; of every segment as many chunks as they manage in that time, and not
-    // many more CTAs than it takes (4 x 16 heads, 8192 tokens, d 128, no stash, one call's kernels alone: 465, 441, 430, 440 us
-    // with 0.53, 0.86, 1.0, 1.15 of that rate). Forward calls in a row, without -> with these sums: 504 -> 454 us at that
-    // shape, 146 -> 132 (2048 tokens), 818 -> 745 (8 heads, 65536 tokens, d 64, m 512), 193 -> 183 (48 heads, 4096 tokens, d 64); with a
-    // stash, whose stores slow the scan, 559 -> 535, 154 -> 141, 848 -> 784, 202 -> 189. The surplus of 1.6: the same as with all idle
-    // SMs, and with 1.0 the last tiles are waited for (745 -> 833, 183 -> 199). Not for scans of fewer than 8 chunks, nor where they would sum
-    // less than a fifth.
+    // many more CTAs than it takes. 4 x 16 heads, 8192 tokens, d 128, forward calls in a row with 0, 0.5, 0.7, 0.85, 1.0, 1.15, 1.4 of that rate: with a
+    // stash 550, 518, 508, 500, 492, 522, 577 us, without 477, 449, 435, 428, 430, 456, 512. Without -> with these sums, no stash: 131 -> 119
+    // (2048 tokens), 759 -> 683 (8 heads, 65536 tokens, d 64, m 512), 179 -> 163 (48 heads, 4096 tokens, d 64); with a stash 145 -> 133, 812 -> 740,
+    // 189 -> 171. The surplus of 1.6: the same as with all idle SMs (163, 683), and with 1.0 the last tiles are waited for (163 -> 172, with a
+    // stash 171 -> 181). Not for scans of fewer than 8 chunks, nor where they would sum less than a fifth.
     const long long scan_ctas = units * nsplit, idle = 148 - scan_ctas;
     Y.summers = Y.cut = 0;
     if (D.causal && Y.T / nsplit >= 8 && idle > 0) {
